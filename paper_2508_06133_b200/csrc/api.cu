@@ -32,31 +32,19 @@ int kv_cuda_fail(cudaError_t e, const char* what) {
 namespace {
 
 const i64 kSweepChunk = 1ll << 22;          // candidates per launch inside a sweep
-const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory before striding kicks in
+const int kSnapshots = 256;                 // states of the base run kept for the sweeps
+const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
 
-// Runs CALL(SIM) with SIM = the simulator class of the handle: the register-resident one when the
-// longest window fits 33 registers per lane, else the hybrid one (registers + a shared-memory ring
-// for the far rounds); the all-shared-memory one on request (KVSCHED_SIM=smem).
+// Runs CALL(SIM) with SIM = the simulator class of the handle: the chunked one (NM far registers per
+// lane for decodes up to 1,025 / 2,049 / 4,097 / 8,193 rounds), beyond that the hybrid one, whose
+// per-lane state does not grow with the longest decode.
 #define KV_DISPATCH_SIM(h, CALL)                               \
-    if ((h)->hyb) {                                             \
-        CALL(HybSim);                                           \
-    } else if ((h)->nreg > 0) {                                      \
-        switch ((h)->nreg) {                                    \
-            case 2: CALL(RegSim<2>); break;                     \
-            case 3: CALL(RegSim<3>); break;                     \
-            case 5: CALL(RegSim<5>); break;                     \
-            case 9: CALL(RegSim<9>); break;                     \
-            case 17: CALL(RegSim<17>); break;                   \
-            default: CALL(RegSim<33>); break;                   \
-        }                                                       \
-    } else {                                                    \
-        switch ((h)->nit) {                                     \
-            case 1: CALL(SmemSim<1>); break;                    \
-            case 2: CALL(SmemSim<2>); break;                    \
-            case 4: CALL(SmemSim<4>); break;                    \
-            case 8: CALL(SmemSim<8>); break;                    \
-            default: CALL(SmemSim<0>); break;                   \
-        }                                                       \
+    switch ((h)->nm) {                                          \
+        case 1: CALL(ChunkSim<1>); break;                       \
+        case 2: CALL(ChunkSim<2>); break;                       \
+        case 4: CALL(ChunkSim<4>); break;                       \
+        case 8: CALL(ChunkSim<8>); break;                       \
+        default: CALL(HybSim); break;                           \
     }
 
 int bits_of(u64 v) { int b = 0; while (v) { ++b; v >>= 1; } return b; }
@@ -239,15 +227,7 @@ int k3_warps(const sched_ctx* h) {
     return w;
 }
 
-size_t k3_smem_bytes(const sched_ctx* h, bool* table_in_smem, unsigned* table_bytes) {
-    const size_t rings = (size_t)k3_warps(h) * h->ring_cells * sizeof(int);
-    const unsigned tb = (unsigned)(((size_t)h->n * sizeof(int2) + 15) & ~(size_t)15);
-    const size_t with_table = ((size_t)tb + 127) / 128 * 128 + rings;
-    if (with_table <= (size_t)h->smem_optin - 2048) {
-        *table_in_smem = true; *table_bytes = tb; return with_table;
-    }
-    *table_in_smem = false; *table_bytes = tb; return rings;
-}
+size_t k3_smem_bytes(const sched_ctx* h) { return (size_t)k3_warps(h) * h->ring_cells * sizeof(int); }
 
 int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t* o, i64 M) {
     if (!out) return SCHED_E_INVAL;
@@ -276,21 +256,15 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         h->smem_optin = (int)prop.sharedMemPerBlockOptin;
         h->B = B; h->n = n; h->M = M; h->omax = omax; h->sum_o_max = sum_max;
         h->g_num = 0; h->g_den = 1;
-        h->nreg = sim_pick_nreg(omax);
-        h->hyb = h->nreg == 0;
-        if (const char* kind = getenv("KVSCHED_SIM")) {             // testing knob: "smem" / "hybrid" force that simulator
-            if (strcmp(kind, "smem") == 0) { h->nreg = 0; h->hyb = false; }
-            if (strcmp(kind, "hybrid") == 0) { h->nreg = 0; h->hyb = true; }
-        }
-        h->nit = sim_pick_nit(omax);
-        if (const char* cap = getenv("KVSCHED_MAX_NIT")) {          // tuning knob: windows beyond the cap stream
-            const int c = atoi(cap);
-            if (c == 0 || c == 1 || c == 2 || c == 4 || c == 8) h->nit = c < h->nit ? c : h->nit;
-        }
-        // cells per simulator state: registers x 32 lanes, or a ring whose length is a multiple of
-        // 32 cells (a wrapped 16-byte access then keeps its bank)
-        h->L = h->hyb ? 32 * (HybSim::NREG + sim_pick_far_chunks(omax)) : h->nreg > 0 ? 32 * h->nreg : (omax + 8 + 31) & ~31;
-        h->ring_cells = h->hyb ? HybSim::ring_cells(h->L) : h->nreg > 0 ? 0 : h->L;
+        const int slots = sim_pick_slots(omax);
+        h->nm = slots <= 32 ? 1 : slots <= 256 ? slots / 32 : 0;
+        // the chunked simulator's bounds (M, rounds ahead, at most 31 more per admission) have to fit 31 bits
+        if (M + 32ll * n + 32768 >= (1ll << 31)) h->nm = 0;
+        if (const char* kind = getenv("KVSCHED_SIM"))               // testing knob: force the hybrid simulator
+            if (strcmp(kind, "hybrid") == 0) h->nm = 0;
+        // ints per simulator state, and the part of it that lives in shared memory
+        h->L = h->nm == 0 ? 32 * (HybSim::NREG + sim_pick_far_chunks(omax)) : 32 + 96 * h->nm + 32 * slots;
+        h->ring_cells = h->nm == 0 ? HybSim::ring_cells(h->L) : 32 * slots;
         if (k3_warps(h) < 1) { rc = SCHED_E_UNSUPPORTED; break; }
         if (cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaStreamCreate"); break; }
         h->stream = h->own_stream;
@@ -310,8 +284,10 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             A(dev_alloc(&h->d_prefP, n + 1)); A(dev_alloc(&h->d_prefO, n + 1));
             A(dev_alloc(&h->d_batch_off, n + 1)); A(dev_alloc(&h->d_num_batches, 1)); A(dev_alloc(&h->d_seg_off, 2));
             size_t per = (size_t)h->L * sizeof(int);
-            i64 stride = (i64)(((size_t)n * per + kSnapBudget - 1) / kSnapBudget);
-            if (stride < 1) stride = 1;
+            // a candidate replays (stride - 1) / 2 positions on average to reach its first moved one:
+            // 0.2 % of the list at 256 snapshots, for which the base run stores 256 states instead of n
+            i64 stride = ((i64)n + kSnapshots - 1) / kSnapshots;
+            while ((((i64)n + stride - 1) / stride) * (i64)per > (i64)kSnapBudget) ++stride;
             h->snap_stride = (int)stride;
             h->snap_count = (n + h->snap_stride - 1) / h->snap_stride;
             A(dev_alloc(&h->d_snap_ring, (size_t)h->snap_count * h->L));
@@ -416,10 +392,9 @@ int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, 
     KV_TRY(ensure_base(h));
     MoveEvalParams p;
     memset(&p, 0, sizeof(p));
-    bool in_smem; unsigned tb;
-    const size_t smem = k3_smem_bytes(h, &in_smem, &tb);
+    const size_t smem = k3_smem_bytes(h);
     p.n = h->n; p.L = h->L; p.M = (int)h->M; p.stride = h->snap_stride;
-    p.tbl_base = h->d_tbl_base; p.table_in_smem = in_smem ? 1 : 0; p.table_bytes = tb;
+    p.tbl_base = h->d_tbl_base;
     p.snap_ring = h->d_snap_ring; p.snap_hdr = h->d_snap_hdr; p.snap_count = h->snap_count;
     p.src.mode = mode; p.src.codes = codes; p.src.first = first; p.src.seed = seed; p.src.iteration = iteration;
     p.count = count; p.tel_out = tel_out; p.tel_by_slot = by_slot ? 1 : 0; p.starts_out = starts_out;
@@ -605,10 +580,8 @@ int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* ca
     if (kind == SCHED_CAND_ORDER) {
         OrderEvalParams p;
         memset(&p, 0, sizeof(p));
-        bool in_smem; unsigned tb;
-        const size_t smem = k3_smem_bytes(h, &in_smem, &tb);
+        const size_t smem = k3_smem_bytes(h);
         p.n = n; p.L = h->L; p.M = (int)h->M; p.tbl_id = h->d_tbl_id;
-        p.table_in_smem = in_smem ? 1 : 0; p.table_bytes = tb;
         p.orders = (const int*)candidates; p.count = count; p.tel_out = (i64*)tel_out; p.starts_out = starts_out;
         p.status = h->d_status;
         KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));

@@ -14,7 +14,7 @@ typedef unsigned long long u64;
 #define KV_FULL 0xffffffffu
 
 // Device-side status word (ctx->d_status[0]); non-zero means a bounded loop gave up.
-enum { KV_DEV_OK = 0, KV_DEV_LOOP_CAP = 1, KV_DEV_TMA_TIMEOUT = 2 };
+enum { KV_DEV_OK = 0, KV_DEV_LOOP_CAP = 1 };
 
 struct SnapHeader {          // simulator state in front of one list position (16 bytes)
     int t;                   // current round index (number of completed rounds = next start time)
@@ -28,11 +28,9 @@ struct sched_ctx {
     int B, n;                // instances, requests per instance
     i64 M;
     int omax;                // largest decode length over all instances
-    int L;                   // cells per simulator state (32 * nreg; 32 * (33 + far chunks); or a ring of a multiple of 32 cells >= omax + 8)
-    int nreg;                // > 0: register-resident simulator with this many registers per lane
-    int nit;                 // shared-memory simulator: 128-cell rounds cached in registers (0: streamed)
-    bool hyb;                // hybrid simulator: 33 registers per lane + a shared-memory ring for the rounds after them
-    int ring_cells;          // shared-memory ints one simulator needs (0 for the register simulator)
+    int L;                   // ints per simulator state
+    int nm;                  // chunked simulator with this many far registers per lane; 0: hybrid simulator
+    int ring_cells;          // shared-memory ints one simulator needs
     i64 sum_o_max;           // largest sum of o over instances (bounds every start time)
     int sm_count;
     int smem_optin;          // max dynamic shared memory per block (bytes)

@@ -13,70 +13,24 @@
 //   k3_check_starts   explicit start times: occupancy by the integer program's memory row
 //                     (Section 6.1), flag raised at the first round above M.
 //
-// The request table is staged into shared memory once per CTA with a bulk asynchronous copy
-// (cp.async.bulk + mbarrier, no multicast) when it fits; otherwise it is read through L1/L2.
+// The request table is read through L1/L2, 32 positions (256 consecutive bytes) at a time: one such
+// load per 32 admissions, whereas a copy of it in shared memory takes the room of 20 simulators.
 #pragma once
 
 #include "common.cuh"
 #include "k2_fmetric.cuh"
 #include "k4_moves.cuh"
-#include "sim.cuh"
-#include "sim_reg.cuh"
+#include "sim_chunk.cuh"
 #include "sim_hyb.cuh"
+
+__device__ __forceinline__ int kv_wrap(int idx, int L) {   // idx < 3L
+    if (idx >= L) idx -= L;
+    if (idx >= L) idx -= L;
+    return (int)KV_IDX(idx, L, 301);
+}
 
 #define K3S_WARPS 16                       // warps per CTA of the start-time checker
 
-// ------------------------------------------------------------------------------------------------
-// Bulk copy global -> shared with a bounded wait.  bytes is a multiple of 16, both addresses are
-// 16-byte aligned.  Returns false (in every thread) if the copy did not land within the cap; the
-// caller must then leave without touching the destination.
-// ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ unsigned kv_smem_addr(const void* p) {
-    return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ int kv_mbar_wait(unsigned bar, int max_spins) {
-    for (int spin = 0; spin < max_spins; ++spin) {
-        unsigned done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done) : "r"(bar) : "memory");
-        if (done) return 1;
-    }
-    return 0;
-}
-
-__device__ bool kv_bulk_load(void* smem_dst, const void* gsrc, unsigned bytes, u64* mbar, int* sh_flag, int* status) {
-    const unsigned bar = kv_smem_addr(mbar);
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-        const unsigned chunk = 32768;
-        for (unsigned off = 0; off < bytes; off += chunk) {
-            unsigned sz = bytes - off < chunk ? bytes - off : chunk;
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                ::"r"(kv_smem_addr((const char*)smem_dst + off)), "l"((const char*)gsrc + off), "r"(sz), "r"(bar)
-                : "memory");
-        }
-        // bounded wait; if it runs out, flag the failure and give the copy one more bounded
-        // chance to land so that the CTA does not exit with a transfer still in flight
-        int ok = kv_mbar_wait(bar, 1 << 22);
-        if (!ok) {
-            atomicExch(status, KV_DEV_TMA_TIMEOUT);
-            kv_mbar_wait(bar, 1 << 22);
-        }
-        *sh_flag = ok;
-    }
-    __syncthreads();
-    return *sh_flag != 0;
-}
-
-// ------------------------------------------------------------------------------------------------
 __global__ void k3_gather_table(const int2* __restrict__ tbl_id, const int* __restrict__ order, int n,
                                 int2* __restrict__ tbl_base) {
     int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -95,7 +49,10 @@ __global__ void k3_iota(int* a, int n) {
 
 // ------------------------------------------------------------------------------------------------
 // Base run: positions 0 .. n-1 of the base order; snapshot idx holds the state in front of
-// position idx * stride.  One warp.  Dynamic shared memory: the simulator's ring, if it has one.
+// position idx * stride.  One warp: the run is a chain of n admissions, each of which needs the one
+// before it, so what counts is the latency of one admission.  The next 32 requests are loaded while
+// the 32 in hand are admitted, and their starts are stored together.  Dynamic shared memory: the
+// simulator's ring.
 // ------------------------------------------------------------------------------------------------
 template <class SIM>
 __global__ void __launch_bounds__(32)
@@ -106,23 +63,35 @@ k3_base_run(const int2* __restrict__ tbl_base, int n, int L, int M, int stride, 
     const int lane = threadIdx.x;
     SIM sim;
     sim.attach((int*)smem_raw, L);
-    sim.reset(lane);
+    sim.reset(M);
+    i64 tel = 0;                                         // of the positions before this block
+    int2 next = lane < n ? tbl_base[lane] : make_int2(1, 1);
+    int to_snap = 0, idx = 0;                            // positions until the next snapshot, its number
     for (int q0 = 0; q0 < n; q0 += 32) {
-        const int qq = q0 + lane;
-        int2 so = qq < n ? tbl_base[qq] : make_int2(1, 1);
+        const int2 so = next;
+        if (q0 + 32 + lane < n) next = tbl_base[q0 + 32 + lane];
         const int cnt = min(32, n - q0);
+        int mine = 0;
+        const int sp = so.x + 1, om = so.y - 1;
         for (int k = 0; k < cnt; ++k) {
-            const int q = q0 + k;
-            if (q % stride == 0) {
-                const int idx = (int)KV_IDX(q / stride, snap_count, 401);
-                sim.store(snap_ring + (size_t)idx * L, snap_hdr + idx, lane);
+            if (to_snap == 0) {
+                const int i = (int)KV_IDX(idx, snap_count, 401);
+                i64 before = lane < k ? (i64)mine + so.y : 0;    // this block's completions so far
+                for (int d = 16; d >= 1; d >>= 1) before += __shfl_xor_sync(KV_FULL, before, d);
+                sim.store(snap_ring + (size_t)i * L, snap_hdr + i, tel + before);
+                ++idx;
+                to_snap = stride;
             }
-            const int s = __shfl_sync(KV_FULL, so.x, k), o = __shfl_sync(KV_FULL, so.y, k);
-            const int p = sim.admit(s, o, M, lane, status);
-            if (lane == 0) base_starts_pos[q] = p;
+            --to_snap;
+            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, status);
+            if (lane == k) mine = sim.start();
         }
+        if (q0 + lane < n) base_starts_pos[q0 + lane] = mine;
+        i64 done = lane < cnt ? (i64)mine + so.y : 0;
+        for (int d = 16; d >= 1; d >>= 1) done += __shfl_xor_sync(KV_FULL, done, d);
+        tel += done;
     }
-    if (lane == 0) *base_tel = sim.total();
+    if (lane == 0) *base_tel = tel;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -131,8 +100,6 @@ k3_base_run(const int2* __restrict__ tbl_base, int n, int L, int M, int stride, 
 struct MoveEvalParams {
     int n, L, M, stride, snap_count;
     const int2* tbl_base;
-    int table_in_smem;
-    unsigned table_bytes;              // multiple of 16
     const int* snap_ring;
     const SnapHeader* snap_hdr;
     MoveSource src;
@@ -149,28 +116,20 @@ struct MoveEvalParams {
 
 // One warp per candidate, no loop over candidates (a persistent loop around the simulator costs
 // ~15 % more instructions per admission with this compiler): warp w of CTA b takes launch slot
-// 32 b + w, whose candidate K4 chose so that the warps of a CTA have nearly equal work.
+// kWarps b + w, whose candidate K4 chose so that the warps of a CTA have nearly equal work.
 template <class SIM, bool kStarts>
-__global__ void __launch_bounds__(SIM::kWarps * 32, 1)
+__global__ void __launch_bounds__(SIM::kWarps * 32, SIM::kMinCtas)
 k3_eval_moves(const MoveEvalParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ u64 mbar;
-    __shared__ int sh_flag;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int2* tbl = p.tbl_base;
-    size_t ring_off = 0;
-    if (p.table_in_smem) {
-        if (!kv_bulk_load(smem_raw, p.tbl_base, p.table_bytes, &mbar, &sh_flag, p.status)) return;
-        tbl = (const int2*)smem_raw;
-        ring_off = (p.table_bytes + 127) & ~(size_t)127;
-    }
+    const int2* __restrict__ tbl = p.tbl_base;
     const int n = p.n, L = p.L, M = p.M;
     const i64 slot = (i64)blockIdx.x * (blockDim.x >> 5) + warp;
     if (slot >= p.count) return;
     const i64 c = KV_IDX(p.launch_order[slot], p.count, 402);
     i64* tel_dst = p.tel_out + (p.tel_by_slot ? slot : c);
     SIM sim;
-    sim.attach((int*)(smem_raw + ring_off) + (size_t)warp * SIM::ring_cells(L), L);
+    sim.attach((int*)smem_raw + (size_t)warp * SIM::ring_cells(L), L);
     const Move mv = k4_move_of(p.src, n, c);
     if ((unsigned)mv.i >= (unsigned)n || (unsigned)mv.j >= (unsigned)n) {      // code outside the neighbourhood
         if (lane == 0) *tel_dst = INT64_MAX;
@@ -180,7 +139,8 @@ k3_eval_moves(const MoveEvalParams p) {
     const int idx = (int)KV_IDX(first_pos / p.stride, p.snap_count, 403);
     const int q_start = idx * p.stride;
     // restore the base run's state in front of q_start
-    sim.load(p.snap_ring + (size_t)idx * L, p.snap_hdr[idx], lane);
+    sim.load(p.snap_ring + (size_t)idx * L, p.snap_hdr[idx], M, n - q_start);
+    i64 sum_o = 0;
     int* starts = kStarts ? p.starts_out + (size_t)c * n : nullptr;
     if (kStarts)
         for (int q = lane; q < q_start; q += 32) starts[KV_IDX(p.base_order[q], n, 406)] = p.base_starts_pos[q];
@@ -193,14 +153,17 @@ k3_eval_moves(const MoveEvalParams p) {
             so = tbl[bp];
             if (kStarts) id = p.base_order[bp];
         }
-        const int cnt = min(32, n - q0);
+        const int cnt = min(32, n - q0), sp = so.x + 1, om = so.y - 1;
+        if (lane < cnt) sum_o += so.y;
+        int mine = 0;
         for (int k = 0; k < cnt; ++k) {
-            const int s = __shfl_sync(KV_FULL, so.x, k), o = __shfl_sync(KV_FULL, so.y, k);
-            const int pstart = sim.admit(s, o, M, lane, p.status);
-            if (kStarts && lane == k) starts[KV_IDX(id, n, 405)] = pstart;
+            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, p.status);
+            if (kStarts && lane == k) mine = sim.start();
         }
+        if (kStarts && lane < cnt) starts[KV_IDX(id, n, 405)] = mine;
     }
-    if (lane == 0) *tel_dst = sim.total();
+    for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
+    if (lane == 0) *tel_dst = sim.total(sum_o);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -209,8 +172,6 @@ k3_eval_moves(const MoveEvalParams p) {
 struct OrderEvalParams {
     int n, L, M;
     const int2* tbl_id;
-    int table_in_smem;
-    unsigned table_bytes;
     const int* orders;
     i64 count;
     i64* tel_out;
@@ -219,28 +180,21 @@ struct OrderEvalParams {
 };
 
 template <class SIM, bool kStarts>
-__global__ void __launch_bounds__(SIM::kWarps * 32, 1)
+__global__ void __launch_bounds__(SIM::kWarps * 32, SIM::kMinCtas)
 k3_eval_orders(const OrderEvalParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ u64 mbar;
-    __shared__ int sh_flag;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int2* tbl = p.tbl_id;
-    size_t ring_off = 0;
-    if (p.table_in_smem) {
-        if (!kv_bulk_load(smem_raw, p.tbl_id, p.table_bytes, &mbar, &sh_flag, p.status)) return;
-        tbl = (const int2*)smem_raw;
-        ring_off = (p.table_bytes + 127) & ~(size_t)127;
-    }
+    const int2* __restrict__ tbl = p.tbl_id;
     const int n = p.n, L = p.L, M = p.M;
     const i64 c = (i64)blockIdx.x * (blockDim.x >> 5) + warp;      // every order has the same length
     if (c >= p.count) return;
     SIM sim;
-    sim.attach((int*)(smem_raw + ring_off) + (size_t)warp * SIM::ring_cells(L), L);
+    sim.attach((int*)smem_raw + (size_t)warp * SIM::ring_cells(L), L);
     const int* ord = p.orders + (size_t)c * n;
     int* starts = kStarts ? p.starts_out + (size_t)c * n : nullptr;
-    sim.reset(lane);
+    sim.reset(M);
     int bad = 0;
+    i64 sum_o = 0;
     for (int q0 = 0; q0 < n; q0 += 32) {
         const int qq = q0 + lane;
         int2 so = make_int2(1, 1);
@@ -250,14 +204,17 @@ k3_eval_orders(const OrderEvalParams p) {
             if (lane == 0) p.tel_out[c] = INT64_MAX;
             return;
         }
-        const int cnt = min(32, n - q0);
+        const int cnt = min(32, n - q0), sp = so.x + 1, om = so.y - 1;
+        if (lane < cnt) sum_o += so.y;
+        int mine = 0;
         for (int k = 0; k < cnt; ++k) {
-            const int s = __shfl_sync(KV_FULL, so.x, k), o = __shfl_sync(KV_FULL, so.y, k);
-            const int pstart = sim.admit(s, o, M, lane, p.status);
-            if (kStarts && lane == k) starts[id] = pstart;
+            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, p.status);
+            if (kStarts && lane == k) mine = sim.start();
         }
+        if (kStarts && lane < cnt) starts[id] = mine;
     }
-    if (lane == 0) p.tel_out[c] = sim.total();
+    for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
+    if (lane == 0) p.tel_out[c] = sim.total(sum_o);
 }
 
 // ------------------------------------------------------------------------------------------------

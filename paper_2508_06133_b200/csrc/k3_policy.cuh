@@ -5,16 +5,16 @@
 
 #include "common.cuh"
 #include "k2_fmetric.cuh"
-#include "sim.cuh"
-#include "sim_reg.cuh"
+#include "sim_chunk.cuh"
 #include "sim_hyb.cuh"
 
 // ------------------------------------------------------------------------------------------------
 // Policy sweep: one warp per (instance, policy) pair, up to K3P_MAX_WARPS pairs of one instance per
-// CTA.  Dynamic shared memory: int s[n], o[n] once per CTA; per warp the simulator's ring
-// (SIM::ring_cells(L) ints), PT P[n+2], O[n+2] (PT = int32 when n * M < 2^31, else int64), int
-// boff[n+2], a 256-bin histogram, and 16-bit: three id buffers [n] and batch numbers [n].  Orders are built by
-// a single-warp radix sort (k3_warp_radix_sort) on the fields of the policy's key.
+// CTA.  Dynamic shared memory: int s[n], o[n] once per CTA; per warp the finished order (16-bit ids)
+// and one area that first holds what the order is built with -- PT P[n+2], O[n+2] (PT = int32 when
+// n * M < 2^31, else int64), int boff[n+2], a 256-bin histogram, and 16-bit: three id buffers [n] and
+// batch numbers [n] -- and then the simulator's ring (SIM::ring_cells(L) ints).  Orders are built by a
+// single-warp radix sort (k3_warp_radix_sort) on the fields of the policy's key.
 // ------------------------------------------------------------------------------------------------
 // One pass of a stable least-significant-digit radix sort run by a single warp on shared memory:
 // the m ids of `in` are written to `out` in ascending order of digit(id), an 8-bit value; ids with
@@ -128,11 +128,14 @@ __device__ __forceinline__ int k3_warp_select_batches(const PT* P, const PT* O, 
     return nb;
 }
 
-// Bytes of shared memory one warp of the policy kernel needs besides the instance's (s, o):
-// the simulator's ring, P and O, the batch offsets, the radix histogram and four 16-bit id arrays.
+// Bytes of shared memory one warp of the policy kernel needs besides the instance's (s, o): the order,
+// and the larger of the simulator's ring and the order's scratch (P and O, the batch offsets, the
+// radix histogram, four 16-bit id arrays).
+__host__ __device__ inline size_t k3_policy_order_bytes(int n) { return ((size_t)n * 2 + 15) & ~(size_t)15; }
 __host__ __device__ inline size_t k3_policy_warp_bytes(int n, int ring_cells, int pt_bytes) {
-    const size_t b = (size_t)ring_cells * 4 + (size_t)(n + 2) * 2 * pt_bytes + (size_t)(n + 2) * 4 + 256 * 4 + (size_t)n * 8;
-    return (b + 15) & ~(size_t)15;
+    const size_t ring = (size_t)ring_cells * 4;
+    const size_t scratch = (size_t)(n + 2) * 2 * pt_bytes + (size_t)(n + 2) * 4 + 256 * 4 + (size_t)n * 8;
+    return k3_policy_order_bytes(n) + (((ring > scratch ? ring : scratch) + 15) & ~(size_t)15);
 }
 
 // grid = B * groups CTAs of W = blockDim.x / 32 warps; CTA (b, g) evaluates instance b under
@@ -156,8 +159,9 @@ k3_eval_policy(const int* __restrict__ s_all, const int* __restrict__ o_all, int
     const int policy = policies[kpol];
     unsigned char* mine = smem_raw + (((size_t)n * 8 + 15) & ~(size_t)15) +
                           (size_t)warp * k3_policy_warp_bytes(n, SIM::ring_cells(L), (int)sizeof(PT));
-    int* ring = (int*)mine;                           // first: 16-byte aligned for the vector loads
-    PT* P = (PT*)(ring + SIM::ring_cells(L));         // a multiple of 4 ints: 8-byte aligned
+    k3_id_t* fin = (k3_id_t*)mine;                    // the finished order
+    int* ring = (int*)(mine + k3_policy_order_bytes(n));   // 16-byte aligned; the scratch until the order is finished
+    PT* P = (PT*)ring;
     PT* O = P + (n + 2);
     int* boff = (int*)(O + (n + 2));                  // n + 2 batch offsets
     int* hist = boff + n + 2;                         // 256 bins of the radix passes
@@ -193,15 +197,25 @@ k3_eval_policy(const int* __restrict__ s_all, const int* __restrict__ o_all, int
         auto f_b = [&](int id) { return bat[id]; };
         ord = k3_warp_radix_sort(byo, ord == bufa ? bufb : bufa, n, hist, lane, f_b, k3_bytes_of((unsigned)nb));
     }
+    for (int i = lane; i < n; i += 32) fin[i] = ord[i];
+    __syncwarp();                                     // from here on the scratch is the simulator's
     SIM sim;
     sim.attach(ring, L);
-    sim.reset(lane);
+    sim.reset(M);
+    i64 sum_o = 0;
     int* starts = starts_out ? starts_out + ((size_t)b * num_policies + kpol) * n : nullptr;
-    for (int q = 0; q < n; ++q) {
-        const int id = (int)KV_IDX(ord[q], n, 906);
-        const int pstart = sim.admit(s[id], o[id], M, lane, status);
-        if (starts && lane == 0) starts[id] = pstart;
+    for (int q0 = 0; q0 < n; q0 += 32) {
+        int id = 0, sp = 2, om = 0;
+        const int cnt = min(32, n - q0);
+        if (lane < cnt) { id = (int)KV_IDX(fin[q0 + lane], n, 906); sp = s[id] + 1; om = o[id] - 1; sum_o += om + 1; }
+        int mine = 0;
+        for (int k = 0; k < cnt; ++k) {
+            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, status);
+            if (lane == k) mine = sim.start();
+        }
+        if (starts && lane < cnt) starts[id] = mine;
     }
-    if (lane == 0) tel_out[(size_t)b * num_policies + kpol] = sim.total();
+    for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
+    if (lane == 0) tel_out[(size_t)b * num_policies + kpol] = sim.total(sum_o);
 }
 

@@ -1,7 +1,9 @@
-// Hybrid schedule simulator for decode lengths beyond what the register-resident simulator covers:
-// the first 32 * 33 rounds of the timeline live in registers exactly as in sim_reg.cuh (same cell
-// encoding V = U + round index, same rotation at every 32-round boundary), the rounds after them in
-// a per-warp ring of FC chunks of 32 cells in shared memory ("far" part).  Lane l owns column l of
+// Hybrid schedule simulator, for decode lengths beyond what the chunked simulator (sim_chunk.cuh)
+// covers: every cell of the timeline is kept.  The first 32 * 33 rounds live in registers: register
+// R[c] of lane l holds the cell of round T0 + 32 c + l (T0 = t rounded down to a multiple of 32) as
+// V = U + round index (an unoccupied cell holds its round index), and the registers rotate by one
+// whenever t crosses a multiple of 32.  The rounds after them are in a per-warp ring of FC chunks of
+// 32 cells in shared memory ("far" part).  Lane l owns column l of
 // every chunk, in registers and in the ring alike, so no lane ever reads another lane's cell and no
 // warp synchronisation is needed around the shared-memory accesses.
 //
@@ -9,7 +11,7 @@
 // one whole span later) goes to the slot of the first far chunk, and that chunk's cells become the
 // last register.  A request whose window ends inside the registers -- nch = ceil((t%32 + o)/32) <=
 // 33, the common case: most decode lengths are short even when the longest is not -- never touches
-// shared memory and costs what it costs in the register simulator; a longer window continues over
+// shared memory; a longer window continues over
 // the first nch - 33 far chunks with one shared load (test) or load + store (ramp add) per chunk.
 //
 // State size (snapshot layout): L = 32 * (33 + FC) ints, the registers first (R[c] of lane l at
@@ -18,12 +20,116 @@
 #pragma once
 
 #include "common.cuh"
-#include "sim_reg.cuh"
+
+// The passes over the window are specialised on the chunk count nch by a tree of warp-uniform
+// branches.  STMT(KLO, KHI) is expanded once per leaf and handles nch in (KLO, KHI]: chunks
+// 1 .. KLO-1 are certainly inside the window (one instruction each per pass), chunks KLO .. KHI-1 are
+// masked by lane, and no other register is touched.  Exact up to 16 chunks, two chunk counts per leaf
+// beyond.
+#define KV_RS_BUCKETS_MIX(nch, STMT) \
+    if (nch <= 7) { \
+      if (nch <= 4) { \
+        if (nch <= 2) { \
+          if (nch <= 1) { \
+            STMT(0, 1) \
+          } else { \
+            STMT(1, 2) \
+          } \
+        } else { \
+          if (nch <= 3) { \
+            STMT(2, 3) \
+          } else { \
+            STMT(3, 4) \
+          } \
+        } \
+      } else { \
+        if (nch <= 5) { \
+          STMT(4, 5) \
+        } else { \
+          if (nch <= 6) { \
+            STMT(5, 6) \
+          } else { \
+            STMT(6, 7) \
+          } \
+        } \
+      } \
+    } else { \
+      if (nch <= 12) { \
+        if (nch <= 9) { \
+          if (nch <= 8) { \
+            STMT(7, 8) \
+          } else { \
+            STMT(8, 9) \
+          } \
+        } else { \
+          if (nch <= 10) { \
+            STMT(9, 10) \
+          } else { \
+            if (nch <= 11) { \
+              STMT(10, 11) \
+            } else { \
+              STMT(11, 12) \
+            } \
+          } \
+        } \
+      } else { \
+        if (nch <= 15) { \
+          if (nch <= 13) { \
+            STMT(12, 13) \
+          } else { \
+            if (nch <= 14) { \
+              STMT(13, 14) \
+            } else { \
+              STMT(14, 15) \
+            } \
+          } \
+        } else { \
+          if (nch <= 18) { \
+            if (nch <= 16) { \
+              STMT(15, 16) \
+            } else { \
+              STMT(16, 18) \
+            } \
+          } else { \
+            if (nch <= 24) { \
+              if (nch <= 20) { \
+                STMT(18, 20) \
+              } else { \
+                if (nch <= 22) { \
+                  STMT(20, 22) \
+                } else { \
+                  STMT(22, 24) \
+                } \
+              } \
+            } else { \
+              if (nch <= 32) { \
+                if (nch <= 28) { \
+                  if (nch <= 26) { \
+                    STMT(24, 26) \
+                  } else { \
+                    STMT(26, 28) \
+                  } \
+                } else { \
+                  if (nch <= 30) { \
+                    STMT(28, 30) \
+                  } else { \
+                    STMT(30, 32) \
+                  } \
+                } \
+              } else { \
+                STMT(32, 33) \
+              } \
+            } \
+          } \
+        } \
+      } \
+    }
+
 
 struct HybSim {
     static constexpr int NREG = 33;
-    static constexpr bool kUsesSmem = true;
     static constexpr int kWarps = 24;                 // 33 timeline registers + the ring bookkeeping need more than 64 registers
+    static constexpr int kMinCtas = 1;
     __host__ __device__ static constexpr int ring_cells(int L) { return L - 32 * NREG; }
 
     int R[NREG];
@@ -34,22 +140,28 @@ struct HybSim {
     int FC, fb;              // chunks in the far ring; slot of the first far chunk
     int span;                // 32 * (NREG + FC): rounds covered by the whole state
 
+    int M, lane;
+
     __device__ __forceinline__ void attach(int* ring, int L) {
-        far = ring + (threadIdx.x & 31);
+        lane = kv_lane();
+        far = ring + lane;
         FC = (L >> 5) - NREG;
         span = L;
         fb = 0;
     }
-    __device__ __forceinline__ i64 total() const { return tel; }
+    __device__ __forceinline__ i64 total(i64) const { return tel; }
+    __device__ __forceinline__ int start() const { return t; }             // of the request admitted last
     __device__ __forceinline__ int slot_of(int k) const { const int x = fb + k; return (int)KV_IDX(x >= FC ? x - FC : x, FC, 201); }
 
-    __device__ __forceinline__ void reset(int lane) {
+    __device__ __forceinline__ void reset(int M_) {
+        M = M_;
 #pragma unroll
         for (int c = 0; c < NREG; ++c) R[c] = 32 * c + lane;
         for (int k = 0; k < FC; ++k) far[32 * k] = 32 * (NREG + k) + lane;
         fb = 0; t = 0; tel = 0; tm = 0; rl = lane;
     }
-    __device__ __forceinline__ void load(const int* __restrict__ snap, const SnapHeader& h, int lane) {
+    __device__ __forceinline__ void load(const int* __restrict__ snap, const SnapHeader& h, int M_, int) {
+        M = M_;
 #pragma unroll
         for (int c = 0; c < NREG; ++c) R[c] = snap[KV_IDX(32 * c + lane, span, 202)];
         for (int k = 0; k < FC; ++k) far[32 * k] = snap[KV_IDX(32 * (NREG + k) + lane, span, 203)];
@@ -57,7 +169,7 @@ struct HybSim {
         t = h.t; tm = t & 31; rl = lane - tm;
         tel = ((i64)h.tel_hi << 32) | (i64)(unsigned)h.tel_lo;
     }
-    __device__ __forceinline__ void store(int* __restrict__ snap, SnapHeader* hdr, int lane) const {
+    __device__ __forceinline__ void store(int* __restrict__ snap, SnapHeader* hdr, i64) const {
 #pragma unroll
         for (int c = 0; c < NREG; ++c) snap[KV_IDX(32 * c + lane, span, 204)] = R[c];
         for (int k = 0; k < FC; ++k) snap[KV_IDX(32 * (NREG + k) + lane, span, 205)] = far[32 * slot_of(k)];
@@ -80,7 +192,7 @@ struct HybSim {
         fb = fb + 1 == FC ? 0 : fb + 1;
     }
 
-    __device__ __forceinline__ void advance(int delta, int lane) {
+    __device__ __forceinline__ void advance(int delta) {
         const int step = min(delta, 32 - tm);
         if ((unsigned)rl < (unsigned)step) R[0] = t + rl + span;
         t += step;
@@ -96,7 +208,7 @@ struct HybSim {
         rl = lane - tm;
     }
 
-    // ---- passes over a window that ends inside the registers (as in the register simulator)
+    // ---- passes over a window that ends inside the registers
     template <int KLO, int KHI>
     __device__ __forceinline__ int pass_max_from(int v, int ol) const {
         constexpr int KI = KLO < KHI ? KLO : KHI;
@@ -126,11 +238,11 @@ struct HybSim {
         return need;
     }
 
-    // Admit one request; returns its start.  All 32 lanes call this with identical (s, o).  Same
-    // turn structure as the register simulator: the first chunk alone decides whether the request
+    // Admit one request (sp = s + 1, om = o - 1).  All 32 lanes call this with identical arguments.  The first chunk alone decides whether the request
     // has to wait and for how long at least; otherwise the whole window is tested and, if it fits,
     // the ramp is added; a window that reaches beyond the registers continues over the far ring.
-    __device__ __forceinline__ int admit(int s, int o, int M, int lane, int* status) {
+    __device__ __forceinline__ void admit(int sp, int om, int, int* status) {
+        const int s = sp - 1, o = om + 1;
         int kadm = s + 1 - M - t;                      // V + kadm > 0  <=>  the cell is over budget
         for (int guard = 0;; ++guard) {
             const int ol = o - rl;
@@ -146,7 +258,7 @@ struct HybSim {
                         if (vmax + kadm <= 0) {                                    \
                             pass_add<A, (B < NREG ? B : NREG)>(rl, ol, s + 1 + rl); \
                             tel += t + o;                                          \
-                            return t;                                              \
+                            return;                                              \
                         }                                                          \
                     }
                     KV_RS_BUCKETS_MIX(nch, KV_HS_TRY)
@@ -176,14 +288,14 @@ struct HybSim {
                             }
                         }
                         tel += t + o;
-                        return t;
+                        return;
                     }
                     delta = kv_warp_max(need_behind(ol, kadm, nfar));
                 }
             }
             kadm -= delta;                             // >= 1: the worst cell alone asks for it
-            advance(delta, lane);
-            if (guard > kv_loop_cap(span)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); return t; }
+            advance(delta);
+            if (guard > kv_loop_cap(span)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); return; }
         }
     }
 };
