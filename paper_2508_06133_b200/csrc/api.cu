@@ -736,17 +736,23 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
         KV_TRY(phase1_quantile(h, seed));
     } else {
         // Algorithm 3: ascending (s+o, index), then first fit + improving swaps, batch after batch
-        if (!h->d_ls) KV_TRY(dev_alloc(&h->d_ls, 7 * (size_t)n + 32));
         k1_keys_total_size<<<(n + 255) / 256, 256, 0, st>>>(h->d_s, h->d_o, n, h->d_keys_a, h->d_vals_a, SCHED_POLICY_TOTAL_SIZE);
         KV_TRY(check_launch(h));
         k1_radix_sort_segments<<<1, K1_THREADS, 0, st>>>(h->d_keys_a, h->d_vals_a, h->d_keys_b, h->d_vals_b, h->d_seg_off, nullptr, 1,
                                                           key_byte_mask(0, bits_of((u64)h->M)));
         KV_TRY(check_launch(h));
-        int* ls = h->d_ls;
         if ((i64)h->g_num * h->M + (i64)h->g_den * h->omax >= (1ll << 31)) return SCHED_E_UNSUPPORTED;   // 32-bit weights
-        k2_local_swap<<<1, K2L_THREADS, 0, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, ls, ls + n, ls + 2 * (size_t)n,
-                                                 ls + 3 * (size_t)n, ls + 4 * (size_t)n, ls + 5 * (size_t)n, ls + 6 * (size_t)n,
-                                                 h->d_vals_b, h->d_batch_off, h->d_num_batches, h->d_status);
+        // the solver's arrays in shared memory (20 bytes per request) up to about 11,000 requests
+        const size_t bytes = k2l_bytes<unsigned short>(n);
+        if (n < 65536 && bytes <= (size_t)h->smem_optin - 2048) {
+            KV_CUDA(cudaFuncSetAttribute(k2_local_swap<unsigned short>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 2048));
+            k2_local_swap<unsigned short><<<1, K2L_THREADS, bytes, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, nullptr,
+                                                                         h->d_vals_b, h->d_batch_off, h->d_num_batches, h->d_status);
+        } else {
+            if (!h->d_ls) KV_TRY(dev_alloc(&h->d_ls, 7 * (size_t)n + 32));
+            k2_local_swap<int><<<1, K2L_THREADS, 0, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, h->d_ls,
+                                                          h->d_vals_b, h->d_batch_off, h->d_num_batches, h->d_status);
+        }
         KV_TRY(check_launch(h));
         KV_CUDA(cudaMemcpyAsync(h->d_vals_a, h->d_vals_b, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, st));
     }
@@ -1062,43 +1068,49 @@ int sched_online_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const
     OnlineParams P;
     memset(&P, 0, sizeof(P));
     P.n_max = n_max; P.M = (int)M; P.policy = policy; P.period = period; P.lookahead = lookahead;
-    P.L = 32; while (P.L < omax) P.L <<= 1;
-    P.npow2 = 2; while (P.npow2 < n_max) P.npow2 <<= 1;
-    const size_t smem = sizeof(u64) * (size_t)P.npow2 + sizeof(int) * ((size_t)5 * n_max + P.L + (size_t)9 * lookahead);
+    const int slots = sim_pick_slots(omax), nm = slots <= 32 ? 1 : slots / 32;
+    P.L = 32 + 96 * nm + 32 * slots;
+    const size_t smem = k6_smem_bytes(32 * slots, n_max, lookahead);
     int dev = 0, optin = 0;
     KV_CUDA(cudaGetDevice(&dev));
     KV_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (smem + 4096 > (size_t)optin) return SCHED_E_UNSUPPORTED;
-    KV_CUDA(cudaFuncSetAttribute(k6_online, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem + 1024 > (size_t)optin) return SCHED_E_UNSUPPORTED;
+    void (*kernel)(const OnlineParams) = nm == 1 ? k6_online<ChunkSim<1>> : nm == 2 ? k6_online<ChunkSim<2>>
+                                       : nm == 4 ? k6_online<ChunkSim<4>> : k6_online<ChunkSim<8>>;
+    // the same value for every call: callers on other threads may be between this and their launch
+    KV_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024));
 
+    // one block: latency [B], status (8 bytes) | n_each [B] | a, s, o, start [cells each]
     const size_t cells = (size_t)B * n_max;
-    int *d_n = nullptr, *d_a = nullptr, *d_s = nullptr, *d_o = nullptr, *d_start = nullptr, *d_status = nullptr;
-    i64* d_lat = nullptr;
+    const size_t bytes = sizeof(i64) * ((size_t)B + 1) + sizeof(int) * ((size_t)B + 4 * cells);
+    char* block = nullptr;
+    KV_TRY(dev_alloc(&block, bytes < kPoolMinBlock ? kPoolMinBlock : bytes));
+    i64* d_lat = (i64*)block;
+    int* d_status = (int*)(d_lat + B);
+    int* d_n = (int*)(d_lat + B + 1);
+    int* d_a = d_n + B;
+    int* d_s = d_a + cells;
+    int* d_o = d_s + cells;
+    int* d_start = d_o + cells;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     int rc = SCHED_OK;
     do {
 #define ON_CUDA(call) if ((call) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), #call); break; }
-        if ((rc = dev_alloc(&d_n, (size_t)B)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_a, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_s, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_o, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_start, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_lat, (size_t)B)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_status, 1)) != SCHED_OK) break;
-        ON_CUDA(cudaEventCreate(&e0));
-        ON_CUDA(cudaEventCreate(&e1));
+        if (kernel_ms_out) {
+            ON_CUDA(cudaEventCreate(&e0));
+            ON_CUDA(cudaEventCreate(&e1));
+        }
         ON_CUDA(cudaMemcpy(d_n, n_each, sizeof(int) * (size_t)B, cudaMemcpyHostToDevice));
         ON_CUDA(cudaMemcpy(d_a, arrival, sizeof(int) * cells, cudaMemcpyHostToDevice));
         ON_CUDA(cudaMemcpy(d_s, s, sizeof(int) * cells, cudaMemcpyHostToDevice));
         ON_CUDA(cudaMemcpy(d_o, o, sizeof(int) * cells, cudaMemcpyHostToDevice));
-        ON_CUDA(cudaMemset(d_start, 0xff, sizeof(int) * cells));          // -1 where there is no request
-        ON_CUDA(cudaMemset(d_status, 0, sizeof(int)));
+        ON_CUDA(cudaMemsetAsync(d_start, 0xff, sizeof(int) * cells, 0));          // -1 where there is no request
+        ON_CUDA(cudaMemsetAsync(d_lat, 0, sizeof(i64) * ((size_t)B + 1), 0));
         P.n_each = d_n; P.a = d_a; P.s = d_s; P.o = d_o; P.start_out = d_start; P.latency_out = d_lat; P.status = d_status;
-        ON_CUDA(cudaEventRecord(e0, 0));
-        k6_online<<<B, K6_THREADS, smem, 0>>>(P);
+        if (e0) ON_CUDA(cudaEventRecord(e0, 0));
+        kernel<<<B, K6_THREADS, smem, 0>>>(P);
         ON_CUDA(cudaGetLastError());
-        ON_CUDA(cudaEventRecord(e1, 0));
-        ON_CUDA(cudaDeviceSynchronize());
+        if (e1) ON_CUDA(cudaEventRecord(e1, 0));
         int status = 0;
         ON_CUDA(cudaMemcpy(&status, d_status, sizeof(int), cudaMemcpyDeviceToHost));
         if (status != 0) { rc = SCHED_E_INTERNAL; break; }
@@ -1110,9 +1122,7 @@ int sched_online_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const
     } while (0);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    int* frees[] = {d_n, d_a, d_s, d_o, d_start, d_status};
-    for (int* ptr : frees) if (ptr) kv_free(ptr);
-    if (d_lat) kv_free(d_lat);
+    kv_free(block);
     return rc;
 }
 

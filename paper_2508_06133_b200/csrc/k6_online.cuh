@@ -1,5 +1,5 @@
 // K6 -- online arrivals (Section 6.2 "Heuristics under Online Arrival"; Section 7, "Experiment under
-// Online Poisson Arrivals"): many independent arrival streams, one CTA each, one policy per launch.
+// Online Poisson Arrivals"): many independent arrival streams, one warp each, one policy per launch.
 //
 // Model.  Request i arrives at the integer time a_i >= 0 (non-decreasing in i) and may start at any
 // p_i >= a_i: it is first seen by iteration a_i + 1.  In iteration t the policy orders the pending
@@ -20,14 +20,22 @@
 // budget by e at offset r needs min(e, r+1) more rounds), so the loop jumps to the earliest of:
 // that bound, the next arrival, the next due plan.
 //
-// Memory profile: a ring of L >= o_max rounds in shared memory, cell (tau mod L) = tokens in use in
-// round tau for tau in [t, t + L); rounds that are over are cleared when t moves.
+// What bounds it: one stream is a chain of admissions, plans and waits (about 1,240, 540 and 1,200 for
+// the busiest stream of the paper's experiment), so the latency of each of them:
+//   - a plan's batches are built when the head of the list reaches them.  A plan lives a few
+//     iterations, in which the first of its batches (of up to 18) is hardly ever used up: one batch
+//     per plan is built instead of 16, and 1/25 of the swaps is made.  What the list would have held
+//     behind that point is a function of the window alone, so nothing else changes;
+//   - the pending requests stay sorted from plan to plan, new ones are merged in;
+//   - the memory profile is the chunked simulator (sim_chunk.cuh), so a test costs the same for every
+//     decode length; one warp does everything, without block barriers.
 #pragma once
 
 #include "common.cuh"
 #include "k2_local_swap.cuh"
+#include "sim_chunk.cuh"
 
-#define K6_THREADS K2L_THREADS
+#define K6_THREADS 32
 #define K6_MAX_N 2048            // requests per stream
 #define K6_MAX_LOOKAHEAD 1024
 #define K6_MAX_O 8192
@@ -41,168 +49,200 @@ struct OnlineParams {
     const int* o;
     int M;
     int policy, period, lookahead;
-    int L;                       // ring length, a power of two >= the longest decode
-    int npow2;                   // power of two >= n_max
+    int L;                       // ints per simulator state
     int* start_out;              // [B, n_max]
     i64* latency_out;            // [B]  sum of (p + o - a)
     int* status;
 };
 
-struct K6Shared {
-    K2lShared ls;
-    int red[32];
+typedef unsigned short k6_ix;
+
+// dynamic shared memory: the simulator's ring; a, s, o, started flags and two id lists of n_max; the
+// local swap scratch and one batch for `lookahead` requests
+__host__ __device__ inline size_t k6_smem_bytes(int ring_cells, int n_max, int lookahead) {
+    return ((size_t)ring_cells + 6 * (size_t)n_max + lookahead) * sizeof(int) + k2l_bytes<k6_ix>(lookahead) + 64;
+}
+
+struct K6Stream {
+    int *sa, *ss, *so, *started;
+    int *S, *S2;                 // pending requests of the last plan by ascending (s+o, index); scratch
+    int* B;                      // the batch in hand by ascending (o, index)
+    K2lArrays<k6_ix> win;        // what is left of the plan's window
+    int n, nvis;
+    int slen, sused;             // S[0 .. slen): the window first; sused: how far the list has come in it
+    int wlen;                    // requests left in the window
+    int blen, bused;
+    int tail;                    // next arrival behind the plan
+
+    __device__ __forceinline__ int size_of(int id) const { return ss[id] + so[id]; }
+
+    // S <- the requests of S that have not started, with the arrivals tail .. nvis-1 that have not
+    // started merged in by (s+o, index); arrivals have higher indices than everything in S
+    __device__ void merge(int lane) {
+        int m = 0;
+        for (int base = 0; base < slen; base += 32) {
+            const int k = base + lane;
+            const int id = k < slen ? S[k] : 0;
+            const bool keep = k < slen && !started[id];
+            const unsigned v = __ballot_sync(KV_FULL, keep);
+            if (keep) S[m + __popc(v & ((1u << lane) - 1u))] = id;
+            m += __popc(v);
+            __syncwarp();
+        }
+        int c = 0;                                       // new ones, in arrival order, at the end of S2
+        int* fresh = S2 + n - (nvis - tail);
+        for (int base = tail; base < nvis; base += 32) {
+            const int id = base + lane;
+            const bool keep = id < nvis && !started[id];
+            const unsigned v = __ballot_sync(KV_FULL, keep);
+            if (keep) fresh[c + __popc(v & ((1u << lane) - 1u))] = id;
+            c += __popc(v);
+        }
+        __syncwarp();
+        if (c > 0) {
+            // new position of a new one: the old ones not above its size + its rank among the new;
+            // of an old one: its old position + the new ones below its size
+            for (int k = lane; k < c; k += 32) {
+                const int id = fresh[k], T = size_of(id);
+                int lo = 0, hi = m;
+                while (lo < hi) { const int mid = (lo + hi) >> 1; if (size_of(S[mid]) <= T) lo = mid + 1; else hi = mid; }
+                int r = lo;
+                for (int j = 0; j < c; ++j) { const int Tj = size_of(fresh[j]); r += (Tj < T || (Tj == T && j < k)) ? 1 : 0; }
+                started[id] = -1 - r;                    // its position, until everything has moved
+            }
+            __syncwarp();
+            // old ones move up, from the end so that nothing is overwritten before it is read
+            for (int base = (m - 1) & ~31; base >= 0 && m > 0; base -= 32) {
+                const int k = base + lane;
+                int id = 0, r = 0;
+                if (k < m) {
+                    id = S[k];
+                    const int T = size_of(id);
+                    for (int j = 0; j < c; ++j) r += size_of(fresh[j]) < T ? 1 : 0;
+                }
+                __syncwarp();
+                if (k < m) S[KV_IDX(k + r, n, 1002)] = id;
+                __syncwarp();
+            }
+            for (int k = lane; k < c; k += 32) {
+                const int id = fresh[k];
+                S[KV_IDX(-1 - started[id], n, 1003)] = id;
+                started[id] = 0;
+            }
+            __syncwarp();
+        }
+        slen = m + c;
+    }
+
+    // a new plan over everything pending
+    __device__ void plan(int lookahead, int lane) {
+        merge(lane);
+        tail = nvis;
+        wlen = min(slen, lookahead);
+        for (int k = lane; k < wlen; k += 32) {
+            const int id = S[k];
+            win.id[k] = id; win.T[k] = size_of(id); win.O[k] = so[id];
+        }
+        sused = wlen; blen = 0; bused = 0;
+        __syncwarp();
+    }
+
+    // head of the priority list, -1: nothing pending
+    __device__ int head(int M, int lane, int* status, K2lShared<32>& sh) {
+        if (bused == blen && wlen > 0) {
+            const int k0 = k2l_batch<32, k6_ix>(win, wlen, (i64)M, status, sh);
+            if (k0 < 1) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); wlen = 0; return -1; }
+            // the batch by ascending (o, index): rank of every member among the members
+            for (int k = lane; k < k0; k += 32) {
+                const int id = win.id[win.xpos[k]] & ~K2L_IN;
+                S2[k] = (so[id] << K6_IDX_BITS) | id;
+            }
+            __syncwarp();
+            for (int k = lane; k < k0; k += 32) {
+                const int key = S2[k];
+                int rank = 0;
+                for (int j = 0; j < k0; ++j) rank += S2[j] < key ? 1 : 0;
+                B[rank] = key & ((1 << K6_IDX_BITS) - 1);
+            }
+            __syncwarp();
+            wlen = k2l_compact<32, k6_ix>(win, wlen, sh);
+            blen = k0; bused = 0;
+        }
+        if (bused < blen) return B[bused];
+        if (sused < slen) return S[sused];
+        return tail < nvis ? tail : -1;
+    }
+    __device__ __forceinline__ void pop() {
+        if (bused < blen) ++bused;
+        else if (sused < slen) ++sused;
+        else ++tail;
+    }
 };
 
-__device__ __forceinline__ int k6_block_max(int v, int* red) {
-    const int tid = threadIdx.x;
-    v = kv_warp_max(v);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    int r = red[0];
-    for (int k = 1; k < K6_THREADS / 32; ++k) r = max(r, red[k]);
-    __syncthreads();
-    return r;
-}
-__device__ __forceinline__ int k6_block_min(int v, int* red) {
-    const int tid = threadIdx.x;
-    v = kv_warp_min(v);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    int r = red[0];
-    for (int k = 1; k < K6_THREADS / 32; ++k) r = min(r, red[k]);
-    __syncthreads();
-    return r;
-}
-
-// ascending bitonic sort of keys[0 .. len), len a power of two, by all threads of the CTA
-__device__ void k6_bitonic_sort(u64* keys, int len) {
-    const int tid = threadIdx.x;
-    for (int size = 2; size <= len; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int k = tid; k < (len >> 1); k += K6_THREADS) {
-                const int lo = ((k / stride) * (stride << 1)) + (k % stride);
-                const int hi = lo + stride;
-                const bool up = ((lo & size) == 0);
-                const u64 x = keys[lo], y = keys[hi];
-                if ((x > y) == up) { keys[lo] = y; keys[hi] = x; }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// Smallest wait (in iterations) that the window of (s, o) at iteration t asks for; <= 0: it fits.
-__device__ __forceinline__ int k6_window_need(const int* ring, int mask, int t, int s, int o, int M, int* red) {
-    int need = INT_MIN;
-    for (int x = threadIdx.x; x < o; x += K6_THREADS) {
-        const int e = ring[(t + x) & mask] + s + 1 + x - M;
-        need = max(need, min(e, x + 1));
-    }
-    return k6_block_max(need, red);
-}
-
+template <class SIM>
 __global__ void __launch_bounds__(K6_THREADS) k6_online(const OnlineParams P) {
     extern __shared__ __align__(16) unsigned char k6_smem[];
-    __shared__ K6Shared sh;
-    const int tid = threadIdx.x;
+    __shared__ K2lShared<32> sh;
+    const int lane = threadIdx.x;
     const int b = blockIdx.x;
     const int n = P.n_each[b];
-    const int W = P.lookahead;
-    // dynamic shared memory: sort keys first (8-byte aligned), then the int arrays
-    u64* keys = reinterpret_cast<u64*>(k6_smem);
-    int* sa = reinterpret_cast<int*>(keys + P.npow2);
-    int* ss = sa + P.n_max;
-    int* so = ss + P.n_max;
-    int* ring = so + P.n_max;
-    int* C = ring + P.L;                 // Sorted-F-Online: the cached list; SOF: started flags
-    int* C2 = C + P.n_max;
-    int* win = C2 + P.n_max;             // 9 arrays of `lookahead` ints for Algorithm 3
-    int* removed = win + W;
-    int* rem = removed + W;
-    int* remT = rem + W;
-    int* remO = remT + W;
-    int* inX = remO + W;
-    int* pm = inX + W;
-    int* xpos = pm + W;
-    int* bout = xpos + W;
-
-    const size_t base = (size_t)b * P.n_max;
-    i64 horizon = 2;
-    for (int i = tid; i < n; i += K6_THREADS) {
-        sa[i] = P.a[base + i]; ss[i] = P.s[base + i]; so[i] = P.o[base + i];
-        C[i] = 0;
+    const int nm = P.n_max;
+    K6Stream q;
+    int* ring = reinterpret_cast<int*>(k6_smem);
+    q.sa = ring + SIM::ring_cells(P.L);
+    q.ss = q.sa + nm; q.so = q.ss + nm; q.started = q.so + nm; q.S = q.started + nm; q.S2 = q.S + nm;
+    q.B = q.S2 + nm;
+    {
+        const size_t at = (size_t)((unsigned char*)(q.B + P.lookahead) - k6_smem);
+        q.win = k2l_arrays<k6_ix>(k6_smem + ((at + 15) & ~(size_t)15), P.lookahead);
     }
-    for (int k = tid; k < P.L; k += K6_THREADS) ring[k] = 0;
-    __syncthreads();
-    for (int i = 0; i < n; ++i) horizon += so[i];      // same in every thread
-    horizon += sa[n - 1];
-    const i64 turn_cap = 4 * (horizon + n) + 64;       // every turn is an arrival, a plan or a wait that ends
+    q.n = n; q.nvis = 0; q.slen = 0; q.sused = 0; q.wlen = 0; q.blen = 0; q.bused = 0; q.tail = 0;
 
-    const int mask = P.L - 1;
-    const int M = P.M;
-    int t = 1, nvis = 0, remaining = n;
-    int fcfs_next = 0;                                  // FCFS: next request in arrival order
-    int ch = 0, ce = 0;                                 // Sorted-F-Online: pending = C[ch .. ce)
+    const size_t base = (size_t)b * nm;
+    i64 sum_o = 0;
+    for (int i = lane; i < n; i += 32) {
+        q.sa[i] = P.a[base + i]; q.ss[i] = P.s[base + i]; q.so[i] = P.o[base + i];
+        q.started[i] = 0;
+        sum_o += q.so[i];
+    }
+    for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
+    __syncwarp();
+    const i64 horizon = 2 + sum_o + q.sa[n - 1];
+    const i64 turn_cap = kv_loop_cap(4 * (horizon + n) + 64);   // every turn is an arrival, a plan or a wait that ends
+
+    SIM sim;
+    sim.attach(ring, P.L);
+    sim.reset(P.M);
+
+    int t = 1, remaining = n;                           // iteration t: the simulator stands at round t - 1
     bool computed = false;
     int t_last = 0, backlog_last = 0, new_since = 0;
     bool changed = true;                                // pending set differs from the one last planned
     i64 latency = 0;
 
     for (i64 turn = 0; remaining > 0; ++turn) {
-        if (turn > kv_loop_cap(turn_cap)) { if (tid == 0) atomicExch(P.status, KV_DEV_LOOP_CAP); break; }
+        if (turn > turn_cap) { if (lane == 0) atomicExch(P.status, KV_DEV_LOOP_CAP); break; }
         // arrivals seen by iteration t
-        const int old = nvis;
-        while (nvis < n && sa[nvis] <= t - 1) ++nvis;
-        const int newly = nvis - old;
+        const bool was_empty = q.nvis == n - remaining;
+        const int old = q.nvis;
+        for (;;) {                                      // 32 at a time: arrivals are in order
+            const int i = q.nvis + lane;
+            const int c = __popc(__ballot_sync(KV_FULL, i < n && q.sa[i] <= t - 1));
+            q.nvis += c;
+            if (c < 32) break;
+        }
+        const int newly = q.nvis - old, pending = q.nvis - (n - remaining);
         if (P.policy == SCHED_POLICY_SORTED_F) {
-            const bool was_empty = (ce == ch);
-            for (int k = tid; k < newly; k += K6_THREADS) C[ce + k] = old + k;
-            ce += newly;
             new_since += newly;
-            __syncthreads();
             if (newly > 0) changed = true;
-            const bool due = ce > ch && (!computed || t - t_last >= P.period || was_empty || 2 * new_since >= backlog_last);
+            const bool due = pending > 0 && (!computed || t - t_last >= P.period || was_empty || 2 * new_since >= backlog_last);
             if (due && !changed) {
                 // same pending set as at the last plan (no arrival, no start since): the plan is a
                 // function of that set alone, so it would come out as the list already is
                 t_last = t;
             } else if (due) {
-                // ---- plan: pending by ascending (s+o, index)
-                const int m = ce - ch;
-                int len = 2;
-                while (len < m) len <<= 1;
-                for (int k = tid; k < len; k += K6_THREADS) {
-                    u64 key = ~0ull;
-                    if (k < m) { const int id = C[ch + k]; key = ((u64)(unsigned)(ss[id] + so[id]) << 32) | (u64)(unsigned)id; }
-                    keys[k] = key;
-                }
-                __syncthreads();
-                k6_bitonic_sort(keys, len);
-                const int wn = m < W ? m : W;
-                for (int k = tid; k < wn; k += K6_THREADS) { win[k] = (int)(keys[k] & 0xffffffffu); removed[k] = 0; }
-                __syncthreads();
-                int done = 0;
-                while (done < wn) {                     // every batch places at least one request
-                    const int k0 = k2l_batch(ss, so, win, wn, (i64)M, 0, 1, removed, rem, remT, remO, inX, pm, xpos,
-                                             bout, P.status, sh.ls);
-                    if (k0 < 1) { if (tid == 0) atomicExch(P.status, KV_DEV_LOOP_CAP); done = wn; break; }
-                    // the batch by ascending (o, index): rank of every member among the members
-                    for (int k = tid; k < k0; k += K6_THREADS) {
-                        const int id = bout[k];
-                        const int key = (so[id] << K6_IDX_BITS) | id;
-                        int rank = 0;
-                        for (int j = 0; j < k0; ++j) { const int jd = bout[j]; rank += (((so[jd] << K6_IDX_BITS) | jd) < key) ? 1 : 0; }
-                        C2[done + rank] = id;
-                    }
-                    done += k0;
-                    __syncthreads();
-                }
-                for (int k = wn + tid; k < m; k += K6_THREADS) C2[k] = (int)(keys[k] & 0xffffffffu);
-                __syncthreads();
-                for (int k = tid; k < m; k += K6_THREADS) C[k] = C2[k];
-                __syncthreads();
-                ch = 0; ce = m;
-                computed = true; t_last = t; backlog_last = m; new_since = 0;
+                q.plan(P.lookahead, lane);
+                computed = true; t_last = t; backlog_last = pending; new_since = 0;
                 changed = false;
             }
         }
@@ -210,43 +250,41 @@ __global__ void __launch_bounds__(K6_THREADS) k6_online(const OnlineParams P) {
         int r = -1, need = 0;
         for (;;) {
             if (P.policy == SCHED_POLICY_FCFS) {
-                r = fcfs_next < nvis ? fcfs_next : -1;
+                r = q.tail < q.nvis ? q.tail : -1;
             } else if (P.policy == SCHED_POLICY_SOF) {
                 int best = INT_MAX;
-                for (int i = tid; i < nvis; i += K6_THREADS)
-                    if (!C[i]) best = min(best, (so[i] << K6_IDX_BITS) | i);
-                best = k6_block_min(best, sh.red);
+                for (int i = lane; i < q.nvis; i += 32)
+                    if (!q.started[i]) best = min(best, (q.so[i] << K6_IDX_BITS) | i);
+                best = kv_warp_min(best);
                 r = best == INT_MAX ? -1 : (best & ((1 << K6_IDX_BITS) - 1));
             } else {
-                r = ch < ce ? C[ch] : -1;
+                r = q.head(P.M, lane, P.status, sh);
             }
             if (r < 0) break;
-            const int s = ss[r], o = so[r];
-            need = k6_window_need(ring, mask, t, s, o, M, sh.red);
+            const int s = q.ss[r], o = q.so[r];
+            need = sim.test(s + 1, o - 1);
             if (need > 0) break;
-            for (int x = tid; x < o; x += K6_THREADS) ring[(t + x) & mask] += s + 1 + x;
-            if (tid == 0) P.start_out[base + KV_IDX(r, n, 1001)] = t - 1;
-            latency += (i64)(t - 1) + o - sa[r];
+            sim.add(s + 1, o - 1);
+            if (lane == 0) { P.start_out[base + KV_IDX(r, n, 1001)] = t - 1; q.started[r] = 1; }
+            latency += (i64)(t - 1) + o - q.sa[r];
             --remaining;
-            if (P.policy == SCHED_POLICY_FCFS) ++fcfs_next;
-            else if (P.policy == SCHED_POLICY_SOF) { if (tid == 0) C[r] = 1; }
-            else { ++ch; changed = true; }
-            __syncthreads();
+            if (P.policy == SCHED_POLICY_FCFS) ++q.tail;
+            else if (P.policy == SCHED_POLICY_SORTED_F) { q.pop(); changed = true; }
+            __syncwarp();
         }
         if (remaining == 0) break;
         // ---- the next iteration at which anything can change
         i64 t_next;
         if (r < 0) {
-            t_next = (i64)sa[nvis] + 1;                 // nothing pending: wait for the next arrival
+            if (q.nvis == n) { if (lane == 0) atomicExch(P.status, KV_DEV_LOOP_CAP); break; }   // a batch gave up
+            t_next = (i64)q.sa[q.nvis] + 1;             // nothing pending: wait for the next arrival
         } else {
             t_next = (i64)t + need;
-            if (nvis < n) t_next = min(t_next, (i64)sa[nvis] + 1);
+            if (q.nvis < n) t_next = min(t_next, (i64)q.sa[q.nvis] + 1);
             if (P.policy == SCHED_POLICY_SORTED_F) t_next = min(t_next, (i64)t_last + P.period);
         }
-        const int d = (int)(t_next - t);
-        for (int k = tid; k < min(d, P.L); k += K6_THREADS) ring[(t + k) & mask] = 0;
+        sim.skip((int)(t_next - t), P.M);
         t = (int)t_next;
-        __syncthreads();
     }
-    if (tid == 0) P.latency_out[b] = latency;
+    if (lane == 0) P.latency_out[b] = latency;
 }
