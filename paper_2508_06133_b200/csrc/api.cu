@@ -7,6 +7,7 @@
 
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -147,6 +148,43 @@ void kv_free(void* p) {
     g_pool_cached += b.bytes;
 }
 
+// Pinned host memory of the handles' read-backs, cached like the device blocks (at most 64 MiB).
+struct PinnedBlock { void* p; size_t bytes; };
+std::vector<PinnedBlock> g_pinned_free;
+size_t g_pinned_cached = 0;
+const size_t kPinnedCap = 64ull << 20;
+
+cudaError_t kv_host_malloc(void** out, size_t* bytes) {        // rounds *bytes up
+    size_t want = 4096;
+    while (want < *bytes) want <<= 1;
+    *bytes = want;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        for (size_t k = 0; k < g_pinned_free.size(); ++k)
+            if (g_pinned_free[k].bytes == want) {
+                *out = g_pinned_free[k].p;
+                g_pinned_cached -= want;
+                g_pinned_free[k] = g_pinned_free.back();
+                g_pinned_free.pop_back();
+                return cudaSuccess;
+            }
+    }
+    return cudaHostAlloc(out, want, cudaHostAllocPortable);
+}
+// no copy from or to the block may be in flight
+void kv_host_free(void* p, size_t bytes) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (g_pinned_cached + bytes <= kPinnedCap) {
+            g_pinned_free.push_back(PinnedBlock{p, bytes});
+            g_pinned_cached += bytes;
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
 template <typename T>
 int dev_alloc(T** p, size_t count) {
     *p = nullptr;
@@ -202,13 +240,9 @@ int validate_instance(i64 total, const int32_t* s, const int32_t* o, i64 M) {
 
 void free_ctx(sched_ctx* h) {
     if (!h) return;
-    void* ptrs[] = {h->d_s, h->d_o, h->d_tbl_id, h->d_tbl_base, h->d_order, h->d_snap_ring, h->d_snap_hdr,
-                    h->d_base_tel, h->d_counter, h->d_status, h->d_tel, h->d_best, h->d_partials, h->d_ticket,
-                    h->d_keys_a, h->d_keys_b, h->d_vals_a, h->d_vals_b, h->d_prefP, h->d_prefO,
-                    h->d_batch_off, h->d_num_batches, h->d_seg_off, h->d_stage, h->d_base_starts,
-                    h->d_state, h->d_sort, h->d_k4, h->d_ls};
+    void* ptrs[] = {h->d_arena, h->d_tel, h->d_stage, h->d_sort, h->d_k4, h->d_ls};
     for (void* p : ptrs) if (p) kv_free(p);
-    if (h->h_pinned) cudaFreeHost(h->h_pinned);
+    kv_host_free(h->h_pinned, h->pinned_bytes);
     if (h->ev_k3_begin) cudaEventDestroy(h->ev_k3_begin);
     if (h->ev_k3_end) cudaEventDestroy(h->ev_k3_end);
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
@@ -228,6 +262,11 @@ int k3_warps(const sched_ctx* h) {
 }
 
 size_t k3_smem_bytes(const sched_ctx* h) { return (size_t)k3_warps(h) * h->ring_cells * sizeof(int); }
+
+// d_result, d_order and d_batch_off as create_common lays them out: {TEL, batches, status}, n, n + 1 ints
+size_t order_at() { return 256; }
+size_t offsets_at(int n) { return order_at() + (((size_t)n * sizeof(int) + 255) & ~(size_t)255); }
+size_t result_bytes(int n) { return offsets_at(n) + ((size_t)n + 1) * sizeof(int); }
 
 int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t* o, i64 M) {
     if (!out) return SCHED_E_INVAL;
@@ -250,10 +289,10 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
     int rc = SCHED_OK;
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaGetDevice"); break; }
-        cudaDeviceProp prop;
-        if (cudaGetDeviceProperties(&prop, h->device) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaGetDeviceProperties"); break; }
-        h->sm_count = prop.multiProcessorCount;
-        h->smem_optin = (int)prop.sharedMemPerBlockOptin;
+        if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
+            cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) {
+            rc = kv_cuda_fail(cudaGetLastError(), "cudaDeviceGetAttribute"); break;
+        }
         h->B = B; h->n = n; h->M = M; h->omax = omax; h->sum_o_max = sum_max;
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
@@ -269,20 +308,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         if (cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaStreamCreate"); break; }
         h->stream = h->own_stream;
         if (cudaEventCreate(&h->ev_k3_begin) != cudaSuccess || cudaEventCreate(&h->ev_k3_end) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaEventCreate"); break; }
-#define A(call) if ((rc = (call)) != SCHED_OK) break
-        A(dev_alloc(&h->d_s, total)); A(dev_alloc(&h->d_o, total));
-        A(dev_alloc(&h->d_tbl_id, total + 2));
-        A(dev_alloc(&h->d_counter, 4)); A(dev_alloc(&h->d_status, 1));
-        A(dev_alloc(&h->d_best, 2)); A(dev_alloc(&h->d_partials, 2 * 4096)); A(dev_alloc(&h->d_ticket, 1));
-        A(dev_alloc(&h->d_state, 4));
-        if (cudaMallocHost(&h->h_pinned, 64) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaMallocHost"); break; }
         if (B == 1) {
-            A(dev_alloc(&h->d_tbl_base, n + 2)); A(dev_alloc(&h->d_order, n));
-            A(dev_alloc(&h->d_base_starts, n)); A(dev_alloc(&h->d_base_tel, 1));
-            A(dev_alloc(&h->d_keys_a, n)); A(dev_alloc(&h->d_keys_b, n));
-            A(dev_alloc(&h->d_vals_a, n)); A(dev_alloc(&h->d_vals_b, n));
-            A(dev_alloc(&h->d_prefP, n + 1)); A(dev_alloc(&h->d_prefO, n + 1));
-            A(dev_alloc(&h->d_batch_off, n + 1)); A(dev_alloc(&h->d_num_batches, 1)); A(dev_alloc(&h->d_seg_off, 2));
             size_t per = (size_t)h->L * sizeof(int);
             // a candidate replays (stride - 1) / 2 positions on average to reach its first moved one:
             // 0.2 % of the list at 256 snapshots, for which the base run stores 256 states instead of n
@@ -290,10 +316,42 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             while ((((i64)n + stride - 1) / stride) * (i64)per > (i64)kSnapBudget) ++stride;
             h->snap_stride = (int)stride;
             h->snap_count = (n + h->snap_stride - 1) / h->snap_stride;
-            A(dev_alloc(&h->d_snap_ring, (size_t)h->snap_count * h->L));
-            A(dev_alloc(&h->d_snap_hdr, h->snap_count));
         }
-#undef A
+        // every array of a fixed size in one block; first pass: its size, second: the addresses
+        size_t used = 0;
+        for (int pass = 0; pass < 2 && rc == SCHED_OK; ++pass) {
+            if (pass == 1 && (rc = dev_alloc(&h->d_arena, used < kPoolMinBlock ? kPoolMinBlock : used)) != SCHED_OK) break;
+            used = 0;
+            auto take = [&](auto** ptr, size_t count) {
+                typedef typename std::remove_reference<decltype(**ptr)>::type T;
+                if (pass == 1) *ptr = (T*)(h->d_arena + used);
+                used += (count * sizeof(T) + 255) & ~(size_t)255;
+            };
+            // what a solver call hands back lies in a row: base TEL, batches, status | order | batch offsets
+            take(&h->d_result, 4);
+            if (B == 1) { take(&h->d_order, n); take(&h->d_batch_off, n + 1); }
+            take(&h->d_s, total); take(&h->d_o, total);
+            take(&h->d_tbl_id, total + 2);
+            take(&h->d_counter, 4);
+            take(&h->d_best, 2); take(&h->d_partials, 2 * 4096); take(&h->d_ticket, 1);
+            take(&h->d_state, 4);
+            if (B == 1) {
+                take(&h->d_tbl_base, n + 2);
+                take(&h->d_base_starts, n);
+                take(&h->d_keys_a, n); take(&h->d_keys_b, n);
+                take(&h->d_vals_a, n); take(&h->d_vals_b, n);
+                take(&h->d_prefP, n + 1); take(&h->d_prefO, n + 1);
+                take(&h->d_seg_off, 2);
+                take(&h->d_snap_ring, (size_t)h->snap_count * h->L);
+                take(&h->d_snap_hdr, h->snap_count);
+            }
+        }
+        if (rc != SCHED_OK) break;
+        h->d_base_tel = (i64*)h->d_result;
+        h->d_num_batches = h->d_result + 2;
+        h->d_status = h->d_result + 3;
+        h->pinned_bytes = 256 + (B == 1 ? result_bytes(n) : 0);
+        if (kv_host_malloc(&h->h_pinned, &h->pinned_bytes) != cudaSuccess) { h->h_pinned = nullptr; rc = kv_cuda_fail(cudaGetLastError(), "cudaHostAlloc"); break; }
         cudaStream_t st = h->stream;
 #define C(call) if ((call) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), #call); break; }
         C(cudaMemcpyAsync(h->d_s, s, total * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -329,12 +387,30 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
                 rc = kv_cuda_fail(cudaGetLastError(), "cudaFuncSetAttribute(MaxDynamicSharedMemorySize)"); break;
             }
         }
-        C(cudaFuncSetAttribute(k3_check_starts, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 2048));
         C(cudaStreamSynchronize(st));       // s, o may be pageable host memory owned by the caller
 #undef C
     } while (0);
     if (rc != SCHED_OK) { free_ctx(h); return rc; }
     *out = h;
+    return SCHED_OK;
+}
+
+// `rows` lists of n entries in ascending (key, value) order -> out.  More than one tile: through
+// tmp_keys / tmp_vals (rows * n entries each).
+template <class KEY>
+int sort_rows(sched_ctx* h, const KEY& src, int n, i64 rows, u64* tmp_keys, int* tmp_vals, int* out) {
+    const int tiles = (n + K1_TILE - 1) / K1_TILE;
+    const i64 total = rows * n, ctas = rows * tiles;
+    if (total >= (1ll << 31) || ctas >= (1ll << 31)) return SCHED_E_UNSUPPORTED;
+    int threads = 32;
+    while (threads < n && threads < K1_TILE) threads <<= 1;
+    k1_tile_sort<<<(unsigned)ctas, threads, 0, h->stream>>>(src, n, tiles, tiles > 1 ? tmp_keys : nullptr, tiles > 1 ? tmp_vals : out);
+    KV_TRY(check_launch(h));
+    if (tiles > 1) {
+        k1_tile_merge<<<(unsigned)((total + K1_MERGE_THREADS - 1) / K1_MERGE_THREADS), K1_MERGE_THREADS, 0, h->stream>>>(
+            tmp_keys, tmp_vals, n, total, out);
+        KV_TRY(check_launch(h));
+    }
     return SCHED_OK;
 }
 
@@ -453,15 +529,20 @@ int read_checked_word() {
     return SCHED_OK;
 }
 
-int read_status(sched_ctx* h) {
-    int* hp = (int*)h->h_pinned;
-    KV_CUDA(cudaMemcpyAsync(hp, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    KV_CUDA(cudaStreamSynchronize(h->stream));
-    if (*hp != KV_DEV_OK) {
+// what the status word of an idle stream says
+int after_status(sched_ctx* h, int status) {
+    if (status != KV_DEV_OK) {
         cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream);
         return SCHED_E_INTERNAL;
     }
     return read_checked_word();
+}
+
+int read_status(sched_ctx* h) {
+    int* hp = (int*)h->h_pinned;
+    KV_CUDA(cudaMemcpyAsync(hp, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    KV_CUDA(cudaStreamSynchronize(h->stream));
+    return after_status(h, *hp);
 }
 
 #ifdef KVSCHED_CHECKED
@@ -601,32 +682,45 @@ int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* ca
         if (starts_out) return SCHED_E_INVAL;
         const i64 total = count * n;
         if (total >= (1ll << 31)) return SCHED_E_UNSUPPORTED;
-        // ids of every candidate by ascending (start, id): K1 with one segment per candidate
-        const size_t need = (size_t)total * (2 * sizeof(u64) + 2 * sizeof(int)) + (size_t)(count + 1) * sizeof(int) + 64;
+        // ids of every candidate by ascending (start, id)
+        const bool tiled = n > K1_TILE;
+        const size_t need = (size_t)total * (sizeof(int) + (tiled ? sizeof(u64) + sizeof(int) : 0)) + 64;
         if (h->sort_cap < need) {
             if (h->d_sort) { kv_free(h->d_sort); h->d_sort = nullptr; h->sort_cap = 0; }
             KV_CUDA(kv_malloc((void**)&h->d_sort, need));
             h->sort_cap = need;
         }
-        u64* ka = (u64*)h->d_sort; u64* kb = ka + total;
-        int* va = (int*)(kb + total); int* vb = va + total; int* seg = vb + total;
-        k1_keys_start_then_id<<<(unsigned)((total + 255) / 256), 256, 0, h->stream>>>((const int*)candidates, n, total, ka, va, seg, (int)count);
-        KV_TRY(check_launch(h));
-        const unsigned mask = key_byte_mask(bits_of((u64)n), 31);
-        k1_radix_sort_segments<<<(unsigned)(count < 65535 ? count : 65535), K1_THREADS, 0, h->stream>>>(ka, va, kb, vb, seg, nullptr, (int)count, mask);
-        KV_TRY(check_launch(h));
+        u64* tmp_keys = tiled ? (u64*)h->d_sort : nullptr;
+        int* tmp_vals = tiled ? (int*)(tmp_keys + total) : nullptr;
+        int* ids = tiled ? tmp_vals + total : (int*)h->d_sort;
+        KV_TRY(sort_rows(h, K1StartKey{(const int*)candidates}, n, count, tmp_keys, tmp_vals, ids));
         StartsEvalParams p;
         memset(&p, 0, sizeof(p));
-        p.n = n; p.L = (h->omax + 8 + 31) & ~31; p.M = (int)h->M; p.tbl_id = h->d_tbl_id;
-        p.starts = (const int*)candidates; p.sorted_ids = va; p.count = count;
-        p.tel_out = (i64*)tel_out; p.feasible_out = feasible_out; p.counter = h->d_counter;
-        KV_CUDA(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned), h->stream));
-        int sw = (int)(((size_t)h->smem_optin - 2048) / ((size_t)p.L * sizeof(int)));
-        if (sw > K3S_WARPS) sw = K3S_WARPS;
-        if (sw < 1) return SCHED_E_UNSUPPORTED;
-        const i64 sctas = (count + sw - 1) / sw;
-        k3_check_starts<<<(unsigned)(sctas < h->sm_count ? sctas : h->sm_count), sw * 32,
-                          (size_t)sw * p.L * sizeof(int), h->stream>>>(p);
+        p.n = n; p.M = (int)h->M; p.tbl_id = h->d_tbl_id;
+        p.starts = (const int*)candidates; p.sorted_ids = ids; p.count = count;
+        p.tel_out = (i64*)tel_out; p.feasible_out = feasible_out;
+        if (h->nm > 0) {
+            p.L = h->L;
+            const size_t smem = k3_smem_bytes(h);
+            switch (h->nm) {
+#define RUN(N) k3_check_starts<ChunkSim<N>><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p)
+                case 1: RUN(1); break;
+                case 2: RUN(2); break;
+                case 4: RUN(4); break;
+                default: RUN(8); break;
+#undef RUN
+            }
+        } else {
+            p.L = (h->omax + 8 + 31) & ~31; p.counter = h->d_counter;
+            KV_CUDA(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned), h->stream));
+            int sw = (int)(((size_t)h->smem_optin - 2048) / ((size_t)p.L * sizeof(int)));
+            if (sw > K3S_WARPS) sw = K3S_WARPS;
+            if (sw < 1) return SCHED_E_UNSUPPORTED;
+            const i64 sctas = (count + sw - 1) / sw;
+            KV_CUDA(cudaFuncSetAttribute(k3_check_starts_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 2048));
+            k3_check_starts_cells<<<(unsigned)(sctas < h->sm_count ? sctas : h->sm_count), sw * 32,
+                                    (size_t)sw * p.L * sizeof(int), h->stream>>>(p);
+        }
         KV_TRY(check_launch(h));
         h->evaluations += count;
         return SCHED_OK;
@@ -719,16 +813,17 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
     if (h->batch_handle) return SCHED_E_INVAL;
     const int n = h->n;
     cudaStream_t st = h->stream;
+    const int* list = h->d_vals_a;              // the batches one behind the other
     if (solver == 0) {
         // S1: ascending (s+o, o, index)
-        k1_keys_total_size<<<(n + 255) / 256, 256, 0, st>>>(h->d_s, h->d_o, n, h->d_keys_a, h->d_vals_a, SCHED_POLICY_SORTED_F);
-        KV_TRY(check_launch(h));
-        k1_radix_sort_segments<<<1, K1_THREADS, 0, st>>>(h->d_keys_a, h->d_vals_a, h->d_keys_b, h->d_vals_b, h->d_seg_off, nullptr, 1,
-                                                          key_byte_mask(bits_of((u64)h->omax), bits_of((u64)h->M)));
-        KV_TRY(check_launch(h));
-        // S2: prefix sums + F-metric batch boundaries
-        k2_prefix_f<<<1, 1024, 0, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->d_prefP, h->d_prefO, h->d_batch_off, h->d_num_batches,
-                                        (i64)h->g_num, (i64)h->g_den);
+        KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_SORTED_F}, n, 1, h->d_keys_a, h->d_vals_b, h->d_vals_a));
+        // S2: prefix sums + F-metric batch boundaries; the sums in shared memory where they fit
+        const size_t bytes = 2 * ((size_t)n + 1) * sizeof(i64);
+        const bool fits = bytes <= (size_t)h->smem_optin - 4096;
+        KV_CUDA(cudaFuncSetAttribute(k2_prefix_f, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 4096));
+        k2_prefix_f<<<1, K2_THREADS, fits ? bytes : 0, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, fits ? nullptr : h->d_prefP,
+                                                             fits ? nullptr : h->d_prefO, h->d_batch_off, h->d_num_batches,
+                                                             (i64)h->g_num, (i64)h->g_den);
         KV_TRY(check_launch(h));
     } else if (solver == 2) {
         KV_TRY(phase1_dp(h));
@@ -736,11 +831,7 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
         KV_TRY(phase1_quantile(h, seed));
     } else {
         // Algorithm 3: ascending (s+o, index), then first fit + improving swaps, batch after batch
-        k1_keys_total_size<<<(n + 255) / 256, 256, 0, st>>>(h->d_s, h->d_o, n, h->d_keys_a, h->d_vals_a, SCHED_POLICY_TOTAL_SIZE);
-        KV_TRY(check_launch(h));
-        k1_radix_sort_segments<<<1, K1_THREADS, 0, st>>>(h->d_keys_a, h->d_vals_a, h->d_keys_b, h->d_vals_b, h->d_seg_off, nullptr, 1,
-                                                          key_byte_mask(0, bits_of((u64)h->M)));
-        KV_TRY(check_launch(h));
+        KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_TOTAL_SIZE}, n, 1, h->d_keys_a, h->d_vals_b, h->d_vals_a));
         if ((i64)h->g_num * h->M + (i64)h->g_den * h->omax >= (1ll << 31)) return SCHED_E_UNSUPPORTED;   // 32-bit weights
         // the solver's arrays in shared memory (20 bytes per request) up to about 11,000 requests
         const size_t bytes = k2l_bytes<unsigned short>(n);
@@ -754,16 +845,11 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
                                                           h->d_vals_b, h->d_batch_off, h->d_num_batches, h->d_status);
         }
         KV_TRY(check_launch(h));
-        KV_CUDA(cudaMemcpyAsync(h->d_vals_a, h->d_vals_b, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, st));
+        list = h->d_vals_b;
     }
     // each batch by ascending (o, index)
-    k1_keys_output_then_id<<<(n + 255) / 256, 256, 0, st>>>(h->d_o, h->d_vals_a, n, h->d_keys_a, h->d_vals_a);
-    KV_TRY(check_launch(h));
-    int grid = n < 4 * h->sm_count ? n : 4 * h->sm_count;
-    k1_radix_sort_segments<<<grid, K1_THREADS, 0, st>>>(h->d_keys_a, h->d_vals_a, h->d_keys_b, h->d_vals_b, h->d_batch_off, h->d_num_batches, 0,
-                                                         key_byte_mask(bits_of((u64)n), bits_of((u64)h->omax)));
-    KV_TRY(check_launch(h));
-    KV_CUDA(cudaMemcpyAsync(h->d_order, h->d_vals_a, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, st));
+    KV_TRY(sort_rows(h, K1BatchKey{h->d_o, list, h->d_batch_off, h->d_num_batches}, n, 1, h->d_keys_a,
+                     list == h->d_vals_a ? h->d_vals_b : h->d_vals_a, h->d_order));
     h->base_ready = false;
     KV_TRY(ensure_base(h));
     if (order_out) KV_CUDA(cudaMemcpyAsync(order_out, h->d_order, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, st));
@@ -778,17 +864,16 @@ static int sorted_f_common_host(sched_handle h, int solver, int32_t* order_out, 
     KV_ENTER(h);
     KV_TRY(sorted_f_common_dev(h, solver, nullptr, nullptr, nullptr, nullptr, seed));
     const int n = h->n;
-    cudaStream_t st = h->stream;
-    int nb = 0;
-    KV_CUDA(cudaMemcpyAsync(&nb, h->d_num_batches, sizeof(int), cudaMemcpyDeviceToHost, st));
-    if (order_out) KV_CUDA(cudaMemcpyAsync(order_out, h->d_order, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, st));
-    if (tel_out) KV_CUDA(cudaMemcpyAsync(tel_out, h->d_base_tel, sizeof(i64), cudaMemcpyDeviceToHost, st));
-    KV_CUDA(cudaStreamSynchronize(st));
+    char* hp = (char*)h->h_pinned;
+    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, result_bytes(n), cudaMemcpyDeviceToHost, h->stream));
+    KV_CUDA(cudaStreamSynchronize(h->stream));
+    const int nb = ((int*)hp)[2], status = ((int*)hp)[3];
+    KV_TRY(after_status(h, status));
+    if (tel_out) *tel_out = *(i64*)hp;
     if (num_batches_out) *num_batches_out = nb;
-    if (batch_offsets_out) {
-        KV_CUDA(cudaMemcpyAsync(batch_offsets_out, h->d_batch_off, (size_t)(nb + 1) * sizeof(int), cudaMemcpyDeviceToHost, st));
-    }
-    return read_status(h);
+    if (order_out) memcpy(order_out, hp + order_at(), (size_t)n * sizeof(int));
+    if (batch_offsets_out) memcpy(batch_offsets_out, hp + offsets_at(n), ((size_t)nb + 1) * sizeof(int));
+    return SCHED_OK;
 }
 
 // Algorithm 2 batch after batch; leaves the batches (members in ascending index) in d_vals_a and the
@@ -1285,6 +1370,9 @@ int sched_debug_set_loop_cap(int32_t cap) {
 int sched_release_cached_memory(void) {
     std::lock_guard<std::mutex> lock(g_pool_mu);
     pool_trim_locked(-1);
+    for (const PinnedBlock& b : g_pinned_free) cudaFreeHost(b.p);
+    g_pinned_free.clear();
+    g_pinned_cached = 0;
     return SCHED_OK;
 }
 

@@ -35,6 +35,9 @@ struct sched_ctx {
     int sm_count;
     int smem_optin;          // max dynamic shared memory per block (bytes)
 
+    unsigned char* d_arena;  // one block that holds every array of a fixed size
+    int* d_result;           // {base TEL (two words), batches, status}; d_order and d_batch_off follow it
+
     int *d_s, *d_o;          // [B*n]
     int2* d_tbl_id;          // (s, o) by request id [B*n]
     int2* d_tbl_base;        // (s, o) by base position [n]
@@ -43,7 +46,8 @@ struct sched_ctx {
     bool batch_handle;       // created by sched_init_batch
     int* d_base_starts;      // start of every position of the base order [n]
     i64* d_state;            // local-search state {current TEL, accepted flag}
-    void* h_pinned;          // 64 bytes of pinned host memory for small read-backs
+    void* h_pinned;          // pinned host memory for read-backs
+    size_t pinned_bytes;
     void* d_sort;            // grow-only scratch for sorting explicit start times
     size_t sort_cap;
     int g_num, g_den;        // prefill weight alpha = g_num / g_den of the batch metric (0/1: the F-metric)

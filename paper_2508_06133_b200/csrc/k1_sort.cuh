@@ -1,139 +1,130 @@
-// K1 -- segmented LSD radix sort of (64-bit key, int32 value) pairs, one CTA per segment
-// (CTAs stride over the segments when there are more segments than CTAs).
+// K1 -- sorting of (64-bit key, 32-bit value) pairs in ascending (key, value) order, in independent rows
+// of n entries; the keys are made on the fly from what they are a function of.
 //
-// Used for the request orderings the method needs: ascending (s+o, o, index) over the whole
-// backlog (the order Algorithm 3 starts from), ascending (o, index) inside every selected batch
-// (Algorithm 1, Phase 1: "sort requests in X* in nondecreasing order of o_i"), and the order
-// policies.  Keys are built so that they are unique (the request index is part of the key or the
-// input is in index order), hence the result does not depend on anything but the keys.
+// Used for the request orderings the method needs: ascending (s+o, o, index) over the whole backlog
+// (the order Algorithm 3 starts from), ascending (o, index) inside every selected batch (Algorithm 1,
+// Phase 1: "sort requests in X* in nondecreasing order of o_i"), and the requests of explicit schedules
+// by start time.  Values are distinct within a row (request ids), so the result does not depend on
+// anything but the pairs.
 //
-// A pass handles one 8-bit digit: a shared-memory histogram, an exclusive scan over the 256 bins,
-// then tiles of 256 elements in order; inside a tile, __match_any_sync groups the lanes of a warp
-// by digit, the per-warp counts are turned into offsets by one thread per digit, and every
-// element is scattered to  bin offset + elements of its digit in earlier tiles/warps + its rank
-// among equal digits in its warp  -- which keeps each pass stable.  Digits whose byte is zero in
-// `byte_mask` are skipped (the host knows how many bits the keys use).
+//   k1_tile_sort    one CTA sorts a tile of up to 1,024 pairs: a bitonic network, exchanges within a
+//                   warp by shuffles, the others through shared memory.
+//   k1_tile_merge   the place of a pair in its row is its place in its tile plus, for every other tile
+//                   of the row, the pairs there that come before it: a binary search each, four tiles
+//                   at a time.  Neighbouring lanes hold neighbouring pairs, so their searches read the
+//                   same lines.
+// Two launches for any n (one up to 1,024) and n / 1024 * 11 search steps per pair.  What bounded the
+// radix sort this replaces, one CTA per row and a chain of 6 to 8 passes over it, was latency.
 #pragma once
 
 #include "common.cuh"
 
-#define K1_THREADS 256
-#define K1_WARPS (K1_THREADS / 32)
+#define K1_TILE 1024
+#define K1_MERGE_THREADS 256
 
-__global__ void __launch_bounds__(K1_THREADS)
-k1_radix_sort_segments(u64* __restrict__ keys_a, int* __restrict__ vals_a,
-                       u64* __restrict__ keys_b, int* __restrict__ vals_b,
-                       const int* __restrict__ seg_off, const int* __restrict__ num_segments_ptr,
-                       int num_segments, unsigned byte_mask) {
-    __shared__ int hist[256];
-    __shared__ int digit_off[256];
-    __shared__ int warp_cnt[K1_WARPS][256];
-    __shared__ int warp_tot[K1_WARPS];
+__device__ __forceinline__ bool k1_less(u64 ka, int va, u64 kb, int vb) { return ka < kb || (ka == kb && va < vb); }
 
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (num_segments_ptr) num_segments = *num_segments_ptr;     // count produced on the device
-    for (int seg = blockIdx.x; seg < num_segments; seg += gridDim.x) {
-    const int lo = seg_off[seg], hi = seg_off[seg + 1];
-    const int m = hi - lo;
-    if (m <= 1) continue;
-    u64* ksrc = keys_a; int* vsrc = vals_a;
-    u64* kdst = keys_b; int* vdst = vals_b;
-
-    for (int byte = 0; byte < 8; ++byte) {
-        if (!((byte_mask >> byte) & 1u)) continue;
-        const int shift = byte * 8;
-        hist[tid] = 0;
-        __syncthreads();
-        for (int i = lo + tid; i < hi; i += K1_THREADS)
-            atomicAdd(&hist[(int)((ksrc[i] >> shift) & 0xff)], 1);
-        __syncthreads();
-        // exclusive scan of the 256 bins: warp scans, then the 8 warp totals
-        {
-            int v = hist[tid], incl = v;
-            for (int d = 1; d < 32; d <<= 1) {
-                int y = __shfl_up_sync(KV_FULL, incl, d);
-                if (lane >= d) incl += y;
+// KEY: a struct with  __device__ u64 key(row, i, n, val&)  for entry i of a row.  blockDim.x: the tile,
+// a power of two of 32 .. K1_TILE; grid: rows * tiles per row.
+template <class KEY>
+__global__ void __launch_bounds__(K1_TILE)
+k1_tile_sort(const KEY src, int n, int tiles, u64* __restrict__ keys, int* __restrict__ vals) {
+    __shared__ u64 sk[K1_TILE];
+    __shared__ int sv[K1_TILE];
+    const int tid = threadIdx.x, size_max = blockDim.x;
+    const int row = blockIdx.x / tiles, i = (blockIdx.x % tiles) * K1_TILE + tid;
+    u64 key = ~0ull;                                     // the padding sorts to the end of a row's last tile
+    int val = 0x7fffffff;
+    if (i < n) key = src.key(row, i, n, val);
+    for (int size = 2; size <= size_max; size <<= 1) {
+        const bool up = (tid & size) == 0 || size == size_max;
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            u64 ok; int ov;
+            if (stride >= 32) {
+                __syncthreads();
+                sk[tid] = key; sv[tid] = val;
+                __syncthreads();
+                ok = sk[tid ^ stride]; ov = sv[tid ^ stride];
+            } else {
+                ok = __shfl_xor_sync(KV_FULL, key, stride); ov = __shfl_xor_sync(KV_FULL, val, stride);
             }
-            if (lane == 31) warp_tot[w] = incl;
-            __syncthreads();
-            int base = 0;
-            for (int k = 0; k < w; ++k) base += warp_tot[k];
-            digit_off[tid] = base + incl - v;
+            const bool low = (tid & stride) == 0;
+            if (k1_less(ok, ov, key, val) == (low == up)) { key = ok; val = ov; }
         }
-        __syncthreads();
-        for (int tile = 0; tile < m; tile += K1_THREADS) {
-            const int i = lo + tile + tid;
-            const bool valid = i < hi;
-            u64 key = 0; int val = 0; int d = 256;
-            if (valid) { key = ksrc[i]; val = vsrc[i]; d = (int)((key >> shift) & 0xff); }
-            for (int k = 0; k < K1_WARPS; ++k) warp_cnt[k][tid] = 0;
-            __syncthreads();
-            const unsigned peers = __match_any_sync(KV_FULL, d);
-            const int rank = __popc(peers & ((1u << lane) - 1u));
-            if (valid && rank == 0) warp_cnt[w][d] = __popc(peers);
-            __syncthreads();
-            {
-                int acc = digit_off[tid];
-                for (int k = 0; k < K1_WARPS; ++k) {
-                    int c = warp_cnt[k][tid];
-                    warp_cnt[k][tid] = acc;
-                    acc += c;
+    }
+    if (i < n) {
+        const size_t at = (size_t)row * n + i;
+        if (keys) keys[at] = key;
+        vals[at] = val;
+    }
+}
+
+// grid: total entries / K1_MERGE_THREADS
+static __global__ void __launch_bounds__(K1_MERGE_THREADS)
+k1_tile_merge(const u64* __restrict__ keys_all, const int* __restrict__ vals_all, int n, i64 total,
+              int* __restrict__ vals_out) {
+    const i64 at = (i64)blockIdx.x * K1_MERGE_THREADS + threadIdx.x;
+    if (at >= total) return;
+    const i64 row0 = at / n * n;
+    const u64* keys = keys_all + row0;
+    const int* vals = vals_all + row0;
+    const int i = (int)(at - row0);
+    const u64 key = keys[i];
+    const int val = vals[i];
+    const int mine = i / K1_TILE, tiles = (n + K1_TILE - 1) / K1_TILE;
+    int rank = i - mine * K1_TILE;
+    for (int t0 = 0; t0 < tiles; t0 += 4) {
+        int lo[4], hi[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int t = t0 + q;
+            lo[q] = t * K1_TILE;
+            hi[q] = t < tiles && t != mine ? min(n, lo[q] + K1_TILE) : lo[q];
+        }
+        for (int step = 0; step < 11; ++step) {          // 1,024 entries: 1,025 answers
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (lo[q] < hi[q]) {
+                    const int mid = (lo[q] + hi[q]) >> 1;
+                    const u64 k = keys[mid];
+                    if (k < key || (k == key && vals[mid] < val)) lo[q] = mid + 1; else hi[q] = mid;
                 }
-                digit_off[tid] = acc;
             }
-            __syncthreads();
-            if (valid) {
-                const int dst = lo + (int)KV_IDX(warp_cnt[w][d] + rank, hi - lo, 701);
-                kdst[dst] = key;
-                vdst[dst] = val;
-            }
-            __syncthreads();
         }
-        u64* tk = ksrc; ksrc = kdst; kdst = tk;
-        int* tv = vsrc; vsrc = vdst; vdst = tv;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rank += lo[q] - (t0 + q) * K1_TILE;
     }
-    if (ksrc != keys_a) {                      // odd number of passes: bring the result home
-        for (int i = lo + tid; i < hi; i += K1_THREADS) { keys_a[i] = ksrc[i]; vals_a[i] = vsrc[i]; }
+    vals_out[row0 + KV_IDX(rank, n, 701)] = val;
+}
+
+// Whole-backlog orders: ascending (s+o, o, index) / (s+o, index) / (o, index).
+struct K1RequestKey {
+    const int *s, *o;
+    int policy;
+    __device__ __forceinline__ u64 key(int, int i, int, int& val) const {
+        val = i;
+        const u64 T = (u64)(s[i] + o[i]), O = (u64)o[i];
+        return policy == SCHED_POLICY_SOF ? O : policy == SCHED_POLICY_TOTAL_SIZE ? T : (T << 32) | O;
     }
-    __syncthreads();
-    }   // segments
-}
+};
 
-// Keys for the whole-backlog sort: (s+o) in the high word, o in the low word; values = request ids
-// in index order, so equal keys keep ascending index.
-__global__ void k1_keys_total_size(const int* __restrict__ s, const int* __restrict__ o, int n,
-                                   u64* __restrict__ keys, int* __restrict__ vals, int policy) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    u64 T = (u64)(s[i] + o[i]), O = (u64)o[i];
-    u64 k;
-    if (policy == SCHED_POLICY_SOF) k = O << 32;
-    else if (policy == SCHED_POLICY_TOTAL_SIZE) k = T << 32;
-    else if (policy == SCHED_POLICY_FCFS) k = 0;
-    else k = (T << 32) | O;
-    keys[i] = k;
-    vals[i] = i;
-}
+// Every batch by ascending (o, index): (batch, o) of the request at list position q.
+struct K1BatchKey {
+    const int *o, *list, *batch_off, *num_batches;
+    __device__ __forceinline__ u64 key(int, int q, int n, int& val) const {
+        const int id = (int)KV_IDX(list[q], n, 702);
+        val = id;
+        int lo = 0, hi = *num_batches - 1;               // the batch with batch_off[b] <= q < batch_off[b+1]
+        while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (batch_off[mid] <= q) lo = mid; else hi = mid - 1; }
+        return ((u64)(unsigned)lo << 32) | (u64)(unsigned)o[id];
+    }
+};
 
-// Keys for the per-batch sort: (o, request id) of the request at every position of `order`.
-__global__ void k1_keys_output_then_id(const int* __restrict__ o, const int* __restrict__ order, int n,
-                                       u64* __restrict__ keys, int* __restrict__ vals) {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    int id = order[q];
-    keys[q] = ((u64)o[id] << 32) | (u64)(unsigned)id;
-    vals[q] = id;
-}
-
-// Keys for checking explicit start times: (start, request id) per candidate; also writes the
-// segment offsets c * n, c = 0 .. count.
-__global__ void k1_keys_start_then_id(const int* __restrict__ starts, int n, long long total,
-                                      u64* __restrict__ keys, int* __restrict__ vals,
-                                      int* __restrict__ seg_off, int count) {
-    long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k <= count) seg_off[k] = (int)(k * n);
-    if (k >= total) return;
-    const int id = (int)(k % n);
-    keys[k] = ((u64)(unsigned)starts[k] << 32) | (u64)(unsigned)id;
-    vals[k] = id;
-}
+// Explicit schedules: (start, id) of request i of schedule `row`.
+struct K1StartKey {
+    const int* starts;
+    __device__ __forceinline__ u64 key(int row, int i, int n, int& val) const {
+        val = i;
+        return (u64)(unsigned)starts[(size_t)row * n + i];
+    }
+};

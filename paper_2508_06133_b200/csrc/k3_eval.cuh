@@ -11,7 +11,7 @@
 //   (k3_policy.cuh)   k3_eval_policy: one warp per (instance, policy) pair: order construction,
 //                     optional prefix-F batching, simulation -- all in shared memory.
 //   k3_check_starts   explicit start times: occupancy by the integer program's memory row
-//                     (Section 6.1), flag raised at the first round above M.
+//                     (Section 6.1), flag raised where a request takes a round above M.
 //
 // The request table is read through L1/L2, 32 positions (256 consecutive bytes) at a time: one such
 // load per 32 admissions, whereas a copy of it in shared memory takes the room of 20 simulators.
@@ -219,9 +219,11 @@ k3_eval_orders(const OrderEvalParams p) {
 
 // ------------------------------------------------------------------------------------------------
 // Explicit start times p[c][i].  One warp per candidate.  Requests are visited in ascending start
-// order (ids sorted by K1 beforehand: sorted_ids[c][k]); the ring then only has to cover omax
-// rounds ahead of the current start.  feasible[c] = 0 as soon as a cell exceeds M (the remaining
-// requests are still summed into the TEL but no longer placed).
+// order (ids sorted by K1 beforehand: sorted_ids[c][k]), so a window never begins before the ones in
+// front of it and the simulator's test answers the question: the schedule stays within M in every
+// round  <=>  every request fits at its start beside those with an earlier start (or a lower id).
+// feasible[c] = 0 from the first that does not (the remaining requests are still summed into the TEL
+// but no longer placed).
 // ------------------------------------------------------------------------------------------------
 struct StartsEvalParams {
     int n, L, M;
@@ -234,8 +236,48 @@ struct StartsEvalParams {
     unsigned int* counter;
 };
 
-__global__ void __launch_bounds__(K3S_WARPS * 32, 1)
+template <class SIM>
+__global__ void __launch_bounds__(SIM::kWarps * 32)
 k3_check_starts(const StartsEvalParams p) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const i64 c = (i64)blockIdx.x * SIM::kWarps + warp;
+    if (c >= p.count) return;
+    const int n = p.n, M = p.M;
+    const int* st_c = p.starts + (size_t)c * n;
+    const int* ids = p.sorted_ids + (size_t)c * n;
+    SIM sim;
+    sim.attach((int*)smem_raw + (size_t)warp * SIM::ring_cells(p.L), p.L);
+    sim.reset(M);
+    i64 tel = 0;
+    bool ok = true;
+    int id_next = lane < n ? ids[lane] : 0;
+    for (int q0 = 0; q0 < n; q0 += 32) {
+        const int cnt = min(32, n - q0), id = id_next;
+        if (q0 + 32 + lane < n) id_next = ids[q0 + 32 + lane];
+        int2 so = make_int2(1, 1);
+        int pi = 0;
+        if (lane < cnt) { so = p.tbl_id[KV_IDX(id, n, 407)]; pi = st_c[id]; tel += (i64)pi + so.y; }
+        if (__any_sync(KV_FULL, pi < 0)) ok = false;                           // the simulator cannot go back
+        for (int k = 0; k < cnt && ok; ++k) {
+            const int sp = __shfl_sync(KV_FULL, so.x, k) + 1, om = __shfl_sync(KV_FULL, so.y, k) - 1;
+            const int wait = __shfl_sync(KV_FULL, pi, k) - sim.start();
+            if (wait < 0) { ok = false; break; }
+            if (wait > 0) sim.skip(wait, M);
+            if (sim.test(sp, om) > 0) ok = false;
+            else sim.add(sp, om);
+        }
+    }
+    for (int d = 16; d >= 1; d >>= 1) tel += __shfl_xor_sync(KV_FULL, tel, d);
+    if (lane == 0) {
+        p.tel_out[c] = tel;
+        if (p.feasible_out) p.feasible_out[c] = ok ? 1 : 0;
+    }
+}
+
+// The same on a ring of single rounds, for decodes beyond what the chunked simulator covers.
+__global__ void __launch_bounds__(K3S_WARPS * 32, 1)
+k3_check_starts_cells(const StartsEvalParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* ring = (int*)smem_raw + (size_t)warp * p.L;
