@@ -50,14 +50,6 @@ const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
 
 int bits_of(u64 v) { int b = 0; while (v) { ++b; v >>= 1; } return b; }
 
-// byte mask for a 64-bit key whose low word uses lo_bits and high word hi_bits
-unsigned key_byte_mask(int lo_bits, int hi_bits) {
-    unsigned m = 0;
-    for (int b = 0; b < (lo_bits + 7) / 8; ++b) m |= 1u << b;
-    for (int b = 0; b < (hi_bits + 7) / 8; ++b) m |= 1u << (4 + b);
-    return m;
-}
-
 // ------------------------------------------------------------------------------------------------
 // Device-memory cache.  Creating and destroying a handle allocates and frees a few hundred MB (base
 // run snapshots, staging, per-candidate scratch); cudaFree of such blocks was seen to take from 2 ms
@@ -341,7 +333,6 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
                 take(&h->d_keys_a, n); take(&h->d_keys_b, n);
                 take(&h->d_vals_a, n); take(&h->d_vals_b, n);
                 take(&h->d_prefP, n + 1); take(&h->d_prefO, n + 1);
-                take(&h->d_seg_off, 2);
                 take(&h->d_snap_ring, (size_t)h->snap_count * h->L);
                 take(&h->d_snap_hdr, h->snap_count);
             }
@@ -366,8 +357,6 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             C(cudaMemsetAsync(h->d_tbl_base, 0, (n + 2) * sizeof(int2), st));
             k3_iota<<<(n + 255) / 256, 256, 0, st>>>(h->d_order, n);
             if ((rc = check_launch(h)) != SCHED_OK) break;
-            int seg[2] = {0, n};
-            C(cudaMemcpyAsync(h->d_seg_off, seg, sizeof(seg), cudaMemcpyHostToDevice, st));
         }
         // opt in to large dynamic shared memory once
         {
@@ -877,7 +866,9 @@ static int sorted_f_common_host(sched_handle h, int solver, int32_t* order_out, 
 }
 
 // Algorithm 2 batch after batch; leaves the batches (members in ascending index) in d_vals_a and the
-// boundaries in d_batch_off / d_num_batches.  Synchronises once per batch (n <= 128 batches).
+// boundaries in d_batch_off / d_num_batches.  Where two tables fit into shared memory ((n+1)(M+1) up to
+// 28,000 cells) in one launch; larger ones with one launch per request, synchronised once per batch
+// (n <= 128 batches).
 static int phase1_dp(sched_handle h) {
     const int n = h->n;
     if (n > 128) return SCHED_E_UNSUPPORTED;
@@ -885,6 +876,14 @@ static int phase1_dp(sched_handle h) {
     const i64 cells_max = (i64)(n + 1) * W;
     if (cells_max > (1ll << 26)) return SCHED_E_UNSUPPORTED;
     cudaStream_t st = h->stream;
+    const size_t small_bytes = k2d_small_bytes(n, W);
+    if (small_bytes <= (size_t)h->smem_optin - 4096) {
+        KV_TRY(ensure_stage(h, (size_t)n * (n + 1) * words * sizeof(unsigned)));
+        KV_CUDA(cudaFuncSetAttribute(k2d_small, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 4096));
+        k2d_small<<<1, K2D_SMALL_THREADS, small_bytes, st>>>(h->d_s, h->d_o, n, W, words, (unsigned*)h->d_stage, h->d_vals_a,
+                                                             h->d_batch_off, h->d_num_batches);
+        return check_launch(h);
+    }
     int *dpA = nullptr, *dpB = nullptr, *small = nullptr;
     unsigned* took = nullptr;
     int rc = SCHED_OK;
@@ -940,64 +939,31 @@ static int phase1_dp(sched_handle h) {
 }
 
 // Algorithm 4 batch after batch; leaves the batches (members in ascending (o, index)) in d_vals_a and
-// the boundaries in d_batch_off / d_num_batches.  Reads the batch size back once per batch.
+// the boundaries in d_batch_off / d_num_batches.
 static int phase1_quantile(sched_handle h, u64 seed) {
     const int n = h->n;
     cudaStream_t st = h->stream;
     // fixed-point ratio key: 2^F must exceed the product of two sizes s+o <= M, and o * 2^F must fit
     const int F = 2 * bits_of((u64)h->M);
     if (F + bits_of((u64)h->omax) > 63) return SCHED_E_UNSUPPORTED;
-    if (!h->d_ls) KV_TRY(dev_alloc(&h->d_ls, 7 * (size_t)n + 32));
-    int* rem = h->d_ls;
-    int* rem_next = rem + n;
-    int* chosen = rem + 2 * (size_t)n;
-    int* va = rem + 3 * (size_t)n;
-    int* vb = rem + 4 * (size_t)n;
-    int* small = rem + 5 * (size_t)n + (n & 1);            // even offset: nothing here needs more
-    u64 *ka = h->d_keys_a, *kb = h->d_keys_b;
-    const int blocks = (n + 255) / 256;
-    // the remaining list: everything, ascending (o, index)
-    k1_keys_total_size<<<blocks, 256, 0, st>>>(h->d_s, h->d_o, n, ka, rem, SCHED_POLICY_SOF);
-    KV_TRY(check_launch(h));
-    k1_radix_sort_segments<<<1, K1_THREADS, 0, st>>>(ka, rem, kb, rem_next, h->d_seg_off, nullptr, 1,
-                                                      key_byte_mask(0, bits_of((u64)h->omax)));
-    KV_TRY(check_launch(h));
-    int zero = 0;
-    KV_CUDA(cudaMemcpyAsync(h->d_batch_off, &zero, sizeof(int), cudaMemcpyHostToDevice, st));
-    const unsigned mask_size = key_byte_mask(bits_of((u64)h->M), 0);
-    const unsigned mask_ratio = key_byte_mask(F + 1 < 32 ? F + 1 : 32, F + 1 > 32 ? F + 1 - 32 : 0) | 0x80u;
-    int nr = n, nb = 0, done = 0;
-    int* hp = (int*)h->h_pinned;
-    while (nr > 0) {
-        const int m = nr / 2 > 1 ? nr / 2 : 1;
-        const int g = (nr + 255) / 256;
-        k2q_begin<<<g, 256, 0, st>>>(rem, nr, seed, nb, ka, va, chosen, small);
-        KV_TRY(check_launch(h));
-        k1_radix_sort_segments<<<1, K1_THREADS, 0, st>>>(ka, va, kb, vb, small + K2Q_SEG1, nullptr, 1, 0xffu);
-        KV_TRY(check_launch(h));
-        k2q_sample_keys<<<(m + 255) / 256, 256, 0, st>>>(rem, va, m, h->d_s, h->d_o, ka);
-        KV_TRY(check_launch(h));
-        k1_radix_sort_segments<<<2, K1_THREADS, 0, st>>>(ka, va, kb, vb, small + K2Q_SEG2, nullptr, 2, mask_size);
-        KV_TRY(check_launch(h));
-        k2q_pass1<<<1, K2Q_THREADS, 0, st>>>(rem, nr, m, h->d_s, h->d_o, h->M, ka, chosen, small);
-        KV_TRY(check_launch(h));
-        k2q_ratio_keys<<<g, 256, 0, st>>>(rem, nr, h->d_s, h->d_o, chosen, F, ka, va);
-        KV_TRY(check_launch(h));
-        k1_radix_sort_segments<<<1, K1_THREADS, 0, st>>>(ka, va, kb, vb, small + K2Q_SEG1, nullptr, 1, mask_ratio);
-        KV_TRY(check_launch(h));
-        k2q_pass2_emit<<<1, K2Q_THREADS, 0, st>>>(rem, rem_next, nr, h->d_s, h->d_o, h->M, va, chosen, small,
-                                                  h->d_vals_a, done, h->d_batch_off, nb);
-        KV_TRY(check_launch(h));
-        KV_CUDA(cudaMemcpyAsync(hp, small + K2Q_COUNT, sizeof(int), cudaMemcpyDeviceToHost, st));
-        KV_CUDA(cudaStreamSynchronize(st));
-        const int took = *hp;
-        if (took < 1 || took > nr) return SCHED_E_INTERNAL;      // every batch places at least one request
-        nr -= took; done += took; ++nb;
-        int* tmp = rem; rem = rem_next; rem_next = tmp;
+    // the three orders: the list by (o, index), its places by size, its places by ratio
+    int* list = h->d_vals_b;
+    int* by_size = (int*)h->d_keys_b;
+    int* by_ratio = by_size + n;
+    KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_SOF}, n, 1, h->d_keys_a, h->d_vals_a, list));
+    KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, 0}, n, 1, h->d_keys_a, h->d_vals_a, by_size));
+    KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, F}, n, 1, h->d_keys_a, h->d_vals_a, by_ratio));
+    const size_t bytes = k2q_bytes<unsigned short>(n), room = (size_t)h->smem_optin - sizeof(K2qShared) - 1024;
+    if (n < 65536 && bytes <= room) {
+        KV_CUDA(cudaFuncSetAttribute(k2_quantile<unsigned short>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
+        k2_quantile<unsigned short><<<1, K2Q_THREADS, bytes, st>>>(h->d_s, h->d_o, list, by_size, by_ratio, n, h->M, seed, nullptr,
+                                                                  h->d_vals_a, h->d_batch_off, h->d_num_batches, h->d_status);
+    } else {
+        if (!h->d_ls) KV_TRY(dev_alloc(&h->d_ls, 7 * (size_t)n + 32));
+        k2_quantile<int><<<1, K2Q_THREADS, 0, st>>>(h->d_s, h->d_o, list, by_size, by_ratio, n, h->M, seed, h->d_ls,
+                                                    h->d_vals_a, h->d_batch_off, h->d_num_batches, h->d_status);
     }
-    KV_CUDA(cudaMemcpyAsync(h->d_num_batches, &nb, sizeof(int), cudaMemcpyHostToDevice, st));
-    KV_CUDA(cudaStreamSynchronize(st));                          // nb lives on this stack frame
-    return SCHED_OK;
+    return check_launch(h);
 }
 
 int sched_sorted_f_dev(sched_handle h, int32_t* order_out, int32_t* batch_offsets_out,

@@ -76,7 +76,6 @@ struct sched_ctx {
     i64 *d_prefP, *d_prefO;  // [n+1]
     int* d_batch_off;        // [n+1]
     int* d_num_batches;      // [1]
-    int* d_seg_off;          // [2] offsets {0, n} for whole-array sorts
 
     // staging for the host-pointer entry points
     void* d_stage;

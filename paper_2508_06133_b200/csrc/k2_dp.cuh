@@ -113,3 +113,93 @@ k2d_apply(const int* __restrict__ s, const int* __restrict__ o, const unsigned* 
         *nb_io = nb; *done_io = done; *nr_io = left;
     }
 }
+
+// ---- small backlogs: everything in one launch of one CTA ---------------------------------------------
+// Both tables in shared memory (rows * (M+1) ints each), `took` in global memory, all batches one after
+// the other.  A warp takes 32 consecutive m of one row at a time, so the 32 answers are one vote.  What
+// bounds the many-launch form at these sizes is the launches: n per batch, and a read-back per batch.
+#define K2D_SMALL_THREADS 1024
+
+__host__ __device__ inline size_t k2d_small_bytes(int n, i64 W) { return (size_t)(n + 1) * (size_t)W * 2 * sizeof(int); }
+
+__global__ void __launch_bounds__(K2D_SMALL_THREADS)
+k2d_small(const int* __restrict__ s, const int* __restrict__ o, int n, int W /* M + 1 */, int words, unsigned* took,
+          int* __restrict__ order_out, int* __restrict__ batch_off, int* __restrict__ num_batches) {
+    extern __shared__ __align__(16) int k2d_smem[];
+    __shared__ int rem[128], mi[128], oi[128];           // the remaining list: ids, sizes, decode lengths
+    __shared__ unsigned char chosen[128];
+    __shared__ int sv[32], sk[32], sm[32], sh_done, sh_left;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int* cur = k2d_smem;
+    int* nxt = cur + (size_t)(n + 1) * W;
+    if (tid < n) rem[tid] = tid;
+    if (tid == 0) batch_off[0] = 0;
+    __syncthreads();
+    int nr = n, nb = 0, done = 0;
+    while (nr > 0) {
+        if (tid < nr) { const int id = rem[tid]; oi[tid] = o[id]; mi[tid] = s[id] + oi[tid]; chosen[tid] = 0; }
+        const int rows = nr + 1;
+        for (int i = tid; i < rows * W; i += K2D_SMALL_THREADS) { const int v = i == 0 ? 0 : K2D_INF; cur[i] = v; nxt[i] = v; }
+        __syncthreads();
+        for (int a = 0; a < nr; ++a) {
+            const int size = mi[a], out = oi[a];
+            unsigned* slab = took + (size_t)a * rows * words;
+            // rows 1 .. a+1 can change; of the others both tables hold the same
+            const int units = (a + 1) * words;
+            for (int u = w; u < units; u += K2D_SMALL_THREADS / 32) {
+                const int k = 1 + u / words, word = u % words, m = word * 32 + lane;
+                bool take = false;
+                if (m < W) {
+                    const int old = cur[k * W + m];
+                    const int src = m >= size ? cur[(k - 1) * W + m - size] : K2D_INF;
+                    take = src != K2D_INF && src + out < old;
+                    nxt[k * W + m] = take ? src + out : old;
+                }
+                const unsigned bits = __ballot_sync(KV_FULL, take);
+                if (lane == 0) slab[(size_t)k * words + word] = bits;
+            }
+            __syncthreads();
+            int* x = cur; cur = nxt; nxt = x;
+        }
+        // best cell by (F ascending, k descending, m ascending)
+        int bv = 0, bk = 0, bm = 0;
+        for (int i = W + tid; i < rows * W; i += K2D_SMALL_THREADS) {
+            const int v = cur[i];
+            if (v == K2D_INF) continue;
+            const int k = i / W, m = i % W;
+            if (k2d_better(v, k, m, bv, bk, bm)) { bv = v; bk = k; bm = m; }
+        }
+        for (int d = 16; d >= 1; d >>= 1) {
+            const int ov = __shfl_xor_sync(KV_FULL, bv, d), ok = __shfl_xor_sync(KV_FULL, bk, d), om = __shfl_xor_sync(KV_FULL, bm, d);
+            if (k2d_better(ov, ok, om, bv, bk, bm)) { bv = ov; bk = ok; bm = om; }
+        }
+        if (lane == 0) { sv[w] = bv; sk[w] = bk; sm[w] = bm; }
+        __syncthreads();
+        bv = sv[lane]; bk = sk[lane]; bm = sm[lane];
+        for (int d = 16; d >= 1; d >>= 1) {
+            const int ov = __shfl_xor_sync(KV_FULL, bv, d), ok = __shfl_xor_sync(KV_FULL, bk, d), om = __shfl_xor_sync(KV_FULL, bm, d);
+            if (k2d_better(ov, ok, om, bv, bk, bm)) { bv = ov; bk = ok; bm = om; }
+        }
+        // walk the requests backwards from the chosen cell (row k can have been reached by request a >= k-1 only)
+        if (tid == 0) {
+            int k = bk, m = bm;
+            for (int a = nr - 1; a >= 0 && k > 0; --a) {
+                if (k > a + 1) continue;
+                const unsigned bits = took[(size_t)a * rows * words + (size_t)k * words + (m >> 5)];
+                if ((bits >> (m & 31)) & 1u) { chosen[a] = 1; k -= 1; m -= mi[a]; }
+            }
+            int left = 0;
+            for (int a = 0; a < nr; ++a) {
+                if (chosen[a]) order_out[KV_IDX(done++, n, 831)] = rem[a];
+                else rem[left++] = rem[a];
+            }
+            sh_done = done; sh_left = left;
+        }
+        __syncthreads();
+        done = sh_done; nr = sh_left; ++nb;
+        if (tid == 0) batch_off[KV_IDX(nb, n + 1, 832)] = done;
+        __syncthreads();
+        if (bk < 1) break;                               // cannot happen: every request fits on its own
+    }
+    if (tid == 0) *num_batches = nb;
+}

@@ -1,276 +1,290 @@
-// K2d -- Algorithm 4 (Quantile Greedy Selection, Section 5.3) as the Phase-1 solver.
+// K2d -- Algorithm 4 (Quantile Greedy Selection, Section 5.3) as the Phase-1 solver, all batches in one
+// launch of one CTA (every batch is built from what the previous ones left).
 //
-// One batch out of the remaining requests, which are kept as a list `rem` in ascending (o, index)
-// -- the order the algorithm sorts by first; taking a batch out keeps the list sorted, so it is
-// sorted once.  Per batch, the host issues
-//   k2q_begin        sampling keys  mix(seed ^ mix(batch * 2^32 + id))  per list position
-//   K1 sort          positions by key: the first m = max(1, floor(nr/2)) are the sample
-//   k2q_sample_keys  s+o and o of the sample members, as two segments
-//   K1 sort          both segments: Q_p and Q_o are the elements at position floor(3 (m-1) / 10)
-//   k2q_pass1        first fit over the list under both thresholds (one CTA)
-//   k2q_ratio_keys   o/(s+o) of the positions not yet chosen as a fixed-point key
-//   K1 sort          positions by that key (stable: equal ratios keep the list order)
-//   k2q_pass2_emit   first fit over the sorted positions, then the batch (already in ascending
-//                    (o, index), being a sub-list of rem) and the compacted remaining list
-// and reads the batch size back.
+// Per batch, over the nr remaining requests, which the algorithm lists in ascending (o, index):
+//   sample    the m = max(1, floor(nr/2)) requests with the smallest keys
+//             mix(seed ^ mix(batch * 2^32 + id)); Q_p and Q_o are the sample's (s+o) and o at position
+//             floor(3 (m-1) / 10) of their ascending orders;
+//   pass 1    first fit down the list over the requests with s+o <= Q_p and o <= Q_o;
+//   pass 2    first fit over the others in ascending o/(s+o), equal ratios in list order;
+//   batch     the requests taken, in list order.
+//
+// Nothing is sorted per batch.  The three orders (list, size, ratio) do not change, so they are sorted
+// once and what has been taken is skipped (and dropped from the lists when it makes up half of them).
+// The m-th smallest key is found with one histogram of the keys' leading 12 bits and a ranking of the
+// few keys of the bin it falls in (further bits where a bin holds more than K2Q_CAND); the elements at
+// a position of the sample's orders by counting sample members along the lists.
 //
 // The ratio key floor(o * 2^F / (s+o)) orders the requests exactly as the rationals do when
 // 2^F exceeds the product of any two denominators: two different ratios differ by at least
 // 1 / ((s_a+o_a)(s_b+o_b)) > 2^-F, so their keys differ; equal ratios give equal keys.
 //
 // First fit is sequential by definition (whether a request is admitted depends on the memory the
-// earlier ones took).  Here a CTA takes 1024 list positions at a time: requests that cannot fit
+// earlier ones took).  Here a CTA takes 1,024 list positions at a time: requests that cannot fit
 // even alone in what is left are dropped (the free memory only shrinks, so they would be refused
 // at their turn anyway), an inclusive scan over the sizes of the others finds the first one that
 // no longer fits after its predecessors; everything before it is admitted, it is refused, and the
-// walk goes on right after it.  Every turn either finishes a tile or admits at least one request.
+// walk goes on right after it.  Every turn either finishes a tile or admits at least one request; the
+// walk ends when not even the smallest request would fit.
+//
+// What bounds it: barriers, about 15 per batch and 2 per turn.  The arrays are in shared memory (19
+// bytes per request, 10,000 requests) where they fit.
 #pragma once
 
 #include "common.cuh"
 
-#define K1_THREADS 256
-#define K1_WARPS (K1_THREADS / 32)
-
-__global__ void __launch_bounds__(K1_THREADS)
-k1_radix_sort_segments(u64* __restrict__ keys_a, int* __restrict__ vals_a,
-                       u64* __restrict__ keys_b, int* __restrict__ vals_b,
-                       const int* __restrict__ seg_off, const int* __restrict__ num_segments_ptr,
-                       int num_segments, unsigned byte_mask) {
-    __shared__ int hist[256];
-    __shared__ int digit_off[256];
-    __shared__ int warp_cnt[K1_WARPS][256];
-    __shared__ int warp_tot[K1_WARPS];
-
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (num_segments_ptr) num_segments = *num_segments_ptr;     // count produced on the device
-    for (int seg = blockIdx.x; seg < num_segments; seg += gridDim.x) {
-    const int lo = seg_off[seg], hi = seg_off[seg + 1];
-    const int m = hi - lo;
-    if (m <= 1) continue;
-    u64* ksrc = keys_a; int* vsrc = vals_a;
-    u64* kdst = keys_b; int* vdst = vals_b;
-
-    for (int byte = 0; byte < 8; ++byte) {
-        if (!((byte_mask >> byte) & 1u)) continue;
-        const int shift = byte * 8;
-        hist[tid] = 0;
-        __syncthreads();
-        for (int i = lo + tid; i < hi; i += K1_THREADS)
-            atomicAdd(&hist[(int)((ksrc[i] >> shift) & 0xff)], 1);
-        __syncthreads();
-        // exclusive scan of the 256 bins: warp scans, then the 8 warp totals
-        {
-            int v = hist[tid], incl = v;
-            for (int d = 1; d < 32; d <<= 1) {
-                int y = __shfl_up_sync(KV_FULL, incl, d);
-                if (lane >= d) incl += y;
-            }
-            if (lane == 31) warp_tot[w] = incl;
-            __syncthreads();
-            int base = 0;
-            for (int k = 0; k < w; ++k) base += warp_tot[k];
-            digit_off[tid] = base + incl - v;
-        }
-        __syncthreads();
-        for (int tile = 0; tile < m; tile += K1_THREADS) {
-            const int i = lo + tile + tid;
-            const bool valid = i < hi;
-            u64 key = 0; int val = 0; int d = 256;
-            if (valid) { key = ksrc[i]; val = vsrc[i]; d = (int)((key >> shift) & 0xff); }
-            for (int k = 0; k < K1_WARPS; ++k) warp_cnt[k][tid] = 0;
-            __syncthreads();
-            const unsigned peers = __match_any_sync(KV_FULL, d);
-            const int rank = __popc(peers & ((1u << lane) - 1u));
-            if (valid && rank == 0) warp_cnt[w][d] = __popc(peers);
-            __syncthreads();
-            {
-                int acc = digit_off[tid];
-                for (int k = 0; k < K1_WARPS; ++k) {
-                    int c = warp_cnt[k][tid];
-                    warp_cnt[k][tid] = acc;
-                    acc += c;
-                }
-                digit_off[tid] = acc;
-            }
-            __syncthreads();
-            if (valid) {
-                const int dst = lo + (int)KV_IDX(warp_cnt[w][d] + rank, hi - lo, 701);
-                kdst[dst] = key;
-                vdst[dst] = val;
-            }
-            __syncthreads();
-        }
-        u64* tk = ksrc; ksrc = kdst; kdst = tk;
-        int* tv = vsrc; vsrc = vdst; vdst = tv;
-    }
-    if (ksrc != keys_a) {                      // odd number of passes: bring the result home
-        for (int i = lo + tid; i < hi; i += K1_THREADS) { keys_a[i] = ksrc[i]; vals_a[i] = vsrc[i]; }
-    }
-    __syncthreads();
-    }   // segments
-}
-
-__global__ void k1_keys_total_size(const int* __restrict__ s, const int* __restrict__ o, int n,
-                                   u64* __restrict__ keys, int* __restrict__ vals, int policy) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    u64 T = (u64)(s[i] + o[i]), O = (u64)o[i];
-    u64 k;
-    if (policy == SCHED_POLICY_SOF) k = O << 32;
-    else if (policy == SCHED_POLICY_TOTAL_SIZE) k = T << 32;
-    else if (policy == SCHED_POLICY_FCFS) k = 0;
-    else k = (T << 32) | O;
-    keys[i] = k;
-    vals[i] = i;
-}
-
-
 #define K2Q_THREADS 1024
-#define K2Q_CHOSEN_KEY (1ull << 63)
+#define K2Q_BINS 4096
+#define K2Q_CAND 512
+enum { K2Q_SAMPLE = 1, K2Q_NEW = 2, K2Q_GONE = 4 };
 
-// layout of the small device state (ints)
-#define K2Q_COUNT 0        // size of the batch just selected
-#define K2Q_MEM_LO 2       // memory used after pass 1 (low / high word)
-#define K2Q_MEM_HI 3
-#define K2Q_SEG1 4         // {0, nr}
-#define K2Q_SEG2 6         // {0, m, 2m}
-#define K2Q_SMALL_INTS 16
-
-__global__ void k2q_begin(const int* __restrict__ rem, int nr, u64 seed, int batch,
-                          u64* __restrict__ keys, int* __restrict__ vals, int* __restrict__ chosen,
-                          int* __restrict__ small) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a == 0) {
-        const int m = nr / 2 > 1 ? nr / 2 : 1;
-        small[K2Q_SEG1] = 0; small[K2Q_SEG1 + 1] = nr;
-        small[K2Q_SEG2] = 0; small[K2Q_SEG2 + 1] = m; small[K2Q_SEG2 + 2] = 2 * m;
+// Entry i of the list in ascending (o, index): its size, or its ratio key; the value is the place i.
+struct K2qSlotKey {
+    const int *s, *o, *list;
+    int F;                       // 0: size
+    __device__ __forceinline__ u64 key(int, int i, int n, int& val) const {
+        val = i;
+        const int id = (int)KV_IDX(list[i], n, 821);
+        const u64 T = (u64)(s[id] + o[id]);
+        return F ? ((u64)o[id] << F) / T : T;
     }
-    if (a >= nr) return;
-    const int id = rem[a];
-    keys[a] = kv_mix64(seed ^ kv_mix64(((u64)(unsigned)batch << 32) + (u64)id));
-    vals[a] = a;
-    chosen[a] = 0;
-}
-
-__global__ void k2q_sample_keys(const int* __restrict__ rem, const int* __restrict__ by_key, int m,
-                                const int* __restrict__ s, const int* __restrict__ o, u64* __restrict__ keys) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= m) return;
-    const int id = rem[by_key[r]];
-    keys[r] = (u64)(s[id] + o[id]);
-    keys[m + r] = (u64)o[id];
-}
-
-__global__ void k2q_ratio_keys(const int* __restrict__ rem, int nr, const int* __restrict__ s, const int* __restrict__ o,
-                               const int* __restrict__ chosen, int F, u64* __restrict__ keys, int* __restrict__ vals) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= nr) return;
-    const int id = rem[a];
-    keys[a] = chosen[a] ? K2Q_CHOSEN_KEY : (((u64)o[id] << F) / (u64)(s[id] + o[id]));
-    vals[a] = a;
-}
-
-struct K2qShared {
-    i64 warp_tot[32];
-    i64 sum;
-    int first;
-    int iwarp[32];
 };
 
-// First fit over list[0 .. cnt) (list == nullptr: the positions 0 .. cnt-1 themselves).  elig(a, T, o)
-// says whether position a may be admitted at all.  Returns the memory in use afterwards; sets
-// chosen[a] = 1 for every admitted position.  Called by all K2Q_THREADS threads.
-template <typename Elig>
-__device__ i64 k2q_first_fit(const int* __restrict__ list, int cnt, const int* __restrict__ rem,
-                             const int* __restrict__ s, const int* __restrict__ o, i64 M, i64 mem,
-                             int* __restrict__ chosen, Elig elig, K2qShared& sh) {
+template <typename IX>
+struct K2qArrays {               // by place in the list of all requests
+    int *T, *O, *id;
+    IX *L, *TL, *RL;             // places in list / size / ratio order
+    unsigned char* flag;
+};
+template <typename IX>
+__host__ __device__ inline size_t k2q_bytes(int n) { return (size_t)n * (3 * sizeof(int) + 3 * sizeof(IX) + 1) + 16; }
+
+struct K2qShared {
+    int hist[K2Q_BINS];
+    u64 cand_key[K2Q_CAND];
+    int cand[K2Q_CAND];
+    u64 tot[32];
+    u64 pick[2];
+    int bin, bin_count, bin_before, ncand, Qp, Qo, min_T;
+};
+
+// exclusive scan of one value per thread over the CTA; `total` in every thread.  Ends with a barrier
+// between its reads of sh.tot and the caller.
+__device__ __forceinline__ u64 k2q_scan(u64 v, u64& total, K2qShared& sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    u64 incl = v;
+    for (int d = 1; d < 32; d <<= 1) { const u64 y = __shfl_up_sync(KV_FULL, incl, d); if (lane >= d) incl += y; }
+    if (lane == 31) sh.tot[w] = incl;
+    __syncthreads();
+    u64 t = sh.tot[lane];
+    for (int d = 1; d < 32; d <<= 1) { const u64 y = __shfl_up_sync(KV_FULL, t, d); if (lane >= d) t += y; }
+    total = __shfl_sync(KV_FULL, t, 31);
+    const u64 before = __shfl_sync(KV_FULL, t, w > 0 ? w - 1 : 0);
+    __syncthreads();
+    return incl - v + (w > 0 ? before : 0);
+}
+
+// First fit over list[0 .. len); kRatio: everything not taken yet, otherwise sizes up to Qp and decodes
+// up to Qo of a list in ascending o.  Flags what it takes; returns the memory in use afterwards.
+template <bool kRatio, typename IX>
+__device__ i64 k2q_first_fit(const K2qArrays<IX>& a, const IX* list, int len, i64 M, i64 mem, K2qShared& sh) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    int pos = 0;
-    while (pos < cnt) {                                   // pos grows by at least one per turn
+    const int Qp = sh.Qp, Qo = sh.Qo, min_T = sh.min_T;
+    int pos = 0, par = 0;
+    while (pos < len) {                                   // pos grows by at least one per turn
         const i64 slack = M - mem;
-        if (slack < 2) break;                             // every request has s + o >= 2
-        if (tid == 0) sh.first = K2Q_THREADS;
+        if (slack < min_T) break;
+        if (!kRatio && a.O[list[pos]] > Qo) break;
         const int idx = pos + tid;
-        int a = -1;
-        i64 T = 0;
-        if (idx < cnt) {
-            a = list ? list[idx] : idx;
-            const int id = rem[a];
-            const int oi = o[id];
-            const i64 Ti = (i64)s[id] + oi;
-            if (Ti <= slack && elig(a, Ti, oi)) T = Ti;
+        int slot = 0;
+        u64 T = 0;
+        if (idx < len) {
+            slot = list[idx];
+            const int t = a.T[slot];
+            if (!(a.flag[slot] & (K2Q_NEW | K2Q_GONE)) && t <= slack && (kRatio || (t <= Qp && a.O[slot] <= Qo))) T = (u64)t;
         }
-        i64 incl = T;
-        for (int d = 1; d < 32; d <<= 1) {
-            const i64 y = __shfl_up_sync(KV_FULL, incl, d);
-            if (lane >= d) incl += y;
+        u64 incl = T;
+        for (int d = 1; d < 32; d <<= 1) { const u64 y = __shfl_up_sync(KV_FULL, incl, d); if (lane >= d) incl += y; }
+        if (lane == 31) sh.tot[w] = incl;
+        __syncthreads();
+        u64 t = sh.tot[lane];
+        for (int d = 1; d < 32; d <<= 1) { const u64 y = __shfl_up_sync(KV_FULL, t, d); if (lane >= d) t += y; }
+        const u64 total = __shfl_sync(KV_FULL, t, 31), before = __shfl_sync(KV_FULL, t, w > 0 ? w - 1 : 0);
+        if (w > 0) incl += before;
+        // the first refused one and the memory taken in front of it, in one word (sums stay below 2^41)
+        if (total > (u64)slack) {
+            const unsigned v = __ballot_sync(KV_FULL, T > 0 && incl > (u64)slack);
+            if (v && lane == __ffs(v) - 1) atomicMin(&sh.pick[par], ((u64)tid << 44) | (incl - T));
         }
-        if (lane == 31) sh.warp_tot[w] = incl;
         __syncthreads();
-        for (int k = 0; k < w; ++k) incl += sh.warp_tot[k];
-        if (T > 0 && incl > slack) atomicMin(&sh.first, tid);
-        __syncthreads();
-        const int f = sh.first;
-        if (T > 0 && tid < f) chosen[a] = 1;
-        if (f < K2Q_THREADS ? tid == f : tid == K2Q_THREADS - 1) sh.sum = f < K2Q_THREADS ? incl - T : incl;
-        __syncthreads();
-        mem += sh.sum;
-        pos += f < K2Q_THREADS ? f + 1 : K2Q_THREADS;
+        const u64 pick = sh.pick[par];
+        const int first = pick == ~0ull ? K2Q_THREADS : (int)(pick >> 44);
+        if (T > 0 && tid < first) a.flag[slot] |= K2Q_NEW;
+        mem += (i64)(pick == ~0ull ? total : pick & ((1ull << 44) - 1));
+        pos += first < K2Q_THREADS ? first + 1 : K2Q_THREADS;
+        par ^= 1;
+        if (tid == 0) sh.pick[par] = ~0ull;               // read again two barriers from here
     }
+    __syncthreads();
+    if (tid == 0) { sh.pick[0] = ~0ull; sh.pick[1] = ~0ull; }
+    __syncthreads();
     return mem;
 }
 
-__global__ void __launch_bounds__(K2Q_THREADS)
-k2q_pass1(const int* __restrict__ rem, int nr, int m, const int* __restrict__ s, const int* __restrict__ o, i64 M,
-          const u64* __restrict__ sorted_sample /* s+o at [0,m), o at [m,2m) */, int* __restrict__ chosen,
-          int* __restrict__ small) {
-    __shared__ K2qShared sh;
-    const int q = (int)((3ll * (m - 1)) / 10);
-    const i64 Qp = (i64)sorted_sample[q], Qo = (i64)sorted_sample[m + q];
-    const i64 mem = k2q_first_fit(nullptr, nr, rem, s, o, M, 0,
-                                  chosen, [=](int, i64 T, int oi) { return T <= Qp && (i64)oi <= Qo; }, sh);
-    if (threadIdx.x == 0) {
-        small[K2Q_MEM_LO] = (int)(mem & 0xffffffffll);
-        small[K2Q_MEM_HI] = (int)(mem >> 32);
+// list[0 .. len) without what is gone, in the same order; returns the new length
+template <typename IX>
+__device__ int k2q_compact(const K2qArrays<IX>& a, IX* list, int len, K2qShared& sh) {
+    int left = 0;
+    for (int base = 0; base < len; base += K2Q_THREADS) {
+        const int idx = base + threadIdx.x;
+        const IX slot = idx < len ? list[idx] : (IX)0;
+        const bool keep = idx < len && !(a.flag[slot] & K2Q_GONE);
+        u64 total;
+        const int rank = (int)k2q_scan(keep ? 1 : 0, total, sh);
+        if (keep) list[left + rank] = slot;
+        left += (int)total;
     }
+    __syncthreads();
+    return left;
 }
 
-// Pass 2, then hand the batch out.  by_ratio: the list positions in ascending ratio (positions
-// chosen in pass 1 sort to the end and are not eligible).  The batch is appended to order_out at
-// `done`, batch_off[nb + 1] is set, rem_next receives the positions not chosen, in list order.
+// list: request ids by ascending (o, index); by_size, by_ratio: places in it.  scratch: k2q_bytes<int>(n)
+// bytes of global memory, or nullptr: the arrays are in dynamic shared memory.  Leaves the batches one
+// behind the other in order_out, their members in list order, and the boundaries in batch_off.
+template <typename IX>
 __global__ void __launch_bounds__(K2Q_THREADS)
-k2q_pass2_emit(const int* __restrict__ rem, int* __restrict__ rem_next, int nr, const int* __restrict__ s,
-               const int* __restrict__ o, i64 M, const int* __restrict__ by_ratio, int* __restrict__ chosen,
-               int* __restrict__ small, int* __restrict__ order_out, int done, int* __restrict__ batch_off, int nb) {
+k2_quantile(const int* __restrict__ s, const int* __restrict__ o, const int* __restrict__ list,
+            const int* __restrict__ by_size, const int* __restrict__ by_ratio, int n, i64 M, u64 seed, void* scratch,
+            int* __restrict__ order_out, int* __restrict__ batch_off, int* __restrict__ num_batches, int* status) {
+    extern __shared__ __align__(16) unsigned char k2q_smem[];
     __shared__ K2qShared sh;
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const i64 mem0 = ((i64)small[K2Q_MEM_HI] << 32) | (i64)(unsigned)small[K2Q_MEM_LO];
-    k2q_first_fit(by_ratio, nr, rem, s, o, M, mem0, chosen,
-                  [=](int a, i64, int) { return chosen[a] == 0; }, sh);
-    __syncthreads();                                      // chosen[] of this CTA is complete
-    int taken = 0;                                        // chosen positions before this tile
-    for (int base = 0; base < nr; base += K2Q_THREADS) {
-        const int a = base + tid;
-        const int flag = (a < nr) ? chosen[a] : 0;
-        int incl = flag;
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(KV_FULL, incl, d);
-            if (lane >= d) incl += y;
-        }
-        if (lane == 31) sh.iwarp[w] = incl;
-        __syncthreads();
-        int before = 0, total = 0;
-        for (int k = 0; k < 32; ++k) { const int c = sh.iwarp[k]; if (k < w) before += c; total += c; }
-        const int rank = taken + before + incl - flag;    // chosen positions before a
-        if (a < nr) {
-            if (flag) order_out[done + rank] = rem[a];
-            else rem_next[a - rank] = rem[a];
-        }
-        taken += total;
-        __syncthreads();
+    const int tid = threadIdx.x, lane = tid & 31;
+    K2qArrays<IX> a;
+    {
+        int* p = scratch ? (int*)scratch : (int*)k2q_smem;
+        a.T = p; a.O = p + n; a.id = p + 2 * (size_t)n;
+        a.L = (IX*)(p + 3 * (size_t)n); a.TL = a.L + n; a.RL = a.TL + n;
+        a.flag = (unsigned char*)(a.RL + n);
     }
-    if (tid == 0) {
-        small[K2Q_COUNT] = taken;
-        batch_off[nb + 1] = done + taken;
+    for (int p = tid; p < n; p += K2Q_THREADS) {
+        const int id = list[p];
+        a.T[p] = s[id] + o[id]; a.O[p] = o[id]; a.id[p] = id;
+        a.L[p] = (IX)p; a.TL[p] = (IX)by_size[p]; a.RL[p] = (IX)by_ratio[p];
+        a.flag[p] = 0;
     }
+    if (tid == 0) { batch_off[0] = 0; sh.pick[0] = ~0ull; sh.pick[1] = ~0ull; }
+    __syncthreads();
+    int len = n, nr = n, done = 0, nb = 0;
+    while (nr > 0) {
+        const int m = nr / 2 > 1 ? nr / 2 : 1;
+        auto key_of = [&](int slot) { return kv_mix64(seed ^ kv_mix64(((u64)(unsigned)nb << 32) + (u64)a.id[slot])); };
+        // ---- the sample: keys whose leading bits are below `top`, and the first of those that have them equal
+        int shift = 64 - 12, before = 0;
+        u64 top = 0;
+        for (;;) {
+            for (int k = tid; k < K2Q_BINS; k += K2Q_THREADS) sh.hist[k] = 0;
+            if (tid == 0) { sh.ncand = 0; sh.min_T = INT_MAX; }
+            __syncthreads();
+            for (int i = tid; i < len; i += K2Q_THREADS) {
+                const int slot = a.L[i];
+                if (a.flag[slot] & K2Q_GONE) continue;
+                const u64 h = key_of(slot);
+                if (shift == 64 - 12 || (h >> (shift + 12)) == top) atomicAdd(&sh.hist[(int)(h >> shift) & (K2Q_BINS - 1)], 1);
+            }
+            __syncthreads();
+            int c[K2Q_BINS / K2Q_THREADS], sum = 0;
+            u64 total;
+#pragma unroll
+            for (int k = 0; k < K2Q_BINS / K2Q_THREADS; ++k) { c[k] = sh.hist[tid * (K2Q_BINS / K2Q_THREADS) + k]; sum += c[k]; }
+            int ex = (int)k2q_scan((u64)sum, total, sh);
+            const int want = m - before;
+            if (ex < want && want <= ex + sum) {
+#pragma unroll
+                for (int k = 0; k < K2Q_BINS / K2Q_THREADS; ++k) {
+                    if (ex < want && want <= ex + c[k]) { sh.bin = tid * (K2Q_BINS / K2Q_THREADS) + k; sh.bin_count = c[k]; sh.bin_before = ex; }
+                    ex += c[k];
+                }
+            }
+            __syncthreads();
+            top = (top << 12) | (u64)sh.bin;
+            before += sh.bin_before;
+            if (sh.bin_count <= K2Q_CAND || shift < 12) break;             // 4 bits: at most 16 distinct keys
+            shift -= 12;
+            __syncthreads();
+        }
+        for (int i = tid; i < len; i += K2Q_THREADS) {
+            const int slot = a.L[i];
+            if (a.flag[slot] & K2Q_GONE) continue;
+            const u64 h = key_of(slot), lead = h >> shift;
+            a.flag[slot] = lead < top ? K2Q_SAMPLE : 0;
+            if (lead == top) {
+                const int k = (int)KV_IDX(atomicAdd(&sh.ncand, 1), K2Q_CAND, 822);
+                sh.cand_key[k] = h; sh.cand[k] = slot;
+            }
+        }
+        __syncthreads();
+        if (tid < sh.ncand) {
+            const u64 h = sh.cand_key[tid];
+            int rank = 0;
+            for (int k = 0; k < sh.ncand; ++k) rank += sh.cand_key[k] < h ? 1 : 0;
+            if (rank < m - before) a.flag[sh.cand[tid]] = K2Q_SAMPLE;
+        }
+        __syncthreads();
+        // ---- quantiles: the q-th sample member along the list (o) and along the sizes (s+o)
+        const int E = (len + K2Q_THREADS - 1) / K2Q_THREADS, i0 = min(len, tid * E), i1 = min(len, i0 + E);
+        {
+            const int q = (int)((3ll * (m - 1)) / 10);
+            int cl = 0, ct = 0, least = INT_MAX;
+            for (int i = i0; i < i1; ++i) {
+                const int fl = a.flag[a.L[i]], slot = a.TL[i], ft = a.flag[slot];
+                cl += (fl & (K2Q_SAMPLE | K2Q_GONE)) == K2Q_SAMPLE;
+                ct += (ft & (K2Q_SAMPLE | K2Q_GONE)) == K2Q_SAMPLE;
+                if (!(ft & K2Q_GONE) && least == INT_MAX) least = a.T[slot];
+            }
+            least = kv_warp_min(least);
+            if (lane == 0 && least != INT_MAX) atomicMin(&sh.min_T, least);
+            u64 total;
+            const u64 ex = k2q_scan(((u64)(unsigned)ct << 32) | (u64)(unsigned)cl, total, sh);
+            const int el = (int)(ex & 0xffffffffu), et = (int)(ex >> 32);
+            if (el <= q && q < el + cl) {
+                int k = el;
+                for (int i = i0; i < i1; ++i) {
+                    const int slot = a.L[i];
+                    if ((a.flag[slot] & (K2Q_SAMPLE | K2Q_GONE)) == K2Q_SAMPLE && k++ == q) { sh.Qo = a.O[slot]; break; }
+                }
+            }
+            if (et <= q && q < et + ct) {
+                int k = et;
+                for (int i = i0; i < i1; ++i) {
+                    const int slot = a.TL[i];
+                    if ((a.flag[slot] & (K2Q_SAMPLE | K2Q_GONE)) == K2Q_SAMPLE && k++ == q) { sh.Qp = a.T[slot]; break; }
+                }
+            }
+            __syncthreads();
+        }
+        // ---- the two passes
+        i64 mem = k2q_first_fit<false>(a, a.L, len, M, 0, sh);
+        mem = k2q_first_fit<true>(a, a.RL, len, M, mem, sh);
+        // ---- hand the batch out
+        int mine = 0;
+        for (int i = i0; i < i1; ++i) mine += (a.flag[a.L[i]] & K2Q_NEW) ? 1 : 0;
+        u64 total;
+        int at = done + (int)k2q_scan((u64)mine, total, sh);
+        for (int i = i0; i < i1; ++i) {
+            const int slot = a.L[i];
+            if (a.flag[slot] & K2Q_NEW) { order_out[KV_IDX(at++, n, 823)] = a.id[slot]; a.flag[slot] = K2Q_GONE; }
+        }
+        const int taken = (int)total;
+        if (taken < 1) { if (tid == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }      // every batch places a request
+        done += taken; nr -= taken; ++nb;
+        if (tid == 0) batch_off[KV_IDX(nb, n + 1, 824)] = done;
+        __syncthreads();
+        if (2 * nr <= len && len > K2Q_THREADS / 4) {
+            const int kept = k2q_compact(a, a.L, len, sh);
+            k2q_compact(a, a.TL, len, sh);
+            k2q_compact(a, a.RL, len, sh);
+            len = kept;
+        }
+    }
+    if (tid == 0) *num_batches = nb;
 }
