@@ -33,6 +33,7 @@ int kv_cuda_fail(cudaError_t e, const char* what) {
 namespace {
 
 const i64 kSweepChunk = 1ll << 22;          // candidates per launch inside a sweep
+const i64 kAcceptSmall = 16384;              // sweep results that one CTA reduces (4 us against a launch of its own)
 const int kSnapshots = 256;                 // states of the base run kept for the sweeps
 const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
 
@@ -319,14 +320,13 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
                 if (pass == 1) *ptr = (T*)(h->d_arena + used);
                 used += (count * sizeof(T) + 255) & ~(size_t)255;
             };
-            // what a solver call hands back lies in a row: base TEL, batches, status | order | batch offsets
-            take(&h->d_result, 4);
+            // what a solver call hands back lies in a row: base TEL, batches, status, best move | order | batch offsets
+            take(&h->d_result, 16);
             if (B == 1) { take(&h->d_order, n); take(&h->d_batch_off, n + 1); }
             take(&h->d_s, total); take(&h->d_o, total);
             take(&h->d_tbl_id, total + 2);
             take(&h->d_counter, 4);
-            take(&h->d_best, 2); take(&h->d_partials, 2 * 4096); take(&h->d_ticket, 1);
-            take(&h->d_state, 4);
+            take(&h->d_partials, 2 * 4096); take(&h->d_ticket, 1);
             if (B == 1) {
                 take(&h->d_tbl_base, n + 2);
                 take(&h->d_base_starts, n);
@@ -341,6 +341,8 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         h->d_base_tel = (i64*)h->d_result;
         h->d_num_batches = h->d_result + 2;
         h->d_status = h->d_result + 3;
+        h->d_best = (i64*)(h->d_result + 4);
+        h->d_accepted = h->d_result + 8;
         h->pinned_bytes = 256 + (B == 1 ? result_bytes(n) : 0);
         if (kv_host_malloc(&h->h_pinned, &h->pinned_bytes) != cudaSuccess) { h->h_pinned = nullptr; rc = kv_cuda_fail(cudaGetLastError(), "cudaHostAlloc"); break; }
         cudaStream_t st = h->stream;
@@ -404,19 +406,39 @@ int sort_rows(sched_ctx* h, const KEY& src, int n, i64 rows, u64* tmp_keys, int*
 }
 
 // Base order -> position-ordered table, snapshots, base TEL.
-int ensure_base(sched_ctx* h) {
-    if (h->base_ready) return SCHED_OK;
-    const int n = h->n;
-    k3_gather_table<<<(n + 255) / 256, 256, 0, h->stream>>>(h->d_tbl_id, h->d_order, n, h->d_tbl_base);
-    KV_TRY(check_launch(h));
-#define RUN(N) k3_base_run<N><<<1, 32, (size_t)h->ring_cells * sizeof(int), h->stream>>>(                  \
-        h->d_tbl_base, n, h->L, (int)h->M, h->snap_stride, h->snap_count, h->d_snap_ring, h->d_snap_hdr, \
-        h->d_base_starts, h->d_base_tel, h->d_status)
+BaseRunParams base_run_params(sched_ctx* h) {
+    BaseRunParams p;
+    memset(&p, 0, sizeof(p));
+    p.tbl_id = h->d_tbl_id; p.tbl_base = h->d_tbl_base; p.order = h->d_order;
+    p.n = h->n; p.L = h->L; p.M = (int)h->M; p.stride = h->snap_stride; p.snap_count = h->snap_count;
+    p.snap_ring = h->d_snap_ring; p.snap_hdr = h->d_snap_hdr; p.starts_pos = h->d_base_starts;
+    p.base_tel = h->d_base_tel; p.status = h->d_status;
+    return p;
+}
+
+int run_base(sched_ctx* h, const BaseRunParams& p) {
+#define RUN(N) k3_base_run<N><<<1, K3B_THREADS, (size_t)h->ring_cells * sizeof(int), h->stream>>>(p)
     KV_DISPATCH_SIM(h, RUN);
 #undef RUN
-    KV_TRY(check_launch(h));
+    return check_launch(h);
+}
+
+int ensure_base(sched_ctx* h) {
+    if (h->base_ready) return SCHED_OK;
+    KV_TRY(run_base(h, base_run_params(h)));
     h->base_ready = true;
     return SCHED_OK;
+}
+
+// The best of tel[0 .. count) (launch slots, mapped back through index_map), or of d_best with count = 0,
+// becomes the base order's next move if it improves; the base run follows.  Leaves d_result complete.
+int accept_best(sched_ctx* h, const i64* tel, const int* index_map, i64 count, int sampled, u64 seed, int iteration) {
+    BaseRunParams p = base_run_params(h);
+    p.accept = 1;
+    p.tel = tel; p.index_map = index_map; p.count = count;
+    p.best = h->d_best; p.accepted = h->d_accepted; p.scratch = h->d_vals_b;
+    p.sampled = sampled; p.seed = seed; p.iteration = iteration;
+    return run_base(h, p);
 }
 
 // one warp per candidate: CTAs needed for `count` candidates
@@ -424,6 +446,14 @@ unsigned k3_grid(const sched_ctx* h, i64 count) {
     const int w = k3_warps(h);
     const i64 ctas = (count + w - 1) / w;
     return (unsigned)(ctas < 1 ? 1 : ctas);
+}
+
+// Candidates that run side by side in one wave need no launch order: 8 warps per SM cost four launches
+// less (12 of 33 us of a 120-move sweep) and no longer tail.
+i64 ordered_from(const sched_ctx* h) { return 8ll * h->sm_count; }
+// slot -> candidate of the last launch_moves() of `count` candidates, nullptr: the same
+const int* last_launch_order(const sched_ctx* h, i64 count) {
+    return count > ordered_from(h) ? (const int*)h->d_k4 + h->n + 1 + count : nullptr;
 }
 
 // K4: launch order of `count` candidates, bucketed by first moved position (longest suffix first)
@@ -465,8 +495,10 @@ int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, 
     p.count = count; p.tel_out = tel_out; p.tel_by_slot = by_slot ? 1 : 0; p.starts_out = starts_out;
     p.base_order = h->d_order; p.base_starts_pos = h->d_base_starts;
     p.status = h->d_status;
-    KV_TRY(order_candidates(h, p.src, count));
-    p.launch_order = (const int*)h->d_k4 + h->n + 1 + count;
+    if (count > ordered_from(h)) {
+        KV_TRY(order_candidates(h, p.src, count));
+        p.launch_order = last_launch_order(h, count);
+    }
     KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
 #define RUN(N)                                                                                    \
     if (starts_out) k3_eval_moves<N, true><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p);  \
@@ -479,8 +511,6 @@ int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, 
     h->evaluations += count;
     return SCHED_OK;
 }
-
-const int* last_launch_order(const sched_ctx* h, i64 count) { return (const int*)h->d_k4 + h->n + 1 + count; }
 
 int launch_argmin(sched_ctx* h, const i64* tel, i64 count, i64 index_base, const i64* prior, i64* best_out,
                   const int* index_map = nullptr) {
@@ -521,6 +551,7 @@ int read_checked_word() {
 // what the status word of an idle stream says
 int after_status(sched_ctx* h, int status) {
     if (status != KV_DEV_OK) {
+        h->base_ready = false;                       // the base run may be what gave up
         cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream);
         return SCHED_E_INTERNAL;
     }
@@ -1004,51 +1035,50 @@ int sched_local_search(sched_handle h, int neighbourhood, int32_t iters, uint64_
     if (neighbourhood < SCHED_NBHD_SWAP || neighbourhood > SCHED_NBHD_SAMPLED) return SCHED_E_INVAL;
     if (neighbourhood == SCHED_NBHD_SAMPLED && samples_per_iter < 1) return SCHED_E_INVAL;
     const int n = h->n;
-    if (order_inout) KV_TRY(sched_set_base_order(h, order_inout));
     cudaStream_t st = h->stream;
+    char* hp = (char*)h->h_pinned;
+    if (order_inout) {                               // through the pinned block: every path below waits for the stream
+        std::vector<unsigned char> seen;
+        if (!is_permutation(order_inout, n, seen)) return SCHED_E_NOT_PERMUTATION;
+        KV_CUDA(cudaStreamSynchronize(st));
+        memcpy(hp, order_inout, (size_t)n * sizeof(int));
+        KV_CUDA(cudaMemcpyAsync(h->d_order, hp, (size_t)n * sizeof(int), cudaMemcpyHostToDevice, st));
+        h->base_ready = false;
+    }
     const int sampled = neighbourhood == SCHED_NBHD_SAMPLED ? 1 : 0;
     const i64 total = n >= 2 ? neighbourhood_size(n, neighbourhood, samples_per_iter) : 0;
     KV_TRY(ensure_base(h));
-    i64* d_cur = (i64*)h->d_state;               // {current TEL, accepted flag}
-    int* d_acc = (int*)(d_cur + 1);
-    KV_CUDA(cudaMemcpyAsync(d_cur, h->d_base_tel, sizeof(i64), cudaMemcpyDeviceToDevice, st));
-    i64* hp = (i64*)h->h_pinned;                 // {best TEL, best code, accepted, base TEL}
+    const int* res = (const int*)hp;                 // d_result as read back
     int it = 0;
-    i64 cur_tel = 0;
-    KV_CUDA(cudaMemcpyAsync(&hp[3], h->d_base_tel, sizeof(i64), cudaMemcpyDeviceToHost, st));
-    KV_CUDA(cudaStreamSynchronize(st));
-    cur_tel = hp[3];
     for (; it < iters && total > 0; ++it) {
         KV_TRY(ensure_tel(h, total < kSweepChunk ? total : kSweepChunk));
+        const bool small = total <= kAcceptSmall;    // the accepting CTA looks for the best itself
         for (i64 done = 0; done < total; done += kSweepChunk) {
             const i64 c = total - done < kSweepChunk ? total - done : kSweepChunk;
             KV_TRY(launch_moves(h, sampled ? 2 : 1, nullptr, done, seed, it, c, h->d_tel, nullptr, true));
-            KV_TRY(launch_argmin(h, h->d_tel, c, done, done ? h->d_best : nullptr, h->d_best, last_launch_order(h, c)));
+            if (!small) KV_TRY(launch_argmin(h, h->d_tel, c, done, done ? h->d_best : nullptr, h->d_best, last_launch_order(h, c)));
         }
-        k5_accept_move<<<1, 256, 0, st>>>(h->d_order, n, h->d_best, d_cur, d_acc, h->d_vals_b, sampled, seed, it);
-        KV_TRY(check_launch(h));
-        KV_CUDA(cudaMemcpyAsync(&hp[0], h->d_best, 2 * sizeof(i64), cudaMemcpyDeviceToHost, st));
-        KV_CUDA(cudaMemcpyAsync(&hp[2], d_acc, sizeof(int), cudaMemcpyDeviceToHost, st));
+        KV_TRY(accept_best(h, h->d_tel, small ? last_launch_order(h, total) : nullptr, small ? total : 0, sampled, seed, it));
+        KV_CUDA(cudaMemcpyAsync(hp, h->d_result, 16 * sizeof(int), cudaMemcpyDeviceToHost, st));
         KV_CUDA(cudaStreamSynchronize(st));
-        if (trace_out) { trace_out[2 * it] = hp[1]; trace_out[2 * it + 1] = hp[0]; }
-        const bool accepted = *(int*)&hp[2] != 0;
-        if (accepted) {
-            cur_tel = hp[0];
-            h->base_ready = false;
-            KV_TRY(ensure_base(h));
+        KV_TRY(after_status(h, res[3]));
+        const i64 base_tel = ((const i64*)hp)[0], best_tel = ((const i64*)hp)[2], best_code = ((const i64*)hp)[3];
+        if (trace_out) { trace_out[2 * it] = best_code; trace_out[2 * it + 1] = best_tel; }
+        if (res[8] != 0) {
             // the re-simulated base order must reproduce the TEL that won the sweep
-            KV_CUDA(cudaMemcpyAsync(&hp[3], h->d_base_tel, sizeof(i64), cudaMemcpyDeviceToHost, st));
-            KV_CUDA(cudaStreamSynchronize(st));
-            if (hp[3] != cur_tel) return SCHED_E_INTERNAL;
+            if (base_tel != best_tel) return SCHED_E_INTERNAL;
         } else if (!sampled) {
             ++it;
             break;
         }
     }
-    if (order_inout) KV_CUDA(cudaMemcpyAsync(order_inout, h->d_order, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, st));
-    if (tel_out) *tel_out = cur_tel;
+    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, order_at() + (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, st));
+    KV_CUDA(cudaStreamSynchronize(st));
+    KV_TRY(after_status(h, res[3]));
+    if (order_inout) memcpy(order_inout, hp + order_at(), (size_t)n * sizeof(int));
+    if (tel_out) *tel_out = *(const i64*)hp;
     if (iters_done_out) *iters_done_out = it;
-    return read_status(h);
+    return SCHED_OK;
 }
 
 int sched_accept_move(sched_handle h, int64_t best_tel, int64_t best_index, int sampled, uint64_t seed,
@@ -1059,28 +1089,21 @@ int sched_accept_move(sched_handle h, int64_t best_tel, int64_t best_index, int 
     if (!sampled && best_index >= neighbourhood_size(n, SCHED_NBHD_SWAP_INSERT, 0)) return SCHED_E_INVAL;
     cudaStream_t st = h->stream;
     KV_TRY(ensure_base(h));
-    i64* d_cur = (i64*)h->d_state;               // {current TEL, accepted flag}
-    int* d_acc = (int*)(d_cur + 1);
-    i64* hp = (i64*)h->h_pinned;                 // {best TEL, best index, accepted, base TEL}
+    i64* hp = (i64*)h->h_pinned;
+    KV_CUDA(cudaStreamSynchronize(st));
     hp[0] = best_tel; hp[1] = best_index;
     KV_CUDA(cudaMemcpyAsync(h->d_best, hp, 2 * sizeof(i64), cudaMemcpyHostToDevice, st));
-    KV_CUDA(cudaMemcpyAsync(d_cur, h->d_base_tel, sizeof(i64), cudaMemcpyDeviceToDevice, st));
-    k5_accept_move<<<1, 256, 0, st>>>(h->d_order, n, h->d_best, d_cur, d_acc, h->d_vals_b, sampled ? 1 : 0, seed, iteration);
-    KV_TRY(check_launch(h));
-    KV_CUDA(cudaMemcpyAsync(&hp[2], d_acc, sizeof(int), cudaMemcpyDeviceToHost, st));
+    KV_TRY(accept_best(h, nullptr, nullptr, 0, sampled ? 1 : 0, seed, iteration));
+    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, 16 * sizeof(int), cudaMemcpyDeviceToHost, st));
     KV_CUDA(cudaStreamSynchronize(st));
-    const bool accepted = *(int*)&hp[2] != 0;
-    if (accepted) {
-        h->base_ready = false;
-        KV_TRY(ensure_base(h));
-    }
-    KV_CUDA(cudaMemcpyAsync(&hp[3], h->d_base_tel, sizeof(i64), cudaMemcpyDeviceToHost, st));
-    KV_CUDA(cudaStreamSynchronize(st));
+    const int* res = (const int*)hp;                 // d_result as read back
+    KV_TRY(after_status(h, res[3]));
+    const bool accepted = res[8] != 0;
     // the re-simulated order must reproduce the TEL that the caller's sweep reported for this move
-    if (accepted && hp[3] != best_tel) return SCHED_E_INTERNAL;
+    if (accepted && hp[0] != best_tel) return SCHED_E_INTERNAL;
     if (accepted_out) *accepted_out = accepted ? 1 : 0;
-    if (tel_out) *tel_out = hp[3];
-    return read_status(h);
+    if (tel_out) *tel_out = hp[0];
+    return SCHED_OK;
 }
 
 int sched_last_eval_kernel_ms(sched_handle h, float* ms_out) {

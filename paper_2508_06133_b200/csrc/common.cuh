@@ -36,7 +36,8 @@ struct sched_ctx {
     int smem_optin;          // max dynamic shared memory per block (bytes)
 
     unsigned char* d_arena;  // one block that holds every array of a fixed size
-    int* d_result;           // {base TEL (two words), batches, status}; d_order and d_batch_off follow it
+    int* d_result;           // {base TEL (two words), batches, status, best TEL, best index (two each), accepted}; d_order and
+                             // d_batch_off follow it
 
     int *d_s, *d_o;          // [B*n]
     int2* d_tbl_id;          // (s, o) by request id [B*n]
@@ -45,7 +46,7 @@ struct sched_ctx {
     bool base_ready;         // d_tbl_base + snapshots match d_order
     bool batch_handle;       // created by sched_init_batch
     int* d_base_starts;      // start of every position of the base order [n]
-    i64* d_state;            // local-search state {current TEL, accepted flag}
+    int* d_accepted;         // [1] whether the last accept step changed the base order
     void* h_pinned;          // pinned host memory for read-backs
     size_t pinned_bytes;
     void* d_sort;            // grow-only scratch for sorting explicit start times
@@ -66,7 +67,7 @@ struct sched_ctx {
     int* d_status;           // [1] device status
     i64* d_tel;              // [tel_cap] per-candidate TEL scratch
     i64 tel_cap;
-    i64* d_best;             // [2] (TEL, index) + partials
+    i64* d_best;             // [2] (TEL, index)
     i64* d_partials;         // [2 * max_blocks]
     unsigned int* d_ticket;  // [1]
 

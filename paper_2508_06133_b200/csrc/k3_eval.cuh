@@ -1,7 +1,7 @@
 // K3 (+K4) -- batched schedule evaluation kernels.
 //
-//   k3_gather_table   (s, o) of the request at every position of the base order.
-//   k3_base_run       one warp list-schedules the base order and stores the simulator state in
+//   k3_base_run       accepts the best move of a sweep if asked to, gathers (s, o) of the request at every
+//                     position of the base order, list-schedules it and stores the simulator state in
 //                     front of every `stride`-th position (snapshots) plus the start of every position.
 //   k3_eval_moves     one warp per candidate; the candidate is a move applied to the base order
 //                     (K4: index -> (type, i, j) -> position map, never materialised; launch order
@@ -20,6 +20,7 @@
 #include "common.cuh"
 #include "k2_fmetric.cuh"
 #include "k4_moves.cuh"
+#include "k5_argmin.cuh"
 #include "sim_chunk.cuh"
 #include "sim_hyb.cuh"
 
@@ -30,12 +31,6 @@ __device__ __forceinline__ int kv_wrap(int idx, int L) {   // idx < 3L
 }
 
 #define K3S_WARPS 16                       // warps per CTA of the start-time checker
-
-__global__ void k3_gather_table(const int2* __restrict__ tbl_id, const int* __restrict__ order, int n,
-                                int2* __restrict__ tbl_base) {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < n) tbl_base[q] = tbl_id[order[q]];
-}
 
 __global__ void k3_make_table(const int* __restrict__ s, const int* __restrict__ o, int total, int2* __restrict__ tbl) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -49,16 +44,98 @@ __global__ void k3_iota(int* a, int n) {
 
 // ------------------------------------------------------------------------------------------------
 // Base run: positions 0 .. n-1 of the base order; snapshot idx holds the state in front of
-// position idx * stride.  One warp: the run is a chain of n admissions, each of which needs the one
-// before it, so what counts is the latency of one admission.  The next 32 requests are loaded while
-// the 32 in hand are admitted, and their starts are stored together.  Dynamic shared memory: the
-// simulator's ring.
+// position idx * stride.  One CTA; all of it gathers the table, one warp runs: the run is a chain of n
+// admissions, each of which needs the one before it, so what counts is the latency of one admission.
+// The next 32 requests are loaded while the 32 in hand are admitted, and their starts are stored
+// together.  Dynamic shared memory: the simulator's ring.
+//
+// With `accept`, the best move of a sweep comes first, so that an iteration of a small local search is
+// two launches: the smallest (TEL, index) of tel[0 .. count) (or what `best` already holds, count = 0)
+// is applied to the order if it strictly improves the base TEL (Section 5.2's rule); if it does not,
+// nothing else happens.
 // ------------------------------------------------------------------------------------------------
+#define K3B_THREADS 256
+
+struct BaseRunParams {
+    const int2* tbl_id;
+    int2* tbl_base;
+    int* order;
+    int n, L, M, stride, snap_count;
+    int* snap_ring;
+    SnapHeader* snap_hdr;
+    int* starts_pos;
+    i64* base_tel;
+    int* status;
+    int accept;
+    const i64* tel;
+    const int* index_map;
+    i64 count;
+    i64* best;                         // (TEL, index)
+    int* accepted;
+    int* scratch;                      // [n]
+    int sampled, iteration;
+    u64 seed;
+};
+
+// Applies the best move to the order if it improves; the same answer in every thread.
+__device__ bool k3_accept(const BaseRunParams& p) {
+    __shared__ i64 sh_v[K3B_THREADS / 32], sh_i[K3B_THREADS / 32];
+    __shared__ Move mv;
+    __shared__ int sh_do;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, n = p.n;
+    if (p.count > 0) {
+        i64 bv = INT64_MAX, bi = INT64_MAX;
+        for (i64 k = tid; k < p.count; k += K3B_THREADS) k5_take(bv, bi, p.tel[k], p.index_map ? (i64)p.index_map[k] : k);
+        for (int d = 16; d >= 1; d >>= 1) {
+            const i64 ov = __shfl_xor_sync(KV_FULL, bv, d), oi = __shfl_xor_sync(KV_FULL, bi, d);
+            k5_take(bv, bi, ov, oi);
+        }
+        if (lane == 0) { sh_v[w] = bv; sh_i[w] = bi; }
+        __syncthreads();
+        if (tid == 0) {
+            for (int k = 1; k < K3B_THREADS / 32; ++k) k5_take(bv, bi, sh_v[k], sh_i[k]);
+            p.best[0] = bv; p.best[1] = bi;
+        }
+    }
+    if (tid == 0) {
+        const i64 bv = p.best[0], bi = p.best[1];
+        bool improve = bi != INT64_MAX && bv < *p.base_tel;
+        if (improve) {
+            mv = p.sampled ? kv_sample_move(n, p.seed, p.iteration, bi) : kv_decode_move(n, bi);
+            if ((unsigned)mv.i >= (unsigned)n || (unsigned)mv.j >= (unsigned)n) improve = false;   // not a move of this list
+        }
+        sh_do = improve ? 1 : 0;
+        *p.accepted = sh_do;
+    }
+    __syncthreads();
+    if (!sh_do) return false;
+    const Move m = mv;
+    if (m.type == 0) {
+        if (tid == 0) { const int x = p.order[m.i]; p.order[m.i] = p.order[m.j]; p.order[m.j] = x; }
+    } else {
+        // insert: build the moved range in scratch, then copy it back
+        const int lo = min(m.i, m.j), hi = max(m.i, m.j);
+        for (int q = lo + tid; q <= hi; q += K3B_THREADS) p.scratch[q] = p.order[kv_map_pos(m, q)];
+        __syncthreads();
+        for (int q = lo + tid; q <= hi; q += K3B_THREADS) p.order[q] = p.scratch[q];
+    }
+    __syncthreads();
+    return true;
+}
+
 template <class SIM>
-__global__ void __launch_bounds__(32)
-k3_base_run(const int2* __restrict__ tbl_base, int n, int L, int M, int stride, int snap_count,
-            int* __restrict__ snap_ring, SnapHeader* __restrict__ snap_hdr,
-            int* __restrict__ base_starts_pos, i64* __restrict__ base_tel, int* status) {
+__global__ void __launch_bounds__(K3B_THREADS)
+k3_base_run(const BaseRunParams p) {
+    if (p.accept && !k3_accept(p)) return;
+    for (int q = threadIdx.x; q < p.n; q += K3B_THREADS) p.tbl_base[q] = p.tbl_id[KV_IDX(p.order[q], p.n, 409)];
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int2* tbl_base = p.tbl_base;
+    const int n = p.n, L = p.L, M = p.M, stride = p.stride;
+    int* const snap_ring = p.snap_ring;
+    SnapHeader* const snap_hdr = p.snap_hdr;
+    int* const base_starts_pos = p.starts_pos;
+    int* const status = p.status;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x;
     SIM sim;
@@ -73,9 +150,10 @@ k3_base_run(const int2* __restrict__ tbl_base, int n, int L, int M, int stride, 
         const int cnt = min(32, n - q0);
         int mine = 0;
         const int sp = so.x + 1, om = so.y - 1;
+        int sp_next = __shfl_sync(KV_FULL, sp, 0), om_next = __shfl_sync(KV_FULL, om, 0);
         for (int k = 0; k < cnt; ++k) {
             if (to_snap == 0) {
-                const int i = (int)KV_IDX(idx, snap_count, 401);
+                const int i = (int)KV_IDX(idx, p.snap_count, 401);
                 i64 before = lane < k ? (i64)mine + so.y : 0;    // this block's completions so far
                 for (int d = 16; d >= 1; d >>= 1) before += __shfl_xor_sync(KV_FULL, before, d);
                 sim.store(snap_ring + (size_t)i * L, snap_hdr + i, tel + before);
@@ -83,7 +161,9 @@ k3_base_run(const int2* __restrict__ tbl_base, int n, int L, int M, int stride, 
                 to_snap = stride;
             }
             --to_snap;
-            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, status);
+            const int sp_k = sp_next, om_k = om_next;
+            sp_next = __shfl_sync(KV_FULL, sp, k + 1); om_next = __shfl_sync(KV_FULL, om, k + 1);
+            sim.admit(sp_k, om_k, n - q0 - k, status);
             if (lane == k) mine = sim.start();
         }
         if (q0 + lane < n) base_starts_pos[q0 + lane] = mine;
@@ -91,7 +171,7 @@ k3_base_run(const int2* __restrict__ tbl_base, int n, int L, int M, int stride, 
         for (int d = 16; d >= 1; d >>= 1) done += __shfl_xor_sync(KV_FULL, done, d);
         tel += done;
     }
-    if (lane == 0) *base_tel = tel;
+    if (lane == 0) *p.base_tel = tel;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -104,7 +184,7 @@ struct MoveEvalParams {
     const SnapHeader* snap_hdr;
     MoveSource src;
     i64 count;
-    const int* launch_order;           // candidate index of every launch slot (K4)
+    const int* launch_order;           // candidate index of every launch slot (K4), nullptr: the slot itself
     i64* tel_out;
     int tel_by_slot;                   // 1: tel_out is indexed by launch slot (full-sector writes; the arg-min maps
                                        // slots back through launch_order), 0: by candidate index
@@ -126,7 +206,7 @@ k3_eval_moves(const MoveEvalParams p) {
     const int n = p.n, L = p.L, M = p.M;
     const i64 slot = (i64)blockIdx.x * (blockDim.x >> 5) + warp;
     if (slot >= p.count) return;
-    const i64 c = KV_IDX(p.launch_order[slot], p.count, 402);
+    const i64 c = p.launch_order ? KV_IDX(p.launch_order[slot], p.count, 402) : slot;
     i64* tel_dst = p.tel_out + (p.tel_by_slot ? slot : c);
     SIM sim;
     sim.attach((int*)smem_raw + (size_t)warp * SIM::ring_cells(L), L);

@@ -76,34 +76,3 @@ k5_argmin(const i64* __restrict__ tel, i64 count, i64 index_base, const int* __r
         *ticket = 0;
     }
 }
-
-// Accept the best move if it strictly improves the current TEL (Section 5.2's rule), applying it
-// to the base order in place.  One thread block; state = {cur_tel, accepted flag, iterations}.
-__global__ void k5_accept_move(int* __restrict__ order, int n, const i64* __restrict__ best,
-                               i64* __restrict__ cur_tel, int* __restrict__ accepted,
-                               int* __restrict__ scratch /* [n] */, int sampled, u64 seed, int iteration) {
-    __shared__ int sh_do;
-    __shared__ Move mv;
-    if (threadIdx.x == 0) {
-        bool improve = best[1] != INT64_MAX && best[0] < *cur_tel;
-        if (improve) {
-            mv = sampled ? kv_sample_move(n, seed, iteration, best[1]) : kv_decode_move(n, best[1]);
-            if ((unsigned)mv.i >= (unsigned)n || (unsigned)mv.j >= (unsigned)n) improve = false;   // not a move of this list
-        }
-        if (improve) *cur_tel = best[0];
-        sh_do = improve ? 1 : 0;
-        *accepted = improve ? 1 : 0;
-    }
-    __syncthreads();
-    if (!sh_do) return;
-    const Move m = mv;
-    if (m.type == 0) {
-        if (threadIdx.x == 0) { int x = order[m.i]; order[m.i] = order[m.j]; order[m.j] = x; }
-        return;
-    }
-    // insert: build the moved range in scratch, then copy it back
-    const int lo = min(m.i, m.j), hi = max(m.i, m.j);
-    for (int q = lo + threadIdx.x; q <= hi; q += blockDim.x) scratch[q] = order[kv_map_pos(m, q)];
-    __syncthreads();
-    for (int q = lo + threadIdx.x; q <= hi; q += blockDim.x) order[q] = scratch[q];
-}

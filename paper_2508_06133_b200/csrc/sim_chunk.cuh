@@ -175,14 +175,16 @@ struct ChunkSim {
     // 0: (sp, om) fits at t; otherwise a lower bound of the rounds it has to wait
     __device__ __forceinline__ int test(int sp, int om) {
         const int nk = nkt - sp;                         // it fits  <=>  V[x] <= nk in every round of the window
-        bool over = (unsigned)rl <= (unsigned)om && cur > nk;
-        over = over || (xr <= om && U[0] > nk);
+        // one reduction answers for all lanes: above 0 the wait that chunk 0 asks for, 0 where a far bound
+        // says "perhaps" (or a round fits exactly), below 0 everything is clear
+        int v = (unsigned)rl <= (unsigned)om ? __viaddmin_s32(cur, -nk, rl + 1) : INT_MIN;
+        if (xr <= om && U[0] > nk) v = max(v, 0);
         if (NM > 1 && tau + om >= 1024 + 32) {
 #pragma unroll
-            for (int m = 1; m < NM; ++m) over = over || (xr + 1024 * m <= om && U[m] > nk);
+            for (int m = 1; m < NM; ++m) if (xr + 1024 * m <= om && U[m] > nk) v = max(v, 0);
         }
-        if (!__any_sync(KV_FULL, over)) return 0;
-        const int d = kv_warp_max((unsigned)rl <= (unsigned)om ? __viaddmin_s32(cur, -nk, rl + 1) : 0);
+        const int d = kv_warp_max(v);
+        if (d < 0) return 0;
         return d > 0 ? d : far_need(om, nk);
     }
     // t moves on by d rounds
@@ -208,7 +210,8 @@ struct ChunkSim {
             }
         }
         const int last = tau + om, back = (last & 31) - lane;       // the chunk the window ends in
-        if (last > 31 && back >= 0) *cells_of(T0 + last) += sp + om - back;
+        // an atomic without a result: nothing behind it waits for the old value
+        if (last > 31 && back >= 0) atomicAdd(cells_of(T0 + last), sp + om - back);
     }
 
     // Admit one request (sp = s + 1, om = o - 1) at the earliest start; all 32 lanes call this with
