@@ -33,6 +33,8 @@ int kv_cuda_fail(cudaError_t e, const char* what) {
 namespace {
 
 const i64 kSweepChunk = 1ll << 22;          // candidates per launch inside a sweep
+const int kResultBad = 9;                   // word of d_result: the candidates of a host call are not what they should be
+const int kDeviceCheckMax = 1 << 20;        // requests whose bits fit a CTA's shared memory
 const i64 kAcceptSmall = 16384;              // sweep results that one CTA reduces (4 us against a launch of its own)
 const int kSnapshots = 256;                 // states of the base run kept for the sweeps
 const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
@@ -757,9 +759,11 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
     size_t cand_bytes = 0; i64 outs = count;
     if (kind == SCHED_CAND_ORDER) {
         if (h->batch_handle) return SCHED_E_INVAL;
-        std::vector<unsigned char> seen;
-        for (i64 c = 0; c < count; ++c)
-            if (!is_permutation((const int32_t*)candidates + c * n, n, seen)) return SCHED_E_NOT_PERMUTATION;
+        if (n > kDeviceCheckMax) {
+            std::vector<unsigned char> seen;
+            for (i64 c = 0; c < count; ++c)
+                if (!is_permutation((const int32_t*)candidates + c * n, n, seen)) return SCHED_E_NOT_PERMUTATION;
+        }
         cand_bytes = (size_t)count * n * sizeof(int);
     } else if (kind == SCHED_CAND_MOVE) {
         if (h->batch_handle || n < 2) return SCHED_E_INVAL;
@@ -771,10 +775,6 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
         cand_bytes = (size_t)count * sizeof(i64);
     } else if (kind == SCHED_CAND_START_TIMES) {
         if (h->batch_handle || starts_out) return SCHED_E_INVAL;
-        for (i64 k = 0; k < count * n; ++k) {
-            int v = ((const int32_t*)candidates)[k];
-            if (v < 0 || v >= (1 << 30)) return SCHED_E_INVAL;
-        }
         cand_bytes = (size_t)count * n * sizeof(int);
     } else if (kind == SCHED_CAND_POLICY) {
         for (i64 c = 0; c < count; ++c) {
@@ -794,10 +794,33 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
     KV_TRY(ensure_stage(h, off_starts + starts_bytes + 256));
     char* base = (char*)h->d_stage;
     KV_CUDA(cudaMemcpyAsync(base, candidates, cand_bytes, cudaMemcpyHostToDevice, h->stream));
+    // orders and start times are checked where they have been copied to (a pass over 777 orders of 1,531
+    // takes 8 us there and 1.2 ms here); the evaluation in between reads nothing out of place whatever
+    // they hold, and nothing is handed out before the answer is known
+    const bool on_device = (kind == SCHED_CAND_ORDER && n <= kDeviceCheckMax) || kind == SCHED_CAND_START_TIMES;
+    if (on_device) {
+        KV_CUDA(cudaMemsetAsync(h->d_result + kResultBad, 0, sizeof(int), h->stream));
+        if (kind == SCHED_CAND_ORDER) {
+            const size_t bits = (((size_t)n + 31) / 32) * sizeof(unsigned);
+            KV_CUDA(cudaFuncSetAttribute(k3_check_orders, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 1024));
+            k3_check_orders<<<(unsigned)(count < 65535 ? count : 65535), 256, bits, h->stream>>>((const int*)base, n, count, h->d_result + kResultBad);
+        } else {
+            const i64 total = count * n;
+            const i64 blocks = (total + 1023) / 1024;
+            k3_check_start_range<<<(unsigned)(blocks < 65535 ? blocks : 65535), 256, 0, h->stream>>>((const int*)base, total, h->d_result + kResultBad);
+        }
+        KV_TRY(check_launch(h));
+    }
     int rc = sched_eval_batch_dev(h, kind, count, base, (int64_t*)(base + off_tel),
                                   feasible_out ? (uint8_t*)(base + off_feas) : nullptr,
                                   starts_out ? (int32_t*)(base + off_starts) : nullptr);
     if (rc != SCHED_OK) { cudaStreamSynchronize(h->stream); return rc; }
+    if (on_device) {
+        const int* res = (const int*)h->h_pinned;
+        KV_CUDA(cudaMemcpyAsync(h->h_pinned, h->d_result, 16 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+        KV_CUDA(cudaStreamSynchronize(h->stream));
+        if (res[kResultBad]) return kind == SCHED_CAND_ORDER ? SCHED_E_NOT_PERMUTATION : SCHED_E_INVAL;
+    }
     KV_CUDA(cudaMemcpyAsync(tel_out, base + off_tel, (size_t)outs * sizeof(i64), cudaMemcpyDeviceToHost, h->stream));
     if (feasible_out) KV_CUDA(cudaMemcpyAsync(feasible_out, base + off_feas, (size_t)outs, cudaMemcpyDeviceToHost, h->stream));
     if (starts_out) KV_CUDA(cudaMemcpyAsync(starts_out, base + off_starts, starts_bytes, cudaMemcpyDeviceToHost, h->stream));
@@ -1235,63 +1258,69 @@ static int amin_run(int32_t B, int32_t n_max, const int32_t* n_each, const int32
     memset(&P, 0, sizeof(P));
     P.n_max = n_max; P.M = (int)M;
     P.L = 32; while (P.L < omax + 2) P.L <<= 1;
-    const size_t smem = sizeof(int) * ((size_t)5 * n_max + (size_t)4 * P.L);
+    const int slots = sim_pick_slots(omax), nm = slots <= 32 ? 1 : slots / 32;
+    P.sim_L = 32 + 96 * nm + 32 * slots;
+    const size_t smem = k7_smem_bytes(32 * slots, n_max, P.L);
     int dev = 0, optin = 0;
     KV_CUDA(cudaGetDevice(&dev));
     KV_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     if (smem + 1024 > (size_t)optin) return SCHED_E_UNSUPPORTED;
-    KV_CUDA(cudaFuncSetAttribute(k7_amin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    void (*kernel)(const AminParams) = nm == 1 ? k7_amin<ChunkSim<1>> : nm == 2 ? k7_amin<ChunkSim<2>>
+                                     : nm == 4 ? k7_amin<ChunkSim<4>> : k7_amin<ChunkSim<8>>;
+    // the same value for every call: callers on other threads may be between this and their launch
+    KV_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024));
 
-    const size_t cells = (size_t)B * n_max;
-    int *d_n = nullptr, *d_s = nullptr, *d_l = nullptr, *d_o = nullptr, *d_ord = nullptr, *d_start = nullptr, *d_status = nullptr;
-    i64* d_res = nullptr;                                   // tel | evictions | peak, B each
+    // one block: tel | evictions | peak [B each], status (8 bytes) | n_each [B] | s, lower, o, order, start [cells each]
+    const size_t cells = (size_t)B * n_max, row = sizeof(int) * cells;
+    const size_t bytes = sizeof(i64) * (3 * (size_t)B + 1) + sizeof(int) * (size_t)B + 5 * row;
+    char* block = nullptr;
+    KV_TRY(dev_alloc(&block, bytes < kPoolMinBlock ? kPoolMinBlock : bytes));
+    i64* d_res = (i64*)block;
+    int* d_status = (int*)(d_res + 3 * (size_t)B);
+    int* d_n = (int*)(d_res + 3 * (size_t)B + 1);
+    int* d_s = d_n + B;
+    int* d_l = d_s + cells;
+    int* d_o = d_l + cells;
+    int* d_ord = d_o + cells;
+    int* d_start = d_ord + cells;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     int rc = SCHED_OK;
     do {
 #define AM_CUDA(call) if ((call) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), #call); break; }
-        if ((rc = dev_alloc(&d_n, (size_t)B)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_s, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_l, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_o, cells)) != SCHED_OK) break;
-        if (order_host && (rc = dev_alloc(&d_ord, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_start, cells)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_res, (size_t)3 * B)) != SCHED_OK) break;
-        if ((rc = dev_alloc(&d_status, 1)) != SCHED_OK) break;
-        AM_CUDA(cudaEventCreate(&e0));
-        AM_CUDA(cudaEventCreate(&e1));
+        if (kernel_ms_out) {
+            AM_CUDA(cudaEventCreate(&e0));
+            AM_CUDA(cudaEventCreate(&e1));
+        }
         AM_CUDA(cudaMemcpy(d_n, n_each, sizeof(int) * (size_t)B, cudaMemcpyHostToDevice));
-        AM_CUDA(cudaMemcpy(d_s, s, sizeof(int) * cells, cudaMemcpyHostToDevice));
-        AM_CUDA(cudaMemcpy(d_l, lower, sizeof(int) * cells, cudaMemcpyHostToDevice));
-        AM_CUDA(cudaMemcpy(d_o, o, sizeof(int) * cells, cudaMemcpyHostToDevice));
-        if (order_host) AM_CUDA(cudaMemcpy(d_ord, order_host, sizeof(int) * cells, cudaMemcpyHostToDevice));
-        AM_CUDA(cudaMemset(d_start, 0xff, sizeof(int) * cells));           // -1 where a row has no request
-        AM_CUDA(cudaMemset(d_status, 0, sizeof(int)));
+        AM_CUDA(cudaMemcpy(d_s, s, row, cudaMemcpyHostToDevice));
+        AM_CUDA(cudaMemcpy(d_l, lower, row, cudaMemcpyHostToDevice));
+        AM_CUDA(cudaMemcpy(d_o, o, row, cudaMemcpyHostToDevice));
+        if (order_host) AM_CUDA(cudaMemcpy(d_ord, order_host, row, cudaMemcpyHostToDevice));
+        AM_CUDA(cudaMemsetAsync(d_start, 0xff, row, 0));                   // -1 where a row has no request
+        AM_CUDA(cudaMemsetAsync(d_status, 0, sizeof(i64), 0));
         P.n_each = d_n; P.s = d_s; P.lower = d_l; P.o = d_o;
         P.order = order_host ? d_ord : order_dev;
         P.order_stride = order_host ? (size_t)n_max : 0;
         P.start_out = d_start; P.tel_out = d_res; P.evict_out = d_res + B; P.peak_out = d_res + 2 * (size_t)B;
         P.status = d_status;
-        AM_CUDA(cudaEventRecord(e0, 0));
-        k7_amin<<<B, K7_THREADS, smem, 0>>>(P);
+        if (e0) AM_CUDA(cudaEventRecord(e0, 0));
+        kernel<<<B, K7_THREADS, smem, 0>>>(P);
         AM_CUDA(cudaGetLastError());
-        AM_CUDA(cudaEventRecord(e1, 0));
-        AM_CUDA(cudaDeviceSynchronize());
-        int status = 0;
-        AM_CUDA(cudaMemcpy(&status, d_status, sizeof(int), cudaMemcpyDeviceToHost));
-        if (status != 0) { rc = SCHED_E_INTERNAL; break; }
+        if (e1) AM_CUDA(cudaEventRecord(e1, 0));
+        std::vector<i64> res(3 * (size_t)B + 1);
+        AM_CUDA(cudaMemcpy(res.data(), d_res, res.size() * sizeof(i64), cudaMemcpyDeviceToHost));
+        if (*(const int*)&res[3 * (size_t)B] != 0) { rc = SCHED_E_INTERNAL; break; }
         if ((rc = read_checked_word()) != SCHED_OK) break;
-        AM_CUDA(cudaMemcpy(start_out, d_start, sizeof(int) * cells, cudaMemcpyDeviceToHost));
-        AM_CUDA(cudaMemcpy(tel_out, d_res, sizeof(i64) * (size_t)B, cudaMemcpyDeviceToHost));
-        if (evictions_out) AM_CUDA(cudaMemcpy(evictions_out, d_res + B, sizeof(i64) * (size_t)B, cudaMemcpyDeviceToHost));
-        if (peak_out) AM_CUDA(cudaMemcpy(peak_out, d_res + 2 * (size_t)B, sizeof(i64) * (size_t)B, cudaMemcpyDeviceToHost));
+        AM_CUDA(cudaMemcpy(start_out, d_start, row, cudaMemcpyDeviceToHost));
+        memcpy(tel_out, res.data(), sizeof(i64) * (size_t)B);
+        if (evictions_out) memcpy(evictions_out, res.data() + B, sizeof(i64) * (size_t)B);
+        if (peak_out) memcpy(peak_out, res.data() + 2 * (size_t)B, sizeof(i64) * (size_t)B);
         if (kernel_ms_out) AM_CUDA(cudaEventElapsedTime(kernel_ms_out, e0, e1));
 #undef AM_CUDA
     } while (0);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    int* frees[] = {d_n, d_s, d_l, d_o, d_ord, d_start, d_status};
-    for (int* ptr : frees) if (ptr) kv_free(ptr);
-    if (d_res) kv_free(d_res);
+    kv_free(block);
     return rc;
 }
 

@@ -36,8 +36,8 @@ struct sched_ctx {
     int smem_optin;          // max dynamic shared memory per block (bytes)
 
     unsigned char* d_arena;  // one block that holds every array of a fixed size
-    int* d_result;           // {base TEL (two words), batches, status, best TEL, best index (two each), accepted}; d_order and
-                             // d_batch_off follow it
+    int* d_result;           // {base TEL (two words), batches, status, best TEL, best index (two each), accepted, bad input};
+                             // d_order and d_batch_off follow it
 
     int *d_s, *d_o;          // [B*n]
     int2* d_tbl_id;          // (s, o) by request id [B*n]

@@ -247,6 +247,36 @@ k3_eval_moves(const MoveEvalParams p) {
 }
 
 // ------------------------------------------------------------------------------------------------
+// Checks of the host entry point's candidates: every order a permutation of 0 .. n-1 (one bit per id in
+// dynamic shared memory), every start time in 0 .. 2^30 - 1.
+// ------------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256)
+k3_check_orders(const int* __restrict__ orders, int n, i64 count, int* bad) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned* seen = (unsigned*)smem_raw;
+    const int words = (n + 31) >> 5;
+    for (i64 c = blockIdx.x; c < count; c += gridDim.x) {
+        for (int k = threadIdx.x; k < words; k += 256) seen[k] = 0u;
+        __syncthreads();
+        bool wrong = false;
+        for (int q = threadIdx.x; q < n; q += 256) {
+            const int id = orders[(size_t)c * n + q];
+            if ((unsigned)id >= (unsigned)n) { wrong = true; continue; }
+            const unsigned bit = 1u << (id & 31);
+            if (atomicOr(&seen[id >> 5], bit) & bit) wrong = true;
+        }
+        if (wrong) *bad = 1;
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k3_check_start_range(const int* __restrict__ starts, i64 total, int* bad) {
+    bool wrong = false;
+    for (i64 k = (i64)blockIdx.x * 256 + threadIdx.x; k < total; k += (i64)gridDim.x * 256) wrong = wrong || (unsigned)starts[k] >= (1u << 30);
+    if (wrong) *bad = 1;
+}
+
+// ------------------------------------------------------------------------------------------------
 // Explicit orders: orders[c][q] = request id at position q.
 // ------------------------------------------------------------------------------------------------
 struct OrderEvalParams {

@@ -1,7 +1,7 @@
 // K7 -- Sorted-F + A_min, Phase 2 (Section 5.5 "Handling Prediction Uncertainty via Adaptive Output
 // Length Refinement"; Algorithm 5, the supplement to Section 5): the executor when only a lower bound l_i <= o_i of
 // every decode length is known.  Many independent scenarios (a backlog, its list and one vector of
-// lower bounds each), one CTA per scenario.
+// lower bounds each), one warp per scenario.
 //
 // Every request carries a running estimate e_i (initially l_i).  Iteration t = 1, 2, ...:
 //   1. requests that have run their o_i rounds leave; every other running request is about to run
@@ -15,30 +15,35 @@
 //   4. the round runs.
 //
 // How the kernel avoids touching every running request in every round.
-//   occ[tau] is the projected memory of round tau: request j contributes s_j + (tau - p_j) for
+//   The projected memory of the rounds from t on is a chunked timeline (sim_chunk.cuh; a start p is the
+//   simulator's round p + 1): request j contributes s_j + (tau - p_j) for
 //   tau in [p_j + 1, p_j + e_j].  A request whose estimate e (fixed at its admission) is below its
 //   true length o is OVERDUE in rounds p+e+1 .. p+o: there its estimate is t - p, i.e. step 1 extends
 //   its projection by exactly the current round.  The overdue requests are kept as two aggregates,
-//   cnt = how many and A = sum of (s_j - p_j), so step 1 is occ[t] += A + cnt * t; a request joins the
+//   cnt = how many and A = sum of (s_j - p_j), so step 1 adds A + cnt * t to round t; a request joins the
 //   aggregates at p+e+1 and leaves them at p+o+1 through per-round event cells (dc, dA) written when
 //   it is admitted (and taken back if it is evicted).  A is kept modulo 2^32: the sum A + cnt * t is
 //   a memory amount and fits, its two terms need not.  The estimate of a running request is never
 //   stored: it is max(e at admission, t - p).
 //   The projection is within M in every round >= t at the end of an iteration, so only step 1 can
-//   break it, and only in round t: "the projection exceeds M" is occ[t] > M.
-//   While the head of the queue is refused nothing is admitted and occ only grows, so the bound on
-//   its wait that the window test gives (a cell over budget by x at offset r needs min(x, r+1) more
-//   rounds) stays valid until the next eviction.  Rounds in which nothing can happen (no overflow;
-//   head still bound to wait, or not even its first round fits) are walked by one warp, 32 rounds
-//   per step (the running aggregates of a round are prefix sums of the event cells).
+//   break it, and only in round t.
+//   While the head of the queue is refused nothing is admitted and the projection only grows, so the
+//   bound on its wait that the window test gives (a cell over budget by x at offset r needs min(x, r+1)
+//   more rounds) stays valid until the next eviction.  Rounds in which nothing can happen (no overflow;
+//   head still bound to wait, or not even its first round fits) are walked up to 32 at a time, one lane
+//   each (the running aggregates of a round are prefix sums of the event cells).
+//   The running requests are a compact list, so an eviction looks at them and not at everything that
+//   has ever started.
+// What bounds it: a scenario is a chain (2,000 requests of the paper's lengths: 2,400 admissions, 380
+// evictions, 1,400 walks), so the latency of each; one warp needs no block barriers for them.
 #pragma once
 
 #include "common.cuh"
+#include "sim_chunk.cuh"
 
-#define K7_THREADS 256
+#define K7_THREADS 32
 #define K7_MAX_N 4096
 #define K7_MAX_O 8192
-#define K7_ID_BITS 20
 
 struct AminParams {
     int n_max;
@@ -49,7 +54,8 @@ struct AminParams {
     const int* order;            // [B, n_max] the list: request ids; or one row shared by all (order_stride 0)
     size_t order_stride;
     int M;
-    int L;                       // ring length, a power of two >= the longest decode + 2
+    int L;                       // event ring length, a power of two >= the longest decode + 2
+    int sim_L;                   // ints per simulator state
     int* start_out;              // [B, n_max] by request id
     i64* tel_out;                // [B] sum of (p + o)
     i64* evict_out;              // [B] evictions
@@ -57,122 +63,78 @@ struct AminParams {
     int* status;
 };
 
-enum { K7_ACT_WORK = 0, K7_ACT_DONE = 1, K7_ACT_CAP = 2 };
-
-struct K7Ctl {
-    int t, remaining, peak, act;
-    unsigned cnt, A;
-};
-
-__device__ __forceinline__ int k7_block_max(int v, int* red) {
-    const int tid = threadIdx.x;
-    v = kv_warp_max(v);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    int r = red[0];
-#pragma unroll
-    for (int k = 1; k < K7_THREADS / 32; ++k) r = max(r, red[k]);
-    __syncthreads();
-    return r;
-}
-__device__ __forceinline__ int k7_block_min(int v, int* red) {
-    const int tid = threadIdx.x;
-    v = kv_warp_min(v);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    int r = red[0];
-#pragma unroll
-    for (int k = 1; k < K7_THREADS / 32; ++k) r = min(r, red[k]);
-    __syncthreads();
-    return r;
-}
-__device__ __forceinline__ u64 k7_block_min64(u64 v, u64* red) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) { const u64 w = __shfl_xor_sync(KV_FULL, v, d); v = w < v ? w : v; }
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    u64 r = red[0];
-#pragma unroll
-    for (int k = 1; k < K7_THREADS / 32; ++k) r = red[k] < r ? red[k] : r;
-    __syncthreads();
-    return r;
+__host__ __device__ inline size_t k7_smem_bytes(int ring_cells, int n_max, int L) {
+    return ((size_t)ring_cells + 4 * (size_t)n_max + 3 * (size_t)L) * sizeof(int) + 2 * (size_t)n_max * sizeof(unsigned short) + 16;
 }
 
+template <class SIM>
 __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
     extern __shared__ __align__(16) unsigned char k7_smem[];
-    __shared__ K7Ctl ctl;
-    __shared__ int red[K7_THREADS / 32];
-    __shared__ u64 red64[K7_THREADS / 32];
-    __shared__ u64 acc;
-    const int tid = threadIdx.x;
+    const int lane = threadIdx.x;
     const int b = blockIdx.x;
     const int n = P.n_each[b];
     const int nm = P.n_max;
     // per list position: prefill, true length, estimate while pending, start (-1: pending), request id
-    int* ps = reinterpret_cast<int*>(k7_smem);
+    int* ring = reinterpret_cast<int*>(k7_smem);
+    int* ps = ring + SIM::ring_cells(P.sim_L);
     int* po = ps + nm;
     int* pe = po + nm;
     int* pp = pe + nm;
-    int* pid = pp + nm;
-    int* occ = pid + nm;                                          // projected memory per round
-    int* dc = occ + P.L;                                          // change of cnt at the start of a round
+    int* dc = pp + nm;                                            // change of cnt at the start of a round
     unsigned* dA = reinterpret_cast<unsigned*>(dc + P.L);         // change of A
     int* fin = reinterpret_cast<int*>(dA + P.L);                  // requests that leave at the start of a round
+    unsigned short* pid = reinterpret_cast<unsigned short*>(fin + P.L);
+    unsigned short* run = pid + nm;                               // positions that run (and some that have finished)
 
     const size_t base = (size_t)b * nm;
     const int* ord = P.order + (size_t)b * P.order_stride;
-    if (tid == 0) acc = 0;
-    __syncthreads();
+    i64 sum_o = 0;
     {
-        u64 part = 0;
         bool bad = false;
-        for (int q = tid; q < n; q += K7_THREADS) {
+        for (int q = lane; q < n; q += 32) {
             const int id = ord[q];
             if (id < 0 || id >= n) { bad = true; continue; }      // never read outside the row
             ps[q] = P.s[base + id]; po[q] = P.o[base + id]; pe[q] = P.lower[base + id];
-            pp[q] = -1; pid[q] = id;
-            part += (u64)po[q];
+            pp[q] = -1; pid[q] = (unsigned short)id;
+            sum_o += po[q];
         }
-        for (int k = tid; k < P.L; k += K7_THREADS) { occ[k] = 0; dc[k] = 0; dA[k] = 0u; fin[k] = 0; }
-        if (part) atomicAdd(&acc, part);
-        if (__syncthreads_or(bad ? 1 : 0)) {
-            if (tid == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
+        for (int k = lane; k < P.L; k += 32) { dc[k] = 0; dA[k] = 0u; fin[k] = 0; }
+        if (__any_sync(KV_FULL, bad)) {
+            if (lane == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
             return;
         }
+        for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
+        __syncwarp();
     }
-    const i64 sum_o = (i64)acc;
-    __syncthreads();
     i64 round_cap = 16 + sum_o * (i64)(n + 1);
     if (round_cap > (1ll << 30)) round_cap = 1ll << 30;           // t stays a 32-bit round index
-    const i64 turn_cap = round_cap;
 
     const int mask = P.L - 1;
     const int M = P.M;
-    int t = 1, remaining = n, peak = 0;
+    SIM sim;
+    sim.attach(ring, P.sim_L);
+    sim.reset(M, 1);                                              // the simulator's round is the iteration t
+    int remaining = n, peak = 0, nrun = 0;
     unsigned cnt = 0, A = 0;
     int head = 0, frontier = 0, npe = 0;     // first pending position; first never-started one; pending ones below it
     int t_ok = 1;                            // the head cannot start in an iteration before this one
     i64 evictions = 0;
-    bool failed = false;
+    bool failed = false, done = false;
 
     for (i64 turn = 0;; ++turn) {
-        if (turn > turn_cap) { failed = true; break; }
-        if (tid < 32) {
-            // rounds in which nothing can be decided (step 1 only), 32 at a time: lane l takes round
-            // t + l.  A round reads only its own cells and the running (cnt, A, remaining), which are
-            // prefix sums of the event cells, so the 32 rounds are evaluated together and the walk
-            // stops at the first lane whose round needs the whole CTA (or ends the run).
-            const int lane = tid;
-            int act = K7_ACT_WORK;
-            const int head_s = head < n ? ps[head] : 0;
-            for (;;) {
-                const int tau = t + lane;
-                const int k = tau & mask;
-                int cs = dc[k];
-                unsigned as = dA[k];
-                int fs = fin[k];
-                const int oc = occ[k];
+        if (turn > round_cap) { failed = true; break; }
+        // rounds in which nothing can be decided (step 1 only): the lanes whose round of chunk 0 is still
+        // to come take one each.  A round reads only its own cell and the running (cnt, A, remaining),
+        // which are prefix sums of the event cells; the walk stops at the first round that needs a
+        // decision (or ends the run).
+        const int head_s = head < n ? ps[head] : 0;
+        for (;;) {
+            const bool live = sim.rl >= 0;
+            const int round = sim.T0 + lane, k = round & mask;
+            int cs = live ? dc[k] : 0;
+            unsigned as = live ? dA[k] : 0u;
+            int fs = live ? fin[k] : 0;
+            if (__any_sync(KV_FULL, cs != 0 || as != 0u || fs != 0)) {
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
                     const int c2 = __shfl_up_sync(KV_FULL, cs, d);
@@ -180,55 +142,46 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
                     const int f2 = __shfl_up_sync(KV_FULL, fs, d);
                     if (lane >= d) { cs += c2; as += a2; fs += f2; }
                 }
-                const unsigned cnt_l = cnt + (unsigned)cs, A_l = A + as;
-                const int rem_l = remaining - fs;
-                const int u = oc + (int)(A_l + cnt_l * (unsigned)tau);
-                const bool done = rem_l == 0;
-                // the head's first round is the current one: if it does not fit there, the window
-                // test cannot succeed in this iteration and the CTA need not be woken for it
-                const bool work = u > M || (head < n && tau >= t_ok && u + head_s + 1 <= M);
-                const bool cap = (i64)tau >= round_cap;
-                const unsigned stops = __ballot_sync(KV_FULL, done || work || cap);
-                const int first = stops ? __ffs(stops) - 1 : 32;
-                if (lane <= first) { dc[k] = 0; dA[k] = 0u; fin[k] = 0; }          // events consumed
-                if (lane < first) occ[k] = 0;                                        // a round that is over
-                else if (lane == first) occ[k] = u;
-                peak = max(peak, kv_warp_max(lane < first ? u : 0));
-                const int src = first < 32 ? first : 31;
-                cnt = __shfl_sync(KV_FULL, cnt_l, src);
-                A = __shfl_sync(KV_FULL, A_l, src);
-                remaining = __shfl_sync(KV_FULL, rem_l, src);
-                if (first < 32) {
-                    t += first;
-                    const int why = done ? K7_ACT_DONE : (work ? K7_ACT_WORK : K7_ACT_CAP);
-                    act = __shfl_sync(KV_FULL, why, first);
-                    break;
-                }
-                t += 32;
             }
-            if (lane == 0) { ctl.t = t; ctl.remaining = remaining; ctl.peak = peak; ctl.act = act; ctl.cnt = cnt; ctl.A = A; }
+            const unsigned cnt_l = cnt + (unsigned)cs, A_l = A + as;
+            const int rem_l = remaining - fs;
+            const int u = sim.cur - lane + (int)(A_l + cnt_l * (unsigned)round);
+            const bool end = live && rem_l == 0;
+            // the head's first round is the current one: if it does not fit there, the window test cannot
+            // succeed in this iteration
+            const bool work = live && (u > M || (head < n && round >= t_ok && u + head_s + 1 <= M));
+            const bool cap = (i64)round >= round_cap;
+            const unsigned stops = __ballot_sync(KV_FULL, end || work || (live && cap));
+            const int first = stops ? __ffs(stops) - 1 : 32;
+            if (live && lane <= first) { dc[k] = 0; dA[k] = 0u; fin[k] = 0; }            // events consumed
+            const int run_max = kv_warp_max(live && lane < first ? u : 0);
+            peak = max(peak, run_max);
+            const int src = first < 32 ? first : 31;
+            cnt = __shfl_sync(KV_FULL, cnt_l, src);
+            A = __shfl_sync(KV_FULL, A_l, src);
+            remaining = __shfl_sync(KV_FULL, rem_l, src);
+            if (first < 32) {
+                if (lane == first) sim.cur = u + lane;                                  // step 1 of the round that is decided
+                sim.advance(__shfl_sync(KV_FULL, sim.rl, first), 0);
+                if (__shfl_sync(KV_FULL, (int)end, first)) done = true;
+                else if (!__shfl_sync(KV_FULL, (int)work, first)) failed = true;
+                break;
+            }
+            sim.advance(32 - sim.tau, 0);
         }
-        __syncthreads();
-        t = ctl.t; remaining = ctl.remaining; peak = ctl.peak; cnt = ctl.cnt; A = ctl.A;
-        const int act = ctl.act;
-        __syncthreads();
-        if (act == K7_ACT_DONE) break;
-        if (act == K7_ACT_CAP) { failed = true; break; }
+        if (done || failed) break;
+        const int t = sim.T0 + sim.tau;
 
         // ---- step 2: admissions of iteration t
         if (head < n && t >= t_ok) {
             for (;;) {
                 const int q = head;
                 const int s = ps[q], o = po[q], e = pe[q];
-                int need = INT_MIN;
-                for (int x = tid; x < e; x += K7_THREADS) {
-                    const int over = occ[(t + x) & mask] + s + 1 + x - M;
-                    need = max(need, min(over, x + 1));
-                }
-                need = k7_block_max(need, red);
+                const int need = sim.test(s + 1, e - 1);
                 if (need > 0) { t_ok = t + need; break; }
-                for (int x = tid; x < e; x += K7_THREADS) occ[(t + x) & mask] += s + 1 + x;
-                if (tid == 0) {
+                sim.add(s + 1, e - 1);
+                __syncwarp();
+                if (lane == 0) {
                     pp[q] = t - 1;
                     if (e < o) {                                   // overdue in rounds t+e .. t+o-1
                         const unsigned v = (unsigned)(s - (t - 1));
@@ -237,46 +190,59 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
                     }
                     fin[(t + o) & mask] += 1;
                 }
+                if (lane == 0) run[KV_IDX(nrun, nm, 1102)] = (unsigned short)q;
+                ++nrun;
+                __syncwarp();
                 if (q == frontier) ++frontier; else --npe;
                 if (npe == 0) {
                     head = frontier;
-                    __syncthreads();
                 } else {                                           // an evicted request further down the list
-                    int first = INT_MAX;
-                    for (int k = q + 1 + tid; k < frontier; k += K7_THREADS)
-                        if (pp[k] < 0) { first = k; break; }
-                    head = k7_block_min(first, red);
+                    int found = INT_MAX;
+                    for (int k0 = q + 1; k0 < frontier && found == INT_MAX; k0 += 32) {
+                        const unsigned v = __ballot_sync(KV_FULL, k0 + lane < frontier && pp[k0 + lane] < 0);
+                        if (v) found = k0 + __ffs(v) - 1;
+                    }
+                    head = found;
                     if (head == INT_MAX) { failed = true; break; }
                 }
                 if (head >= n) break;
             }
             if (failed) break;
         }
-        __syncthreads();
 
         // ---- step 3: ordered eviction while round t is over budget
-        while (occ[t & mask] > M) {
-            u64 best = ~0ull;
-            for (int q = tid; q < frontier; q += K7_THREADS) {
-                const int p = pp[q];
-                if (p >= 0 && t <= p + po[q]) {
-                    const int est = max(pe[q], t - p);
-                    const u64 key = ((u64)(unsigned)est << (2 * K7_ID_BITS)) | ((u64)(unsigned)pid[q] << K7_ID_BITS) | (u64)(unsigned)q;
-                    best = key < best ? key : best;
+        for (;;) {
+            const int used = __shfl_sync(KV_FULL, sim.cur - lane, sim.tau);
+            if (used <= M) { peak = max(peak, used); break; }
+            // smallest (estimate, request id) among the running; the list loses what has finished
+            int kept = 0, est_min = INT_MAX, id_min = INT_MAX, at_min = 0;
+            for (int k0 = 0; k0 < nrun; k0 += 32) {
+                const int k = k0 + lane, r = k < nrun ? run[k] : 0, p = pp[r];
+                const bool keep = k < nrun && p >= 0 && t <= p + po[r];
+                const unsigned v = __ballot_sync(KV_FULL, keep);
+                if (keep) {
+                    const int at = kept + __popc(v & ((1u << lane) - 1u)), est = max(pe[r], t - p), id = pid[r];
+                    run[at] = (unsigned short)r;
+                    if (est < est_min || (est == est_min && id < id_min)) { est_min = est; id_min = id; at_min = at; }
                 }
+                kept += __popc(v);
+                __syncwarp();
             }
-            best = k7_block_min64(best, red64);
-            if (best == ~0ull) { failed = true; break; }
-            const int q = (int)(best & ((1u << K7_ID_BITS) - 1));
-            const int est = (int)(best >> (2 * K7_ID_BITS));
+            nrun = kept;
+            const int est = kv_warp_min(est_min);
+            const int id = kv_warp_min(est_min == est ? id_min : INT_MAX);
+            if (est == INT_MAX) { failed = true; break; }
+            const int at = __shfl_sync(KV_FULL, at_min, __ffs(__ballot_sync(KV_FULL, est_min == est && id_min == id)) - 1);
+            const int q = run[KV_IDX(at, nm, 1103)];
             const int p = pp[q], s = ps[q], o = po[q], e0 = pe[q];
-            const int cells = p + est - t + 1;                     // what is left of its projection
-            for (int x = tid; x < cells; x += K7_THREADS) occ[(t + x) & mask] -= s + (t + x - p);
+            sim.remove(s - (p - sim.T0), p + est - sim.T0);        // what is left of its projection
             const unsigned v = (unsigned)(s - p);
             const bool overdue = e0 < o && t >= p + e0 + 1;
             if (overdue) { cnt -= 1u; A -= v; }
-            __syncthreads();
-            if (tid == 0) {
+            __syncwarp();
+            --nrun;
+            if (lane == 0) {
+                run[at] = run[nrun];
                 if (e0 < o) {
                     if (!overdue) { dc[(p + e0 + 1) & mask] -= 1; dA[(p + e0 + 1) & mask] -= v; }
                     dc[(p + o + 1) & mask] += 1; dA[(p + o + 1) & mask] += v;
@@ -288,29 +254,21 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
             ++evictions; ++npe;
             head = min(head, q);
             t_ok = t + 1;
-            __syncthreads();
+            __syncwarp();
         }
         if (failed) break;
-
         // ---- step 4: the round runs
-        const int used = occ[t & mask];
-        __syncthreads();
-        peak = max(peak, used);
-        if (tid == 0) occ[t & mask] = 0;
-        ++t;
+        sim.advance(1, 0);
     }
     if (failed) {
-        if (tid == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
+        if (lane == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
         return;
     }
-    if (tid == 0) acc = 0;
-    __syncthreads();
-    u64 part = 0;
-    for (int q = tid; q < n; q += K7_THREADS) {
+    i64 part = 0;
+    for (int q = lane; q < n; q += 32) {
         P.start_out[base + KV_IDX(pid[q], n, 1101)] = pp[q];
-        part += (u64)((i64)pp[q] + po[q]);
+        part += (i64)pp[q] + po[q];
     }
-    if (part) atomicAdd(&acc, part);
-    __syncthreads();
-    if (tid == 0) { P.tel_out[b] = (i64)acc; P.evict_out[b] = evictions; P.peak_out[b] = peak; }
+    for (int d = 16; d >= 1; d >>= 1) part += __shfl_xor_sync(KV_FULL, part, d);
+    if (lane == 0) { P.tel_out[b] = part; P.evict_out[b] = evictions; P.peak_out[b] = peak; }
 }

@@ -214,6 +214,20 @@ struct ChunkSim {
         if (last > 31 && back >= 0) atomicAdd(cells_of(T0 + last), sp + om - back);
     }
 
+    // Takes back what is left (from t on) of a window whose ramp is a + x in round x, counted from T0, and
+    // whose last round is `last`.  The bounds fall by the least the ramp has in a chunk it covers whole.
+    __device__ __forceinline__ void remove(int a, int last) {
+        if (rl >= 0 && lane <= last) cur -= a + lane;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const int x = 32 * (lane + 1) + 1024 * m;
+            if (x + 31 <= last) U[m] -= a + x;
+            if (x + 31 < last) { A[m] -= a; C[m] -= 1; }
+        }
+        const int x = (last & ~31) + lane;                          // the chunk the window ends in
+        if (last > 31 && x <= last) atomicAdd(cells_of(T0 + last), -(a + x));
+    }
+
     // Admit one request (sp = s + 1, om = o - 1) at the earliest start; all 32 lanes call this with
     // identical arguments.  left: requests still to be admitted, this one included.
     __device__ __forceinline__ void admit(int sp, int om, int left, int* status) {
