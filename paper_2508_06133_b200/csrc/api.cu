@@ -308,7 +308,9 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             // a candidate replays (stride - 1) / 2 positions on average to reach its first moved one:
             // 0.2 % of the list at 256 snapshots, for which the base run stores 256 states instead of n
             i64 stride = ((i64)n + kSnapshots - 1) / kSnapshots;
-            while ((((i64)n + stride - 1) / stride) * (i64)per > (i64)kSnapBudget) ++stride;
+            stride = (stride + 3) & ~3ll;               // requests are admitted four at a time
+            if (stride < 16) stride = 16;               // the base run stops for every snapshot
+            while ((((i64)n + stride - 1) / stride) * (i64)per > (i64)kSnapBudget) stride += 4;
             h->snap_stride = (int)stride;
             h->snap_count = (n + h->snap_stride - 1) / h->snap_stride;
         }

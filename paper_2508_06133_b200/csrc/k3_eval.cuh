@@ -141,36 +141,29 @@ k3_base_run(const BaseRunParams p) {
     SIM sim;
     sim.attach((int*)smem_raw, L);
     sim.reset(M);
-    i64 tel = 0;                                         // of the positions before this block
+    i64 tel = 0;                                         // this lane's share of the completion times so far
     int2 next = lane < n ? tbl_base[lane] : make_int2(1, 1);
     int to_snap = 0, idx = 0;                            // positions until the next snapshot, its number
-    for (int q0 = 0; q0 < n; q0 += 32) {
+    for (int q0 = 0; q0 < n;) {
         const int2 so = next;
-        if (q0 + 32 + lane < n) next = tbl_base[q0 + 32 + lane];
-        const int cnt = min(32, n - q0);
-        int mine = 0;
-        const int sp = so.x + 1, om = so.y - 1;
-        int sp_next = __shfl_sync(KV_FULL, sp, 0), om_next = __shfl_sync(KV_FULL, om, 0);
-        for (int k = 0; k < cnt; ++k) {
-            if (to_snap == 0) {
-                const int i = (int)KV_IDX(idx, p.snap_count, 401);
-                i64 before = lane < k ? (i64)mine + so.y : 0;    // this block's completions so far
-                for (int d = 16; d >= 1; d >>= 1) before += __shfl_xor_sync(KV_FULL, before, d);
-                sim.store(snap_ring + (size_t)i * L, snap_hdr + i, tel + before);
-                ++idx;
-                to_snap = stride;
-            }
-            --to_snap;
-            const int sp_k = sp_next, om_k = om_next;
-            sp_next = __shfl_sync(KV_FULL, sp, k + 1); om_next = __shfl_sync(KV_FULL, om, k + 1);
-            sim.admit(sp_k, om_k, n - q0 - k, status);
-            if (lane == k) mine = sim.start();
+        // a block ends where a snapshot is due (the stride is a multiple of 4, so is every block but the last)
+        if (to_snap == 0) {
+            const int i = (int)KV_IDX(idx, p.snap_count, 401);
+            i64 before = tel;
+            for (int d = 16; d >= 1; d >>= 1) before += __shfl_xor_sync(KV_FULL, before, d);
+            sim.store(snap_ring + (size_t)i * L, snap_hdr + i, before);
+            ++idx;
+            to_snap = stride;
         }
-        if (q0 + lane < n) base_starts_pos[q0 + lane] = mine;
-        i64 done = lane < cnt ? (i64)mine + so.y : 0;
-        for (int d = 16; d >= 1; d >>= 1) done += __shfl_xor_sync(KV_FULL, done, d);
-        tel += done;
+        const int cnt = min(min(32, n - q0), to_snap);
+        if (q0 + cnt + lane < n) next = tbl_base[q0 + cnt + lane];
+        const int mine = sim_run_block<true>(sim, so, cnt, n - q0, status);
+        if (lane < cnt) base_starts_pos[q0 + lane] = mine;
+        if (lane < cnt) tel += (i64)mine + so.y;
+        q0 += cnt;
+        to_snap -= cnt;
     }
+    for (int d = 16; d >= 1; d >>= 1) tel += __shfl_xor_sync(KV_FULL, tel, d);
     if (lane == 0) *p.base_tel = tel;
 }
 
@@ -233,13 +226,9 @@ k3_eval_moves(const MoveEvalParams p) {
             so = tbl[bp];
             if (kStarts) id = p.base_order[bp];
         }
-        const int cnt = min(32, n - q0), sp = so.x + 1, om = so.y - 1;
+        const int cnt = min(32, n - q0);
         if (lane < cnt) sum_o += so.y;
-        int mine = 0;
-        for (int k = 0; k < cnt; ++k) {
-            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, p.status);
-            if (kStarts && lane == k) mine = sim.start();
-        }
+        const int mine = sim_run_block<false>(sim, so, cnt, n - q0, p.status);
         if (kStarts && lane < cnt) starts[KV_IDX(id, n, 405)] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
@@ -314,13 +303,9 @@ k3_eval_orders(const OrderEvalParams p) {
             if (lane == 0) p.tel_out[c] = INT64_MAX;
             return;
         }
-        const int cnt = min(32, n - q0), sp = so.x + 1, om = so.y - 1;
+        const int cnt = min(32, n - q0);
         if (lane < cnt) sum_o += so.y;
-        int mine = 0;
-        for (int k = 0; k < cnt; ++k) {
-            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, p.status);
-            if (kStarts && lane == k) mine = sim.start();
-        }
+        const int mine = sim_run_block<false>(sim, so, cnt, n - q0, p.status);
         if (kStarts && lane < cnt) starts[id] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);

@@ -205,14 +205,11 @@ k3_eval_policy(const int* __restrict__ s_all, const int* __restrict__ o_all, int
     i64 sum_o = 0;
     int* starts = starts_out ? starts_out + ((size_t)b * num_policies + kpol) * n : nullptr;
     for (int q0 = 0; q0 < n; q0 += 32) {
-        int id = 0, sp = 2, om = 0;
+        int id = 0;
+        int2 so = make_int2(1, 1);
         const int cnt = min(32, n - q0);
-        if (lane < cnt) { id = (int)KV_IDX(fin[q0 + lane], n, 906); sp = s[id] + 1; om = o[id] - 1; sum_o += om + 1; }
-        int mine = 0;
-        for (int k = 0; k < cnt; ++k) {
-            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), n - q0 - k, status);
-            if (lane == k) mine = sim.start();
-        }
+        if (lane < cnt) { id = (int)KV_IDX(fin[q0 + lane], n, 906); so = make_int2(s[id], o[id]); sum_o += so.y; }
+        const int mine = sim_run_block<false>(sim, so, cnt, n - q0, status);
         if (starts && lane < cnt) starts[id] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);

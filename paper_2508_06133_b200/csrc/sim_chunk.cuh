@@ -50,6 +50,7 @@ template <int NM>
 struct ChunkSim {
     static constexpr int kWarps = NM == 1 ? 4 : NM == 2 ? 2 : 1;    // warps per CTA: 16 KB of rings
     static constexpr int kMinCtas = 10;                             // CTAs per SM the registers have to allow
+    static constexpr bool kGroups = true;                           // has surely()
     static constexpr int kMeta = 32 + 96 * NM;                      // state ints besides the ring
     __host__ __device__ static constexpr int ring_cells(int L) { return L - kMeta; }   // shared-memory ints per warp
 
@@ -210,8 +211,9 @@ struct ChunkSim {
             }
         }
         const int last = tau + om, back = (last & 31) - lane;       // the chunk the window ends in
-        // an atomic without a result: nothing behind it waits for the old value
-        if (last > 31 && back >= 0) atomicAdd(cells_of(T0 + last), sp + om - back);
+        // an atomic without a result, by every lane: nothing waits for the old value, and adding zero costs
+        // less than a branch around it (a window that ends in chunk 0 meets that chunk's own slot, unused)
+        atomicAdd(cells_of(T0 + last), last > 31 && back >= 0 ? sp + om - back : 0);
     }
 
     // Takes back what is left (from t on) of a window whose ramp is a + x in round x, counted from T0, and
@@ -228,19 +230,78 @@ struct ChunkSim {
         if (last > 31 && x <= last) atomicAdd(cells_of(T0 + last), -(a + x));
     }
 
+    // Whether requests of `size` tokens in all (s + o each), the longest with om = o - 1, certainly fit at t
+    // one beside the other: none of them uses more than its s + o in any round.
+    __device__ __forceinline__ bool surely(int size, int om) const {
+        const int nk = nkt - size;
+        bool over = (unsigned)rl <= (unsigned)om && cur > nk;
+        over = over || (xr <= om && U[0] > nk);
+        if (NM > 1 && tau + om >= 1024 + 32) {
+#pragma unroll
+            for (int m = 1; m < NM; ++m) over = over || (xr + 1024 * m <= om && U[m] > nk);
+        }
+        return !__any_sync(KV_FULL, over);
+    }
+
     // Admit one request (sp = s + 1, om = o - 1) at the earliest start; all 32 lanes call this with
-    // identical arguments.  left: requests still to be admitted, this one included.
-    __device__ __forceinline__ void admit(int sp, int om, int left, int* status) {
+    // identical arguments.  left: requests still to be admitted, this one included.  Returns whether it
+    // had to wait.
+    __device__ __forceinline__ bool admit(int sp, int om, int left, int* status) {
+        bool waited = false;
         for (int guard = 0;; ++guard) {
             const int d = test(sp, om);
             if (d <= 0) break;
+            waited = true;
             advance(d, left);
-            if (guard > kv_loop_cap(32 * mask + 2048)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); return; }
+            if (guard > kv_loop_cap(32 * mask + 2048)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); return true; }
         }
         add(sp, om);
         acc += tau;
+        return waited;
     }
 };
+
+// Up to 32 consecutive requests of a list, (s, o) of the k-th in lane k, the list going on with
+// left - cnt behind them.  Returns the start of the k-th in lane k.
+//
+// kGroups: where memory is not short, several requests start in the same round; four at a time are then
+// asked for together, and if their sizes certainly fit they are added one behind the other without a test
+// each, so that the additions overlap.  Tried only behind a request that did not wait.  For a run that
+// stands alone, where the latency of an admission counts: 0.251 -> 0.226 ms for 1,000 requests, 1.83 ->
+// 1.69 ms for 10,000.  Many runs side by side are bound by instructions, of which the tries cost more than
+// they save (8.70 -> 9.49 ms for 16,384 moves of the 10,000), so they go without.
+template <bool kGroups, class SIM>
+__device__ __forceinline__ int sim_run_block(SIM& sim, int2 so, int cnt, int left, int* status) {
+    const int lane = threadIdx.x & 31, sp = so.x + 1, om = so.y - 1;
+    int mine = 0;
+    if constexpr (kGroups && SIM::kGroups) {
+        int size = so.x + so.y, longest = om;                       // of the aligned four this lane is in
+        size += __shfl_xor_sync(KV_FULL, size, 1); size += __shfl_xor_sync(KV_FULL, size, 2);
+        longest = max(longest, __shfl_xor_sync(KV_FULL, longest, 1));
+        longest = max(longest, __shfl_xor_sync(KV_FULL, longest, 2));
+        bool waited = false;
+        for (int k = 0; k < cnt;) {
+            if ((k & 3) == 0 && !waited && k + 4 <= cnt &&
+                sim.surely(__shfl_sync(KV_FULL, size, k), __shfl_sync(KV_FULL, longest, k))) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sim.add(__shfl_sync(KV_FULL, sp, k + j), __shfl_sync(KV_FULL, om, k + j));
+                sim.acc += 4 * sim.tau;
+                if ((lane & ~3) == k) mine = sim.start();
+                k += 4;
+                continue;
+            }
+            waited = sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), left - k, status);
+            if (lane == k) mine = sim.start();
+            ++k;
+        }
+    } else {
+        for (int k = 0; k < cnt; ++k) {
+            sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), left - k, status);
+            if (lane == k) mine = sim.start();
+        }
+    }
+    return mine;
+}
 
 // Ring slots (32 cells each, a power of two) for the longest decode of a handle: a window that starts
 // in the last round of its chunk ends (30 + omax) / 32 chunks further on.

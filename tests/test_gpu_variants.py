@@ -1,0 +1,147 @@
+"""Kernel variants at the sizes where one takes over from another, against the CPU oracle."""
+import numpy as np
+import pytest
+
+import oracle as orc
+from paper_2508_06133_b200 import binding as kv
+from paper_2508_06133_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def oracle_moves(s, o, M, base, codes):
+    mv = [orc.decode_move(len(s), int(c)) for c in codes]
+    return orc.eval_moves(s, o, M, base, [m[0] for m in mv], [m[1] for m in mv], [m[2] for m in mv])
+
+
+@pytest.mark.parametrize("omax", [1, 2, 31, 32, 33, 34, 65, 1025, 1026, 2049, 2050, 4097, 4098, 8193, 8194])
+def test_timeline_sizes(omax):
+    """The longest decode at and beside the numbers of far chunks and far registers a timeline is built
+    for, and the first length of the simulator that keeps every cell: explicit orders with starts, moves
+    from snapshots (n = 70 has five), the starts checked again and one of them broken."""
+    rng = np.random.default_rng(7 * omax)
+    n, M = 70, 5 * omax + 40
+    s = rng.integers(1, M - omax, n).astype(np.int32)
+    o = rng.integers(1, omax + 1, n).astype(np.int32)
+    o[:4] = omax
+    s[:2] = 1
+    s[::9] = M - o[::9]
+    s[4:40:3] = 1                                            # several fit beside each other
+    orders = np.stack([rng.permutation(n) for _ in range(3)]).astype(np.int32)
+    codes = np.arange(0, 3 * n * (n - 1) // 2, 61, dtype=np.int64)
+    with kv.Scheduler(s, o, M) as h:
+        tel, _, starts = h.eval_batch(kv.CAND_ORDER, orders, want_starts=True)
+        broken = starts.copy()
+        broken[:, orders[0][n - 1]] = starts[:, 0]            # two requests at the start of the first
+        again, ok, _ = h.eval_batch(kv.CAND_START_TIMES, np.concatenate([starts, broken]), want_feasible=True)
+        h.set_base_order(orders[0])
+        mtel, _, _ = h.eval_batch(kv.CAND_MOVE, codes)
+        mtel2, _, mstarts = h.eval_batch(kv.CAND_MOVE, codes[:5], want_starts=True)
+    for c in range(3):
+        p, t, _ = orc.list_schedule_rounds(s, o, M, orders[c])
+        assert tel[c] == t and (starts[c] == p).all()
+        assert again[c] == t and ok[c]
+        ref = orc.check_schedule(s, o, M, broken[c])
+        assert again[3 + c] == ref["tel"] and bool(ok[3 + c]) == ref["feasible"]
+    ref = oracle_moves(s, o, M, orders[0], codes)
+    assert (mtel == ref).all() and (mtel2 == ref[:5]).all()
+    assert (mstarts.astype(np.int64).sum(1) + int(o.sum()) == ref[:5]).all()
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 1023, 1024, 1025, 2049, 12000, 20000])
+def test_sorting_and_batch_selection_sizes(n):
+    """One tile, its edges, several, and sizes beyond what the solvers keep in shared memory."""
+    inst = W.mixed_backlog(n, 5 + n, 70000)
+    s, o, M = inst.s, inst.o, inst.M
+    s[: n // 3] = 17; o[: n // 3] = 9                         # ties in size and in decode length
+    with kv.Scheduler(s, o, M) as h:
+        order, offs, tel = h.sorted_f()
+    r_order, r_offs = orc.sorted_f_prefix(s, o, M)
+    assert (order == r_order).all() and (offs == r_offs).all()
+    assert tel == orc.list_schedule_rounds(s, o, M, r_order)[1]
+
+
+@pytest.mark.parametrize("n", [2, 63, 65, 513, 1500])
+@pytest.mark.parametrize("weight", [0, 1])
+def test_local_swap_sizes(n, weight):
+    """Blocks of the prefix minima and their edges; a large prefill weight (many swaps)."""
+    rng = np.random.default_rng(n)
+    M = 4000
+    s = rng.integers(1, 900, n).astype(np.int32)
+    o = rng.integers(1, 400, n).astype(np.int32)
+    with kv.Scheduler(s, o, M) as h:
+        if weight:
+            h.set_prefill_weight(3, 2)
+        order, offs, _ = h.sorted_f_local_swap()
+    ref = orc.sorted_g_local_swap(s, o, M, 3, 2) if weight else orc.sorted_f_local_swap(s, o, M)
+    assert (order == ref[0]).all() and (offs == ref[1]).all()
+
+
+def test_solvers_beyond_shared_memory():
+    """Local swap and quantile selection where their arrays are in global memory (more than 11,000)."""
+    inst = W.mixed_backlog(12500, 3, 1 << 22)
+    with kv.Scheduler(inst.s, inst.o, inst.M) as h:
+        order, offs, _ = h.sorted_f_quantile(9)
+    ref = orc.sorted_f_quantile(inst.s, inst.o, inst.M, 9)
+    assert (order == ref[0]).all() and (offs == ref[1]).all()
+    rng = np.random.default_rng(8)
+    n, M = 12500, 1 << 21                                    # few batches and swaps: the oracle walks every pair
+    s = np.full(n, 200, dtype=np.int32)
+    o = np.sort(rng.integers(100, 400, n)).astype(np.int32)
+    with kv.Scheduler(s, o, M) as h:
+        order, offs, _ = h.sorted_f_local_swap()
+    ref = orc.sorted_f_local_swap(s, o, M)
+    assert (order == ref[0]).all() and (offs == ref[1]).all()
+
+
+@pytest.mark.parametrize("n,M", [(9, 200), (40, 600), (24, 1100), (24, 1250)])
+def test_dynamic_programme_sizes(n, M):
+    """The last tables that fit shared memory and the first that do not."""
+    rng = np.random.default_rng(n + M)
+    s = rng.integers(1, M // 3, n).astype(np.int32)
+    o = rng.integers(1, M // 4, n).astype(np.int32)
+    with kv.Scheduler(s, o, M) as h:
+        order, offs, _ = h.sorted_f_dp()
+    ref = orc.sorted_f_exact(s, o, M, orc.DP)
+    assert (order == ref[0]).all() and (offs == ref[1]).all()
+
+
+@pytest.mark.parametrize("lookahead", [127, 128, 129, 400])
+def test_online_windows(lookahead):
+    """A burst of arrivals: windows up to and beyond what a plan keeps in registers, plans that live so
+    long that several of their batches, the requests behind the window and late arrivals are used."""
+    rng = np.random.default_rng(lookahead)
+    n, M = 420, 3000
+    s = rng.integers(1, 500, n).astype(np.int32)
+    o = rng.integers(1, 120, n).astype(np.int32)
+    a = np.sort(np.where(rng.random(n) < 0.7, 0, rng.integers(0, 2000, n))).astype(np.int32)
+    for period in (10, 100000):
+        starts, lat, _ = kv.online_simulate([n], a[None], s[None], o[None], M, kv.POLICY_SORTED_F, period, lookahead)
+        p, tot = orc.online_schedule(a, s, o, M, kv.POLICY_SORTED_F, period, lookahead)
+        assert (starts[0] == p).all() and lat[0] == tot
+
+
+@pytest.mark.parametrize("n", [2, 40, 1531])
+def test_host_candidates_are_checked(n):
+    """An order with a repeated id, one with an id outside 0 .. n-1, a negative start and one of 2^30 are
+    refused, wherever they stand; the handle goes on."""
+    rng = np.random.default_rng(n)
+    s = rng.integers(1, 50, n).astype(np.int32)
+    o = rng.integers(1, 50, n).astype(np.int32)
+    good = np.stack([rng.permutation(n) for _ in range(7)]).astype(np.int32)
+    with kv.Scheduler(s, o, 4000) as h:
+        tel, _, starts = h.eval_batch(kv.CAND_ORDER, good, want_starts=True)
+        for row, col, value in ((6, n - 1, good[6, 0]), (0, 0, n), (3, n // 2, -1)):
+            bad = good.copy()
+            bad[row, col] = value
+            with pytest.raises(kv.SchedError) as e:
+                h.eval_batch(kv.CAND_ORDER, bad)
+            assert e.value.code == kv.E_NOT_PERMUTATION
+        for row, col, value in ((6, n - 1, -1), (0, 0, 1 << 30)):
+            bad = starts.copy()
+            bad[row, col] = value
+            with pytest.raises(kv.SchedError) as e:
+                h.eval_batch(kv.CAND_START_TIMES, bad, want_feasible=True)
+            assert e.value.code == kv.E_INVAL
+        again, ok, _ = h.eval_batch(kv.CAND_START_TIMES, starts, want_feasible=True)
+    assert ok.all() and (again == tel).all()
