@@ -878,15 +878,15 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
         // Algorithm 3: ascending (s+o, index), then first fit + improving swaps, batch after batch
         KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_TOTAL_SIZE}, n, 1, h->d_keys_a, h->d_vals_b, h->d_vals_a));
         if ((i64)h->g_num * h->M + (i64)h->g_den * h->omax >= (1ll << 31)) return SCHED_E_UNSUPPORTED;   // 32-bit weights
-        // the solver's arrays in shared memory (20 bytes per request) up to about 11,000 requests
+        // the solver's arrays in shared memory (21 bytes per request) up to about 11,000 requests
         const size_t bytes = k2l_bytes<unsigned short>(n);
         if (n < 65536 && bytes <= (size_t)h->smem_optin - 2048) {
-            KV_CUDA(cudaFuncSetAttribute(k2_local_swap<unsigned short>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 2048));
-            k2_local_swap<unsigned short><<<1, K2L_THREADS, bytes, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, nullptr,
+            KV_CUDA(cudaFuncSetAttribute(k2_local_swap<unsigned short, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 2048));
+            k2_local_swap<unsigned short, true><<<1, K2L_THREADS, bytes, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, nullptr,
                                                                          h->d_vals_b, h->d_batch_off, h->d_num_batches, h->d_status);
         } else {
             if (!h->d_ls) KV_TRY(dev_alloc(&h->d_ls, 7 * (size_t)n + 32));
-            k2_local_swap<int><<<1, K2L_THREADS, 0, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, h->d_ls,
+            k2_local_swap<int, false><<<1, K2L_THREADS, 0, st>>>(h->d_s, h->d_o, h->d_vals_a, n, h->M, h->g_num, h->g_den, h->d_ls,
                                                           h->d_vals_b, h->d_batch_off, h->d_num_batches, h->d_status);
         }
         KV_TRY(check_launch(h));
