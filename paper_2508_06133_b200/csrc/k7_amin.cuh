@@ -35,7 +35,9 @@
 //   The running requests are a compact list, so an eviction looks at them and not at everything that
 //   has ever started.
 // What bounds it: a scenario is a chain (2,000 requests of the paper's lengths: 2,400 admissions, 380
-// evictions, 1,400 walks), so the latency of each; one warp needs no block barriers for them.
+// evictions among 550 running, 1,300 walks: 1,000,000 instructions of one warp at 5 cycles each), so the
+// number of instructions; one warp needs no block barriers for them.  64 scenarios 2.34 ms; 2.44 with 256
+// threads that test every round of a window and look at everything that has ever started.
 #pragma once
 
 #include "common.cuh"
@@ -180,17 +182,15 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
                 const int need = sim.test(s + 1, e - 1);
                 if (need > 0) { t_ok = t + need; break; }
                 sim.add(s + 1, e - 1);
-                __syncwarp();
-                if (lane == 0) {
+                // its events, one lane each: overdue in rounds t+e .. t+o-1 if the estimate is short, then over
+                {
+                    const unsigned v = (unsigned)(s - (t - 1));
+                    unsigned* cell = (lane < 4 ? (lane & 1 ? dA : (unsigned*)dc) : (unsigned*)fin) + ((lane < 2 ? t + e : t + o) & mask);
+                    const unsigned add = lane == 0 || lane == 4 ? 1u : lane == 1 ? v : lane == 2 ? ~0u : 0u - v;
+                    if (lane < 5) atomicAdd(cell, lane == 4 || e < o ? add : 0u);
                     pp[q] = t - 1;
-                    if (e < o) {                                   // overdue in rounds t+e .. t+o-1
-                        const unsigned v = (unsigned)(s - (t - 1));
-                        dc[(t + e) & mask] += 1; dA[(t + e) & mask] += v;
-                        dc[(t + o) & mask] -= 1; dA[(t + o) & mask] -= v;
-                    }
-                    fin[(t + o) & mask] += 1;
+                    run[KV_IDX(nrun, nm, 1102)] = (unsigned short)q;
                 }
-                if (lane == 0) run[KV_IDX(nrun, nm, 1102)] = (unsigned short)q;
                 ++nrun;
                 __syncwarp();
                 if (q == frontier) ++frontier; else --npe;
@@ -214,21 +214,17 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
         for (;;) {
             const int used = __shfl_sync(KV_FULL, sim.cur - lane, sim.tau);
             if (used <= M) { peak = max(peak, used); break; }
-            // smallest (estimate, request id) among the running; the list loses what has finished
-            int kept = 0, est_min = INT_MAX, id_min = INT_MAX, at_min = 0;
-            for (int k0 = 0; k0 < nrun; k0 += 32) {
-                const int k = k0 + lane, r = k < nrun ? run[k] : 0, p = pp[r];
-                const bool keep = k < nrun && p >= 0 && t <= p + po[r];
-                const unsigned v = __ballot_sync(KV_FULL, keep);
-                if (keep) {
-                    const int at = kept + __popc(v & ((1u << lane) - 1u)), est = max(pe[r], t - p), id = pid[r];
-                    run[at] = (unsigned short)r;
-                    if (est < est_min || (est == est_min && id < id_min)) { est_min = est; id_min = id; at_min = at; }
-                }
-                kept += __popc(v);
-                __syncwarp();
+            // smallest (estimate, request id) among the running
+            int est_min = INT_MAX, id_min = INT_MAX, at_min = 0, live = 0;
+#pragma unroll 4
+            for (int k = lane; k < nrun; k += 32) {
+                const int r = run[k], p = pp[r];
+                const bool runs = t <= p + po[r];
+                const int est = runs ? max(pe[r], t - p) : INT_MAX, id = pid[r];
+                live += runs ? 1 : 0;
+                const bool less = est < est_min || (est == est_min && id < id_min);
+                est_min = less ? est : est_min; id_min = less ? id : id_min; at_min = less ? k : at_min;
             }
-            nrun = kept;
             const int est = kv_warp_min(est_min);
             const int id = kv_warp_min(est_min == est ? id_min : INT_MAX);
             if (est == INT_MAX) { failed = true; break; }
@@ -250,6 +246,19 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
                 fin[(p + o + 1) & mask] -= 1;
                 pe[q] = est;
                 pp[q] = -1;
+            }
+            __syncwarp();
+            if (2 * __reduce_add_sync(KV_FULL, live) < nrun) {     // drop what has finished
+                int kept = 0;
+                for (int k0 = 0; k0 < nrun; k0 += 32) {
+                    const int k = k0 + lane, r = k < nrun ? run[k] : 0;
+                    const bool keep = k < nrun && t <= pp[r] + po[r];
+                    const unsigned v = __ballot_sync(KV_FULL, keep);
+                    if (keep) run[kept + __popc(v & ((1u << lane) - 1u))] = (unsigned short)r;
+                    kept += __popc(v);
+                    __syncwarp();
+                }
+                nrun = kept;
             }
             ++evictions; ++npe;
             head = min(head, q);

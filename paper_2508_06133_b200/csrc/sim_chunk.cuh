@@ -173,20 +173,23 @@ struct ChunkSim {
         return kv_warp_max(d);
     }
 
-    // 0: (sp, om) fits at t; otherwise a lower bound of the rounds it has to wait
-    __device__ __forceinline__ int test(int sp, int om) {
+    // One reduction answers for all lanes: above 0 the wait that chunk 0 asks for, 0 where a far bound
+    // says "perhaps" (or a round fits exactly), below 0 everything is clear
+    __device__ __forceinline__ int ask(int sp, int om) const {
         const int nk = nkt - sp;                         // it fits  <=>  V[x] <= nk in every round of the window
-        // one reduction answers for all lanes: above 0 the wait that chunk 0 asks for, 0 where a far bound
-        // says "perhaps" (or a round fits exactly), below 0 everything is clear
         int v = (unsigned)rl <= (unsigned)om ? __viaddmin_s32(cur, -nk, rl + 1) : INT_MIN;
         if (xr <= om && U[0] > nk) v = max(v, 0);
         if (NM > 1 && tau + om >= 1024 + 32) {
 #pragma unroll
             for (int m = 1; m < NM; ++m) if (xr + 1024 * m <= om && U[m] > nk) v = max(v, 0);
         }
-        const int d = kv_warp_max(v);
+        return kv_warp_max(v);
+    }
+    // 0: (sp, om) fits at t; otherwise a lower bound of the rounds it has to wait
+    __device__ __forceinline__ int test(int sp, int om) {
+        const int d = ask(sp, om);
         if (d < 0) return 0;
-        return d > 0 ? d : far_need(om, nk);
+        return d > 0 ? d : far_need(om, nkt - sp);
     }
     // t moves on by d rounds
     __device__ __forceinline__ void advance(int d, int left) {
@@ -243,6 +246,25 @@ struct ChunkSim {
         return !__any_sync(KV_FULL, over);
     }
 
+    // The same result for a run that stands alone: one branch where the request does not wait.
+    __device__ __forceinline__ bool admit_alone(int sp, int om, int left, int* status) {
+        int v = ask(sp, om);
+        const bool waited = v >= 0;                      // or a far bound had to be looked at
+        if (waited) {
+            for (int guard = 0;; ++guard) {
+                const int d = v > 0 ? v : far_need(om, nkt - sp);
+                if (d <= 0) break;
+                advance(d, left);
+                if (guard > kv_loop_cap(32 * mask + 2048)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); return true; }
+                v = ask(sp, om);
+                if (v < 0) break;
+            }
+        }
+        add(sp, om);
+        acc += tau;
+        return waited;
+    }
+
     // Admit one request (sp = s + 1, om = o - 1) at the earliest start; all 32 lanes call this with
     // identical arguments.  left: requests still to be admitted, this one included.  Returns whether it
     // had to wait.
@@ -280,19 +302,27 @@ __device__ __forceinline__ int sim_run_block(SIM& sim, int2 so, int cnt, int lef
         longest = max(longest, __shfl_xor_sync(KV_FULL, longest, 1));
         longest = max(longest, __shfl_xor_sync(KV_FULL, longest, 2));
         bool waited = false;
-        for (int k = 0; k < cnt;) {
-            if ((k & 3) == 0 && !waited && k + 4 <= cnt &&
-                sim.surely(__shfl_sync(KV_FULL, size, k), __shfl_sync(KV_FULL, longest, k))) {
+        int k = 0;
+        for (; k + 4 <= cnt; k += 4) {
+            int s4[4], o4[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) sim.add(__shfl_sync(KV_FULL, sp, k + j), __shfl_sync(KV_FULL, om, k + j));
+            for (int j = 0; j < 4; ++j) { s4[j] = __shfl_sync(KV_FULL, sp, k + j); o4[j] = __shfl_sync(KV_FULL, om, k + j); }
+            if (!waited && sim.surely(__shfl_sync(KV_FULL, size, k), __shfl_sync(KV_FULL, longest, k))) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sim.add(s4[j], o4[j]);
                 sim.acc += 4 * sim.tau;
                 if ((lane & ~3) == k) mine = sim.start();
-                k += 4;
-                continue;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    waited = sim.admit_alone(s4[j], o4[j], left - k - j, status);
+                    if (lane == k + j) mine = sim.start();
+                }
             }
-            waited = sim.admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), left - k, status);
+        }
+        for (; k < cnt; ++k) {
+            sim.admit_alone(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), left - k, status);
             if (lane == k) mine = sim.start();
-            ++k;
         }
     } else {
         for (int k = 0; k < cnt; ++k) {
