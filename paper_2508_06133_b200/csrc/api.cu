@@ -18,6 +18,7 @@
 #include "k2_dp.cuh"
 #include "k2_quantile.cuh"
 #include "k3_eval.cuh"
+#include "k3_lanes.cuh"
 #include "k3_policy.cuh"
 #include "k5_argmin.cuh"
 #include "k6_online.cuh"
@@ -235,7 +236,7 @@ int validate_instance(i64 total, const int32_t* s, const int32_t* o, i64 M) {
 
 void free_ctx(sched_ctx* h) {
     if (!h) return;
-    void* ptrs[] = {h->d_arena, h->d_tel, h->d_stage, h->d_sort, h->d_k4, h->d_ls};
+    void* ptrs[] = {h->d_arena, h->d_lanes, h->d_tel, h->d_stage, h->d_sort, h->d_k4, h->d_ls};
     for (void* p : ptrs) if (p) kv_free(p);
     kv_host_free(h->h_pinned, h->pinned_bytes);
     if (h->ev_k3_begin) cudaEventDestroy(h->ev_k3_begin);
@@ -270,10 +271,16 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
     if (M >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
     const i64 total = (i64)B * n;
     KV_TRY(validate_instance(total, s, o, M));
-    int omax = 0; i64 sum_max = 0;
+    int omax = 0, least = INT32_MAX; i64 sum_max = 0; double volume = 0;
     for (int b = 0; b < B; ++b) {
         i64 sum = 0;
-        for (int i = 0; i < n; ++i) { int v = o[(i64)b * n + i]; sum += v; if (v > omax) omax = v; }
+        for (int i = 0; i < n; ++i) {
+            const int v = o[(i64)b * n + i], size = s[(i64)b * n + i] + v;
+            sum += v;
+            volume += (double)v * (size - 0.5 * v);
+            omax = v > omax ? v : omax;
+            least = size < least ? size : least;
+        }
         if (sum > sum_max) sum_max = sum;
     }
     if (sum_max + omax >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
@@ -288,7 +295,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) {
             rc = kv_cuda_fail(cudaGetLastError(), "cudaDeviceGetAttribute"); break;
         }
-        h->B = B; h->n = n; h->M = M; h->omax = omax; h->sum_o_max = sum_max;
+        h->B = B; h->n = n; h->M = M; h->omax = omax; h->least = least; h->volume = volume; h->sum_o_max = sum_max;
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
         h->nm = slots <= 32 ? 1 : slots <= 256 ? slots / 32 : 0;
@@ -482,6 +489,57 @@ int order_candidates(sched_ctx* h, const MoveSource& src, i64 count) {
     return SCHED_OK;
 }
 
+// One thread per candidate instead of one warp (k3_lanes.cuh)?  Its work goes with the rounds that pass, the
+// other kernel's with the admissions: rounds per request is the backlog's volume (sum of s o + o^2 / 2) over
+// n M, within a few per cent of the base run's.  Measured on 64,000 moves, a warp against a thread per
+// candidate: 1.9 rounds per request 9.2 / 5.4 ms, 2.9 rounds 33.0 / 23.6, 5.1 rounds 11.0 / 11.0, 7.6 rounds
+// 40.6 / 51.3, 12.9 rounds 14.7 / 25.7; from 32,000 moves on (1,000 warps) it is ahead at 2.9 rounds too
+// (16.6 / 13.5), with fewer the device is not full.  Decodes longer than its ring of events, and backlogs
+// whose candidate could pass 32 bits of waiting time in one partial sum, keep the warp.
+constexpr double LANE_ROUNDS = 3.5;
+constexpr i64 LANE_MIN = 32000;
+constexpr int LANE_CTAS = 5;               // resident per SM: the kernel's launch bound
+
+bool lanes_fit(const sched_ctx* h, i64 count, bool want_starts) {
+    return !want_starts && h->nm == 1 && count >= LANE_MIN && count > ordered_from(h) &&
+           h->volume <= LANE_ROUNDS * (double)h->M * h->n &&
+           (i64)h->n * (h->omax + LaneSim<unsigned>::CH) <= INT32_MAX;
+}
+
+// SCHED_OK with *done = false: no memory for the rings of events, nothing was launched.
+template <typename WORD>
+int run_lanes(sched_ctx* h, LaneParams& q, bool* done) {
+    typedef LaneSim<WORD> S;
+    const i64 need = ((i64)q.groups + S::kWarps - 1) / S::kWarps, most = (i64)LANE_CTAS * h->sm_count;
+    const int grid = (int)(need < most ? need : most);
+    const size_t bytes = (size_t)grid * S::kWarps * S::kRingWords * sizeof(WORD);
+    *done = false;
+    if (h->lanes_cap < bytes) {
+        if (h->d_lanes) { kv_free(h->d_lanes); h->d_lanes = nullptr; h->lanes_cap = 0; }
+        if (kv_malloc(&h->d_lanes, bytes) != cudaSuccess) { cudaGetLastError(); h->d_lanes = nullptr; return SCHED_OK; }
+        h->lanes_cap = bytes;
+    }
+    q.rings = h->d_lanes;
+    q.counter = h->d_counter + 1;
+    KV_CUDA(cudaMemsetAsync(q.counter, 0, sizeof(unsigned), h->stream));
+    KV_CUDA(cudaFuncSetAttribute(k3_lane_moves<WORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem));
+    k3_lane_moves<WORD><<<grid, 32 * S::kWarps, S::kSmem, h->stream>>>(q);
+    *done = true;
+    return SCHED_OK;
+}
+
+int launch_lanes(sched_ctx* h, const MoveEvalParams& p, bool* done) {
+    LaneParams q;
+    memset(&q, 0, sizeof(q));
+    q.m = p; q.omax = h->omax; q.least = h->least;
+    q.groups = (int)((p.count + 31) / 32);
+    // the requests that end in one round hold M tokens at most: sum of (s+o - least) and number in 32 bits?
+    q.shift = bits_of((u64)(h->M - h->least));
+    if (q.shift + bits_of((u64)(h->M / h->least)) <= 32) return run_lanes<unsigned>(h, q, done);
+    q.shift = 32;
+    return run_lanes<u64>(h, q, done);
+}
+
 // by_slot: TELs are left in launch-slot order (h->d_k4's launch_order maps a slot to its candidate
 // until the next call); the sweeps that only need the arg-min use it, see launch_argmin.
 int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, int iteration,
@@ -504,11 +562,15 @@ int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, 
         p.launch_order = last_launch_order(h, count);
     }
     KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
+    bool lanes = lanes_fit(h, count, starts_out != nullptr);
+    if (lanes) KV_TRY(launch_lanes(h, p, &lanes));
+    if (!lanes) {
 #define RUN(N)                                                                                    \
     if (starts_out) k3_eval_moves<N, true><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p);  \
     else k3_eval_moves<N, false><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p)
     KV_DISPATCH_SIM(h, RUN);
 #undef RUN
+    }
     KV_TRY(check_launch(h));
     KV_CUDA(cudaEventRecord(h->ev_k3_end, h->stream));
     h->ev_valid = true;

@@ -28,6 +28,8 @@ struct sched_ctx {
     int B, n;                // instances, requests per instance
     i64 M;
     int omax;                // largest decode length over all instances
+    int least;               // smallest s+o over all instances
+    double volume;           // tokens times rounds: sum of s o + o^2 / 2 over all instances
     int L;                   // ints per simulator state
     int nm;                  // chunked simulator with this many far registers per lane; 0: hybrid simulator
     int ring_cells;          // shared-memory ints one simulator needs
@@ -55,6 +57,8 @@ struct sched_ctx {
     int* d_ls;               // scratch of the Local Swap Search kernel: 7 arrays of n ints (lazy)
     void* d_k4;              // grow-only scratch of the launch ordering: bins[n+1], first_pos[count], order[count]
     size_t k4_cap;
+    void* d_lanes;           // grow-only scratch of the one-thread-per-candidate kernel: event rings
+    size_t lanes_cap;
 
     // snapshots of the base run
     int snap_stride, snap_count;

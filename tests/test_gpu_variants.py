@@ -145,3 +145,29 @@ def test_host_candidates_are_checked(n):
             assert e.value.code == kv.E_INVAL
         again, ok, _ = h.eval_batch(kv.CAND_START_TIMES, starts, want_feasible=True)
     assert ok.all() and (again == tel).all()
+
+
+@pytest.mark.parametrize("least", [1, 300])
+@pytest.mark.parametrize("omax", [1, 31, 32, 33, 64, 65, 1024, 1025])
+def test_moves_by_lanes(omax, least):
+    """One thread per candidate: every move of 150 requests (33,525) with a budget that lets 1.5 to 3.3 rounds
+    pass per request, event words of both widths, decodes at the edges of its chunks."""
+    rng = np.random.default_rng(omax + least)
+    n = 150
+    s = rng.integers(least, 3000, n).astype(np.int32)
+    o = rng.integers(1, omax + 1, n).astype(np.int32)
+    o[::20] = omax
+    s[0], o[0] = least, 1
+    volume = int((s.astype(np.int64) * o + o.astype(np.int64) ** 2 // 2).sum())
+    for rounds in (1.5, 3.3):
+        M = max(int((s + o).max()), int(volume / (rounds * n)) + n)
+        base = rng.permutation(n).astype(np.int32)
+        codes = np.arange(3 * n * (n - 1) // 2, dtype=np.int64)
+        with kv.Scheduler(s, o, M) as h:
+            h.set_base_order(base)
+            tel, _, _ = h.eval_batch(kv.CAND_MOVE, codes)
+        assert (tel[::11] == oracle_moves(s, o, M, base, codes[::11])).all()
+        with kv.Scheduler(s, o, M) as h:                     # the same in calls that take a warp per candidate
+            h.set_base_order(base)
+            parts = [h.eval_batch(kv.CAND_MOVE, c)[0] for c in np.array_split(codes, 3)]
+        assert (tel == np.concatenate(parts)).all()
