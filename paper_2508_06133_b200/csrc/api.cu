@@ -491,26 +491,34 @@ int order_candidates(sched_ctx* h, const MoveSource& src, i64 count) {
 
 // One thread per candidate instead of one warp (k3_lanes.cuh)?  Its work goes with the rounds that pass, the
 // other kernel's with the admissions: rounds per request is the backlog's volume (sum of s o + o^2 / 2) over
-// n M, within a few per cent of the base run's.  Measured on 64,000 moves, a warp against a thread per
-// candidate: 1.9 rounds per request 9.2 / 5.4 ms, 2.9 rounds 33.0 / 23.6, 5.1 rounds 11.0 / 11.0, 7.6 rounds
-// 40.6 / 51.3, 12.9 rounds 14.7 / 25.7; from 32,000 moves on (1,000 warps) it is ahead at 2.9 rounds too
-// (16.6 / 13.5), with fewer the device is not full.  Decodes longer than its ring of events, and backlogs
-// whose candidate could pass 32 bits of waiting time in one partial sum, keep the warp.
-constexpr double LANE_ROUNDS = 3.5;
-constexpr i64 LANE_MIN = 32000;
-constexpr int LANE_CTAS = 5;               // resident per SM: the kernel's launch bound
+// n M, within a few per cent of the base run's.  Up to 94,720 candidates (56,832 for decodes beyond 1,025) run
+// side by side, so its time hardly moves below that and the other's is proportional to the count.  Measured,
+// warp against thread, ms:
+//   rounds per request  2.9 (n = 10,000)   7.6 (10,000)   12.4 (1,000)   18.9 (4,000)   24.8 (1,000)
+//   16,000 moves          8.4 /  8.9       10.4 / 15.8     1.2 / 1.9      6.1 / 12.4     1.7 / 3.2
+//   32,000               16.6 / 10.2       20.5 / 17.9     2.4 / 2.2     12.0 / 14.2     3.4 / 3.7
+//   48,000                                                 3.6 / 2.6     17.8 / 16.7     5.1 / 4.4
+//   96,000                                                 7.1 / 3.9     35.4 / 24.1    10.1 / 6.3
+//   decodes to 2,048    4.5 (n = 2,000)   10.8 (2,000)    14.8 (2,000)
+//   32,000                4.6 /  3.8        6.1 / 7.5      7.0 /  9.5
+//   48,000                6.9 /  4.3        9.1 / 8.5     10.5 / 10.9
+//   96,000               13.7 /  6.6       18.0 / 13.8    20.9 / 18.3
+// Longer decodes than its ring of events, schedules with more rounds per request than were measured, and
+// backlogs whose candidate could pass 32 bits of waiting time in its sum of starts keep the warp.
+constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.4;
 
 bool lanes_fit(const sched_ctx* h, i64 count, bool want_starts) {
-    return !want_starts && h->nm == 1 && count >= LANE_MIN && count > ordered_from(h) &&
-           h->volume <= LANE_ROUNDS * (double)h->M * h->n &&
-           (i64)h->n * (h->omax + LaneSim<unsigned>::CH) <= INT32_MAX;
+    if (want_starts || (h->nm != 1 && h->nm != 2) || count <= ordered_from(h)) return false;
+    const double rounds = h->volume / ((double)h->n * (double)h->M);
+    return rounds <= LANE_ROUNDS && (double)count >= (h->nm == 1 ? 1.0 : LANE_LONG) * (LANE_MIN + LANE_MIN_PER_ROUND * rounds) &&
+           (i64)h->n * (h->omax + 64) <= INT32_MAX;
 }
 
 // SCHED_OK with *done = false: no memory for the rings of events, nothing was launched.
-template <typename WORD>
+template <int CH, typename WORD>
 int run_lanes(sched_ctx* h, LaneParams& q, bool* done) {
-    typedef LaneSim<WORD> S;
-    const i64 need = ((i64)q.groups + S::kWarps - 1) / S::kWarps, most = (i64)LANE_CTAS * h->sm_count;
+    typedef LaneSim<CH, WORD> S;
+    const i64 need = ((i64)q.groups + S::kWarps - 1) / S::kWarps, most = (i64)S::kCtas * h->sm_count;
     const int grid = (int)(need < most ? need : most);
     const size_t bytes = (size_t)grid * S::kWarps * S::kRingWords * sizeof(WORD);
     *done = false;
@@ -522,8 +530,8 @@ int run_lanes(sched_ctx* h, LaneParams& q, bool* done) {
     q.rings = h->d_lanes;
     q.counter = h->d_counter + 1;
     KV_CUDA(cudaMemsetAsync(q.counter, 0, sizeof(unsigned), h->stream));
-    KV_CUDA(cudaFuncSetAttribute(k3_lane_moves<WORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem));
-    k3_lane_moves<WORD><<<grid, 32 * S::kWarps, S::kSmem, h->stream>>>(q);
+    KV_CUDA(cudaFuncSetAttribute(k3_lane_moves<CH, WORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem));
+    k3_lane_moves<CH, WORD><<<grid, 32 * S::kWarps, S::kSmem, h->stream>>>(q);
     *done = true;
     return SCHED_OK;
 }
@@ -535,9 +543,10 @@ int launch_lanes(sched_ctx* h, const MoveEvalParams& p, bool* done) {
     q.groups = (int)((p.count + 31) / 32);
     // the requests that end in one round hold M tokens at most: sum of (s+o - least) and number in 32 bits?
     q.shift = bits_of((u64)(h->M - h->least));
-    if (q.shift + bits_of((u64)(h->M / h->least)) <= 32) return run_lanes<unsigned>(h, q, done);
-    q.shift = 32;
-    return run_lanes<u64>(h, q, done);
+    const bool narrow = q.shift + bits_of((u64)(h->M / h->least)) <= 32;
+    if (!narrow) q.shift = 32;
+    if (h->nm == 1) return narrow ? run_lanes<32, unsigned>(h, q, done) : run_lanes<32, u64>(h, q, done);
+    return narrow ? run_lanes<64, unsigned>(h, q, done) : run_lanes<64, u64>(h, q, done);
 }
 
 // by_slot: TELs are left in launch-slot order (h->d_k4's launch_order maps a slot to its candidate

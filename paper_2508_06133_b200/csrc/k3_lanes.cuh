@@ -12,10 +12,10 @@
 //       (shared memory, a column per thread).  Admissions since then add d_A + d_C x to a whole chunk;
 //       a window that ends inside one of the two takes its share back from the cells behind its end.
 //   events    for the chunks behind these: per round x, the requests whose last round is x, their sum of
-//       s+o and their number in one word (global memory, a ring of NCH chunks; a lane's chunk is one
-//       line of 128 or 256 bytes), and the running totals A = sum of (s+1-p), C = how many over the requests
-//       that run into them.  An admission is two additions and at most one word, whatever its window; a
-//       chunk's words are read once, when its cells are put together from the totals.
+//       s+o and their number in one word (global memory, a ring of NCH chunks), and the running totals
+//       A = sum of (s+1-p), C = how many over the requests that run into them.  An admission is two
+//       additions and at most one word, whatever its window; a chunk's words are read once, when its
+//       cells are put together from the totals.
 //   bounds    W0, W1 of V over the two chunks, U[c] over the NF behind them (registers), Uall their
 //       maximum: each raised by a ramp's value in the chunk's last round.  All below the limit: it fits.
 // Where W0 says "perhaps", one walk back over the chunk's cells gives the first round from which the
@@ -23,11 +23,14 @@
 // so a turn nearly always ends with an admission in every lane (1.25 turns per admission).  W1 is
 // answered from the next chunk's cells, U (2 of 1,000 turns) from the events.
 //
-// What bounds it: integer issue, as in the kernel with a warp per candidate, but by the work of a chunk (two
-// builds of 32 cells, 34 event words) and not by that of an admission: it pays when few rounds pass per
-// admission.  Measured, kernel against k3_eval_moves: 10,000 requests, budget 262,144 (2.9 rounds per
-// request), 64,000 moves 33.0 -> 23.6 ms; 3,000 requests, budget 400,000 (1.9), 256,000 moves 36.6 -> 18.9 ms.
-// lanes_fit (api.cu) has the rule and the other side.
+// What bounds it: latency.  20 warps per SM (the cells of two chunks fill shared memory) execute about 500
+// instructions per turn of 32 candidates where the kernel with a warp per candidate executes 32 x 77, but the
+// event rings of all resident candidates are 412 MB and do not stay in L2 (126 MB).  So a chunk's words are
+// read with eight 16-byte loads in flight, laid out so that a warp's load is 512 contiguous bytes, called to L2 one
+// chunk ahead, and cleared only where they are not zero; the request behind the next is on its way a turn early.
+// 65,536 moves of 10,000 requests, budget 262,144, other seeds: 33.8 ms with a warp per candidate; 20.5 with one load of a
+// lane's own line at a time, 16.0 with four coalesced loads, 14.9 with eight.  256,000 moves of 1,000
+// requests, budget 65,536: 18.9 -> 8.8 ms.  lanes_fit (api.cu) has the rule and the other side.
 #pragma once
 
 #include "common.cuh"
@@ -35,7 +38,7 @@
 
 struct LaneParams {
     MoveEvalParams m;
-    int omax;                // largest decode length, <= CH * NCH - CH + 1
+    int omax;                // largest decode length, at most CH * NF + 1
     int shift;               // events: sum of (s+o - least) in the low `shift` bits, number above them
     int least;               // smallest s+o
     void* rings;             // per resident warp: NCH * 32 * CH words
@@ -43,38 +46,41 @@ struct LaneParams {
     int groups;
 };
 
-template <typename WORD_>
+template <int CH_, typename WORD_>
 struct LaneSim {
     typedef WORD_ WORD;
-    static constexpr int CH = 32, NF = 32, NCH = NF + 2;
-    static constexpr int kWarps = 4;
+    static constexpr int CH = CH_, NF = 32, NCH = NF + 2;
+    static constexpr int kWarps = 4, kCtas = CH == 32 ? 5 : 3;            // CTAs per SM: shared memory
     static constexpr size_t kRingWords = (size_t)NCH * 32 * CH;            // per warp
     static constexpr size_t kSmem = (size_t)2 * CH * 32 * kWarps * sizeof(int);
 };
 
-template <typename WORD>
-__global__ void __launch_bounds__(128, 5)
+template <int CH, typename WORD>
+__global__ void __launch_bounds__(128, LaneSim<CH, WORD>::kCtas)
 k3_lane_moves(const LaneParams P) {
-    typedef LaneSim<WORD> S;
-    constexpr int CH = S::CH, NF = S::NF, NCH = S::NCH, VS = 32 * S::kWarps;           // cell x of a chunk: [x * VS]
+    typedef LaneSim<CH, WORD> S;
+    constexpr int NF = S::NF, NCH = S::NCH, VS = 4 * 32 * S::kWarps;
+    constexpr int GROUP = 8;                                               // 16-byte loads of events in flight
     constexpr int PER = 16 / (int)sizeof(WORD);                            // words per 16-byte load
     extern __shared__ __align__(16) int lane_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int* b0 = lane_smem + threadIdx.x;
-    int* b1 = b0 + CH * VS;
-    WORD* const ring = (WORD*)P.rings + ((size_t)blockIdx.x * S::kWarps + warp) * S::kRingWords + (size_t)lane * CH;
+    int* b0 = lane_smem + 4 * threadIdx.x;                                 // cells in fours: at(x)
+    int* b1 = b0 + CH / 4 * VS;
+    auto at = [](int x) -> int { return (x >> 2) * VS + (x & 3); };
+    WORD* const ring = (WORD*)P.rings + ((size_t)blockIdx.x * S::kWarps + warp) * S::kRingWords + lane * PER;
     const int n = P.m.n, M = P.m.M, least = P.least, shift = P.shift;
     const WORD vmask = ((WORD)1 << shift) - 1, one = (WORD)1 << shift;
     auto unpack = [](const uint4& v, WORD* ev) {                           // the words of 16 bytes
         if (sizeof(WORD) == 4) { ev[0] = (WORD)v.x; ev[1] = (WORD)v.y; ev[2] = (WORD)v.z; ev[3] = (WORD)v.w; }
         else { ev[0] = (WORD)((u64)v.x | ((u64)v.y << 32)); ev[1] = (WORD)((u64)v.z | ((u64)v.w << 32)); }
     };
-    auto line_of = [&](int k) -> WORD* {                                   // this lane's words of slot k (k < 2 NCH)
+    // words of slot k (k < 2 NCH): 16 bytes of each lane side by side, then the next 16 bytes
+    auto line_of = [&](int k) -> WORD* {
         if (k >= NCH) k -= NCH;
         return ring + (size_t)KV_IDX(k, NCH, 421) * (32 * CH);
     };
     // the word of the x-th round behind the beginning of slot `slot`
-    auto word_of = [&](int slot, int x) -> WORD* { return line_of(slot + x / CH) + (x & (CH - 1)); };
+    auto word_of = [&](int slot, int x) -> WORD* { return line_of(slot + x / CH) + (x & (CH - 1)) / PER * (32 * PER) + (x & (PER - 1)); };
     for (;;) {
         unsigned group = 0;
         if (lane == 0) group = atomicAdd(P.counter, 1u);
@@ -98,7 +104,7 @@ k3_lane_moves(const LaneParams P) {
         // ---- the base run's state in front of q: events, totals and bounds of the requests that still run
         for (int c = 0; c < NCH; ++c) {
             uint4* z = reinterpret_cast<uint4*>(line_of(c));
-            for (int k = 0; k < CH / PER; ++k) __stcg(z + k, make_uint4(0, 0, 0, 0));
+            for (int k = 0; k < CH / PER; ++k) __stcg(z + 32 * k, make_uint4(0, 0, 0, 0));
         }
         int A = 0, C = 0;                                                  // from the beginning of the chunk built next
         int U[NF];                                                         // U[c]: chunk c + 2
@@ -107,14 +113,17 @@ k3_lane_moves(const LaneParams P) {
         {
             int lo = 0, hi = q;                                            // first position that can still run at t
             while (lo < hi) { const int mid = (lo + hi) >> 1; if (P.m.base_starts_pos[mid] + P.omax > hdr.t) hi = mid; else lo = mid + 1; }
+            int2 so1 = P.m.tbl_base[lo < n ? lo : 0];
+            int p1 = P.m.base_starts_pos[lo < n ? lo : 0];
             for (int k = lo; k < q; ++k) {
-                const int2 so = P.m.tbl_base[k];
-                const int p = P.m.base_starts_pos[k] - T0, last = p + so.y - 1;
+                const int2 so = so1;
+                const int p = p1 - T0, last = p + so.y - 1;
+                so1 = P.m.tbl_base[k + 1 < n ? k + 1 : 0];
+                p1 = P.m.base_starts_pos[k + 1 < n ? k + 1 : 0];
                 if (last < hdr.t - T0) continue;
                 const int a = so.x + 1 - p;
                 A += a; ++C;
-                WORD* w = word_of(0, last);
-                __stcg(w, __ldcg(w) + (WORD)(so.x + so.y - least) + one);
+                atomicAdd(word_of(0, last), (WORD)(so.x + so.y - least) + one);
 #pragma unroll
                 for (int c = 0; c < NF; ++c) if (last >= CH * (c + 2)) U[c] += a + CH * (c + 3) - 1;
             }
@@ -124,22 +133,34 @@ k3_lane_moves(const LaneParams P) {
         auto build = [&](int* cells, int slot) -> int {
             WORD* line = line_of(slot);
             int w = INT_MIN;
-#pragma unroll 4
-            for (int x0 = 0; x0 < CH; x0 += PER) {
-                const uint4 v = __ldcg(reinterpret_cast<const uint4*>(line + x0));
-                __stcg(reinterpret_cast<uint4*>(line + x0), make_uint4(0, 0, 0, 0));
-                WORD ev[4];
-                unpack(v, ev);
+            for (int x0 = 0; x0 < CH; x0 += GROUP * PER) {
+                uint4 v[GROUP];
 #pragma unroll
-                for (int k = 0; k < PER; ++k) {
-                    const int x = x0 + k, cell = A + C * x;
-                    cells[x * VS] = cell;
-                    w = max(w, cell + x);
-                    const int num = (int)(ev[k] >> shift);
-                    A -= (int)(ev[k] & vmask) + num * (least - x);
-                    C -= num;
+                for (int g = 0; g < GROUP; ++g) v[g] = __ldcg(reinterpret_cast<const uint4*>(line + 32 * x0) + 32 * g);
+#pragma unroll
+                for (int g = 0; g < GROUP; ++g) if (v[g].x | v[g].y | v[g].z | v[g].w) __stcg(reinterpret_cast<uint4*>(line + 32 * x0) + 32 * g, make_uint4(0, 0, 0, 0));
+                WORD ev[GROUP * PER];
+#pragma unroll
+                for (int g = 0; g < GROUP; ++g) unpack(v[g], ev + g * PER);
+#pragma unroll
+                for (int x4 = 0; x4 < GROUP * PER; x4 += 4) {
+                    int cell[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int x = x0 + x4 + k;
+                        cell[k] = A + C * x;
+                        w = max(w, cell[k] + x);
+                        const int num = (int)(ev[x4 + k] >> shift);
+                        A -= (int)(ev[x4 + k] & vmask) + num * (least - x);
+                        C -= num;
+                    }
+                    *reinterpret_cast<int4*>(cells + at(x0 + x4)) = make_int4(cell[0], cell[1], cell[2], cell[3]);
                 }
             }
+            // the words that are read next: the admissions of a chunk are time enough to have them in L2
+#pragma unroll
+            for (int x = 0; x < CH; x += 128 / (int)sizeof(WORD))
+                asm volatile("prefetch.global.L2 [%0];" :: "l"(line_of(slot + 1) + lane * (CH - PER) + x));
             A += CH * C;
             return w;
         };
@@ -153,16 +174,16 @@ k3_lane_moves(const LaneParams P) {
         const int d_in = mv.type == 1 ? (mv.i < mv.j ? 1 : -1) : 0;
         const int x1 = mv.j, y1 = mv.i, x2 = mv.type == 0 ? mv.i : n, y2 = mv.j;
         const int in_lo = min(mv.i, mv.j), in_len = max(mv.i, mv.j) - in_lo;
-        auto fetch = [&](int at, int& sp_, int& om_) {
-            int q = (unsigned)(at - in_lo) <= (unsigned)in_len ? at + d_in : at;
-            q = at == x1 ? y1 : at == x2 ? y2 : q;
-            const int2 so = P.m.tbl_base[KV_IDX(at < n ? q : 0, n, 424)];
-            sp_ = so.x + 1; om_ = so.y - 1;
+        auto fetch = [&](int pos) -> int2 {
+            int from = (unsigned)(pos - in_lo) <= (unsigned)in_len ? pos + d_in : pos;
+            from = pos == x1 ? y1 : pos == x2 ? y2 : from;
+            return P.m.tbl_base[KV_IDX(pos < n ? from : 0, n, 424)];
         };
         if (!valid) q = n;
-        int sp = 2, om = 0, sp1 = 2, om1 = 0;                              // the request at q and the one behind it
-        fetch(q, sp, om);
-        fetch(q + 1, sp1, om1);
+        // the request at q, and the one behind it as it was read: nothing waits for it before it is needed
+        const int2 so0 = fetch(q);
+        int sp = so0.x + 1, om = so0.y - 1;
+        int2 next = fetch(q + 1);
 
         for (i64 chunk = 0;; ++chunk) {
             int Uall = INT_MIN;
@@ -177,15 +198,31 @@ k3_lane_moves(const LaneParams P) {
                 const bool ask0 = act && W0 > lim + tau;
                 if (__any_sync(KV_FULL, ask0)) {
                     const int x_lo = kv_warp_min(ask0 ? tau : CH - 1) & ~3;
-                    const int lim0 = lim - dA0, slope = dC0 + 1;
-                    int mx = INT_MIN, best = CH, best_w = 0;
+                    const int lim0 = lim - dA0;
+                    // y: maximum of V behind a round, less the round; grows strictly towards the front.  First the
+                    // four cells in which it passes the limit, then the cell.
+                    const int rise = dC0;
+                    int y = INT_MIN / 2, y_in = y, x_in = CH - 4;
+#pragma unroll 2
                     for (int x4 = CH - 4; x4 >= x_lo; x4 -= 4) {
+                        const int4 four = *reinterpret_cast<const int4*>(b0 + at(x4));
+                        if (y <= lim0) { y_in = y; x_in = x4; }
+                        y = __viaddmax_s32(y, 1, four.w + rise * (x4 + 3));
+                        y = __viaddmax_s32(y, 1, four.z + rise * (x4 + 2));
+                        y = __viaddmax_s32(y, 1, four.y + rise * (x4 + 1));
+                        y = __viaddmax_s32(y, 1, four.x + rise * x4);
+                    }
+                    int best = x_in + 4, best_w;
+                    {
+                        const int4 four = *reinterpret_cast<const int4*>(b0 + at(x_in));
+                        const int cell[4] = {four.x, four.y, four.z, four.w};
+                        y = y_in;
 #pragma unroll
                         for (int k = 3; k >= 0; --k) {
-                            const int x = x4 + k;
-                            mx = max(mx, b0[x * VS] + slope * x);
-                            if (mx <= lim0 + x) { best = x; best_w = mx; }
+                            y = __viaddmax_s32(y, 1, cell[k] + rise * (x_in + k));
+                            if (y <= lim0) { y_in = y; best = x_in + k; }
                         }
+                        best_w = y_in + best;
                     }
                     const bool cut = ask0 && tau + om < CH - 1;            // the window ends inside the chunk
                     if (ask0 && !cut) {
@@ -194,9 +231,17 @@ k3_lane_moves(const LaneParams P) {
                     }
                     if (__any_sync(KV_FULL, cut)) {
                         int d = 0;
-                        if (cut)
-                            for (int x = tau; x <= tau + om; ++x)
-                                d = max(d, __viaddmin_s32(b0[x * VS] + slope * x, -(lim0 + tau), x - tau + 1));
+#pragma unroll 2
+                        for (int x4 = x_lo; x4 < CH; x4 += 4) {
+                            const int4 four = *reinterpret_cast<const int4*>(b0 + at(x4));
+                            const int cell[4] = {four.x, four.y, four.z, four.w};
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const int x = x4 + k - tau;
+                                if (cut && (unsigned)x <= (unsigned)om)
+                                    d = max(d, __viaddmin_s32(cell[k] + (dC0 + 1) * (x4 + k), -(lim0 + tau), x + 1));
+                            }
+                        }
                         if (d > 0) { tau += d; fits = false; }
                     }
                 }
@@ -205,11 +250,16 @@ k3_lane_moves(const LaneParams P) {
                 if (__any_sync(KV_FULL, ask1)) {
                     const int lim1 = lim + tau - dA1 - CH, slope = dC1 + 1, end = tau + om - CH;
                     int w = INT_MIN, d = 0;
-#pragma unroll 4
-                    for (int x = 0; x < CH; ++x) {
-                        const int v = b1[x * VS] + slope * x;
-                        w = max(w, v);
-                        if (x <= end) d = max(d, __viaddmin_s32(v, -lim1, x + CH + 1 - tau));
+#pragma unroll 2
+                    for (int x4 = 0; x4 < CH; x4 += 4) {
+                        const int4 four = *reinterpret_cast<const int4*>(b1 + at(x4));
+                        const int cell[4] = {four.x, four.y, four.z, four.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int x = x4 + k, v = cell[k] + slope * x;
+                            w = max(w, v);
+                            if (x <= end) d = max(d, __viaddmin_s32(v, -lim1, x + CH + 1 - tau));
+                        }
                     }
                     if (ask1) {
                         W1 = w + dA1 + CH;
@@ -235,7 +285,7 @@ k3_lane_moves(const LaneParams P) {
                         int w = INT_MIN;
 #pragma unroll 4
                         for (int x0 = 0; x0 < CH; x0 += PER) {
-                            const uint4 l = __ldcg(reinterpret_cast<const uint4*>(line + x0));
+                            const uint4 l = __ldcg(reinterpret_cast<const uint4*>(line + 32 * x0));
                             WORD ev[4];
                             unpack(l, ev);
 #pragma unroll
@@ -267,15 +317,15 @@ k3_lane_moves(const LaneParams P) {
                     atomicAdd(word_of(slot, last - 2 * CH), (WORD)(sp + om - least) + one);
                 }
                 if (__any_sync(KV_FULL, fits && !far2)) {                  // a window that ends in one of the two chunks
-                    if (far1 && !far2) { for (int x = last + 1 - CH; x < CH; ++x) b1[x * VS] -= a + CH + x; }
-                    if (fits && !far1) { for (int x = last + 1; x < CH; ++x) b0[x * VS] -= a + x; }
+                    if (far1 && !far2) { for (int x = last + 1 - CH; x < CH; ++x) b1[at(x)] -= a + CH + x; }
+                    if (fits && !far1) { for (int x = last + 1; x < CH; ++x) b0[at(x)] -= a + x; }
                 }
                 const int reach = fits ? last : 0;
                 if (fits) {
-                    sp = sp1; om = om1;
+                    sp = next.x + 1; om = next.y - 1;
                     ++q;
                 }
-                fetch(q + 1, sp1, om1);
+                next = fetch(q + 1);
                 // bounds of the far chunks the new windows reach
 #pragma unroll
                 for (int c0 = 0; c0 < NF; c0 += 8) {

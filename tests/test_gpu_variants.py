@@ -148,7 +148,7 @@ def test_host_candidates_are_checked(n):
 
 
 @pytest.mark.parametrize("least", [1, 300])
-@pytest.mark.parametrize("omax", [1, 31, 32, 33, 64, 65, 1024, 1025])
+@pytest.mark.parametrize("omax", [1, 31, 32, 33, 64, 65, 1024, 1025, 1026, 2049])
 def test_moves_by_lanes(omax, least):
     """One thread per candidate: every move of 150 requests (33,525) with a budget that lets 1.5 to 3.3 rounds
     pass per request, event words of both widths, decodes at the edges of its chunks."""
