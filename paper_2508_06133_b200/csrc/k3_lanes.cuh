@@ -28,9 +28,10 @@
 // event rings of all resident candidates are 412 MB and do not stay in L2 (126 MB).  So a chunk's words are
 // read with eight 16-byte loads in flight, laid out so that a warp's load is 512 contiguous bytes, called to L2 one
 // chunk ahead, and cleared only where they are not zero; the request behind the next is on its way a turn early.
-// 65,536 moves of 10,000 requests, budget 262,144, other seeds: 33.8 ms with a warp per candidate; 20.5 with one load of a
-// lane's own line at a time, 16.0 with four coalesced loads, 14.9 with eight.  256,000 moves of 1,000
-// requests, budget 65,536: 18.9 -> 8.8 ms.  lanes_fit (api.cu) has the rule and the other side.
+// 64,000 moves of 10,000 requests, budget 262,144: 33.0 ms with a warp per candidate; 23.6 with one load of a
+// lane's own line at a time, 18.6 with four of them, 16.0 with these side by side and the walk in two levels, 14.7 with
+// eight.  256,000 moves of 1,000 requests, budget 65,536: 18.9 -> 8.8 ms.  4,194,304 moves of the 10,000: 2,741 ->
+// 569 ms.  lanes_fit (api.cu) has the rule and the other side.
 #pragma once
 
 #include "common.cuh"

@@ -24,9 +24,9 @@
 //       0.01 to 0.1 chunks per admission on the synthetic backlogs (and 0.3 to 1.1 waits).
 // Measured against a register-resident timeline that tested and filled every cell of the window (one and
 // a half instructions per 32 cells and admission), k3_eval_moves: 10,000 requests (decodes to 1,024),
-// 65,536 moves 43.3 -> 35.1 ms; 100,000 requests (decodes to 4,096), 7,000 moves 108.8 -> 64.8 ms, where
+// 65,536 moves 43.3 -> 33.0 ms; 100,000 requests (decodes to 4,096), 7,000 moves 108.8 -> 50.7 ms, where
 // the far part of the timeline was read and written in shared memory; one run of the 100,000 from the
-// empty state (sorted_f) 71.6 -> 24.4 ms.  Bound by the issue rate: 85 instructions per admission.
+// empty state (sorted_f) 71.6 -> 15.6 ms.  Bound by the issue rate: 77 instructions per admission.
 // When t enters the next chunk its cells are put together from own, A and C, and the lanes' far
 // values move down by one.
 //
