@@ -236,7 +236,7 @@ int validate_instance(i64 total, const int32_t* s, const int32_t* o, i64 M) {
 
 void free_ctx(sched_ctx* h) {
     if (!h) return;
-    void* ptrs[] = {h->d_arena, h->d_lanes, h->d_tel, h->d_stage, h->d_sort, h->d_k4, h->d_ls};
+    void* ptrs[] = {h->d_arena, h->d_rings, h->d_tel, h->d_stage, h->d_sort, h->d_k4, h->d_ls};
     for (void* p : ptrs) if (p) kv_free(p);
     kv_host_free(h->h_pinned, h->pinned_bytes);
     if (h->ev_k3_begin) cudaEventDestroy(h->ev_k3_begin);
@@ -514,6 +514,15 @@ bool lanes_fit(const sched_ctx* h, i64 count, bool want_starts) {
            (i64)h->n * (h->omax + 64) <= INT32_MAX;
 }
 
+// The handle's block of rings in device memory, of at least `bytes`; false if there is no memory for it.
+bool grow_rings(sched_ctx* h, size_t bytes) {
+    if (h->rings_cap >= bytes) return true;
+    if (h->d_rings) { kv_free(h->d_rings); h->d_rings = nullptr; h->rings_cap = 0; }
+    if (kv_malloc(&h->d_rings, bytes) != cudaSuccess) { cudaGetLastError(); h->d_rings = nullptr; return false; }
+    h->rings_cap = bytes;
+    return true;
+}
+
 // SCHED_OK with *done = false: no memory for the rings of events, nothing was launched.
 template <int CH, typename WORD>
 int run_lanes(sched_ctx* h, LaneParams& q, bool* done) {
@@ -522,12 +531,8 @@ int run_lanes(sched_ctx* h, LaneParams& q, bool* done) {
     const int grid = (int)(need < most ? need : most);
     const size_t bytes = (size_t)grid * S::kWarps * S::kRingWords * sizeof(WORD);
     *done = false;
-    if (h->lanes_cap < bytes) {
-        if (h->d_lanes) { kv_free(h->d_lanes); h->d_lanes = nullptr; h->lanes_cap = 0; }
-        if (kv_malloc(&h->d_lanes, bytes) != cudaSuccess) { cudaGetLastError(); h->d_lanes = nullptr; return SCHED_OK; }
-        h->lanes_cap = bytes;
-    }
-    q.rings = h->d_lanes;
+    if (!grow_rings(h, bytes)) return SCHED_OK;
+    q.rings = h->d_rings;
     q.counter = h->d_counter + 1;
     KV_CUDA(cudaMemsetAsync(q.counter, 0, sizeof(unsigned), h->stream));
     KV_CUDA(cudaFuncSetAttribute(k3_lane_moves<CH, WORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem));
@@ -547,6 +552,31 @@ int launch_lanes(sched_ctx* h, const MoveEvalParams& p, bool* done) {
     if (!narrow) q.shift = 32;
     if (h->nm == 1) return narrow ? run_lanes<32, unsigned>(h, q, done) : run_lanes<32, u64>(h, q, done);
     return narrow ? run_lanes<64, unsigned>(h, q, done) : run_lanes<64, u64>(h, q, done);
+}
+
+// Moves with a warp each whose rings are in device memory (sim_chunk.cuh)?  32 instead of 13 warps per SM
+// against a wait for memory per 32 rounds.  Measured, shared against device memory, decodes to 4,096: 100,000
+// requests, 7,000 moves, 1.0 rounds per request 53.4 / 45.0 ms; 20,000 requests, 4.2 rounds: 35,000 moves 59.4 /
+// 61.2, 2,400 moves (16 warps per SM) 5.1 / 6.5; 2,000 requests, 16 rounds, 200,000 moves 50.7 / 89.5.
+bool device_rings_fit(const sched_ctx* h, i64 count, bool want_starts) {
+    return !want_starts && h->nm == 4 && count >= 27ll * h->sm_count && h->volume <= 2.0 * (double)h->n * (double)h->M;
+}
+
+// 512 MB of rings per launch.  false: no memory for them, nothing was launched.
+bool moves_from_device_rings(sched_ctx* h, MoveEvalParams& p) {
+    typedef ChunkSim<4, true> S;
+    const size_t bytes = (size_t)h->ring_cells * sizeof(int);
+    i64 most = (i64)(((size_t)512 << 20) / bytes);
+    if (most > p.count) most = p.count;
+    if (!grow_rings(h, bytes * most)) return false;
+    p.rings = (int*)h->d_rings;
+    for (i64 at = 0; at < p.count; at += most) {
+        p.first_slot = at;
+        p.end_slot = at + most < p.count ? at + most : p.count;
+        const i64 ctas = (p.end_slot - at + S::kWarps - 1) / S::kWarps;
+        k3_eval_moves<S, false><<<(unsigned)ctas, S::kWarps * 32, 0, h->stream>>>(p);
+    }
+    return true;
 }
 
 // by_slot: TELs are left in launch-slot order (h->d_k4's launch_order maps a slot to its candidate
@@ -573,7 +603,10 @@ int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, 
     KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
     bool lanes = lanes_fit(h, count, starts_out != nullptr);
     if (lanes) KV_TRY(launch_lanes(h, p, &lanes));
-    if (!lanes) {
+    bool done = lanes;
+    if (!done && device_rings_fit(h, count, starts_out != nullptr)) done = moves_from_device_rings(h, p);
+    if (!done) {
+        p.first_slot = 0; p.end_slot = count;
 #define RUN(N)                                                                                    \
     if (starts_out) k3_eval_moves<N, true><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p);  \
     else k3_eval_moves<N, false><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p)

@@ -57,8 +57,8 @@ struct sched_ctx {
     int* d_ls;               // scratch of the Local Swap Search kernel: 7 arrays of n ints (lazy)
     void* d_k4;              // grow-only scratch of the launch ordering: bins[n+1], first_pos[count], order[count]
     size_t k4_cap;
-    void* d_lanes;           // grow-only scratch of the one-thread-per-candidate kernel: event rings
-    size_t lanes_cap;
+    void* d_rings;           // grow-only scratch: rings of candidates whose timelines are not in shared memory
+    size_t rings_cap;
 
     // snapshots of the base run
     int snap_stride, snap_count;

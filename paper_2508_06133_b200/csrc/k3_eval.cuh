@@ -184,6 +184,8 @@ struct MoveEvalParams {
     int* starts_out;                   // nullable [count][n], by request id
     const int* base_order;
     const int* base_starts_pos;
+    i64 first_slot, end_slot;          // launch slots of this launch
+    int* rings;                        // simulators with rings in device memory: one per slot of this launch
     int* status;
 };
 
@@ -197,12 +199,12 @@ k3_eval_moves(const MoveEvalParams p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int2* __restrict__ tbl = p.tbl_base;
     const int n = p.n, L = p.L, M = p.M;
-    const i64 slot = (i64)blockIdx.x * (blockDim.x >> 5) + warp;
-    if (slot >= p.count) return;
+    const i64 at = (i64)blockIdx.x * (blockDim.x >> 5) + warp, slot = p.first_slot + at;
+    if (slot >= p.end_slot) return;
     const i64 c = p.launch_order ? KV_IDX(p.launch_order[slot], p.count, 402) : slot;
     i64* tel_dst = p.tel_out + (p.tel_by_slot ? slot : c);
     SIM sim;
-    sim.attach((int*)smem_raw + (size_t)warp * SIM::ring_cells(L), L);
+    sim.attach((SIM::kGlobal ? p.rings + at * SIM::ring_cells(L) : (int*)smem_raw + (size_t)warp * SIM::ring_cells(L)), L);
     const Move mv = k4_move_of(p.src, n, c);
     if ((unsigned)mv.i >= (unsigned)n || (unsigned)mv.j >= (unsigned)n) {      // code outside the neighbourhood
         if (lane == 0) *tel_dst = INT64_MAX;

@@ -24,7 +24,7 @@
 //       0.01 to 0.1 chunks per admission on the synthetic backlogs (and 0.3 to 1.1 waits).
 // Measured against a register-resident timeline that tested and filled every cell of the window (one and
 // a half instructions per 32 cells and admission), k3_eval_moves: 10,000 requests (decodes to 1,024),
-// 65,536 moves 43.3 -> 33.0 ms; 100,000 requests (decodes to 4,096), 7,000 moves 108.8 -> 50.7 ms, where
+// 65,536 moves 43.3 -> 33.0 ms; 100,000 requests (decodes to 4,096), 7,000 moves 108.8 -> 50.7 ms (40.7 with kGlobal), where
 // the far part of the timeline was read and written in shared memory; one run of the 100,000 from the
 // empty state (sorted_f) 71.6 -> 15.6 ms.  Bound by the issue rate: 77 instructions per admission.
 // When t enters the next chunk its cells are put together from own, A and C, and the lanes' far
@@ -46,10 +46,14 @@
 
 #include "common.cuh"
 
-template <int NM>
+// kGlobal: the rings are in device memory.  A simulator for decodes up to 4,097 rounds has 16 KB of ring,
+// so shared memory holds 13 of them per SM and registers 32; the ring is written without waiting and read once per
+// 32 rounds.  100,000 requests, 7,000 moves, 1.0 rounds per request: 50.7 -> 40.7 ms; device_rings_fit has the rule.
+template <int NM, bool kGlobal_ = false>
 struct ChunkSim {
-    static constexpr int kWarps = NM == 1 ? 4 : NM == 2 ? 2 : 1;    // warps per CTA: 16 KB of rings
-    static constexpr int kMinCtas = 10;                             // CTAs per SM the registers have to allow
+    static constexpr bool kGlobal = kGlobal_;
+    static constexpr int kWarps = NM == 1 || kGlobal ? 4 : NM == 2 ? 2 : 1;    // per CTA: 16 KB of shared rings
+    static constexpr int kMinCtas = kGlobal ? 8 : 10;            // CTAs per SM the registers have to allow
     static constexpr bool kGroups = true;                           // has surely()
     static constexpr int kMeta = 32 + 96 * NM;                      // state ints besides the ring
     __host__ __device__ static constexpr int ring_cells(int L) { return L - kMeta; }   // shared-memory ints per warp
@@ -72,6 +76,7 @@ struct ChunkSim {
         mask = (ring_cells(L) - 1) & ~31;
     }
     __device__ __forceinline__ int* cells_of(int x) const { return ring + KV_IDX(x & mask, mask + 32, 151); }
+    __device__ __forceinline__ static int cell(const int* p) { return kGlobal ? __ldcg(p) : *p; }
     __device__ __forceinline__ void set_time(int t, int M) {
         T0 = t & ~31; tau = t & 31;
         rl = lane - tau; xr = 32 * (lane + 1) - tau; x31 = xr + 31; nkt = M + tau;
@@ -141,7 +146,7 @@ struct ChunkSim {
         }
         // lane 31 has just received the values of the chunk that becomes chunk 0
         const int a = __shfl_sync(KV_FULL, ra[0], 31), c = __shfl_sync(KV_FULL, rc[0], 31) + 1;
-        cur = *p + a + c * lane;
+        cur = cell(p) + a + c * lane;
         *p = 0;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
@@ -164,7 +169,7 @@ struct ChunkSim {
                 todo &= todo - 1;
                 const int x0 = 32 * (j + 1) + 1024 * m;              // counted from T0
                 const int a = __shfl_sync(KV_FULL, A[m], j), c = __shfl_sync(KV_FULL, C[m], j) + 1;
-                const int v = *cells_of(T0 + x0) + a + c * (x0 + lane);
+                const int v = cell(cells_of(T0 + x0)) + a + c * (x0 + lane);
                 const int vmax = kv_warp_max(v);
                 if (lane == j) U[m] = vmax;
                 if (x0 + rl <= om) d = max(d, __viaddmin_s32(v, -nk, x0 + rl + 1));

@@ -130,6 +130,7 @@ struct HybSim {
     static constexpr int NREG = 33;
     static constexpr int kWarps = 24;                 // 33 timeline registers + the ring bookkeeping need more than 64 registers
     static constexpr int kMinCtas = 1;
+    static constexpr bool kGlobal = false;
     static constexpr bool kGroups = false;
     __host__ __device__ static constexpr int ring_cells(int L) { return L - 32 * NREG; }
 

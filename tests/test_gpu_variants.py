@@ -171,3 +171,25 @@ def test_moves_by_lanes(omax, least):
             h.set_base_order(base)
             parts = [h.eval_batch(kv.CAND_MOVE, c)[0] for c in np.array_split(codes, 3)]
         assert (tel == np.concatenate(parts)).all()
+
+
+@pytest.mark.parametrize("omax", [2050, 4097])
+def test_moves_from_device_rings(omax):
+    """A warp per candidate with its ring in device memory: every move of 80 requests (9,480), budgets that let 1
+    and 1.8 rounds pass per request."""
+    rng = np.random.default_rng(omax)
+    n = 80
+    s = rng.integers(1, 3000, n).astype(np.int32)
+    o = rng.integers(1, omax + 1, n).astype(np.int32)
+    o[::20] = omax
+    volume = int((s.astype(np.int64) * o + o.astype(np.int64) ** 2 // 2).sum())
+    for rounds in (1.0, 1.8):
+        M = max(int((s + o).max()), int(volume / (rounds * n)) + n)
+        base = rng.permutation(n).astype(np.int32)
+        codes = np.arange(3 * n * (n - 1) // 2, dtype=np.int64)
+        with kv.Scheduler(s, o, M) as h:
+            h.set_base_order(base)
+            tel, _, _ = h.eval_batch(kv.CAND_MOVE, codes)
+            parts = [h.eval_batch(kv.CAND_MOVE, c)[0] for c in np.array_split(codes, 4)]
+        assert (tel[::7] == oracle_moves(s, o, M, base, codes[::7])).all()
+        assert (tel == np.concatenate(parts)).all()
