@@ -122,7 +122,8 @@ int sched_get_base_order(sched_handle h, int32_t* order_out);
  * ids (SCHED_E_INVAL) and negative start times (SCHED_E_INVAL) before any launch.
  * POLICY builds every order inside the kernel (one warp per instance-policy pair, all of an
  * instance's arrays in shared memory): SCHED_E_UNSUPPORTED when the instance does not fit there
- * (about n > 8,000 requests on a single-instance handle; batch handles are limited to 1,024). */
+ * (n > 8,118 requests on a single-instance handle, n > 6,313 where n * M >= 2^31; batch handles are
+ * limited to 1,024). */
 int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candidates,
                      int64_t* tel_out, uint8_t* feasible_out, int32_t* starts_out);
 

@@ -10,10 +10,12 @@
 
 // ------------------------------------------------------------------------------------------------
 // Policy sweep: one warp per (instance, policy) pair, up to K3P_MAX_WARPS pairs of one instance per
-// CTA.  Dynamic shared memory: int s[n], o[n] once per CTA; per warp the finished order (16-bit ids)
-// and one area that first holds what the order is built with -- PT P[n+2], O[n+2] (PT = int32 when
-// n * M < 2^31, else int64), int boff[n+2], a 256-bin histogram, and 16-bit: three id buffers [n] and
-// batch numbers [n] -- and then the simulator's ring (SIM::ring_cells(L) ints).  Orders are built by a
+// CTA.  Dynamic shared memory: int s[n], o[n] once per CTA; per warp one area that first holds what the
+// order is built with -- PT P[n+2], O[n+2] (PT = int32 when n * M < 2^31, else int64), int boff[n+2], a
+// 256-bin histogram, and 16-bit: three id buffers [n] and batch numbers [n] -- and then the simulator's
+// ring (SIM::ring_cells(L) ints) in front and the finished order (16-bit ids) behind it, at the earliest
+// where the batch numbers were: an array of its own would cost 2 of 28 bytes per request, and with them
+// the longest lists (8,118 requests with 32-bit sums, 6,313 with 64-bit ones).  Orders are built by a
 // single-warp radix sort (k3_warp_radix_sort) on the fields of the policy's key.
 // ------------------------------------------------------------------------------------------------
 // One pass of a stable least-significant-digit radix sort run by a single warp on shared memory:
@@ -128,14 +130,16 @@ __device__ __forceinline__ int k3_warp_select_batches(const PT* P, const PT* O, 
     return nb;
 }
 
-// Bytes of shared memory one warp of the policy kernel needs besides the instance's (s, o): the order,
-// and the larger of the simulator's ring and the order's scratch (P and O, the batch offsets, the
-// radix histogram, four 16-bit id arrays).
-__host__ __device__ inline size_t k3_policy_order_bytes(int n) { return ((size_t)n * 2 + 15) & ~(size_t)15; }
-__host__ __device__ inline size_t k3_policy_warp_bytes(int n, int ring_cells, int pt_bytes) {
+// Bytes of shared memory one warp of the policy kernel needs besides the instance's (s, o): the order's
+// scratch (P and O, the batch offsets, the radix histogram, four 16-bit id arrays) and later the ring and,
+// from k3_policy_order_at on, the order.
+__host__ __device__ inline size_t k3_policy_order_at(int n, int ring_cells, int pt_bytes) {
     const size_t ring = (size_t)ring_cells * 4;
-    const size_t scratch = (size_t)(n + 2) * 2 * pt_bytes + (size_t)(n + 2) * 4 + 256 * 4 + (size_t)n * 8;
-    return k3_policy_order_bytes(n) + (((ring > scratch ? ring : scratch) + 15) & ~(size_t)15);
+    const size_t batch_numbers = (size_t)(n + 2) * 2 * pt_bytes + (size_t)(n + 2) * 4 + 256 * 4 + (size_t)n * 6;
+    return ring > batch_numbers ? ring : batch_numbers;
+}
+__host__ __device__ inline size_t k3_policy_warp_bytes(int n, int ring_cells, int pt_bytes) {
+    return (k3_policy_order_at(n, ring_cells, pt_bytes) + (size_t)n * 2 + 15) & ~(size_t)15;
 }
 
 // grid = B * groups CTAs of W = blockDim.x / 32 warps; CTA (b, g) evaluates instance b under
@@ -159,8 +163,8 @@ k3_eval_policy(const int* __restrict__ s_all, const int* __restrict__ o_all, int
     const int policy = policies[kpol];
     unsigned char* mine = smem_raw + (((size_t)n * 8 + 15) & ~(size_t)15) +
                           (size_t)warp * k3_policy_warp_bytes(n, SIM::ring_cells(L), (int)sizeof(PT));
-    k3_id_t* fin = (k3_id_t*)mine;                    // the finished order
-    int* ring = (int*)(mine + k3_policy_order_bytes(n));   // 16-byte aligned; the scratch until the order is finished
+    k3_id_t* fin = (k3_id_t*)(mine + k3_policy_order_at(n, SIM::ring_cells(L), (int)sizeof(PT)));   // the finished order
+    int* ring = (int*)mine;                           // 16-byte aligned; the scratch until the order is finished
     PT* P = (PT*)ring;
     PT* O = P + (n + 2);
     int* boff = (int*)(O + (n + 2));                  // n + 2 batch offsets
@@ -197,7 +201,7 @@ k3_eval_policy(const int* __restrict__ s_all, const int* __restrict__ o_all, int
         auto f_b = [&](int id) { return bat[id]; };
         ord = k3_warp_radix_sort(byo, ord == bufa ? bufb : bufa, n, hist, lane, f_b, k3_bytes_of((unsigned)nb));
     }
-    for (int i = lane; i < n; i += 32) fin[i] = ord[i];
+    for (int i = lane; i < n; i += 32) fin[i] = ord[i];    // one of the id buffers, all in front of the batch numbers
     __syncwarp();                                     // from here on the scratch is the simulator's
     SIM sim;
     sim.attach(ring, L);

@@ -193,3 +193,24 @@ def test_moves_from_device_rings(omax):
             parts = [h.eval_batch(kv.CAND_MOVE, c)[0] for c in np.array_split(codes, 4)]
         assert (tel[::7] == oracle_moves(s, o, M, base, codes[::7])).all()
         assert (tel == np.concatenate(parts)).all()
+
+
+@pytest.mark.parametrize("n,M", [(7577, 65536), (8118, 65536), (5981, 1 << 22), (6313, 1 << 22)])
+def test_longest_lists_of_the_policy_sweep(n, M):
+    """The longest lists that the policies of one instance fit shared memory with, prefix sums of 32 and of 64
+    bits, and two lengths in front of them; one request more is refused."""
+    inst = W.mixed_backlog(n + 1, 5, M)
+    pols = np.array([kv.POLICY_FCFS, kv.POLICY_SOF, kv.POLICY_TOTAL_SIZE, kv.POLICY_SORTED_F], dtype=np.int32)
+    s, o = inst.s[:n].copy(), inst.o[:n].copy()
+    with kv.Scheduler(s, o, M) as h:
+        tel, _, starts = h.eval_batch(kv.CAND_POLICY, pols, want_starts=True)
+    refs = [orc.policy_order(s, o, orc.FCFS), orc.policy_order(s, o, orc.SHORTEST_OUTPUT_FIRST),
+            orc.policy_order(s, o, orc.TOTAL_SIZE_FIRST), orc.sorted_f_prefix(s, o, M)[0]]
+    for k in range(4):
+        p, t, _ = orc.list_schedule_rounds(s, o, M, refs[k])
+        assert tel[0, k] == t and (starts[0, k] == p).all()
+    if n in (8118, 6313):
+        with kv.Scheduler(inst.s, inst.o, M) as h:
+            with pytest.raises(kv.SchedError) as e:
+                h.eval_batch(kv.CAND_POLICY, pols)
+        assert e.value.code == kv.E_UNSUPPORTED
