@@ -214,3 +214,25 @@ def test_longest_lists_of_the_policy_sweep(n, M):
             with pytest.raises(kv.SchedError) as e:
                 h.eval_batch(kv.CAND_POLICY, pols)
         assert e.value.code == kv.E_UNSUPPORTED
+
+
+@pytest.mark.parametrize("far", [1, 2, 3, 4, 5, 8, 9, 225])
+def test_windows_beyond_the_registers(far):
+    """Decodes whose window ends in the first, second, ... chunk behind the 33 that the long-decode simulator
+    keeps in registers, and beside it: orders, starts and moves (n = 60 has eight states to resume from)."""
+    rng = np.random.default_rng(far)
+    n, top = 60, 32 * (33 + far)
+    o = np.where(rng.random(n) < 0.5, rng.integers(top - 63, top + 1, n), rng.integers(1, top, n)).astype(np.int32)
+    o[0], o[1:3] = 8300, (top, top - 31)                     # the first asks for this simulator
+    s = rng.integers(1, 4000, n).astype(np.int32)
+    M = 2 * int((s.astype(np.int64) + o).max())
+    orders = np.stack([rng.permutation(n) for _ in range(3)]).astype(np.int32)
+    codes = np.arange(0, 3 * n * (n - 1) // 2, 37, dtype=np.int64)
+    with kv.Scheduler(s, o, M) as h:
+        tel, _, starts = h.eval_batch(kv.CAND_ORDER, orders, want_starts=True)
+        h.set_base_order(orders[0])
+        mtel, _, _ = h.eval_batch(kv.CAND_MOVE, codes)
+    for c in range(3):
+        p, t, _ = orc.list_schedule_rounds(s, o, M, orders[c])
+        assert tel[c] == t and (starts[c] == p).all()
+    assert (mtel == oracle_moves(s, o, M, orders[0], codes)).all()
