@@ -37,7 +37,8 @@ const i64 kSweepChunk = 1ll << 22;          // candidates per launch inside a sw
 const int kResultBad = 9;                   // word of d_result: the candidates of a host call are not what they should be
 const int kDeviceCheckMax = 1 << 20;        // requests whose bits fit a CTA's shared memory
 const i64 kAcceptSmall = 16384;              // sweep results that one CTA reduces (4 us against a launch of its own)
-const int kSnapshots = 256;                 // states of the base run kept for the sweeps
+const int kSnapshots = 256;                 // states of the base run kept for the sweeps (chunked simulator)
+const int kSnapStrideHyb = 8;               // positions per state (hybrid simulator)
 const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
 
 // Runs CALL(SIM) with SIM = the simulator class of the handle: the chunked one (NM far registers per
@@ -313,10 +314,13 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         if (B == 1) {
             size_t per = (size_t)h->L * sizeof(int);
             // a candidate replays (stride - 1) / 2 positions on average to reach its first moved one:
-            // 0.2 % of the list at 256 snapshots, for which the base run stores 256 states instead of n
-            i64 stride = ((i64)n + kSnapshots - 1) / kSnapshots;
+            // 0.2 % of the list at 256 snapshots, for which the base run stores 256 states instead of n.
+            // An admission of the hybrid simulator costs as much as storing its state, and late ones ten times
+            // that, so a move near the end of the list counts: one of 20,000 requests with decodes up to 20,000
+            // took 1.65 ms with 256 states and takes 0.20 (the base run 59.8 and 70.7)
+            i64 stride = h->nm ? ((i64)n + kSnapshots - 1) / kSnapshots : kSnapStrideHyb;
             stride = (stride + 3) & ~3ll;               // requests are admitted four at a time
-            if (stride < 16) stride = 16;               // the base run stops for every snapshot
+            if (h->nm && stride < 16) stride = 16;      // the base run stops for every snapshot
             while ((((i64)n + stride - 1) / stride) * (i64)per > (i64)kSnapBudget) stride += 4;
             h->snap_stride = (int)stride;
             h->snap_count = (n + h->snap_stride - 1) / h->snap_stride;
