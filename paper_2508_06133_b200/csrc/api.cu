@@ -1,6 +1,7 @@
 // Host side of the kvsched C-ABI (see include/kvsched.h for the contract of every entry point).
 // All scheduling arithmetic runs in the kernels of k1_sort / k2_fmetric / k3_eval / k5_argmin; this
 // file validates arguments, owns device memory and enqueues launches.  There is no CPU fallback.
+#include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -272,17 +273,20 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
     if (M >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
     const i64 total = (i64)B * n;
     KV_TRY(validate_instance(total, s, o, M));
-    int omax = 0, least = INT32_MAX; i64 sum_max = 0; double volume = 0;
+    int omax = 0, least = INT32_MAX; i64 sum_max = 0, sum_s = 0, sum_o = 0; double volume = 0, short_o = 0;
     for (int b = 0; b < B; ++b) {
         i64 sum = 0;
         for (int i = 0; i < n; ++i) {
             const int v = o[(i64)b * n + i], size = s[(i64)b * n + i] + v;
             sum += v;
+            sum_s += size - v;
             volume += (double)v * (size - 0.5 * v);
+            short_o += v <= 32 ? 1.0 : 32.0 / v;
             omax = v > omax ? v : omax;
             least = size < least ? size : least;
         }
         if (sum > sum_max) sum_max = sum;
+        sum_o += sum;
     }
     if (sum_max + omax >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
 
@@ -297,6 +301,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             rc = kv_cuda_fail(cudaGetLastError(), "cudaDeviceGetAttribute"); break;
         }
         h->B = B; h->n = n; h->M = M; h->omax = omax; h->least = least; h->volume = volume; h->sum_o_max = sum_max;
+        h->mean_s = (double)sum_s / (double)total; h->mean_o = (double)sum_o / (double)total; h->short_share = short_o / (double)total;
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
         h->nm = slots <= 32 ? 1 : slots <= 256 ? slots / 32 : 0;
@@ -507,15 +512,48 @@ int order_candidates(sched_ctx* h, const MoveSource& src, i64 count) {
 //   32,000                4.6 /  3.8        6.1 / 7.5      7.0 /  9.5
 //   48,000                6.9 /  4.3        9.1 / 8.5     10.5 / 10.9
 //   96,000               13.7 /  6.6       18.0 / 13.8    20.9 / 18.3
-// Longer decodes than its ring of events, schedules with more rounds per request than were measured, and
-// backlogs whose candidate could pass 32 bits of waiting time in its sum of starts keep the warp.
+// Two kinds of backlog cost a thread more per admission (log-normal decodes, prefills uniform up to 2,000):
+//   short decodes: a window that ends in one of the two chunks kept as cells takes its share back from them one by one,
+//   which the share of decodes up to a chunk (each counted as 32 / o beyond) tells.  Mean 21 (share 0.94): 40,000 moves of
+//   10,000, 0.5 / 2 / 6 rounds per request 18.6 / 18.4, 22.2 / 30.5, 29.9 / 50.0; mean 84 (0.55): 18.4 / 9.4, 21.9 / 14.6,
+//   25.6 / 25.1;
+//   long decodes on short prefills: memory is used by tokens still to come, what a request waits for lies chunks
+//   ahead, and every wait walks the events up to there.  Prefills up to 20, decodes of mean 340, 10,000 requests, 40,000
+//   moves, 0.5 / 1 / 2 / 6 rounds per request 15.5 / 10.6, 15.7 / 16.0, 16.6 / 40.5, 19.7 / 111; prefills up to 2,000: 18.1 / 8.0,
+//   19.9 / 9.7, 21.6 / 11.9, 26.0 / 24.9; decodes of mean 669 (to 2,048), prefills up to 20: 20.3 / 9.0, 20.7 / 13.4, 21.7 / 16.9,
+//   25.6 / 53.1.  Use of memory falls by s / rounds per round and varies by (s + o) sqrt(rounds ahead / rounds), hence
+//   the form in (1 + o / s) sqrt(rounds); its square and the caps are fitted.  Only where time goes on for
+//   longer than a decode: otherwise nearly everything runs side by side.
+// Of 1,257 sweeps measured in both forms (225 of them on backlogs drawn at random, in Sorted-F, random and index order)
+// 12 take a thread where a warp is faster by more than a tenth (200 by rounds per request alone), 64 the other way round.  Longer decodes than its ring of events, schedules with more rounds per request than
+// were measured (14.8 for decodes beyond 1,025), and backlogs whose candidate could pass 32 bits of waiting
+// time in its sum of starts keep the warp.
 constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.4;
+
+// candidates from which on a thread each is the faster one
+double lanes_from(const sched_ctx* h) {
+    const double rounds = h->volume / ((double)h->n * (double)h->M), n = (double)h->n;
+    double need = LANE_MIN + LANE_MIN_PER_ROUND * rounds, ahead = (1.0 + h->mean_o / h->mean_s) * (1.0 + h->mean_o / h->mean_s);
+    if (rounds > LANE_ROUNDS) return INFINITY;
+    if (h->nm == 1) {
+        if (h->short_share > 0.3) need += 5000.0 * rounds * (h->short_share - 0.3);
+        if (h->short_share > 0.75) need += 150000.0 * (h->short_share - 0.75);
+        ahead = fmin(ahead, 8.0);
+    } else {
+        need *= LANE_LONG;
+        // candidates further apart in a long list also leave one another's rounds: 40,000 moves of 10,000 and of 2,000
+        // requests with a share of 0.57, 6 rounds per request: 30.8 / 44.9 and 6.2 / 5.1
+        if (h->short_share > 0.4 && n > 2000.0) need *= 1.0 + (n - 2000.0) * rounds / 48000.0;
+        ahead = fmin(0.6 * ahead, 3.6);
+    }
+    const double far = ahead * sqrt(rounds);
+    if (n * rounds >= (double)h->omax && far > 5.0) need = far > 8.0 ? INFINITY : need * (1.0 + 0.55 * (far - 5.0));
+    return need;
+}
 
 bool lanes_fit(const sched_ctx* h, i64 count, bool want_starts) {
     if (want_starts || (h->nm != 1 && h->nm != 2) || count <= ordered_from(h)) return false;
-    const double rounds = h->volume / ((double)h->n * (double)h->M);
-    return rounds <= LANE_ROUNDS && (double)count >= (h->nm == 1 ? 1.0 : LANE_LONG) * (LANE_MIN + LANE_MIN_PER_ROUND * rounds) &&
-           (i64)h->n * (h->omax + 64) <= INT32_MAX;
+    return (double)count >= lanes_from(h) && (i64)h->n * (h->omax + 64) <= INT32_MAX;
 }
 
 // The handle's block of rings in device memory, of at least `bytes`; false if there is no memory for it.

@@ -1,12 +1,21 @@
 """Kernel variants at the sizes where one takes over from another, against the CPU oracle."""
 import numpy as np
 import pytest
+import torch
 
 import oracle as orc
 from paper_2508_06133_b200 import binding as kv
 from paper_2508_06133_b200 import workloads as W
 
 pytestmark = pytest.mark.gpu
+
+
+def kernels_of(f):
+    """What f returns, and the names of the kernels that it launched."""
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
+        out = f()
+        torch.cuda.synchronize()
+    return out, " ".join(e.key for e in prof.key_averages())
 
 
 def oracle_moves(s, o, M, base, codes):
@@ -150,8 +159,9 @@ def test_host_candidates_are_checked(n):
 @pytest.mark.parametrize("least", [1, 300])
 @pytest.mark.parametrize("omax", [1, 31, 32, 33, 64, 65, 1024, 1025, 1026, 2049])
 def test_moves_by_lanes(omax, least):
-    """One thread per candidate: every move of 150 requests (33,525) with a budget that lets 1.5 to 3.3 rounds
-    pass per request, event words of both widths, decodes at the edges of its chunks."""
+    """One thread per candidate: every move of 150 requests (33,525, three times over: short decodes keep the warp
+    up to 75,000) with a budget that lets 1.5 to 3.3 rounds pass per request, event words of both widths, decodes at the
+    edges of its chunks."""
     rng = np.random.default_rng(omax + least)
     n = 150
     s = rng.integers(least, 3000, n).astype(np.int32)
@@ -165,12 +175,40 @@ def test_moves_by_lanes(omax, least):
         codes = np.arange(3 * n * (n - 1) // 2, dtype=np.int64)
         with kv.Scheduler(s, o, M) as h:
             h.set_base_order(base)
-            tel, _, _ = h.eval_batch(kv.CAND_MOVE, codes)
-        assert (tel[::11] == oracle_moves(s, o, M, base, codes[::11])).all()
+            (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, np.tile(codes, 3)))
+        assert "k3_lane_moves<%d," % (32 if omax <= 1025 else 64) in names, names
+        tel = tel.reshape(3, -1)
+        assert (tel == tel[0]).all()
+        assert (tel[0, ::11] == oracle_moves(s, o, M, base, codes[::11])).all()
         with kv.Scheduler(s, o, M) as h:                     # the same in calls that take a warp per candidate
             h.set_base_order(base)
-            parts = [h.eval_batch(kv.CAND_MOVE, c)[0] for c in np.array_split(codes, 3)]
-        assert (tel == np.concatenate(parts)).all()
+            parts, names = kernels_of(lambda: [h.eval_batch(kv.CAND_MOVE, c)[0] for c in np.array_split(codes, 3)])
+        assert "k3_lane_moves" not in names, names
+        assert (tel[0] == np.concatenate(parts)).all()
+
+
+@pytest.mark.parametrize("omax,median,smax,rounds,count,thread", [
+    (1024, 200, 4000, 3.0, 24000, True), (1024, 200, 4000, 3.0, 18000, False),
+    (64, 16, 2000, 2.0, 40000, False), (64, 16, 2000, 2.0, 95000, True),      # short decodes
+    (1024, 256, 20, 6.0, 95000, False), (1024, 256, 20, 0.5, 40000, True),    # short prefills: memory grows
+    (2048, 512, 20, 6.0, 95000, False), (2048, 512, 2000, 3.0, 40000, True)])
+def test_which_form_a_sweep_takes(omax, median, smax, rounds, count, thread):
+    """Backlogs on which a thread per candidate is slower than a warp (by up to ten times) keep the warp."""
+    rng = np.random.default_rng(omax + median + smax)
+    n = 2000
+    s = rng.integers(1, smax, n).astype(np.int32)
+    o = np.clip(np.round(rng.lognormal(np.log(median), 0.8, n)), 1, omax).astype(np.int32)
+    o[0] = omax
+    volume = (s.astype(np.float64) * o + o.astype(np.float64) ** 2 / 2).sum()
+    M = max(int((s.astype(np.int64) + o).max()), int(volume / (rounds * n)))
+    best = torch.zeros(2, dtype=torch.int64, device="cuda")
+    with kv.Scheduler(s, o, M) as h:
+        order = h.sorted_f()[0]
+        _, names = kernels_of(lambda: (h.sweep_dev(count, best, sampled=True, seed=3, iteration=2), h.sync()))
+    assert ("k3_lane_moves" in names) == thread and ("k3_eval_moves" in names) != thread, names
+    value, m = best.tolist()
+    i = orc.sample_move(n, 3, 2, m)
+    assert orc.eval_moves(s, o, M, order, [i[0]], [i[1]], [i[2]])[0] == value
 
 
 @pytest.mark.parametrize("omax", [2050, 4097])
