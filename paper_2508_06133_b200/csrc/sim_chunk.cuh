@@ -49,7 +49,12 @@
 // kGlobal: the rings are in device memory.  A simulator for decodes up to 4,097 rounds has 16 KB of ring,
 // so shared memory holds 13 of them per SM and registers 32; the ring is written without waiting and read once per
 // 32 rounds.  100,000 requests, 7,000 moves, 1.0 rounds per request: 50.7 -> 40.7 ms; device_rings_fit has the rule.
-template <int NM, bool kGlobal_ = false>
+//
+// kShort: a window that ends in chunk 0 leaves everything else alone.  Where nearly every decode is a few rounds,
+// a sweep takes 0.75 to 0.99 of the time (mean 2 to 10; without it 1.1 times that of the timeline of single
+// cells that was here before); with longer ones the branches cost more than they save (mean 20: 0.92 to 1.07,
+// mean 200: 1.04 to 1.11).  short_windows (api.cu) has the rule.
+template <int NM, bool kGlobal_ = false, bool kShort = false>
 struct ChunkSim {
     static constexpr bool kGlobal = kGlobal_;
     static constexpr int kWarps = NM == 1 || kGlobal ? 4 : NM == 2 ? 2 : 1;    // per CTA: 16 KB of shared rings
@@ -183,6 +188,7 @@ struct ChunkSim {
     __device__ __forceinline__ int ask(int sp, int om) const {
         const int nk = nkt - sp;                         // it fits  <=>  V[x] <= nk in every round of the window
         int v = (unsigned)rl <= (unsigned)om ? __viaddmin_s32(cur, -nk, rl + 1) : INT_MIN;
+        if (kShort && tau + om <= 31) return kv_warp_max(v);
         if (xr <= om && U[0] > nk) v = max(v, 0);
         if (NM > 1 && tau + om >= 1024 + 32) {
 #pragma unroll
@@ -209,6 +215,7 @@ struct ChunkSim {
     // (sp, om) starts at t
     __device__ __forceinline__ void add(int sp, int om) {
         if ((unsigned)rl <= (unsigned)om) cur += sp + rl;
+        if (kShort && tau + om <= 31) return;
         if (xr <= om) U[0] += sp + x31;
         if (x31 < om) { A[0] += sp - tau; C[0] += 1; }
         if (NM > 1 && tau + om >= 1024 + 32) {

@@ -159,8 +159,8 @@ def test_host_candidates_are_checked(n):
 @pytest.mark.parametrize("least", [1, 300])
 @pytest.mark.parametrize("omax", [1, 31, 32, 33, 64, 65, 1024, 1025, 1026, 2049])
 def test_moves_by_lanes(omax, least):
-    """One thread per candidate: every move of 150 requests (33,525, three times over: short decodes keep the warp
-    up to 75,000) with a budget that lets 1.5 to 3.3 rounds pass per request, event words of both widths, decodes at the
+    """One thread per candidate: every move of 150 requests (33,525, four times over: short decodes keep the warp
+    up to 94,000) with a budget that lets 1.5 to 3.3 rounds pass per request, event words of both widths, decodes at the
     edges of its chunks."""
     rng = np.random.default_rng(omax + least)
     n = 150
@@ -175,9 +175,9 @@ def test_moves_by_lanes(omax, least):
         codes = np.arange(3 * n * (n - 1) // 2, dtype=np.int64)
         with kv.Scheduler(s, o, M) as h:
             h.set_base_order(base)
-            (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, np.tile(codes, 3)))
+            (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, np.tile(codes, 4)))
         assert "k3_lane_moves<%d," % (32 if omax <= 1025 else 64) in names, names
-        tel = tel.reshape(3, -1)
+        tel = tel.reshape(4, -1)
         assert (tel == tel[0]).all()
         assert (tel[0, ::11] == oracle_moves(s, o, M, base, codes[::11])).all()
         with kv.Scheduler(s, o, M) as h:                     # the same in calls that take a warp per candidate
@@ -274,3 +274,24 @@ def test_windows_beyond_the_registers(far):
         p, t, _ = orc.list_schedule_rounds(s, o, M, orders[c])
         assert tel[c] == t and (starts[c] == p).all()
     assert (mtel == oracle_moves(s, o, M, orders[0], codes)).all()
+
+
+@pytest.mark.parametrize("omax", [1, 12, 33, 40])
+def test_moves_of_short_windows(omax):
+    """The simulator for windows that mostly end in the chunk they begin in, and beside them windows that end on
+    its last round and in the two chunks behind it; with a longer mean decode the other one is taken."""
+    rng = np.random.default_rng(omax)
+    n, M = 300, 5000
+    s = rng.integers(1, 2000, n).astype(np.int32)
+    o = rng.integers(1, min(omax, 12) + 1, n).astype(np.int32)
+    o[::30] = omax
+    codes = rng.integers(0, 3 * n * (n - 1) // 2, 3000).astype(np.int64)
+    base = rng.permutation(n).astype(np.int32)
+    with kv.Scheduler(s, o, M) as h:
+        h.set_base_order(base)
+        (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, codes))
+    assert "ChunkSim<1, false, true>" in names, names
+    assert (tel[::5] == oracle_moves(s, o, M, base, codes[::5])).all()
+    with kv.Scheduler(s, 40 * o, M) as h:
+        _, names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, codes))
+    assert ("ChunkSim<1, false, false>" if 40 * omax <= 1025 else "ChunkSim<2, false, false>") in names, names
