@@ -119,7 +119,9 @@ int sched_get_base_order(sched_handle h, int32_t* order_out);
  *   starts_out   : nullable; int32[count][n] start time p_i of every request i, indexed by request
  *                  id (ORDER, MOVE, and POLICY with layout [B][count][n_each]).
  * Host-pointer form: validates ORDER candidates (SCHED_E_NOT_PERMUTATION), MOVE codes and policy
- * ids (SCHED_E_INVAL) and negative start times (SCHED_E_INVAL) before any launch.
+ * ids (SCHED_E_INVAL) and start times outside 0 .. 2^30 - 1 (SCHED_E_INVAL) before anything is evaluated
+ * (more than 8,192 ids or start times by a launch of its own); a refused call writes nothing to the outputs
+ * and counts no evaluation.
  * POLICY builds every order inside the kernel (one warp per instance-policy pair, all of an
  * instance's arrays in shared memory): SCHED_E_UNSUPPORTED when the instance does not fit there
  * (n > 8,118 requests on a single-instance handle, n > 6,313 where n * M >= 2^31; batch handles are

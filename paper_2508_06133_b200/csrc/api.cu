@@ -37,6 +37,7 @@ namespace {
 const i64 kSweepChunk = 1ll << 22;          // candidates per launch inside a sweep
 const int kResultBad = 9;                   // word of d_result: the candidates of a host call are not what they should be
 const int kDeviceCheckMax = 1 << 20;        // requests whose bits fit a CTA's shared memory
+const i64 kHostCheckMax = 1 << 13;          // ids or starts checked by the host: 8 us, a launch and a read-back 13
 const i64 kAcceptSmall = 16384;              // sweep results that one CTA reduces (4 us against a launch of its own)
 const int kSnapshots = 256;                 // states of the base run kept for the sweeps (chunked simulator)
 const int kSnapStrideHyb = 8;               // positions per state (hybrid simulator)
@@ -796,9 +797,9 @@ int sched_get_base_order(sched_handle h, int32_t* order_out) {
     return SCHED_OK;
 }
 
-int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* candidates,
-                         int64_t* tel_out, uint8_t* feasible_out, int32_t* starts_out) {
-    KV_ENTER(h);
+// bad: nullable device word; orders and start times are evaluated only if it is 0 when their kernel starts
+static int eval_batch_dev(sched_handle h, int kind, i64 count, const void* candidates, i64* tel_out, uint8_t* feasible_out,
+                          int32_t* starts_out, const int* bad) {
     if (count < 0 || !tel_out || (count > 0 && !candidates)) return SCHED_E_INVAL;
     if (count == 0) return SCHED_OK;
     if (count >= (1ll << 31)) return SCHED_E_UNSUPPORTED;
@@ -846,7 +847,7 @@ int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* ca
         const size_t smem = k3_smem_bytes(h);
         p.n = n; p.L = h->L; p.M = (int)h->M; p.tbl_id = h->d_tbl_id;
         p.orders = (const int*)candidates; p.count = count; p.tel_out = (i64*)tel_out; p.starts_out = starts_out;
-        p.status = h->d_status;
+        p.bad = bad; p.status = h->d_status;
         KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
 #define RUN(N)                                                                                     \
         if (starts_out) k3_eval_orders<N, true><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p);  \
@@ -880,7 +881,7 @@ int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* ca
         memset(&p, 0, sizeof(p));
         p.n = n; p.M = (int)h->M; p.tbl_id = h->d_tbl_id;
         p.starts = (const int*)candidates; p.sorted_ids = ids; p.count = count;
-        p.tel_out = (i64*)tel_out; p.feasible_out = feasible_out;
+        p.tel_out = (i64*)tel_out; p.feasible_out = feasible_out; p.bad = bad;
         if (h->nm > 0) {
             p.L = h->L;
             const size_t smem = k3_smem_bytes(h);
@@ -910,6 +911,12 @@ int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* ca
     return SCHED_E_INVAL;
 }
 
+int sched_eval_batch_dev(sched_handle h, int kind, int64_t count, const void* candidates,
+                         int64_t* tel_out, uint8_t* feasible_out, int32_t* starts_out) {
+    KV_ENTER(h);
+    return eval_batch_dev(h, kind, count, candidates, (i64*)tel_out, feasible_out, starts_out, nullptr);
+}
+
 int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candidates,
                      int64_t* tel_out, uint8_t* feasible_out, int32_t* starts_out) {
     KV_ENTER(h);
@@ -917,9 +924,10 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
     if (count == 0) return SCHED_OK;
     const int n = h->n;
     size_t cand_bytes = 0; i64 outs = count;
+    const bool on_host = count <= kHostCheckMax / n;
     if (kind == SCHED_CAND_ORDER) {
         if (h->batch_handle) return SCHED_E_INVAL;
-        if (n > kDeviceCheckMax) {
+        if (on_host || n > kDeviceCheckMax) {
             std::vector<unsigned char> seen;
             for (i64 c = 0; c < count; ++c)
                 if (!is_permutation((const int32_t*)candidates + c * n, n, seen)) return SCHED_E_NOT_PERMUTATION;
@@ -935,6 +943,9 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
         cand_bytes = (size_t)count * sizeof(i64);
     } else if (kind == SCHED_CAND_START_TIMES) {
         if (h->batch_handle || starts_out) return SCHED_E_INVAL;
+        if (on_host)
+            for (i64 k = 0; k < count * n; ++k)
+                if ((unsigned)((const int32_t*)candidates)[k] >= (1u << 30)) return SCHED_E_INVAL;
         cand_bytes = (size_t)count * n * sizeof(int);
     } else if (kind == SCHED_CAND_POLICY) {
         for (i64 c = 0; c < count; ++c) {
@@ -954,10 +965,12 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
     KV_TRY(ensure_stage(h, off_starts + starts_bytes + 256));
     char* base = (char*)h->d_stage;
     KV_CUDA(cudaMemcpyAsync(base, candidates, cand_bytes, cudaMemcpyHostToDevice, h->stream));
-    // orders and start times are checked where they have been copied to (a pass over 777 orders of 1,531
-    // takes 8 us there and 1.2 ms here); the evaluation in between reads nothing out of place whatever
-    // they hold, and nothing is handed out before the answer is known
-    const bool on_device = (kind == SCHED_CAND_ORDER && n <= kDeviceCheckMax) || kind == SCHED_CAND_START_TIMES;
+    // orders and start times that are not a few are checked where they have been copied to (a pass over 777
+    // orders of 1,531 takes 8 us there and 1.2 ms here).  The evaluation behind the check does nothing if it
+    // failed: an order of 2^20 times the longest request would be a schedule of hours, of more rounds than
+    // the simulators count
+    const bool on_device = !on_host && ((kind == SCHED_CAND_ORDER && n <= kDeviceCheckMax) || kind == SCHED_CAND_START_TIMES);
+    const int* bad = on_device ? h->d_result + kResultBad : nullptr;
     if (on_device) {
         KV_CUDA(cudaMemsetAsync(h->d_result + kResultBad, 0, sizeof(int), h->stream));
         if (kind == SCHED_CAND_ORDER) {
@@ -971,15 +984,18 @@ int sched_eval_batch(sched_handle h, int kind, int64_t count, const void* candid
         }
         KV_TRY(check_launch(h));
     }
-    int rc = sched_eval_batch_dev(h, kind, count, base, (int64_t*)(base + off_tel),
-                                  feasible_out ? (uint8_t*)(base + off_feas) : nullptr,
-                                  starts_out ? (int32_t*)(base + off_starts) : nullptr);
+    const i64 evaluations = h->evaluations;
+    int rc = eval_batch_dev(h, kind, count, base, (i64*)(base + off_tel), feasible_out ? (uint8_t*)(base + off_feas) : nullptr,
+                            starts_out ? (int32_t*)(base + off_starts) : nullptr, bad);
     if (rc != SCHED_OK) { cudaStreamSynchronize(h->stream); return rc; }
     if (on_device) {
         const int* res = (const int*)h->h_pinned;
         KV_CUDA(cudaMemcpyAsync(h->h_pinned, h->d_result, 16 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
         KV_CUDA(cudaStreamSynchronize(h->stream));
-        if (res[kResultBad]) return kind == SCHED_CAND_ORDER ? SCHED_E_NOT_PERMUTATION : SCHED_E_INVAL;
+        if (res[kResultBad]) {
+            h->evaluations = evaluations;
+            return kind == SCHED_CAND_ORDER ? SCHED_E_NOT_PERMUTATION : SCHED_E_INVAL;
+        }
     }
     KV_CUDA(cudaMemcpyAsync(tel_out, base + off_tel, (size_t)outs * sizeof(i64), cudaMemcpyDeviceToHost, h->stream));
     if (feasible_out) KV_CUDA(cudaMemcpyAsync(feasible_out, base + off_feas, (size_t)outs, cudaMemcpyDeviceToHost, h->stream));

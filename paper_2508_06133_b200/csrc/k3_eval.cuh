@@ -277,6 +277,7 @@ struct OrderEvalParams {
     i64 count;
     i64* tel_out;
     int* starts_out;
+    const int* bad;                    // nullable: not 0, what k3_check_orders has found
     int* status;
 };
 
@@ -288,7 +289,7 @@ k3_eval_orders(const OrderEvalParams p) {
     const int2* __restrict__ tbl = p.tbl_id;
     const int n = p.n, L = p.L, M = p.M;
     const i64 c = (i64)blockIdx.x * (blockDim.x >> 5) + warp;      // every order has the same length
-    if (c >= p.count) return;
+    if (c >= p.count || (p.bad && *p.bad)) return;
     SIM sim;
     sim.attach((int*)smem_raw + (size_t)warp * SIM::ring_cells(L), L);
     const int* ord = p.orders + (size_t)c * n;
@@ -330,6 +331,7 @@ struct StartsEvalParams {
     i64 count;
     i64* tel_out;
     unsigned char* feasible_out;
+    const int* bad;           // nullable: not 0, what k3_check_start_range has found
     unsigned int* counter;
 };
 
@@ -339,7 +341,7 @@ k3_check_starts(const StartsEvalParams p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const i64 c = (i64)blockIdx.x * SIM::kWarps + warp;
-    if (c >= p.count) return;
+    if (c >= p.count || (p.bad && *p.bad)) return;
     const int n = p.n, M = p.M;
     const int* st_c = p.starts + (size_t)c * n;
     const int* ids = p.sorted_ids + (size_t)c * n;
@@ -379,6 +381,7 @@ k3_check_starts_cells(const StartsEvalParams p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* ring = (int*)smem_raw + (size_t)warp * p.L;
     const int n = p.n, L = p.L, M = p.M;
+    if (p.bad && *p.bad) return;
     for (;;) {
         unsigned c32 = 0;
         if (lane == 0) c32 = atomicAdd(p.counter, 1u);

@@ -130,10 +130,10 @@ def test_online_windows(lookahead):
         assert (starts[0] == p).all() and lat[0] == tot
 
 
-@pytest.mark.parametrize("n", [2, 40, 1531])
+@pytest.mark.parametrize("n", [2, 40, 1170, 1171, 1531])
 def test_host_candidates_are_checked(n):
     """An order with a repeated id, one with an id outside 0 .. n-1, a negative start and one of 2^30 are
-    refused, wherever they stand; the handle goes on."""
+    refused, wherever they stand, and not evaluated; the handle goes on.  1,170 are the most that the host checks."""
     rng = np.random.default_rng(n)
     s = rng.integers(1, 50, n).astype(np.int32)
     o = rng.integers(1, 50, n).astype(np.int32)
@@ -143,15 +143,17 @@ def test_host_candidates_are_checked(n):
         for row, col, value in ((6, n - 1, good[6, 0]), (0, 0, n), (3, n // 2, -1)):
             bad = good.copy()
             bad[row, col] = value
+            before = h.stats()[1]
             with pytest.raises(kv.SchedError) as e:
-                h.eval_batch(kv.CAND_ORDER, bad)
-            assert e.value.code == kv.E_NOT_PERMUTATION
+                h.eval_batch(kv.CAND_ORDER, bad, want_starts=True)
+            assert e.value.code == kv.E_NOT_PERMUTATION and h.stats()[1] == before
         for row, col, value in ((6, n - 1, -1), (0, 0, 1 << 30)):
             bad = starts.copy()
             bad[row, col] = value
+            before = h.stats()[1]
             with pytest.raises(kv.SchedError) as e:
                 h.eval_batch(kv.CAND_START_TIMES, bad, want_feasible=True)
-            assert e.value.code == kv.E_INVAL
+            assert e.value.code == kv.E_INVAL and h.stats()[1] == before
         again, ok, _ = h.eval_batch(kv.CAND_START_TIMES, starts, want_feasible=True)
     assert ok.all() and (again == tel).all()
 
