@@ -262,6 +262,9 @@ int k3_warps(const sched_ctx* h) {
 
 size_t k3_smem_bytes(const sched_ctx* h) { return (size_t)k3_warps(h) * h->ring_cells * sizeof(int); }
 
+// A sort of rows of n entries merges more than once: it needs a second pair of buffers.
+bool sort_needs_two(int n) { return n > K1_MERGE_RUNS * K1_TILE; }
+
 // d_result, d_order and d_batch_off as create_common lays them out: {TEL, batches, status}, n, n + 1 ints
 size_t order_at() { return 256; }
 size_t offsets_at(int n) { return order_at() + (((size_t)n * sizeof(int) + 255) & ~(size_t)255); }
@@ -353,6 +356,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
                 take(&h->d_base_starts, n);
                 take(&h->d_keys_a, n); take(&h->d_keys_b, n);
                 take(&h->d_vals_a, n); take(&h->d_vals_b, n);
+                if (sort_needs_two(n)) { take(&h->d_keys_more, n); take(&h->d_vals_more, n); }
                 take(&h->d_prefP, n + 1); take(&h->d_prefO, n + 1);
                 take(&h->d_snap_ring, (size_t)h->snap_count * h->L);
                 take(&h->d_snap_hdr, h->snap_count);
@@ -408,9 +412,9 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
 }
 
 // `rows` lists of n entries in ascending (key, value) order -> out.  More than one tile: through
-// tmp_keys / tmp_vals (rows * n entries each).
+// tmp_keys / tmp_vals (rows * n entries each); more than one merge: and through more_keys / more_vals.
 template <class KEY>
-int sort_rows(sched_ctx* h, const KEY& src, int n, i64 rows, u64* tmp_keys, int* tmp_vals, int* out) {
+int sort_rows(sched_ctx* h, const KEY& src, int n, i64 rows, u64* tmp_keys, int* tmp_vals, u64* more_keys, int* more_vals, int* out) {
     const int tiles = (n + K1_TILE - 1) / K1_TILE;
     const i64 total = rows * n, ctas = rows * tiles;
     if (total >= (1ll << 31) || ctas >= (1ll << 31)) return SCHED_E_UNSUPPORTED;
@@ -418,10 +422,24 @@ int sort_rows(sched_ctx* h, const KEY& src, int n, i64 rows, u64* tmp_keys, int*
     while (threads < n && threads < K1_TILE) threads <<= 1;
     k1_tile_sort<<<(unsigned)ctas, threads, 0, h->stream>>>(src, n, tiles, tiles > 1 ? tmp_keys : nullptr, tiles > 1 ? tmp_vals : out);
     KV_TRY(check_launch(h));
-    if (tiles > 1) {
+    int merges = 0;
+    for (i64 most = 1; most < tiles; most *= K1_MERGE_RUNS) ++merges;
+    i64 run = K1_TILE;
+    for (; merges > 0; --merges) {
+        // as few runs per merge as the merges that are left can do with
+        const int runs = (int)((n + run - 1) / run);
+        int group = 2;
+        for (;; ++group) {
+            i64 reach = 1;
+            for (int k = 0; k < merges && reach < runs; ++k) reach *= group;
+            if (reach >= runs) break;
+        }
         k1_tile_merge<<<(unsigned)((total + K1_MERGE_THREADS - 1) / K1_MERGE_THREADS), K1_MERGE_THREADS, 0, h->stream>>>(
-            tmp_keys, tmp_vals, n, total, out);
+            tmp_keys, tmp_vals, n, total, (int)run, group, bits_of((u64)run), merges > 1 ? more_keys : nullptr, merges > 1 ? more_vals : out);
         KV_TRY(check_launch(h));
+        run *= group;
+        u64* const k = tmp_keys; tmp_keys = more_keys; more_keys = k;
+        int* const v = tmp_vals; tmp_vals = more_vals; more_vals = v;
     }
     return SCHED_OK;
 }
@@ -866,17 +884,20 @@ static int eval_batch_dev(sched_handle h, int kind, i64 count, const void* candi
         const i64 total = count * n;
         if (total >= (1ll << 31)) return SCHED_E_UNSUPPORTED;
         // ids of every candidate by ascending (start, id)
-        const bool tiled = n > K1_TILE;
-        const size_t need = (size_t)total * (sizeof(int) + (tiled ? sizeof(u64) + sizeof(int) : 0)) + 64;
+        const bool tiled = n > K1_TILE, two = sort_needs_two(n);
+        const size_t pair = sizeof(u64) + sizeof(int);
+        const size_t need = (size_t)total * (sizeof(int) + (tiled ? pair : 0) + (two ? pair : 0)) + 64;
         if (h->sort_cap < need) {
             if (h->d_sort) { kv_free(h->d_sort); h->d_sort = nullptr; h->sort_cap = 0; }
             KV_CUDA(kv_malloc((void**)&h->d_sort, need));
             h->sort_cap = need;
         }
         u64* tmp_keys = tiled ? (u64*)h->d_sort : nullptr;
-        int* tmp_vals = tiled ? (int*)(tmp_keys + total) : nullptr;
-        int* ids = tiled ? tmp_vals + total : (int*)h->d_sort;
-        KV_TRY(sort_rows(h, K1StartKey{(const int*)candidates}, n, count, tmp_keys, tmp_vals, ids));
+        u64* more_keys = two ? tmp_keys + total : nullptr;
+        int* tmp_vals = tiled ? (int*)(tmp_keys + (two ? 2 : 1) * total) : nullptr;
+        int* more_vals = two ? tmp_vals + total : nullptr;
+        int* ids = two ? more_vals + total : tiled ? tmp_vals + total : (int*)h->d_sort;
+        KV_TRY(sort_rows(h, K1StartKey{(const int*)candidates}, n, count, tmp_keys, tmp_vals, more_keys, more_vals, ids));
         StartsEvalParams p;
         memset(&p, 0, sizeof(p));
         p.n = n; p.M = (int)h->M; p.tbl_id = h->d_tbl_id;
@@ -1035,7 +1056,7 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
     const int* list = h->d_vals_a;              // the batches one behind the other
     if (solver == 0) {
         // S1: ascending (s+o, o, index)
-        KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_SORTED_F}, n, 1, h->d_keys_a, h->d_vals_b, h->d_vals_a));
+        KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_SORTED_F}, n, 1, h->d_keys_a, h->d_vals_b, h->d_keys_more, h->d_vals_more, h->d_vals_a));
         // S2: prefix sums + F-metric batch boundaries; the sums in shared memory where they fit
         const size_t bytes = 2 * ((size_t)n + 1) * sizeof(i64);
         const bool fits = bytes <= (size_t)h->smem_optin - 4096;
@@ -1050,7 +1071,7 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
         KV_TRY(phase1_quantile(h, seed));
     } else {
         // Algorithm 3: ascending (s+o, index), then first fit + improving swaps, batch after batch
-        KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_TOTAL_SIZE}, n, 1, h->d_keys_a, h->d_vals_b, h->d_vals_a));
+        KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_TOTAL_SIZE}, n, 1, h->d_keys_a, h->d_vals_b, h->d_keys_more, h->d_vals_more, h->d_vals_a));
         if ((i64)h->g_num * h->M + (i64)h->g_den * h->omax >= (1ll << 31)) return SCHED_E_UNSUPPORTED;   // 32-bit weights
         // the solver's arrays in shared memory (21 bytes per request) up to about 11,000 requests
         const size_t bytes = k2l_bytes<unsigned short>(n);
@@ -1068,7 +1089,7 @@ static int sorted_f_common_dev(sched_handle h, int solver, int32_t* order_out, i
     }
     // each batch by ascending (o, index)
     KV_TRY(sort_rows(h, K1BatchKey{h->d_o, list, h->d_batch_off, h->d_num_batches}, n, 1, h->d_keys_a,
-                     list == h->d_vals_a ? h->d_vals_b : h->d_vals_a, h->d_order));
+                     list == h->d_vals_a ? h->d_vals_b : h->d_vals_a, h->d_keys_more, h->d_vals_more, h->d_order));
     h->base_ready = false;
     KV_TRY(ensure_base(h));
     if (order_out) KV_CUDA(cudaMemcpyAsync(order_out, h->d_order, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, st));
@@ -1180,9 +1201,9 @@ static int phase1_quantile(sched_handle h, u64 seed) {
     int* list = h->d_vals_b;
     int* by_size = (int*)h->d_keys_b;
     int* by_ratio = by_size + n;
-    KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_SOF}, n, 1, h->d_keys_a, h->d_vals_a, list));
-    KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, 0}, n, 1, h->d_keys_a, h->d_vals_a, by_size));
-    KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, F}, n, 1, h->d_keys_a, h->d_vals_a, by_ratio));
+    KV_TRY(sort_rows(h, K1RequestKey{h->d_s, h->d_o, SCHED_POLICY_SOF}, n, 1, h->d_keys_a, h->d_vals_a, h->d_keys_more, h->d_vals_more, list));
+    KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, 0}, n, 1, h->d_keys_a, h->d_vals_a, h->d_keys_more, h->d_vals_more, by_size));
+    KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, F}, n, 1, h->d_keys_a, h->d_vals_a, h->d_keys_more, h->d_vals_more, by_ratio));
     const size_t bytes = k2q_bytes<unsigned short>(n), room = (size_t)h->smem_optin - sizeof(K2qShared) - 1024;
     if (n < 65536 && bytes <= room) {
         KV_CUDA(cudaFuncSetAttribute(k2_quantile<unsigned short>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));

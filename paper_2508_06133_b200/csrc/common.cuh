@@ -80,6 +80,8 @@ struct sched_ctx {
     // sort / F-metric scratch (single-instance handles)
     u64 *d_keys_a, *d_keys_b;
     int *d_vals_a, *d_vals_b;
+    u64* d_keys_more;        // [n] each where a sort takes more than one merge
+    int* d_vals_more;
     i64 *d_prefP, *d_prefO;  // [n+1]
     int* d_batch_off;        // [n+1]
     int* d_num_batches;      // [1]

@@ -70,6 +70,29 @@ def test_sorting_and_batch_selection_sizes(n):
     assert tel == orc.list_schedule_rounds(s, o, M, r_order)[1]
 
 
+@pytest.mark.parametrize("n", [32768, 32769, 40000, 70001, 1048577])
+def test_sorting_in_several_merges(n):
+    """The last length that one merge sorts, the first that takes two, groups of runs that do not come out even,
+    and the first that takes three; rows of start times, and through the Phase-1 sorts where n is not too large."""
+    rng = np.random.default_rng(n)
+    s = rng.integers(1, 50, n).astype(np.int32)
+    o = rng.integers(1, 6, n).astype(np.int32)
+    M = 1 << 28                                              # everything fits beside each other
+    with kv.Scheduler(s, o, M) as h:
+        order, _, tel = h.sorted_f()
+        # one batch of everything, by ascending (o, index)
+        assert (order == np.lexsort((np.arange(n), o))).all() and tel == int(o.astype(np.int64).sum())
+        starts = np.stack([rng.integers(0, 300, n), rng.integers(0, 300, n)]).astype(np.int32)
+        for budget in (M, 2000):                             # the second one is exceeded
+            if budget < M:
+                h2 = kv.Scheduler(s, o, budget)
+            got, ok, _ = (h if budget == M else h2).eval_batch(kv.CAND_START_TIMES, starts, want_feasible=True)
+            ref = [orc.check_schedule(s, o, budget, st) for st in starts]
+            assert [int(x) for x in got] == [r["tel"] for r in ref]
+            assert [bool(x) for x in ok] == [r["feasible"] for r in ref]
+        h2.close()
+
+
 @pytest.mark.parametrize("n", [2, 63, 65, 513, 1500])
 @pytest.mark.parametrize("weight", [0, 1])
 def test_local_swap_sizes(n, weight):
