@@ -603,6 +603,7 @@ int run_lanes(sched_ctx* h, LaneParams& q, bool* done) {
     q.counter = h->d_counter + 1;
     KV_CUDA(cudaMemsetAsync(q.counter, 0, sizeof(unsigned), h->stream));
     KV_CUDA(cudaFuncSetAttribute(k3_lane_moves<CH, WORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem));
+    KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
     k3_lane_moves<CH, WORD><<<grid, 32 * S::kWarps, S::kSmem, h->stream>>>(q);
     *done = true;
     return SCHED_OK;
@@ -629,21 +630,24 @@ bool device_rings_fit(const sched_ctx* h, i64 count, bool want_starts) {
     return !want_starts && h->nm == 4 && count >= 27ll * h->sm_count && h->volume <= 2.0 * (double)h->n * (double)h->M;
 }
 
-// 512 MB of rings per launch.  false: no memory for them, nothing was launched.
-bool moves_from_device_rings(sched_ctx* h, MoveEvalParams& p) {
+// 512 MB of rings per launch.  SCHED_OK with *done = false: no memory for them, nothing was launched.
+int moves_from_device_rings(sched_ctx* h, MoveEvalParams& p, bool* done) {
     typedef ChunkSim<4, true> S;
     const size_t bytes = (size_t)h->ring_cells * sizeof(int);
     i64 most = (i64)(((size_t)512 << 20) / bytes);
     if (most > p.count) most = p.count;
-    if (!grow_rings(h, bytes * most)) return false;
+    *done = false;
+    if (!grow_rings(h, bytes * most)) return SCHED_OK;
     p.rings = (int*)h->d_rings;
+    KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
     for (i64 at = 0; at < p.count; at += most) {
         p.first_slot = at;
         p.end_slot = at + most < p.count ? at + most : p.count;
         const i64 ctas = (p.end_slot - at + S::kWarps - 1) / S::kWarps;
         k3_eval_moves<S, false><<<(unsigned)ctas, S::kWarps * 32, 0, h->stream>>>(p);
     }
-    return true;
+    *done = true;
+    return SCHED_OK;
 }
 
 // by_slot: TELs are left in launch-slot order (h->d_k4's launch_order maps a slot to its candidate
@@ -667,13 +671,12 @@ int launch_moves(sched_ctx* h, int mode, const i64* codes, i64 first, u64 seed, 
         KV_TRY(order_candidates(h, p.src, count));
         p.launch_order = last_launch_order(h, count);
     }
-    KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
-    bool lanes = lanes_fit(h, count, starts_out != nullptr);
-    if (lanes) KV_TRY(launch_lanes(h, p, &lanes));
-    bool done = lanes;
-    if (!done && device_rings_fit(h, count, starts_out != nullptr)) done = moves_from_device_rings(h, p);
+    bool done = false;                               // ev_k3_begin is recorded behind the search for memory
+    if (lanes_fit(h, count, starts_out != nullptr)) KV_TRY(launch_lanes(h, p, &done));
+    else if (device_rings_fit(h, count, starts_out != nullptr)) KV_TRY(moves_from_device_rings(h, p, &done));
     if (!done) {
         p.first_slot = 0; p.end_slot = count;
+        KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
         if (short_windows(h, starts_out != nullptr)) {
             k3_eval_moves<ChunkSim<1, false, true>, false><<<k3_grid(h, count), k3_warps(h) * 32, smem, h->stream>>>(p);
             done = true;
