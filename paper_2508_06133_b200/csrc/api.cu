@@ -641,6 +641,7 @@ int moves_from_device_rings(sched_ctx* h, MoveEvalParams& p, bool* done) {
     p.rings = (int*)h->d_rings;
     KV_CUDA(cudaEventRecord(h->ev_k3_begin, h->stream));
     for (i64 at = 0; at < p.count; at += most) {
+        if (at > 0) KV_TRY(check_launch(h));               // the caller counts the last launch
         p.first_slot = at;
         p.end_slot = at + most < p.count ? at + most : p.count;
         const i64 ctas = (p.end_slot - at + S::kWarps - 1) / S::kWarps;

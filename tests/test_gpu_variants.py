@@ -15,7 +15,7 @@ def kernels_of(f):
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA], acc_events=True) as prof:
         out = f()
         torch.cuda.synchronize()
-    return out, " ".join(e.key for e in prof.key_averages())
+    return out, " ".join(" ".join([e.key] * e.count) for e in prof.key_averages())
 
 
 def oracle_moves(s, o, M, base, codes):
@@ -320,6 +320,28 @@ def test_moves_of_short_windows(omax):
     with kv.Scheduler(s, 40 * o, M) as h:
         _, names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, codes))
     assert ("ChunkSim<1, false, false>" if 40 * omax <= 1025 else "ChunkSim<2, false, false>") in names, names
+
+
+@pytest.mark.parametrize("count", [5000, 32768, 32769, 80000])
+def test_launches_of_moves_from_device_rings(count):
+    """32,768 rings of 16 KB per launch: every launch counts, and the candidates of all of them agree with a call
+    that holds them in shared memory."""
+    rng = np.random.default_rng(count)
+    n = 40
+    s = rng.integers(1000, 3000, n).astype(np.int32)
+    o = rng.integers(1, 4098, n).astype(np.int32)
+    o[0] = 4097
+    M = int((s.astype(np.int64) * o + o.astype(np.int64) ** 2 // 2).sum() // n)
+    total = 3 * n * (n - 1) // 2
+    codes = np.arange(count, dtype=np.int64) % total
+    with kv.Scheduler(s, o, M) as h:
+        few, _, _ = h.eval_batch(kv.CAND_MOVE, np.arange(total, dtype=np.int64))
+        before = h.stats()[0]
+        (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, codes))
+        launches = h.stats()[0] - before
+    assert names.count("k3_eval_moves<ChunkSim<4, true") == -(-count // 32768), names
+    assert launches == names.count("k3_eval_moves<") + names.count("k4_"), names
+    assert (tel == few[codes]).all()
 
 
 @pytest.mark.parametrize("omax", [1000, 4000])
