@@ -67,7 +67,7 @@ k3_lane_moves(const LaneParams P) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* b0 = lane_smem + 4 * threadIdx.x;                                 // cells in fours: at(x)
     int* b1 = b0 + CH / 4 * VS;
-    auto at = [](int x) -> int { return (x >> 2) * VS + (x & 3); };
+    auto at = [](int x) -> int { const int c = (int)KV_IDX(x, CH, 425); return (c >> 2) * VS + (c & 3); };
     WORD* const ring = (WORD*)P.rings + ((size_t)blockIdx.x * S::kWarps + warp) * S::kRingWords + lane * PER;
     const int n = P.m.n, M = P.m.M, least = P.least, shift = P.shift;
     const WORD vmask = ((WORD)1 << shift) - 1, one = (WORD)1 << shift;
@@ -81,7 +81,10 @@ k3_lane_moves(const LaneParams P) {
         return ring + (size_t)KV_IDX(k, NCH, 421) * (32 * CH);
     };
     // the word of the x-th round behind the beginning of slot `slot`
-    auto word_of = [&](int slot, int x) -> WORD* { return line_of(slot + x / CH) + (x & (CH - 1)) / PER * (32 * PER) + (x & (PER - 1)); };
+    auto word_of = [&](int slot, int x) -> WORD* {
+        x = (int)KV_IDX(x, NCH * CH, 426);
+        return line_of(slot + x / CH) + (x & (CH - 1)) / PER * (32 * PER) + (x & (PER - 1));
+    };
     for (;;) {
         unsigned group = 0;
         if (lane == 0) group = atomicAdd(P.counter, 1u);

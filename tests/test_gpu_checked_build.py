@@ -1,9 +1,9 @@
 """The checked build of the library (libkvsched_checked.so, -DKVSCHED_CHECKED): every index a kernel
 derives from data or from its own arithmetic is range-checked before use, an index that leaves its
 array is recorded and replaced by 0, and the host call reports SCHED_E_INTERNAL.  It stands in for a
-memory checker: the small-instance parity tests are run once more against it, in a child process
-(the library is chosen when the binding is first loaded), and must pass unchanged -- which also
-means that no index was ever out of range.  The check itself is shown to fire on an out-of-range
+memory checker: the small-instance parity tests and those of the kernel variants are run once more
+against it, in child processes (the library is chosen when the binding is first loaded), and must pass
+unchanged -- which also means that no index was ever out of range.  The check itself is shown to fire on an out-of-range
 value through a probe call that accesses nothing."""
 import os
 import subprocess
@@ -19,6 +19,11 @@ SMALL_CASES = ("small_random or paper_example or long_waits or every_simulator_s
                "local_swap_matches or quantile_greedy or online_policies_match or amin_small or tiny_backlog_all_solvers or "
                "policy_sweep_small or odd_sizes or start_times_checker or local_search_tiny or local_search_random or "
                "sampled_and_resume or bounds_checked_on_the_device or 8_byte_aligned")
+
+# the kernels that only larger calls take, and the edges of what each variant covers
+VARIANT_CASES = ("moves_by_lanes or device_rings or short_windows or beyond_the_registers or timeline_sizes or sorting or "
+                 "several_merges or longest_lists or candidates_are_checked or dynamic_programme or online_windows or "
+                 "local_swap_sizes or beyond_shared_memory")
 
 _PROBE = r"""
 import sys
@@ -59,6 +64,15 @@ def test_checked_build_reports_an_index_outside_its_array():
 def test_small_parity_cases_pass_on_the_checked_build():
     r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(ROOT, "tests", "test_gpu_parity.py"), "-m", "gpu",
                         "-x", "-q", "-p", "no:cacheprovider", "-k", SMALL_CASES],
+                       env=_env(), capture_output=True, text=True, timeout=3000, cwd=ROOT)
+    tail = r.stdout[-3000:] + r.stderr[-2000:]
+    assert r.returncode == 0, tail
+    assert " passed" in r.stdout and "failed" not in r.stdout, tail
+
+
+def test_kernel_variants_pass_on_the_checked_build():
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(ROOT, "tests", "test_gpu_variants.py"), "-m", "gpu",
+                        "-x", "-q", "-p", "no:cacheprovider", "-k", VARIANT_CASES],
                        env=_env(), capture_output=True, text=True, timeout=3000, cwd=ROOT)
     tail = r.stdout[-3000:] + r.stderr[-2000:]
     assert r.returncode == 0, tail
