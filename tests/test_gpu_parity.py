@@ -78,14 +78,14 @@ def test_orders_long_waits_and_ring_wrap():
             assert tel[c] == t and (starts[c] == p).all()
 
 
-@pytest.mark.parametrize("sim", ["", "smem", "hybrid"])
+@pytest.mark.parametrize("sim", ["", "hybrid"])
 def test_orders_wait_decided_behind_the_first_chunk(sim, monkeypatch):
     """The simulators look at the first 32 rounds of a window before anything else.  Here the only
     rounds over budget lie behind them: with M = 195, A = (s 100, o 40) runs from round 0 and peaks at
     140 tokens in round 39; B = (s 20, o 60) fits beside it in rounds 0..31 (at most 132 + 52 = 184)
     and first overflows in round 37 (138 + 58 = 196), so its wait comes from the second chunk alone.
     Also with the pair shifted to every kind of start offset inside a chunk, with longer tails, and
-    in other orders; on the default simulator and on the two with shared-memory timelines."""
+    in other orders; on the default simulator and on the hybrid one."""
     if sim:
         monkeypatch.setenv("KVSCHED_SIM", sim)
     M = 195
@@ -130,10 +130,10 @@ def test_orders_every_simulator_shape(omax):
     assert (mtel == oracle_moves(s, o, M, orders[0], codes)).all()
 
 
-@pytest.mark.parametrize("sim", ["smem", "hybrid"])
+@pytest.mark.parametrize("sim", ["", "hybrid"])
 def test_simulators_with_shared_memory_timelines(sim, monkeypatch):
-    """The all-shared-memory simulator and the hybrid one (33 registers per lane + a shared-memory ring
-    for the rounds after them), each forced for every window length: short windows that never reach
+    """The simulator that the lengths ask for (chunked up to 8,193 rounds) and the hybrid one (33 registers per
+    lane + a shared-memory ring for the rounds after them) forced for every window length: short windows that never reach
     the ring, windows that end in its first chunk, windows over most of it, waits longer than the
     whole state; explicit orders with start times, moves from snapshots, and the policy sweep."""
     monkeypatch.setenv("KVSCHED_SIM", sim)
