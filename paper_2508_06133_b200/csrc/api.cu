@@ -270,6 +270,10 @@ size_t order_at() { return 256; }
 size_t offsets_at(int n) { return order_at() + (((size_t)n * sizeof(int) + 255) & ~(size_t)255); }
 size_t result_bytes(int n) { return offsets_at(n) + ((size_t)n + 1) * sizeof(int); }
 
+// Orders of up to 4,000,000 requests are handed in and out through the handle's pinned block; larger ones are
+// copied from and to the caller's memory (pinning 128 MB for 10,000,000 requests takes sched_init 100 ms).
+bool reads_through_pinned(int n) { return 256 + result_bytes(n) <= ((size_t)32 << 20); }
+
 int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t* o, i64 M) {
     if (!out) return SCHED_E_INVAL;
     *out = nullptr;
@@ -368,7 +372,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         h->d_status = h->d_result + 3;
         h->d_best = (i64*)(h->d_result + 4);
         h->d_accepted = h->d_result + 8;
-        h->pinned_bytes = 256 + (B == 1 ? result_bytes(n) : 0);
+        h->pinned_bytes = 256 + (B == 1 && reads_through_pinned(n) ? result_bytes(n) : 0);
         if (kv_host_malloc(&h->h_pinned, &h->pinned_bytes) != cudaSuccess) { h->h_pinned = nullptr; rc = kv_cuda_fail(cudaGetLastError(), "cudaHostAlloc"); break; }
         cudaStream_t st = h->stream;
 #define C(call) if ((call) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), #call); break; }
@@ -1109,14 +1113,22 @@ static int sorted_f_common_host(sched_handle h, int solver, int32_t* order_out, 
     KV_TRY(sorted_f_common_dev(h, solver, nullptr, nullptr, nullptr, nullptr, seed));
     const int n = h->n;
     char* hp = (char*)h->h_pinned;
-    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, result_bytes(n), cudaMemcpyDeviceToHost, h->stream));
+    const bool pinned = reads_through_pinned(n);
+    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, pinned ? result_bytes(n) : 16 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     KV_CUDA(cudaStreamSynchronize(h->stream));
     const int nb = ((int*)hp)[2], status = ((int*)hp)[3];
     KV_TRY(after_status(h, status));
     if (tel_out) *tel_out = *(i64*)hp;
     if (num_batches_out) *num_batches_out = nb;
-    if (order_out) memcpy(order_out, hp + order_at(), (size_t)n * sizeof(int));
-    if (batch_offsets_out) memcpy(batch_offsets_out, hp + offsets_at(n), ((size_t)nb + 1) * sizeof(int));
+    const size_t order_bytes = (size_t)n * sizeof(int), offset_bytes = ((size_t)nb + 1) * sizeof(int);
+    if (pinned) {
+        if (order_out) memcpy(order_out, hp + order_at(), order_bytes);
+        if (batch_offsets_out) memcpy(batch_offsets_out, hp + offsets_at(n), offset_bytes);
+    } else {
+        if (order_out) KV_CUDA(cudaMemcpyAsync(order_out, h->d_order, order_bytes, cudaMemcpyDeviceToHost, h->stream));
+        if (batch_offsets_out) KV_CUDA(cudaMemcpyAsync(batch_offsets_out, h->d_batch_off, offset_bytes, cudaMemcpyDeviceToHost, h->stream));
+        KV_CUDA(cudaStreamSynchronize(h->stream));
+    }
     return SCHED_OK;
 }
 
@@ -1261,13 +1273,16 @@ int sched_local_search(sched_handle h, int neighbourhood, int32_t iters, uint64_
     const int n = h->n;
     cudaStream_t st = h->stream;
     char* hp = (char*)h->h_pinned;
-    if (order_inout) {                               // through the pinned block: every path below waits for the stream
+    const bool pinned = reads_through_pinned(n);
+    if (order_inout && pinned) {                     // every path below waits for the stream
         std::vector<unsigned char> seen;
         if (!is_permutation(order_inout, n, seen)) return SCHED_E_NOT_PERMUTATION;
         KV_CUDA(cudaStreamSynchronize(st));
         memcpy(hp, order_inout, (size_t)n * sizeof(int));
         KV_CUDA(cudaMemcpyAsync(h->d_order, hp, (size_t)n * sizeof(int), cudaMemcpyHostToDevice, st));
         h->base_ready = false;
+    } else if (order_inout) {
+        KV_TRY(sched_set_base_order(h, order_inout));
     }
     const int sampled = neighbourhood == SCHED_NBHD_SAMPLED ? 1 : 0;
     const i64 total = n >= 2 ? neighbourhood_size(n, neighbourhood, samples_per_iter) : 0;
@@ -1296,10 +1311,11 @@ int sched_local_search(sched_handle h, int neighbourhood, int32_t iters, uint64_
             break;
         }
     }
-    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, order_at() + (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, st));
+    KV_CUDA(cudaMemcpyAsync(hp, h->d_result, pinned ? order_at() + (size_t)n * sizeof(int) : 16 * sizeof(int), cudaMemcpyDeviceToHost, st));
     KV_CUDA(cudaStreamSynchronize(st));
     KV_TRY(after_status(h, res[3]));
-    if (order_inout) memcpy(order_inout, hp + order_at(), (size_t)n * sizeof(int));
+    if (order_inout && pinned) memcpy(order_inout, hp + order_at(), (size_t)n * sizeof(int));
+    else if (order_inout) KV_TRY(sched_get_base_order(h, order_inout));
     if (tel_out) *tel_out = *(const i64*)hp;
     if (iters_done_out) *iters_done_out = it;
     return SCHED_OK;

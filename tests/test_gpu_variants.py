@@ -362,3 +362,22 @@ def test_kernel_time_without_the_search_for_memory(omax):
                 h.sync()
                 ms.append(h.last_eval_kernel_ms())
     assert ms[0] <= 1.5 * min(ms[1:]) + 0.05, ms
+
+
+def test_orders_that_do_not_pass_through_pinned_memory():
+    """4,300,000 requests: the order and the offsets of a solver and a search's order in and out."""
+    n, M = 4300000, 1 << 28
+    rng = np.random.default_rng(4)
+    s = rng.integers(1, 8, n).astype(np.int32)
+    o = rng.integers(1, 4, n).astype(np.int32)
+    total = int(o.astype(np.int64).sum())
+    with kv.Scheduler(s, o, M) as h:                         # everything fits beside each other
+        order, offsets, tel = h.sorted_f()
+        assert (order == np.lexsort((np.arange(n), o))).all() and list(offsets) == [0, n] and tel == total
+        given = rng.permutation(n).astype(np.int32)
+        final, tel, done, trace = h.local_search(kv.NBHD_SAMPLED, 1, order=given, seed=1, samples_per_iter=64)
+        assert (final == given).all() and tel == total and done == 1 and trace[0, 1] == total
+        assert (h.get_base_order() == given).all()
+        with pytest.raises(kv.SchedError) as e:
+            h.local_search(kv.NBHD_SAMPLED, 1, order=np.zeros(n, dtype=np.int32), seed=1, samples_per_iter=64)
+        assert e.value.code == kv.E_NOT_PERMUTATION
