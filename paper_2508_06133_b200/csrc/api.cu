@@ -270,18 +270,6 @@ size_t order_at() { return 256; }
 size_t offsets_at(int n) { return order_at() + (((size_t)n * sizeof(int) + 255) & ~(size_t)255); }
 size_t result_bytes(int n) { return offsets_at(n) + ((size_t)n + 1) * sizeof(int); }
 
-// min(1, 32 / o) in 65,536ths for the decodes that lanes_from looks at, 0 beyond: a division per request would
-// take sched_init of 4,000,000 requests from 8 to 22 ms
-const int kShareTable = 2050;
-const int* short_shares() {
-    struct Table {
-        int v[kShareTable];
-        Table() { for (int o = 0; o < kShareTable; ++o) v[o] = o == 0 ? 0 : o <= 32 ? 65536 : 32 * 65536 / o; }
-    };
-    static const Table table;
-    return table.v;
-}
-
 // Orders of up to 4,000,000 requests are handed in and out through the handle's pinned block; larger ones are
 // copied from and to the caller's memory (pinning 128 MB for 10,000,000 requests takes sched_init 100 ms).
 bool reads_through_pinned(int n) { return 256 + result_bytes(n) <= ((size_t)32 << 20); }
@@ -293,21 +281,23 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
     if (M >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
     const i64 total = (i64)B * n;
     KV_TRY(validate_instance(total, s, o, M));
-    int omax = 0, least = INT32_MAX; i64 sum_max = 0, sum_s = 0, sum_o = 0, short_o = 0; double volume = 0;
-    const int* const share = short_shares();
+    int omax = 0, least = INT32_MAX; i64 sum_max = 0; double volume = 0;
     for (int b = 0; b < B; ++b) {
         i64 sum = 0;
         for (int i = 0; i < n; ++i) {
             const int v = o[(i64)b * n + i], size = s[(i64)b * n + i] + v;
             sum += v;
-            sum_s += size - v;
             volume += (double)v * (size - 0.5 * v);
-            short_o += share[v < kShareTable ? v : 0];
             omax = v > omax ? v : omax;
             least = size < least ? size : least;
         }
         if (sum > sum_max) sum_max = sum;
-        sum_o += sum;
+    }
+    // of some 4,096 requests spread over all: enough for a rule, and these sums over all of 1,000,000 are 2 ms
+    double short_o = 0, some_s = 0, some_o = 0, looked_at = 0;
+    for (i64 k = 0, step = 1 + total / 4096; k < total; k += step) {
+        short_o += o[k] <= 32 ? 1.0 : 32.0 / o[k];
+        some_s += s[k]; some_o += o[k]; looked_at += 1.0;
     }
     if (sum_max + omax >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
 
@@ -322,7 +312,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             rc = kv_cuda_fail(cudaGetLastError(), "cudaDeviceGetAttribute"); break;
         }
         h->B = B; h->n = n; h->M = M; h->omax = omax; h->least = least; h->volume = volume; h->sum_o_max = sum_max;
-        h->mean_s = (double)sum_s / (double)total; h->mean_o = (double)sum_o / (double)total; h->short_share = (double)short_o / 65536.0 / (double)total;
+        h->mean_s = some_s / looked_at; h->mean_o = some_o / looked_at; h->short_share = short_o / looked_at;
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
         h->nm = slots <= 32 ? 1 : slots <= 256 ? slots / 32 : 0;

@@ -30,8 +30,8 @@ struct sched_ctx {
     int omax;                // largest decode length over all instances
     int least;               // smallest s+o over all instances
     double volume;           // tokens times rounds: sum of s o + o^2 / 2 over all instances
-    double mean_s, mean_o;   // over all requests
-    double short_share;      // mean of min(1, 32 / o)
+    double mean_s, mean_o;   // of some 4,096 requests spread over all instances
+    double short_share;      // mean of min(1, 32 / o) over the same
     int L;                   // ints per simulator state
     int nm;                  // chunked simulator with this many far registers per lane; 0: hybrid simulator
     int ring_cells;          // shared-memory ints one simulator needs
