@@ -25,6 +25,12 @@
  *     scratch, outgrown staging buffers) are kept in a process-wide per-device cache -- at most
  *     KVSCHED_POOL_MB MiB in total (environment variable, default 1024, 0 disables the cache) -- and
  *     reused by later calls; sched_release_cached_memory() returns them to the driver.
+ *   - A large sweep (sched_sweep_dev, sched_local_search, MOVE candidates; more than some 18,000 moves on
+ *     decodes up to 2,049 rounds, more than some 4,000 on decodes up to 4,097) keeps simulator state in
+ *     device memory: 4.3 KB per move side by side for decodes up to 1,025 rounds, 8.5 KB up to 2,049 (twice
+ *     that where M * M over the smallest s+o passes some 2^31), 16 KB beyond; 412, 495 (824, 989) and 512 MB
+ *     at most.  It is allocated by the first such sweep of a handle and kept until sched_destroy(); where
+ *     there is no memory for it the sweep runs without.
  *   - A handle is tied to the CUDA device that was current in sched_init(); calls on one handle
  *     must not overlap in time.
  *   - Arrays are dense, row-major, int32 unless stated; TELs are int64.
@@ -191,7 +197,7 @@ int sched_sorted_f_local_swap_dev(sched_handle h, int32_t* order_out, int32_t* b
  * element at 0-based position floor(3 (size-1) / 10) of the ascending values.  Ratios are compared
  * exactly; equal ratios keep the walking order.
  * SCHED_E_UNSUPPORTED when 2*bits(M) + bits(max o) > 63 (the exact ratio key would not fit 64 bits).
- * Host pointers; synchronises once per batch; outputs and side effects as sched_sorted_f(). */
+ * Host pointers; outputs and side effects as sched_sorted_f(). */
 int sched_sorted_f_quantile(sched_handle h, uint64_t seed, int32_t* order_out, int32_t* batch_offsets_out,
                             int32_t* num_batches_out, int64_t* tel_out);
 
@@ -311,8 +317,8 @@ int sched_online_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const
  * All pointers are host memory; the call allocates and frees its own device buffers and synchronises
  * the device.  SCHED_E_INVAL: bad sizes, s < 1, lower < 1, lower > o, s + o > M;
  * SCHED_E_NOT_PERMUTATION: a row of order is not a permutation; SCHED_E_UNSUPPORTED: n_max > 4096,
- * o > 8192, M >= 2^30, or rows too large for the shared memory of one CTA (20 n_max + 16 L bytes,
- * L = the power of two >= max o + 2); SCHED_E_INTERNAL: a scenario did not finish within
+ * o > 8192, M >= 2^30, or rows too large for the shared memory of one CTA (20 n_max + 12 L + 128 R bytes,
+ * L = the power of two >= max o + 2, R = the one >= (max o + 30) / 32); SCHED_E_INTERNAL: a scenario did not finish within
  * 16 + (n+1) sum(o) rounds (capped at 2^30). */
 int sched_amin_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const int32_t* s, const int32_t* lower,
                         const int32_t* o, int64_t M, const int32_t* order, int32_t* start_out, int64_t* tel_out,

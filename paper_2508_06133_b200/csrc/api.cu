@@ -1,5 +1,5 @@
 // Host side of the kvsched C-ABI (see include/kvsched.h for the contract of every entry point).
-// All scheduling arithmetic runs in the kernels of k1_sort / k2_fmetric / k3_eval / k5_argmin; this
+// All scheduling arithmetic runs in the kernels of k1_* .. k7_*; this
 // file validates arguments, owns device memory and enqueues launches.  There is no CPU fallback.
 #include <math.h>
 #include <stdio.h>

@@ -31,7 +31,9 @@
 // 64,000 moves of 10,000 requests, budget 262,144: 33.0 ms with a warp per candidate; 23.6 with one load of a
 // lane's own line at a time, 18.6 with four of them, 16.0 with these side by side and the walk in two levels, 14.7 with
 // eight.  256,000 moves of 1,000 requests, budget 65,536: 18.9 -> 8.8 ms.  4,194,304 moves of the 10,000: 2,741 ->
-// 569 ms.  lanes_fit (api.cu) has the rule and the other side.
+// 569 ms.  These are kernels alone on the chip; 65,536 threads fill 0.7 of it, so sweeps of several handles overlap (9.4
+// ms each).  A handle's first sweep also allocates the rings: 16.5 ms where the next is 14.8, more when the driver
+// takes longer for it (28 ms once in nine).  lanes_from (api.cu) has the rule and the other side.
 #pragma once
 
 #include "common.cuh"

@@ -5,8 +5,8 @@
 // is never materialised as a permutation: the simulator maps positions through kv_map_pos().  What
 // this file adds is the order in which candidates are handed to warps: a candidate only has to be
 // simulated from its first moved position, so its cost is the length of the list suffix behind that
-// position.  The 32 warps of a CTA run one candidate each and the CTA lasts as long as its longest
-// one; candidates are therefore bucketed by first moved position (counting sort: histogram, scan,
+// position.  The warps of a CTA (1 to 24 by simulator) run one candidate each and the CTA lasts as long as
+// its longest one, and the 32 lanes of k3_lane_moves go through time together; candidates are therefore bucketed by first moved position (counting sort: histogram, scan,
 // scatter) so that neighbours in launch order have (almost) equal suffix lengths and the longest
 // candidates are launched first.  The order inside a bucket is arbitrary; results are written per
 // candidate index, so they do not depend on it.

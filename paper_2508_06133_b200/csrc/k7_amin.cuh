@@ -36,8 +36,9 @@
 //   has ever started.
 // What bounds it: a scenario is a chain (2,000 requests of the paper's lengths: 2,400 admissions, 380
 // evictions among 550 running, 1,300 walks: 1,000,000 instructions of one warp at 5 cycles each), so the
-// number of instructions; one warp needs no block barriers for them.  64 scenarios 2.34 ms; 2.44 with 256
-// threads that test every round of a window and look at everything that has ever started.
+// number of instructions.  1 / 64 / 592 scenarios: 2.28 / 2.43 / 4.63 ms, with 256 threads per scenario that test every
+// round of a window and look at everything that has ever started 2.37 / 2.50 / 5.25.  The call around it takes
+// 2.40 / 2.93 / 8.09 ms, with a device block per array 3.44 / 4.58 / 11.3.
 #pragma once
 
 #include "common.cuh"
