@@ -16,9 +16,8 @@ typedef unsigned long long u64;
 // Device-side status word (ctx->d_status[0]); non-zero means a bounded loop gave up.
 enum { KV_DEV_OK = 0, KV_DEV_LOOP_CAP = 1 };
 
-struct SnapHeader {          // simulator state in front of one list position (16 bytes)
+struct SnapHeader {          // simulator state in front of one list position
     int t;                   // current round index (number of completed rounds = next start time)
-    int hz;                  // first round after which the timeline is all zero
     int tel_lo, tel_hi;      // TEL of the positions before this one
 };
 

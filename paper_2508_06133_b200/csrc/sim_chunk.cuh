@@ -128,7 +128,7 @@ struct ChunkSim {
             snap[32 + 96 * m + lane] = A[m]; snap[64 + 96 * m + lane] = C[m]; snap[96 + 96 * m + lane] = U[m];
         }
         if (lane == 0) {
-            SnapHeader h; h.t = T0 + tau; h.hz = 0;
+            SnapHeader h; h.t = T0 + tau;
             h.tel_lo = (int)(tel_before & 0xffffffffll); h.tel_hi = (int)(tel_before >> 32);
             *hdr = h;
         }

@@ -179,7 +179,7 @@ struct HybSim {
         for (int c = 0; c < NREG; ++c) snap[KV_IDX(32 * c + lane, span, 204)] = R[c];
         for (int k = 0; k < FC; ++k) snap[KV_IDX(32 * (NREG + k) + lane, span, 205)] = far[32 * slot_of(k)];
         if (lane == 0) {
-            SnapHeader h; h.t = t; h.hz = 0;
+            SnapHeader h; h.t = t;
             h.tel_lo = (int)(tel & 0xffffffffll); h.tel_hi = (int)(tel >> 32);
             *hdr = h;
         }
