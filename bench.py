@@ -17,9 +17,9 @@ agree on the best (TEL, index) pair with two all-reduce(min) of one int64 over N
 applies that move to its base order.  Time is the max over ranks.
 
 The roofline denominators are measured inside this run by the library's probe kernels
-(`sched_probe_peaks`): `roofline.frac` is read against the measured rate of the integer ALU pipe (the
-pipe every maximum, compare and select of the simulator has to go through); `roofline.frac_vs` gives
-the same achieved figure against the other measured rates -- plain adds, which the compiler spreads
+(`sched_probe_peaks`): `roofline.frac` is the least integer work of a launch read against the measured
+rate of the integer ALU pipe (the pipe every maximum, compare and select of the simulator has to go
+through); `roofline.frac_vs` gives the same achieved figure against the other measured rates -- plain adds, which the compiler spreads
 over two pipes, multiply-adds, a two-pipe mix -- and the instruction-issue limit.
 """
 from __future__ import annotations
@@ -44,10 +44,10 @@ SM_COUNT = 148
 INT_OPS_PER_CLK_PER_SM = 64              # fallback only: 32-bit integer adds per clock and SM when the probe cannot run
 ISSUE_LANES_PER_CLK_PER_SM = 128         # 4 schedulers x 1 warp instruction (32 lanes) per clock
 FALLBACK_HBM_GBS, FALLBACK_SM_MHZ = 6650.0, 1965.0
-OPS_PER_CELL, BYTES_PER_CELL = 4.0, 8.0  # algorithmic cost of one timeline cell: 4 integer operations, 4 B read + 4 B written
+OPS_PER_CELL = 4.0                       # integer operations of a plain timeline per cell
 # dram__bytes_read.sum + dram__bytes_write.sum of one simulator launch, from a one-pass ncu capture of
 # this very launch (summary under profiles/); keyed by (workload, moves per launch) with a digest of
-# the simulator's source files, so that it turns into null when the kernel changes
+# the code lines of the simulator's source files, so that it turns into null when the kernel changes
 K3_TRAFFIC = {("mixed_n10000", 1 << 22): (61.21e6 + 10.59e6, "1e184f7ce88dd053")}
 OPS_PER_ADMISSION = 10.0                 # request read and mapped, one compare per bound, two sums and one cell updated
 DEFAULT_MOVES = {"mixed_10k": 1 << 22, "mixed_1k": 499500, "paper_scale": 1 << 21, "heavy_100k": 1 << 18}
@@ -58,8 +58,8 @@ def simulator_digest() -> str:
     import hashlib
     hsh = hashlib.sha256()
     for name in ("sim_chunk.cuh", "sim_hyb.cuh", "k3_eval.cuh", "k3_lanes.cuh", "k4_moves.cuh", "common.cuh"):
-        with open(os.path.join(ROOT, "paper_2508_06133_b200", "csrc", name), "rb") as f:
-            hsh.update(f.read())
+        with open(os.path.join(ROOT, "paper_2508_06133_b200", "csrc", name)) as f:
+            hsh.update("".join(line.split("//")[0].strip() for line in f).encode())
     return hsh.hexdigest()[:16]
 
 
@@ -208,37 +208,31 @@ def probe_rooflines(kv, stream, sm_mhz):
     return p, source
 
 
-def roofline_block(cells_per_launch, kern_s, probe, probe_source, sm_mhz_load, hbm_gbs, hbm_bytes, traffic, kernel, extra_ops=0.0):
-    """`achieved` = algorithmic integer operations per launch / measured launch time, against the
-    measured integer-add rate; the other measured rates and the issue limit beside it."""
-    ops = OPS_PER_CELL * cells_per_launch + extra_ops
+def roofline_block(ops, ops_note, cells_per_launch, kern_s, probe, probe_source, sm_mhz_load, hbm_gbs, traffic, kernel):
+    """`achieved` = the integer operations that a launch cannot do without / measured launch time, against
+    the measured integer ALU rate; the other measured rates and the issue limit beside it."""
     ach = ops / kern_s                                           # integer operations per second
-    # the pipe that bounds the simulator: maxima, compares, selects and masks execute only on the
-    # integer ALU pipe (measured by the max/xor probe); plain adds alone can also use the
-    # multiply-add pipe, which is what the int_add probe shows -- both fractions are reported
+    # maxima, compares, selects and masks execute only on the integer ALU pipe (measured by the max/xor
+    # probe); plain adds alone can also use the multiply-add pipe, which is what the int_add probe shows
     peak_key = "int_alu" if probe.get("int_alu", 0) > 0 else "int_add"
     peak = probe[peak_key]
     frac_vs = {k: ach / v for k, v in probe.items() if k.startswith(("int_", "sim_")) and v > 0}
     issue_peak = SM_COUNT * ISSUE_LANES_PER_CLK_PER_SM * sm_mhz_load * 1e6
     frac_vs["issue_slots"] = ach / issue_peak
-    rl = {"bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "Tint-op/s", "frac": ach / peak,
-          "traffic": traffic, "kernel": kernel, "kernel_ms": kern_s * 1e3, "cells_per_launch": cells_per_launch,
-          "ops_per_cell": OPS_PER_CELL,
-          "frac_note": "cells of the plain timeline, one update per token-round; the kernels keep far windows as lines or events and "
-                       "do not touch every cell, so the figure can pass 1",
-          "peak_source": probe_source + (" int_alu: measured rate of the integer ALU pipe (max/xor chains, lane-ops/s); frac_vs.int_add is the same "
-                                         "achieved figure against plain adds, which the compiler spreads over the ALU and the multiply-add pipe"
-                                         if peak_key == "int_alu" else " int_add (lane-ops/s)"),
-          "frac_vs": frac_vs,
-          "probe_lane_ops_per_clk_per_sm": {k: v / (SM_COUNT * sm_mhz_load * 1e6) for k, v in probe.items()},
-          "issue_peak_note": "derived: %d SMs x %d lanes/clk x %.0f MHz sampled under load" % (SM_COUNT, ISSUE_LANES_PER_CLK_PER_SM, sm_mhz_load),
-          "hbm_bytes_per_launch": hbm_bytes, "hbm_frac": hbm_bytes / kern_s / 1e9 / hbm_gbs}
-    if "smem_load" in probe and probe["smem_load"] > 0:
-        smem_ach = BYTES_PER_CELL * cells_per_launch / kern_s
-        smem_peak = 0.5 * (probe["smem_load"] + probe.get("smem_store", probe["smem_load"]))
-        rl["smem"] = {"bound": "smem", "achieved": smem_ach / 1e9, "peak": smem_peak / 1e9, "unit": "GB/s",
-                      "frac": smem_ach / smem_peak, "note": "4 B read + 4 B written per cell against the mean of the measured 16-byte load and store rates"}
-    return rl
+    plain = OPS_PER_CELL * cells_per_launch
+    return {"bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "Tint-op/s", "frac": ach / peak,
+            "traffic": traffic, "kernel": kernel, "kernel_ms": kern_s * 1e3, "ops_per_launch": ops, "frac_note": ops_note,
+            "peak_source": probe_source + (" int_alu: measured rate of the integer ALU pipe (max/xor chains, lane-ops/s); frac_vs.int_add is the same "
+                                           "achieved figure against plain adds, which the compiler spreads over the ALU and the multiply-add pipe"
+                                           if peak_key == "int_alu" else " int_add (lane-ops/s)"),
+            "frac_vs": frac_vs,
+            "probe_lane_ops_per_clk_per_sm": {k: v / (SM_COUNT * sm_mhz_load * 1e6) for k, v in probe.items()},
+            "issue_peak_note": "derived: %d SMs x %d lanes/clk x %.0f MHz sampled under load" % (SM_COUNT, ISSUE_LANES_PER_CLK_PER_SM, sm_mhz_load),
+            "plain_timeline": {"cells_per_launch": cells_per_launch, "ops_per_cell": OPS_PER_CELL, "tera_ops_per_s": plain / kern_s / 1e12,
+                               "of_peak": plain / kern_s / peak,
+                               "note": "what a timeline that updates every cell (one per token-round) would have to do in this time; the kernels keep "
+                                       "far windows as lines or events and do not touch every cell, so this is no roofline fraction"},
+            "hbm_frac": traffic / kern_s / 1e9 / hbm_gbs if traffic else None}
 
 
 def cpu_baseline_legs(args, inst, base, ty, mi, mj, tel_check):
@@ -316,14 +310,15 @@ def bench_policy_sweep(args, rank, world, local_rank):
     kern_s = float(np.mean([r[1] for r in res])) * 1e-3
     pairs = B * 4
     value = pairs * args.steps / (sum(step_ms) * 1e-3)
-    cells = 4.0 * float(o.astype(np.int64).sum())                   # every pair simulates its whole list
+    cells = 4.0 * float(o.astype(np.int64).sum())                   # of a plain timeline: every pair simulates its whole list
     # order construction: stable radix passes in shared memory (2 for shortest-decode-first, 2 for total-size-first,
     # 5 for Sorted-F at these sizes), each a count and a scatter visit of n ids, ~3 integer operations per visit
     sort_ops = 6.0 * B * 9 * n
     sm_load = clocks["sm_mhz"] or sm_max
-    roofline = roofline_block(cells, kern_s, probe, probe_source, sm_load, hbm_gbs, 8.0 * B * n + 8.0 * pairs, None,
-                              "k3_eval_policy", extra_ops=sort_ops)
-    roofline["extra_ops_note"] = "order construction: 9 radix passes per instance x 2 visits x n ids x 3 integer operations"
+    roofline = roofline_block(OPS_PER_ADMISSION * pairs * n + sort_ops,
+                              "%g operations per request and pair (request, one window test, one update) and the order construction: 9 radix "
+                              "passes per instance x 2 visits x n ids x 3 integer operations" % OPS_PER_ADMISSION,
+                              cells, kern_s, probe, probe_source, sm_load, hbm_gbs, None, "k3_eval_policy")
     import oracle as orc
     got = tel.cpu().numpy().reshape(B, 4)
     cores = host_cores()
@@ -464,21 +459,21 @@ def main():
         admissions.append(int((n - np.minimum(mi, mj)).sum()))
     cells_per_launch = float(np.mean(cells))
     kern_s = float(np.mean(kern_ms)) * 1e-3
-    hbm_bytes = 8.0 * count + 4.0 * count + 12.0 * n          # TELs out, launch order in, request table and base starts
     traffic = None
     known = K3_TRAFFIC.get((inst.name, count))
     if known is not None and known[1] == simulator_digest():
         traffic = known[0]
     sm_load = clocks["sm_mhz"] or sm_max
-    roofline = roofline_block(cells_per_launch, kern_s, probe, probe_source, sm_load, hbm_gbs, hbm_bytes, traffic, "k3_lane_moves / k3_eval_moves (the library's rule picks)")
     # what the kernels do per candidate is an admission per request, whatever its decode length
     adm = float(np.mean(admissions))
-    roofline["admissions"] = {"per_launch": adm, "per_s": adm / kern_s, "ops_per_admission": OPS_PER_ADMISSION,
-                              "of_peak": OPS_PER_ADMISSION * adm / kern_s / (roofline["peak"] * 1e12),
-                              "note": "least integer work of an admission (request, one window test, one update) against the same peak"}
+    roofline = roofline_block(OPS_PER_ADMISSION * adm,
+                              "%g operations (request, one window test, one update) per request from the first moved one on" % OPS_PER_ADMISSION,
+                              cells_per_launch, kern_s, probe, probe_source, sm_load, hbm_gbs, traffic,
+                              "k3_lane_moves / k3_eval_moves (the library's rule picks)")
+    roofline["admissions"] = {"per_launch": adm, "per_s": adm / kern_s, "ops_per_admission": OPS_PER_ADMISSION}
     # the survey's model-level figure: every evaluation counted as 4 * sum(o) operations, i.e. including the
     # list prefix that the snapshots of the base run make unnecessary -- a statement about the method, not
-    # about how busy the SM is (that is `frac`, which counts only the cells actually re-simulated)
+    # about how busy the SM is
     roofline["model_level"] = {"ops_per_eval": OPS_PER_CELL * sum_o, "tera_ops_per_s": OPS_PER_CELL * sum_o * count / kern_s / 1e12,
                                "of_peak": OPS_PER_CELL * sum_o * count / kern_s / (roofline["peak"] * 1e12),
                                "note": "evals/s x 4 x sum(o) / peak; counts the prefix that snapshot reuse skips (cells re-simulated are %.0f %% of it)"
