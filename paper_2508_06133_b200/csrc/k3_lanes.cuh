@@ -1,7 +1,7 @@
 // K3, many candidates: one THREAD per candidate move.  Same rule, same results as k3_eval_moves
 // (sim_chunk.cuh has the rule; V[x] is the tokens in use in round x, plus x).
 //
-// k3_eval_moves gives a warp to a candidate; nearly all of its 77 instructions per admission are the same
+// k3_eval_moves gives a warp to a candidate; nearly all of its 80 instructions per admission are the same
 // in every lane.  Here the 32 candidates of a warp are neighbours in the launch order (first moved
 // positions next to each other), so they start from the same state of the base run and meet about the
 // same requests in about the same rounds: they are moved through time together, chunk by chunk of CH
@@ -23,9 +23,10 @@
 // so a turn nearly always ends with an admission in every lane (1.25 turns per admission).  W1 is
 // answered from the next chunk's cells, U (2 of 1,000 turns) from the events.
 //
-// What bounds it: latency.  20 warps per SM (the cells of two chunks fill shared memory) execute about 500
-// instructions per turn of 32 candidates where the kernel with a warp per candidate executes 32 x 77, but the
-// event rings of all resident candidates are 412 MB and do not stay in L2 (126 MB).  So a chunk's words are
+// What bounds it: instructions at 20 warps per SM (registers and the cells of two chunks allow no more): 1,250 for 32
+// candidates' admissions at 12 rounds per request where the kernel with a warp per candidate executes 32 x 80, two thirds of
+// the issue slots and of the integer pipe; below a full chip, latency.  The event rings of all resident candidates are
+// 412 MB and do not stay in L2 (126 MB): a third of the memory's rate, and half of all warp cycles in the first form.  So a chunk's words are
 // read with eight 16-byte loads in flight, laid out so that a warp's load is 512 contiguous bytes, called to L2 one
 // chunk ahead, and cleared only where they are not zero; the request behind the next is on its way a turn early.
 // 64,000 moves of 10,000 requests, budget 262,144: 33.0 ms with a warp per candidate; 23.6 with one load of a

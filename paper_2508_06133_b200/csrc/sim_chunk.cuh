@@ -26,7 +26,7 @@
 // a half instructions per 32 cells and admission), k3_eval_moves: 10,000 requests (decodes to 1,024),
 // 65,536 moves 43.3 -> 33.0 ms; 100,000 requests (decodes to 4,096), 7,000 moves 108.8 -> 50.7 ms (40.7 with kGlobal), where
 // the far part of the timeline was read and written in shared memory; one run of the 100,000 from the
-// empty state (sorted_f) 71.6 -> 15.6 ms.  Bound by the issue rate: 77 instructions per admission.
+// empty state (sorted_f) 71.6 -> 15.6 ms.  Bound by the issue rate: 80 instructions per admission, 0.87 of the slots.
 // When t enters the next chunk its cells are put together from own, A and C, and the lanes' far
 // values move down by one.
 //
