@@ -1524,7 +1524,7 @@ static int amin_run(int32_t B, int32_t n_max, const int32_t* n_each, const int32
         P.start_out = d_start; P.tel_out = d_res; P.evict_out = d_res + B; P.peak_out = d_res + 2 * (size_t)B;
         P.status = d_status;
         if (e0) AM_CUDA(cudaEventRecord(e0, 0));
-        kernel<<<B, K7_THREADS, smem, 0>>>(P);
+        kernel<<<B, 32 * K7_WARPS, smem, 0>>>(P);
         AM_CUDA(cudaGetLastError());
         if (e1) AM_CUDA(cudaEventRecord(e1, 0));
         std::vector<i64> res(3 * (size_t)B + 1);

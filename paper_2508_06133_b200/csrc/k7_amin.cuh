@@ -1,7 +1,7 @@
 // K7 -- Sorted-F + A_min, Phase 2 (Section 5.5 "Handling Prediction Uncertainty via Adaptive Output
 // Length Refinement"; Algorithm 5, the supplement to Section 5): the executor when only a lower bound l_i <= o_i of
 // every decode length is known.  Many independent scenarios (a backlog, its list and one vector of
-// lower bounds each), one warp per scenario.
+// lower bounds each), one CTA per scenario.
 //
 // Every request carries a running estimate e_i (initially l_i).  Iteration t = 1, 2, ...:
 //   1. requests that have run their o_i rounds leave; every other running request is about to run
@@ -21,7 +21,7 @@
 //   true length o is OVERDUE in rounds p+e+1 .. p+o: there its estimate is t - p, i.e. step 1 extends
 //   its projection by exactly the current round.  The overdue requests are kept as two aggregates,
 //   cnt = how many and A = sum of (s_j - p_j), so step 1 adds A + cnt * t to round t; a request joins the
-//   aggregates at p+e+1 and leaves them at p+o+1 through per-round event cells (dc, dA) written when
+//   aggregates at p+e+1 and leaves them at p+o+1 through per-round event cells (ev, dA) written when
 //   it is admitted (and taken back if it is evicted).  A is kept modulo 2^32: the sum A + cnt * t is
 //   a memory amount and fits, its two terms need not.  The estimate of a running request is never
 //   stored: it is max(e at admission, t - p).
@@ -33,20 +33,21 @@
 //   head still bound to wait, or not even its first round fits) are walked up to 32 at a time, one lane
 //   each (the running aggregates of a round are prefix sums of the event cells).
 //   The running requests are a compact list, so an eviction looks at them and not at everything that
-//   has ever started.
-// What bounds it: a scenario is a chain (2,000 requests of the paper's lengths: 2,400 admissions, 380
-// evictions among 550 running, 1,300 walks: 1,000,000 instructions of one warp at 5 cycles each), so the
-// number of instructions.  1 / 64 / 592 scenarios: 2.28 / 2.43 / 4.63 ms, with 256 threads per scenario that test every
-// round of a window and look at everything that has ever started 2.37 / 2.50 / 5.25.  The call around it takes
-// 2.40 / 2.93 / 8.09 ms, with a device block per array 3.44 / 4.58 / 11.3.
+//   has ever started; all warps of the CTA do.
+// What bounds it: a scenario is a chain (2,000 requests of the paper's lengths: 2,400 admissions, 440
+// evictions among 620 running, 1,450 walks), so the latency of each of these: about 350 cycles an admission, 750 a walk of up
+// to 32 rounds, and an eviction 4,050 with one warp looking through the list, 1,100 with four.  The events of a round's
+// admissions are put together, a lane each (they were 300 of 890 cycles per admission).  Kernel with 1 / 64 / 592
+// scenarios 2.38 / 2.45 / 4.83 -> 1.61 / 1.65 / 3.31 ms, the call around it 2.51 / 2.97 / 9.03 -> 1.74 / 2.14 / 6.50.
 #pragma once
 
 #include "common.cuh"
 #include "sim_chunk.cuh"
 
-#define K7_THREADS 32
+#define K7_WARPS 4               // one runs the scenario, all of them look for the request to evict
 #define K7_MAX_N 4096
 #define K7_MAX_O 8192
+#define K7_ID_BITS 12            // (estimate << 12) | id fits 32 bits
 
 struct AminParams {
     int n_max;
@@ -67,13 +68,36 @@ struct AminParams {
 };
 
 __host__ __device__ inline size_t k7_smem_bytes(int ring_cells, int n_max, int L) {
-    return ((size_t)ring_cells + 4 * (size_t)n_max + 3 * (size_t)L) * sizeof(int) + 2 * (size_t)n_max * sizeof(unsigned short) + 16;
+    return ((size_t)ring_cells + 4 * (size_t)n_max + 2 * (size_t)L) * sizeof(int) + 2 * (size_t)n_max * sizeof(unsigned short) + 16;
+}
+
+// Smallest (estimate, request id) of the running ones that this warp looks at, and its place in the list: to sh.
+struct K7Scan {
+    int t, nrun;                                                  // nrun < 0: the scenario is over
+    unsigned key[K7_WARPS];
+    int at[K7_WARPS];
+};
+__device__ __forceinline__ void k7_scan(K7Scan& sh, const unsigned short* run, const int* pp, const int* po, const int* pe,
+                                        const unsigned short* pid) {
+    const int warp = threadIdx.x >> 5, nrun = sh.nrun, t = sh.t;
+    unsigned best = ~0u;
+    int at = 0;
+#pragma unroll 2
+    for (int k = threadIdx.x; k < nrun; k += 32 * K7_WARPS) {
+        const int r = run[k], p = pp[r];
+        const unsigned key = t <= p + po[r] ? ((unsigned)max(pe[r], t - p) << K7_ID_BITS) | pid[r] : ~0u;
+        if (key < best) { best = key; at = k; }
+    }
+    const unsigned least = __reduce_min_sync(KV_FULL, best);
+    if (best == least && least != ~0u) { sh.key[warp] = least; sh.at[warp] = at; }      // one lane: ids differ
+    else if (least == ~0u) sh.key[warp] = ~0u;
 }
 
 template <class SIM>
-__global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
+__global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
     extern __shared__ __align__(16) unsigned char k7_smem[];
-    const int lane = threadIdx.x;
+    __shared__ K7Scan scan;
+    const int lane = threadIdx.x & 31;
     const int b = blockIdx.x;
     const int n = P.n_each[b];
     const int nm = P.n_max;
@@ -83,32 +107,38 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
     int* po = ps + nm;
     int* pe = po + nm;
     int* pp = pe + nm;
-    int* dc = pp + nm;                                            // change of cnt at the start of a round
-    unsigned* dA = reinterpret_cast<unsigned*>(dc + P.L);         // change of A
-    int* fin = reinterpret_cast<int*>(dA + P.L);                  // requests that leave at the start of a round
-    unsigned short* pid = reinterpret_cast<unsigned short*>(fin + P.L);
+    int* ev = pp + nm;                                            // at the start of a round: 2^16 times the change of cnt, plus the requests that leave
+    unsigned* dA = reinterpret_cast<unsigned*>(ev + P.L);         // change of A
+    unsigned short* pid = reinterpret_cast<unsigned short*>(dA + P.L);
     unsigned short* run = pid + nm;                               // positions that run (and some that have finished)
 
     const size_t base = (size_t)b * nm;
     const int* ord = P.order + (size_t)b * P.order_stride;
-    i64 sum_o = 0;
     {
         bool bad = false;
-        for (int q = lane; q < n; q += 32) {
+        for (int q = threadIdx.x; q < n; q += 32 * K7_WARPS) {
             const int id = ord[q];
             if (id < 0 || id >= n) { bad = true; continue; }      // never read outside the row
             ps[q] = P.s[base + id]; po[q] = P.o[base + id]; pe[q] = P.lower[base + id];
             pp[q] = -1; pid[q] = (unsigned short)id;
-            sum_o += po[q];
         }
-        for (int k = lane; k < P.L; k += 32) { dc[k] = 0; dA[k] = 0u; fin[k] = 0; }
-        if (__any_sync(KV_FULL, bad)) {
-            if (lane == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
+        for (int k = threadIdx.x; k < P.L; k += 32 * K7_WARPS) { ev[k] = 0; dA[k] = 0u; }
+        if (__syncthreads_or(bad)) {
+            if (threadIdx.x == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
             return;
         }
-        for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
-        __syncwarp();
     }
+    if (threadIdx.x >= 32) {                                      // called at every eviction, and at the end
+        for (;;) {
+            __syncthreads();
+            if (scan.nrun < 0) return;
+            k7_scan(scan, run, pp, po, pe, pid);
+            __syncthreads();
+        }
+    }
+    i64 sum_o = 0;
+    for (int q = lane; q < n; q += 32) sum_o += po[q];
+    for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
     i64 round_cap = 16 + sum_o * (i64)(n + 1);
     if (round_cap > (1ll << 30)) round_cap = 1ll << 30;           // t stays a 32-bit round index
 
@@ -126,7 +156,7 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
 
     for (i64 turn = 0;; ++turn) {
         if (turn > round_cap) { failed = true; break; }
-        // rounds in which nothing can be decided (step 1 only): the lanes whose round of chunk 0 is still
+        // rounds in which nothing can be decided (step 1 only): the lanes whose round of the chunk is still
         // to come take one each.  A round reads only its own cell and the running (cnt, A, remaining),
         // which are prefix sums of the event cells; the walk stops at the first round that needs a
         // decision (or ends the run).
@@ -134,29 +164,28 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
         for (;;) {
             const bool live = sim.rl >= 0;
             const int round = sim.T0 + lane, k = round & mask;
-            int cs = live ? dc[k] : 0;
+            int es = live ? ev[k] : 0;
             unsigned as = live ? dA[k] : 0u;
-            int fs = live ? fin[k] : 0;
-            if (__any_sync(KV_FULL, cs != 0 || as != 0u || fs != 0)) {
+            if (__any_sync(KV_FULL, es != 0 || as != 0u)) {
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
-                    const int c2 = __shfl_up_sync(KV_FULL, cs, d);
+                    const int e2 = __shfl_up_sync(KV_FULL, es, d);
                     const unsigned a2 = __shfl_up_sync(KV_FULL, as, d);
-                    const int f2 = __shfl_up_sync(KV_FULL, fs, d);
-                    if (lane >= d) { cs += c2; as += a2; fs += f2; }
+                    if (lane >= d) { es += e2; as += a2; }
                 }
             }
-            const unsigned cnt_l = cnt + (unsigned)cs, A_l = A + as;
-            const int rem_l = remaining - fs;
+            const unsigned cnt_l = cnt + (unsigned)(es >> 16), A_l = A + as;
+            const int rem_l = remaining - (es & 0xffff);
             const int u = sim.cur - lane + (int)(A_l + cnt_l * (unsigned)round);
             const bool end = live && rem_l == 0;
             // the head's first round is the current one: if it does not fit there, the window test cannot
             // succeed in this iteration
             const bool work = live && (u > M || (head < n && round >= t_ok && u + head_s + 1 <= M));
             const bool cap = (i64)round >= round_cap;
-            const unsigned stops = __ballot_sync(KV_FULL, end || work || (live && cap));
+            const unsigned ends = __ballot_sync(KV_FULL, end), works = __ballot_sync(KV_FULL, work);
+            const unsigned stops = ends | works | __ballot_sync(KV_FULL, live && cap);
             const int first = stops ? __ffs(stops) - 1 : 32;
-            if (live && lane <= first) { dc[k] = 0; dA[k] = 0u; fin[k] = 0; }            // events consumed
+            if (live && lane <= first) { ev[k] = 0; dA[k] = 0u; }                        // events consumed
             const int run_max = kv_warp_max(live && lane < first ? u : 0);
             peak = max(peak, run_max);
             const int src = first < 32 ? first : 31;
@@ -164,10 +193,10 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
             A = __shfl_sync(KV_FULL, A_l, src);
             remaining = __shfl_sync(KV_FULL, rem_l, src);
             if (first < 32) {
-                if (lane == first) sim.cur = u + lane;                                  // step 1 of the round that is decided
-                sim.advance(__shfl_sync(KV_FULL, sim.rl, first), 0);
-                if (__shfl_sync(KV_FULL, (int)end, first)) done = true;
-                else if (!__shfl_sync(KV_FULL, (int)work, first)) failed = true;
+                if (lane == first) sim.cur = u + lane;                              // step 1 of the round that is decided
+                sim.advance(first - sim.tau, 0);
+                if ((ends >> first) & 1u) done = true;
+                else if (!((works >> first) & 1u)) failed = true;
                 break;
             }
             sim.advance(32 - sim.tau, 0);
@@ -177,23 +206,15 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
 
         // ---- step 2: admissions of iteration t
         if (head < n && t >= t_ok) {
+            const int had = nrun;
+            int s = ps[head], e = pe[head];
             for (;;) {
-                const int q = head;
-                const int s = ps[q], o = po[q], e = pe[q];
+                const int q = head, q1 = q + 1 < n ? q + 1 : q, s1 = ps[q1], e1 = pe[q1];      // the next one, mostly
                 const int need = sim.test(s + 1, e - 1);
                 if (need > 0) { t_ok = t + need; break; }
                 sim.add(s + 1, e - 1);
-                // its events, one lane each: overdue in rounds t+e .. t+o-1 if the estimate is short, then over
-                {
-                    const unsigned v = (unsigned)(s - (t - 1));
-                    unsigned* cell = (lane < 4 ? (lane & 1 ? dA : (unsigned*)dc) : (unsigned*)fin) + ((lane < 2 ? t + e : t + o) & mask);
-                    const unsigned add = lane == 0 || lane == 4 ? 1u : lane == 1 ? v : lane == 2 ? ~0u : 0u - v;
-                    if (lane < 5) atomicAdd(cell, lane == 4 || e < o ? add : 0u);
-                    pp[q] = t - 1;
-                    run[KV_IDX(nrun, nm, 1102)] = (unsigned short)q;
-                }
+                run[KV_IDX(nrun, nm, 1102)] = (unsigned short)q;
                 ++nrun;
-                __syncwarp();
                 if (q == frontier) ++frontier; else --npe;
                 if (npe == 0) {
                     head = frontier;
@@ -207,7 +228,22 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
                     if (head == INT_MAX) { failed = true; break; }
                 }
                 if (head >= n) break;
+                s = s1; e = e1;
+                if (head != q1) { s = ps[head]; e = pe[head]; }
             }
+            __syncwarp();
+            // their events: overdue in rounds t+e .. t+o-1 if the estimate is short, then over
+            for (int k = had + lane; k < nrun; k += 32) {
+                const int q = run[k], o = po[q], est = pe[q];
+                const unsigned v = (unsigned)(ps[q] - (t - 1));
+                pp[q] = t - 1;
+                if (est < o) {
+                    atomicAdd(&ev[(t + est) & mask], 1 << 16); atomicAdd(&dA[(t + est) & mask], v);
+                    atomicAdd(&dA[(t + o) & mask], 0u - v);
+                }
+                atomicAdd(&ev[(t + o) & mask], est < o ? 1 - (1 << 16) : 1);
+            }
+            __syncwarp();
             if (failed) break;
         }
 
@@ -216,20 +252,14 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
             const int used = __shfl_sync(KV_FULL, sim.cur - lane, sim.tau);
             if (used <= M) { peak = max(peak, used); break; }
             // smallest (estimate, request id) among the running
-            int est_min = INT_MAX, id_min = INT_MAX, at_min = 0, live = 0;
-#pragma unroll 4
-            for (int k = lane; k < nrun; k += 32) {
-                const int r = run[k], p = pp[r];
-                const bool runs = t <= p + po[r];
-                const int est = runs ? max(pe[r], t - p) : INT_MAX, id = pid[r];
-                live += runs ? 1 : 0;
-                const bool less = est < est_min || (est == est_min && id < id_min);
-                est_min = less ? est : est_min; id_min = less ? id : id_min; at_min = less ? k : at_min;
-            }
-            const int est = kv_warp_min(est_min);
-            const int id = kv_warp_min(est_min == est ? id_min : INT_MAX);
-            if (est == INT_MAX) { failed = true; break; }
-            const int at = __shfl_sync(KV_FULL, at_min, __ffs(__ballot_sync(KV_FULL, est_min == est && id_min == id)) - 1);
+            if (lane == 0) { scan.t = t; scan.nrun = nrun; }
+            __syncthreads();
+            k7_scan(scan, run, pp, po, pe, pid);
+            __syncthreads();
+            const unsigned key = lane < K7_WARPS ? scan.key[lane] : ~0u, least = __reduce_min_sync(KV_FULL, key);
+            if (least == ~0u) { failed = true; break; }
+            const int est = (int)(least >> K7_ID_BITS);
+            const int at = scan.at[__ffs(__ballot_sync(KV_FULL, key == least)) - 1];
             const int q = run[KV_IDX(at, nm, 1103)];
             const int p = pp[q], s = ps[q], o = po[q], e0 = pe[q];
             sim.remove(s - (p - sim.T0), p + est - sim.T0);        // what is left of its projection
@@ -241,35 +271,38 @@ __global__ void __launch_bounds__(K7_THREADS) k7_amin(const AminParams P) {
             if (lane == 0) {
                 run[at] = run[nrun];
                 if (e0 < o) {
-                    if (!overdue) { dc[(p + e0 + 1) & mask] -= 1; dA[(p + e0 + 1) & mask] -= v; }
-                    dc[(p + o + 1) & mask] += 1; dA[(p + o + 1) & mask] += v;
+                    if (!overdue) { ev[(p + e0 + 1) & mask] -= 1 << 16; dA[(p + e0 + 1) & mask] -= v; }
+                    ev[(p + o + 1) & mask] += 1 << 16; dA[(p + o + 1) & mask] += v;
                 }
-                fin[(p + o + 1) & mask] -= 1;
+                ev[(p + o + 1) & mask] -= 1;
                 pe[q] = est;
                 pp[q] = -1;
             }
             __syncwarp();
-            if (2 * __reduce_add_sync(KV_FULL, live) < nrun) {     // drop what has finished
+            ++evictions; ++npe;
+            head = min(head, q);
+            t_ok = t + 1;
+            // as many as have started and neither left nor been evicted; drop what has finished
+            if (2 * (remaining - (n - frontier) - npe) < nrun) {
                 int kept = 0;
                 for (int k0 = 0; k0 < nrun; k0 += 32) {
                     const int k = k0 + lane, r = k < nrun ? run[k] : 0;
                     const bool keep = k < nrun && t <= pp[r] + po[r];
-                    const unsigned v = __ballot_sync(KV_FULL, keep);
-                    if (keep) run[kept + __popc(v & ((1u << lane) - 1u))] = (unsigned short)r;
-                    kept += __popc(v);
+                    const unsigned w = __ballot_sync(KV_FULL, keep);
+                    if (keep) run[kept + __popc(w & ((1u << lane) - 1u))] = (unsigned short)r;
+                    kept += __popc(w);
                     __syncwarp();
                 }
                 nrun = kept;
             }
-            ++evictions; ++npe;
-            head = min(head, q);
-            t_ok = t + 1;
             __syncwarp();
         }
         if (failed) break;
         // ---- step 4: the round runs
         sim.advance(1, 0);
     }
+    if (lane == 0) scan.nrun = -1;
+    __syncthreads();
     if (failed) {
         if (lane == 0) atomicExch(P.status, KV_DEV_LOOP_CAP);
         return;

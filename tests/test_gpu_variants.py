@@ -57,6 +57,22 @@ def test_timeline_sizes(omax):
     assert (mstarts.astype(np.int64).sum(1) + int(o.sum()) == ref[:5]).all()
 
 
+@pytest.mark.parametrize("n", [1, 31, 33, 127, 128, 129, 400, 4096])
+def test_amin_running_lists(n):
+    """Evictions from lists of running requests at and beside the multiples of what the warps of a CTA look at
+    side by side, and the largest ids; nearly everything starts at once, on estimates of one round."""
+    rng = np.random.default_rng(n)
+    s = rng.integers(1, 4, n).astype(np.int32)
+    o = rng.integers(1, 40, n).astype(np.int32)
+    lower = np.where(rng.random(n) < 0.98, 1, o).astype(np.int32)
+    M = max(int((s + o).max()), int(s.sum()) + 2 * n)
+    order = rng.permutation(n).astype(np.int32)
+    starts, tel, ev, peak, _ = kv.amin_simulate([n], s[None], lower[None], o[None], M, order[None])
+    p, rtel, rev, rpeak = orc.amin_schedule_rounds(s, lower, o, M, order)
+    assert (starts[0] == p).all() and (tel[0], ev[0], peak[0]) == (rtel, rev, rpeak)
+    assert n < 100 or rev > n // 8
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 1023, 1024, 1025, 2049, 12000, 20000])
 def test_sorting_and_batch_selection_sizes(n):
     """One tile, its edges, several, and sizes beyond what the solvers keep in shared memory."""
