@@ -321,7 +321,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         if (const char* kind = getenv("KVSCHED_SIM"))               // testing knob: force the hybrid simulator
             if (strcmp(kind, "hybrid") == 0) h->nm = 0;
         // ints per simulator state, and the part of it that lives in shared memory
-        h->L = h->nm == 0 ? 32 * (HybSim::NREG + sim_pick_far_chunks(omax)) : 32 + 96 * h->nm + 32 * slots;
+        h->L = h->nm == 0 ? 32 * (HybSim::NREG + sim_pick_far_chunks(omax)) : sim_state_ints(h->nm, slots);
         h->ring_cells = h->nm == 0 ? HybSim::ring_cells(h->L) : 32 * slots;
         if (k3_warps(h) < 1) { rc = SCHED_E_UNSUPPORTED; break; }
         if (cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking) != cudaSuccess) { rc = kv_cuda_fail(cudaGetLastError(), "cudaStreamCreate"); break; }
@@ -335,7 +335,6 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             // that, so a move near the end of the list counts: one of 20,000 requests with decodes up to 20,000
             // took 1.65 ms with 256 states and takes 0.20 (the base run 59.8 and 70.7)
             i64 stride = h->nm ? ((i64)n + kSnapshots - 1) / kSnapshots : kSnapStrideHyb;
-            stride = (stride + 3) & ~3ll;               // requests are admitted four at a time
             if (h->nm && stride < 16) stride = 16;      // the base run stops for every snapshot
             while ((((i64)n + stride - 1) / stride) * (i64)per > (i64)kSnapBudget) stride += 4;
             h->snap_stride = (int)stride;
@@ -1386,7 +1385,7 @@ int sched_online_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const
     memset(&P, 0, sizeof(P));
     P.n_max = n_max; P.M = (int)M; P.policy = policy; P.period = period; P.lookahead = lookahead;
     const int slots = sim_pick_slots(omax), nm = slots <= 32 ? 1 : slots / 32;
-    P.L = 32 + 96 * nm + 32 * slots;
+    P.L = sim_state_ints(nm, slots);
     const size_t smem = k6_smem_bytes(32 * slots, n_max, lookahead);
     int dev = 0, optin = 0;
     KV_CUDA(cudaGetDevice(&dev));
@@ -1479,7 +1478,7 @@ static int amin_run(int32_t B, int32_t n_max, const int32_t* n_each, const int32
     P.n_max = n_max; P.M = (int)M;
     P.L = 32; while (P.L < omax + 2) P.L <<= 1;
     const int slots = sim_pick_slots(omax), nm = slots <= 32 ? 1 : slots / 32;
-    P.sim_L = 32 + 96 * nm + 32 * slots;
+    P.sim_L = sim_state_ints(nm, slots);
     const size_t smem = k7_smem_bytes(32 * slots, n_max, P.L);
     int dev = 0, optin = 0;
     KV_CUDA(cudaGetDevice(&dev));

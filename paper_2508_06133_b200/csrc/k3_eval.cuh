@@ -146,7 +146,7 @@ k3_base_run(const BaseRunParams p) {
     int to_snap = 0, idx = 0;                            // positions until the next snapshot, its number
     for (int q0 = 0; q0 < n;) {
         const int2 so = next;
-        // a block ends where a snapshot is due (the stride is a multiple of 4, so is every block but the last)
+        // a block ends where a snapshot is due
         if (to_snap == 0) {
             const int i = (int)KV_IDX(idx, p.snap_count, 401);
             i64 before = tel;
@@ -157,7 +157,7 @@ k3_base_run(const BaseRunParams p) {
         }
         const int cnt = min(min(32, n - q0), to_snap);
         if (q0 + cnt + lane < n) next = tbl_base[q0 + cnt + lane];
-        const int mine = sim_run_block<true>(sim, so, cnt, n - q0, status);
+        const int mine = sim.template run<true>(so, cnt, status);
         if (lane < cnt) base_starts_pos[q0 + lane] = mine;
         if (lane < cnt) tel += (i64)mine + so.y;
         q0 += cnt;
@@ -214,7 +214,7 @@ k3_eval_moves(const MoveEvalParams p) {
     const int idx = (int)KV_IDX(first_pos / p.stride, p.snap_count, 403);
     const int q_start = idx * p.stride;
     // restore the base run's state in front of q_start
-    sim.load(p.snap_ring + (size_t)idx * L, p.snap_hdr[idx], M, n - q_start);
+    sim.load(p.snap_ring + (size_t)idx * L, p.snap_hdr[idx], M);
     i64 sum_o = 0;
     int* starts = kStarts ? p.starts_out + (size_t)c * n : nullptr;
     if (kStarts)
@@ -230,7 +230,7 @@ k3_eval_moves(const MoveEvalParams p) {
         }
         const int cnt = min(32, n - q0);
         if (lane < cnt) sum_o += so.y;
-        const int mine = sim_run_block<false>(sim, so, cnt, n - q0, p.status);
+        const int mine = sim.template run<false>(so, cnt, p.status);
         if (kStarts && lane < cnt) starts[KV_IDX(id, n, 405)] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
@@ -308,7 +308,7 @@ k3_eval_orders(const OrderEvalParams p) {
         }
         const int cnt = min(32, n - q0);
         if (lane < cnt) sum_o += so.y;
-        const int mine = sim_run_block<false>(sim, so, cnt, n - q0, p.status);
+        const int mine = sim.template run<false>(so, cnt, p.status);
         if (kStarts && lane < cnt) starts[id] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
@@ -363,7 +363,7 @@ k3_check_starts(const StartsEvalParams p) {
             const int wait = __shfl_sync(KV_FULL, pi, k) - sim.start();
             if (wait < 0) { ok = false; break; }
             if (wait > 0) sim.skip(wait, M);
-            if (sim.test(sp, om) > 0) ok = false;
+            if (sim.need(sp, om) > 0) ok = false;
             else sim.add(sp, om);
         }
     }

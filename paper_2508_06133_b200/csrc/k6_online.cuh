@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(K6_THREADS) k6_online(const OnlineParams P) {
             }
             if (r < 0) break;
             const int s = q.ss[r], o = q.so[r];
-            need = sim.test(s + 1, o - 1);
+            need = sim.need(s + 1, o - 1);
             if (need > 0) break;
             sim.add(s + 1, o - 1);
             if (lane == 0) { P.start_out[base + KV_IDX(r, n, 1001)] = t - 1; q.started[r] = 1; }

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
         // decision (or ends the run).
         const int head_s = head < n ? ps[head] : 0;
         for (;;) {
-            const bool live = sim.rl >= 0;
+            const bool live = lane >= sim.tau;
             const int round = sim.T0 + lane, k = round & mask;
             int es = live ? ev[k] : 0;
             unsigned as = live ? dA[k] : 0u;
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             }
             const unsigned cnt_l = cnt + (unsigned)(es >> 16), A_l = A + as;
             const int rem_l = remaining - (es & 0xffff);
-            const int u = sim.cur - lane + (int)(A_l + cnt_l * (unsigned)round);
+            const int u = sim.cur + M - lane + (int)(A_l + cnt_l * (unsigned)round);
             const bool end = live && rem_l == 0;
             // the head's first round is the current one: if it does not fit there, the window test cannot
             // succeed in this iteration
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             A = __shfl_sync(KV_FULL, A_l, src);
             remaining = __shfl_sync(KV_FULL, rem_l, src);
             if (first < 32) {
-                if (lane == first) sim.cur = u + lane;                              // step 1 of the round that is decided
+                if (lane == first) sim.cur = u + lane - M;                              // step 1 of the round that is decided
                 sim.advance(first - sim.tau, 0);
                 if ((ends >> first) & 1u) done = true;
                 else if (!((works >> first) & 1u)) failed = true;
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             int s = ps[head], e = pe[head];
             for (;;) {
                 const int q = head, q1 = q + 1 < n ? q + 1 : q, s1 = ps[q1], e1 = pe[q1];      // the next one, mostly
-                const int need = sim.test(s + 1, e - 1);
+                const int need = sim.need(s + 1, e - 1);
                 if (need > 0) { t_ok = t + need; break; }
                 sim.add(s + 1, e - 1);
                 run[KV_IDX(nrun, nm, 1102)] = (unsigned short)q;
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
 
         // ---- step 3: ordered eviction while round t is over budget
         for (;;) {
-            const int used = __shfl_sync(KV_FULL, sim.cur - lane, sim.tau);
+            const int used = __shfl_sync(KV_FULL, sim.cur + M - lane, sim.tau);
             if (used <= M) { peak = max(peak, used); break; }
             // smallest (estimate, request id) among the running
             if (lane == 0) { scan.t = t; scan.nrun = nrun; }

@@ -165,7 +165,7 @@ struct HybSim {
         for (int k = 0; k < FC; ++k) far[32 * k] = 32 * (NREG + k) + lane;
         fb = 0; t = 0; tel = 0; tm = 0; rl = lane;
     }
-    __device__ __forceinline__ void load(const int* __restrict__ snap, const SnapHeader& h, int M_, int) {
+    __device__ __forceinline__ void load(const int* __restrict__ snap, const SnapHeader& h, int M_) {
         M = M_;
 #pragma unroll
         for (int c = 0; c < NREG; ++c) R[c] = snap[KV_IDX(32 * c + lane, span, 202)];
@@ -258,7 +258,7 @@ struct HybSim {
     // Admit one request (sp = s + 1, om = o - 1).  All 32 lanes call this with identical arguments.  The first chunk alone decides whether the request
     // has to wait and for how long at least; otherwise the whole window is tested and, if it fits,
     // the ramp is added; a window that reaches beyond the registers continues over the far ring.
-    __device__ __forceinline__ void admit(int sp, int om, int, int* status) {
+    __device__ __forceinline__ void admit(int sp, int om, int* status) {
         const int s = sp - 1, o = om + 1;
         int kadm = s + 1 - M - t;                      // V + kadm > 0  <=>  the cell is over budget
         for (int guard = 0;; ++guard) {
@@ -307,6 +307,18 @@ struct HybSim {
             advance(delta);
             if (guard > kv_loop_cap(span)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); return; }
         }
+    }
+
+    // Up to 32 consecutive requests of a list, (s, o) of the k-th in lane k.  Returns the start of the k-th in lane k.
+    template <bool kAlone>
+    __device__ __forceinline__ int run(int2 so, int cnt, int* status) {
+        const int sp = so.x + 1, om = so.y - 1;
+        int mine = 0;
+        for (int k = 0; k < cnt; ++k) {
+            admit(__shfl_sync(KV_FULL, sp, k), __shfl_sync(KV_FULL, om, k), status);
+            if (lane == k) mine = start();
+        }
+        return mine;
     }
 };
 

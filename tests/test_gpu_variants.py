@@ -57,6 +57,34 @@ def test_timeline_sizes(omax):
     assert (mstarts.astype(np.int64).sum(1) + int(o.sum()) == ref[:5]).all()
 
 
+@pytest.mark.parametrize("omax", [98, 1025, 2049, 4097, 8193])
+@pytest.mark.parametrize("beside", [1.5, 4, 30])
+def test_waits_in_and_behind_the_near_chunks(omax, beside):
+    """Windows of 63 to 66 and 94 to 98 rounds (the shortest that covers the two exact chunks wherever it begins, and
+    those that end on the last round of the next one) among the shortest and the longest, budgets for 1.5 to 30 requests beside
+    each other, so that waits end in the first chunk, in the second and many chunks further on: orders with starts, the same
+    through the run that stands alone, and moves."""
+    rng = np.random.default_rng(omax + int(10 * beside))
+    n = 160
+    o = rng.choice(np.array([1, 2, 31, 32, 33, 62, 63, 64, 65, 66, 67, 94, 95, 96, 97, 98, omax]), n).astype(np.int32)
+    o[0] = omax
+    s = np.where(rng.random(n) < 0.15, rng.integers(1, 6000, n), rng.integers(1, 300, n)).astype(np.int32)
+    M = max(int((s + o).max()), int(beside * (s + o).mean()))
+    orders = np.stack([rng.permutation(n) for _ in range(3)]).astype(np.int32)
+    codes = np.arange(0, 3 * n * (n - 1) // 2, 149, dtype=np.int64)
+    with kv.Scheduler(s, o, M) as h:
+        tel, _, starts = h.eval_batch(kv.CAND_ORDER, orders, want_starts=True)
+        ok = h.eval_batch(kv.CAND_START_TIMES, starts, want_feasible=True)[1]
+        h.set_base_order(orders[0])
+        mtel = h.eval_batch(kv.CAND_MOVE, codes)[0]
+        final, ftel, _, _ = h.local_search(kv.NBHD_SWAP, 0, order=orders[1])
+    for c in range(3):
+        p, t, _ = orc.list_schedule_rounds(s, o, M, orders[c])
+        assert tel[c] == t and (starts[c] == p).all()
+    assert ok.all() and (final == orders[1]).all() and ftel == tel[1]
+    assert (mtel == oracle_moves(s, o, M, orders[0], codes)).all()
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 127, 128, 129, 400, 4096])
 def test_amin_running_lists(n):
     """Evictions from lists of running requests at and beside the multiples of what the warps of a CTA look at
