@@ -534,31 +534,31 @@ bool short_windows(const sched_ctx* h, bool want_starts) { return !want_starts &
 // side by side, so its time hardly moves below that and the other's is proportional to the count.  Measured,
 // warp against thread, ms:
 //   rounds per request  2.9 (n = 10,000)   7.6 (10,000)   12.4 (1,000)   18.9 (4,000)   24.8 (1,000)
-//   16,000 moves          8.4 /  8.9       10.4 / 15.8     1.2 / 1.9      6.1 / 12.4     1.7 / 3.2
-//   32,000               16.6 / 10.2       20.5 / 17.9     2.4 / 2.2     12.0 / 14.2     3.4 / 3.7
-//   48,000                                                 3.6 / 2.6     17.8 / 16.7     5.1 / 4.4
-//   96,000                                                 7.1 / 3.9     35.4 / 24.1    10.1 / 6.3
+//   16,000 moves          7.1 /  8.4        8.6 / 14.4     1.0 / 1.7      4.7 / 11.7     1.3 / 3.2
+//   24,000               10.5 /  8.9       12.7 / 15.9     1.5 / 1.8      7.0 / 12.7     2.0 / 3.5
+//   32,000               13.9 /  9.4       16.8 / 16.2     2.0 / 1.9      9.3 / 13.1     2.6 / 3.6
+//   48,000               20.8 / 10.4       25.2 / 18.4     3.0 / 2.1     13.8 / 14.8     3.9 / 4.1
+//   96,000               41.4 / 15.1       50.1 / 25.9     5.9 / 3.0     27.5 / 21.0     7.7 / 5.7
 //   decodes to 2,048    4.5 (n = 2,000)   10.8 (2,000)    14.8 (2,000)
-//   32,000                4.6 /  3.8        6.1 / 7.5      7.0 /  9.5
-//   48,000                6.9 /  4.3        9.1 / 8.5     10.5 / 10.9
-//   96,000               13.7 /  6.6       18.0 / 13.8    20.9 / 18.3
+//   32,000                3.8 /  4.1        5.1 / 7.6      5.9 /  9.2
+//   48,000                5.7 /  4.3        7.6 / 8.0      8.7 / 10.4
+//   96,000               11.4 /  5.7       15.1 / 12.2    17.4 / 16.4
 // Two kinds of backlog cost a thread more per admission (log-normal decodes, prefills uniform up to 2,000):
 //   short decodes: a window that ends in one of the two chunks kept as cells takes its share back from them one by one,
 //   which the share of decodes up to a chunk (each counted as 32 / o beyond) tells.  Mean 21 (share 0.94): 40,000 moves of
-//   10,000, 0.5 / 2 / 6 rounds per request 18.6 / 18.4, 22.2 / 30.5, 29.9 / 50.0; mean 84 (0.55): 18.4 / 9.4, 21.9 / 14.6,
-//   25.6 / 25.1;
+//   10,000, 0.5 / 2 / 6 rounds per request 16.5 / 19.6, 20.3 / 31.0, 27.8 / 50.0; mean 87 (0.56): 16.4 / 10.1, 18.5 / 15.1,
+//   21.3 / 24.1;
 //   long decodes on short prefills: memory is used by tokens still to come, what a request waits for lies chunks
-//   ahead, and every wait walks the events up to there.  Prefills up to 20, decodes of mean 340, 10,000 requests, 40,000
-//   moves, 0.5 / 1 / 2 / 6 rounds per request 15.5 / 10.6, 15.7 / 16.0, 16.6 / 40.5, 19.7 / 111; prefills up to 2,000: 18.1 / 8.0,
-//   19.9 / 9.7, 21.6 / 11.9, 26.0 / 24.9; decodes of mean 669 (to 2,048), prefills up to 20: 20.3 / 9.0, 20.7 / 13.4, 21.7 / 16.9,
-//   25.6 / 53.1.  Use of memory falls by s / rounds per round and varies by (s + o) sqrt(rounds ahead / rounds), hence
+//   ahead, and every wait walks the events up to there.  Prefills up to 20, decodes of mean 335, 10,000 requests, 40,000
+//   moves, 0.5 / 1 / 2 / 6 rounds per request 16.0 / 10.5, 16.4 / 14.7, 17.4 / 36, 21.2 / 146; prefills up to 2,000: 15.8 / 6.7,
+//   16.2 / 8.5, 16.8 / 10.8, 19.2 / 24.0; decodes of mean 668 (to 2,048), prefills up to 20: 20.7 / 7.9, 21.3 / 14.7, 22.3 / 17.2,
+//   26.9 / 56.  Use of memory falls by s / rounds per round and varies by (s + o) sqrt(rounds ahead / rounds), hence
 //   the form in (1 + o / s) sqrt(rounds); its square and the caps are fitted.  Only where time goes on for
 //   longer than a decode: otherwise nearly everything runs side by side.
-// Of 1,257 sweeps measured in both forms (225 of them on backlogs drawn at random, in Sorted-F, random and index order)
-// 12 take a thread where a warp is faster by more than a tenth (200 by rounds per request alone), 64 the other way round.  Longer decodes than its ring of events, schedules with more rounds per request than
+// Longer decodes than its ring of events, schedules with more rounds per request than
 // were measured (14.8 for decodes beyond 1,025), and backlogs whose candidate could pass 32 bits of waiting
 // time in its sum of starts keep the warp.
-constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.4;
+constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.55;
 
 // candidates from which on a thread each is the faster one
 double lanes_from(const sched_ctx* h) {
@@ -566,14 +566,16 @@ double lanes_from(const sched_ctx* h) {
     double need = LANE_MIN + LANE_MIN_PER_ROUND * rounds, ahead = (1.0 + h->mean_o / h->mean_s) * (1.0 + h->mean_o / h->mean_s);
     if (rounds > LANE_ROUNDS) return INFINITY;
     if (h->nm == 1) {
-        if (h->short_share > 0.3) need += 5000.0 * rounds * (h->short_share - 0.3);
+        if (h->short_share > 0.3) need += 11000.0 * rounds * (h->short_share - 0.3);
+        if (ahead > 1.3) need += 8700.0 * rounds * (fmin(ahead, 3.0) - 1.3);
         if (h->short_share > 0.75) need += 150000.0 * (h->short_share - 0.75);
         if (short_windows(h, false)) need *= 1.3;              // against the warp's simulator for those
         ahead = fmin(ahead, 8.0);
     } else {
         need *= LANE_LONG;
+        if (h->short_share > 0.4) need *= 1.0 + (h->short_share - 0.4) * rounds / 3.0;
         // candidates further apart in a long list also leave one another's rounds: 40,000 moves of 10,000 and of 2,000
-        // requests with a share of 0.57, 6 rounds per request: 30.8 / 44.9 and 6.2 / 5.1
+        // requests with a share of 0.72, 6 rounds per request: 28.1 / 60 and 5.6 / 11.4
         if (h->short_share > 0.4 && n > 2000.0) need *= 1.0 + (n - 2000.0) * rounds / 48000.0;
         ahead = fmin(0.6 * ahead, 3.6);
     }

@@ -1,7 +1,7 @@
 // K3, many candidates: one THREAD per candidate move.  Same rule, same results as k3_eval_moves
 // (sim_chunk.cuh has the rule; V[x] is the tokens in use in round x, plus x).
 //
-// k3_eval_moves gives a warp to a candidate; nearly all of its 80 instructions per admission are the same
+// k3_eval_moves gives a warp to a candidate; nearly all of its 60 to 80 instructions per admission are the same
 // in every lane.  Here the 32 candidates of a warp are neighbours in the launch order (first moved
 // positions next to each other), so they start from the same state of the base run and meet about the
 // same requests in about the same rounds: they are moved through time together, chunk by chunk of CH
@@ -20,21 +20,23 @@
 //       maximum: each raised by a ramp's value in the chunk's last round.  All below the limit: it fits.
 // Where W0 says "perhaps", one walk back over the chunk's cells gives the first round from which the
 // request fits (the maximum of V behind a round falls along the chunk, the limit rises), hence the wait,
-// so a turn nearly always ends with an admission in every lane (1.25 turns per admission).  W1 is
+// so a turn nearly always ends with an admission in every lane.  A request whose window covers the rest of the chunk and that
+// the chunk's last cell keeps out whatever its start leaves the chunk before the turn begins (its last cell is kept in a register):
+// 1.25 to 1.6 turns per admission, 1.4 to 2.2 where the walk had to find that out.  W1 is
 // answered from the next chunk's cells, U (2 of 1,000 turns) from the events.
 //
-// What bounds it: instructions at 20 warps per SM (registers and the cells of two chunks allow no more): 1,250 for 32
-// candidates' admissions at 12 rounds per request where the kernel with a warp per candidate executes 32 x 80, two thirds of
-// the issue slots and of the integer pipe; below a full chip, latency.  The event rings of all resident candidates are
-// 412 MB and do not stay in L2 (126 MB): a third of the memory's rate, and half of all warp cycles in the first form.  So a chunk's words are
-// read with eight 16-byte loads in flight, laid out so that a warp's load is 512 contiguous bytes, called to L2 one
-// chunk ahead, and cleared only where they are not zero; the request behind the next is on its way a turn early.
-// 64,000 moves of 10,000 requests, budget 262,144: 33.0 ms with a warp per candidate; 23.6 with one load of a
-// lane's own line at a time, 18.6 with four of them, 16.0 with these side by side and the walk in two levels, 14.7 with
-// eight.  256,000 moves of 1,000 requests, budget 65,536: 18.9 -> 8.8 ms.  4,194,304 moves of the 10,000: 2,741 ->
-// 569 ms.  These are kernels alone on the chip; 65,536 threads fill 0.7 of it, so sweeps of several handles overlap (9.4
-// ms each).  A handle's first sweep also allocates the rings: 16.5 ms where the next is 14.8, more when the driver
-// takes longer for it (28 ms once in nine).  lanes_from (api.cu) has the rule and the other side.
+// What bounds it: instructions at 20 warps per SM (registers and the cells of two chunks allow no more), 0.72 of the issue
+// slots and 0.68 of the integer pipe; below a full chip, latency.  A turn is about 330 instructions, a chunk 400 more: the
+// walk takes four cells with one maximum (their slopes differ by one, two and three), a chunk's cells follow from
+// the one before by two additions, the bounds' maximum two at a time, and the state in front of a group's first position is summed by
+// reductions with a request per lane instead of by every lane for itself.  The event rings of all resident candidates are
+// 412 MB and do not stay in L2 (126 MB), so a chunk's words are read with eight 16-byte loads in flight, laid out so
+// that a warp's load is 512 contiguous bytes, called to L2 one chunk ahead, and cleared only where they are not zero; the
+// request behind the next is on its way a turn early.
+// 499,500 moves of 1,000 requests, budget 65,536: 13.45 -> 10.45 ms (blocked requests leave early 12.15, the walk by fours and
+// the cells by additions 10.75); 65,536 moves of 10,000, budget 262,144: 14.9 -> 12.2 ms alone on the chip, of which 65,536 threads fill
+// 0.7, so sweeps of several handles overlap (7.8 ms each).  A handle's first sweep also allocates the rings, which can
+// take the driver several ms.  lanes_from (api.cu) has the rule and the other side.
 #pragma once
 
 #include "common.cuh"
@@ -74,6 +76,7 @@ k3_lane_moves(const LaneParams P) {
     WORD* const ring = (WORD*)P.rings + ((size_t)blockIdx.x * S::kWarps + warp) * S::kRingWords + lane * PER;
     const int n = P.m.n, M = P.m.M, least = P.least, shift = P.shift;
     const WORD vmask = ((WORD)1 << shift) - 1, one = (WORD)1 << shift;
+    const int most_turns = kv_loop_cap(1 << 28);
     auto unpack = [](const uint4& v, WORD* ev) {                           // the words of 16 bytes
         if (sizeof(WORD) == 4) { ev[0] = (WORD)v.x; ev[1] = (WORD)v.y; ev[2] = (WORD)v.z; ev[3] = (WORD)v.w; }
         else { ev[0] = (WORD)((u64)v.x | ((u64)v.y << 32)); ev[1] = (WORD)((u64)v.z | ((u64)v.w << 32)); }
@@ -120,23 +123,27 @@ k3_lane_moves(const LaneParams P) {
         {
             int lo = 0, hi = q;                                            // first position that can still run at t
             while (lo < hi) { const int mid = (lo + hi) >> 1; if (P.m.base_starts_pos[mid] + P.omax > hdr.t) hi = mid; else lo = mid + 1; }
-            int2 so1 = P.m.tbl_base[lo < n ? lo : 0];
-            int p1 = P.m.base_starts_pos[lo < n ? lo : 0];
-            for (int k = lo; k < q; ++k) {
-                const int2 so = so1;
-                const int p = p1 - T0, last = p + so.y - 1;
-                so1 = P.m.tbl_base[k + 1 < n ? k + 1 : 0];
-                p1 = P.m.base_starts_pos[k + 1 < n ? k + 1 : 0];
-                if (last < hdr.t - T0) continue;
-                const int a = so.x + 1 - p;
-                A += a; ++C;
-                atomicAdd(word_of(0, last), (WORD)(so.x + so.y - least) + one);
+            // the same for all lanes: one running request each, its sums by reductions, its event in every lane's ring
+            for (int k0 = lo; k0 < q; k0 += 32) {
+                const int k = k0 + lane < q ? k0 + lane : lo;
+                const int2 so = P.m.tbl_base[k];
+                const int p = P.m.base_starts_pos[k] - T0, last = p + so.y - 1;
+                const bool runs = k0 + lane < q && last >= hdr.t - T0;
+                const int a = so.x + 1 - p, size = so.x + so.y - least, reach = runs ? last : -1;
+                unsigned todo = __ballot_sync(KV_FULL, runs);
+                A += __reduce_add_sync(KV_FULL, runs ? a : 0);
+                C += __popc(todo);
 #pragma unroll
-                for (int c = 0; c < NF; ++c) if (last >= CH * (c + 2)) U[c] += a + CH * (c + 3) - 1;
+                for (int c = 0; c < NF; ++c) U[c] += __reduce_add_sync(KV_FULL, reach >= CH * (c + 2) ? a + CH * (c + 3) - 1 : 0);
+                for (; todo; todo &= todo - 1) {
+                    const int j = __ffs(todo) - 1, at_round = __shfl_sync(KV_FULL, last, j);
+                    atomicAdd(word_of(0, at_round), (WORD)__shfl_sync(KV_FULL, size, j) + one);
+                }
             }
         }
         // cells of the chunk whose events are in `slot`, from the totals; the totals move on to the next
         // one.  Returns the maximum of V, x counted from the chunk's own beginning.
+        int end0 = 0, end1 = 0;                                            // the last cell of either chunk
         auto build = [&](int* cells, int slot) -> int {
             WORD* line = line_of(slot);
             int w = INT_MIN;
@@ -145,7 +152,9 @@ k3_lane_moves(const LaneParams P) {
 #pragma unroll
                 for (int g = 0; g < GROUP; ++g) v[g] = __ldcg(reinterpret_cast<const uint4*>(line + 32 * x0) + 32 * g);
 #pragma unroll
-                for (int g = 0; g < GROUP; ++g) if (v[g].x | v[g].y | v[g].z | v[g].w) __stcg(reinterpret_cast<uint4*>(line + 32 * x0) + 32 * g, make_uint4(0, 0, 0, 0));
+                for (int g = 0; g < GROUP; ++g)                            // without a branch
+                    asm volatile("{ .reg .pred q; setp.ne.u32 q, %1, 0; @q st.global.cg.v4.u32 [%0], {%2, %2, %2, %2}; }"
+                                 :: "l"(reinterpret_cast<uint4*>(line + 32 * x0) + 32 * g), "r"(v[g].x | v[g].y | v[g].z | v[g].w), "r"(0) : "memory");
                 WORD ev[GROUP * PER];
 #pragma unroll
                 for (int g = 0; g < GROUP; ++g) unpack(v[g], ev + g * PER);
@@ -154,24 +163,26 @@ k3_lane_moves(const LaneParams P) {
                     int cell[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const int x = x0 + x4 + k;
-                        cell[k] = A + C * x;
-                        w = max(w, cell[k] + x);
+                        cell[k] = A;
+                        w = __viaddmax_s32(A, x0 + x4 + k, w);
+                        // those whose last round this is take their s+o with them, the others use one more each
                         const int num = (int)(ev[x4 + k] >> shift);
-                        A -= (int)(ev[x4 + k] & vmask) + num * (least - x);
                         C -= num;
+                        A += C - (sizeof(WORD) == 4 ? (int)ev[x4 + k] - num * ((1 << (shift & 31)) - least) : (int)ev[x4 + k] + num * least);
                     }
                     *reinterpret_cast<int4*>(cells + at(x0 + x4)) = make_int4(cell[0], cell[1], cell[2], cell[3]);
+                    end1 = cell[3];
                 }
             }
             // the words that are read next: the admissions of a chunk are time enough to have them in L2
 #pragma unroll
             for (int x = 0; x < CH; x += 128 / (int)sizeof(WORD))
                 asm volatile("prefetch.global.L2 [%0];" :: "l"(line_of(slot + 1) + lane * (CH - PER) + x));
-            A += CH * C;
             return w;
         };
-        int W0 = build(b0, 0), W1 = build(b1, 1) + CH;
+        int W0 = build(b0, 0);
+        end0 = end1;
+        int W1 = build(b1, 1) + CH;
         int slot = 2;                                                      // events of the chunk behind the two
         int dA0 = 0, dC0 = 0, dA1 = 0, dC1 = 0;
         int tau = hdr.t - T0;
@@ -195,16 +206,19 @@ k3_lane_moves(const LaneParams P) {
         for (i64 chunk = 0;; ++chunk) {
             int Uall = INT_MIN;
 #pragma unroll
-            for (int c = 0; c < NF; ++c) Uall = max(Uall, U[c]);
+            for (int c = 0; c < NF; c += 2) Uall = __vimax3_s32(Uall, U[c], U[c + 1]);
             // ---- every lane admits and waits until it leaves the chunk
             for (int guard = 0;; ++guard) {
+                const int lim = M - sp;                                    // fits at t  <=>  V[x] <= lim + t over the window
+                // where the window reaches the chunk's last round and that one is over for every start, none is in this chunk
+                if (tau + om >= CH - 1 && end0 + dA0 + (CH - 1) * dC0 > lim) tau = max(tau, CH);
                 const bool act = q < n && tau < CH;
                 if (!__any_sync(KV_FULL, act)) break;
-                const int lim = M - sp;                                    // fits at t  <=>  V[x] <= lim + t over the window
                 bool fits = act;
                 const bool ask0 = act && W0 > lim + tau;
-                if (__any_sync(KV_FULL, ask0)) {
-                    const int x_lo = kv_warp_min(ask0 ? tau : CH - 1) & ~3;
+                const int from = kv_warp_min(ask0 ? tau : CH);
+                if (from < CH) {
+                    const int x_lo = from & ~3;
                     const int lim0 = lim - dA0;
                     // y: maximum of V behind a round, less the round; grows strictly towards the front.  First the
                     // four cells in which it passes the limit, then the cell.
@@ -214,10 +228,8 @@ k3_lane_moves(const LaneParams P) {
                     for (int x4 = CH - 4; x4 >= x_lo; x4 -= 4) {
                         const int4 four = *reinterpret_cast<const int4*>(b0 + at(x4));
                         if (y <= lim0) { y_in = y; x_in = x4; }
-                        y = __viaddmax_s32(y, 1, four.w + rise * (x4 + 3));
-                        y = __viaddmax_s32(y, 1, four.z + rise * (x4 + 2));
-                        y = __viaddmax_s32(y, 1, four.y + rise * (x4 + 1));
-                        y = __viaddmax_s32(y, 1, four.x + rise * x4);
+                        const int m = __viaddmax_s32(four.w, 3 * (rise + 1), __viaddmax_s32(four.z, 2 * (rise + 1), __viaddmax_s32(four.y, rise + 1, four.x)));
+                        y = __viaddmax_s32(y, 4, m + rise * x4);
                     }
                     int best = x_in + 4, best_w;
                     {
@@ -257,20 +269,26 @@ k3_lane_moves(const LaneParams P) {
                 if (__any_sync(KV_FULL, ask1)) {
                     const int lim1 = lim + tau - dA1 - CH, slope = dC1 + 1, end = tau + om - CH;
                     int w = INT_MIN, d = 0;
-#pragma unroll 2
+#pragma unroll 4
                     for (int x4 = 0; x4 < CH; x4 += 4) {
                         const int4 four = *reinterpret_cast<const int4*>(b1 + at(x4));
-                        const int cell[4] = {four.x, four.y, four.z, four.w};
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int x = x4 + k, v = cell[k] + slope * x;
-                            w = max(w, v);
-                            if (x <= end) d = max(d, __viaddmin_s32(v, -lim1, x + CH + 1 - tau));
-                        }
+                        const int m = __viaddmax_s32(four.w, 3 * slope, __viaddmax_s32(four.z, 2 * slope, __viaddmax_s32(four.y, slope, four.x)));
+                        w = max(w, m + slope * x4);
                     }
-                    if (ask1) {
-                        W1 = w + dA1 + CH;
-                        if (d > 0) { tau += d; fits = false; }
+                    if (ask1) W1 = w + dA1 + CH;
+                    const bool over1 = ask1 && w > lim1;                   // somewhere in the chunk: in the window?
+                    if (__any_sync(KV_FULL, over1)) {
+#pragma unroll 2
+                        for (int x4 = 0; x4 < CH; x4 += 4) {
+                            const int4 four = *reinterpret_cast<const int4*>(b1 + at(x4));
+                            const int cell[4] = {four.x, four.y, four.z, four.w};
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const int x = x4 + k;
+                                if (x <= end) d = max(d, __viaddmin_s32(cell[k] + slope * x, -lim1, x + CH + 1 - tau));
+                            }
+                        }
+                        if (over1 && d > 0) { tau += d; fits = false; }
                     }
                 }
                 const bool far = fits && Uall > lim + tau && tau + om >= 2 * CH;
@@ -324,8 +342,14 @@ k3_lane_moves(const LaneParams P) {
                     atomicAdd(word_of(slot, last - 2 * CH), (WORD)(sp + om - least) + one);
                 }
                 if (__any_sync(KV_FULL, fits && !far2)) {                  // a window that ends in one of the two chunks
-                    if (far1 && !far2) { for (int x = last + 1 - CH; x < CH; ++x) b1[at(x)] -= a + CH + x; }
-                    if (fits && !far1) { for (int x = last + 1; x < CH; ++x) b0[at(x)] -= a + x; }
+                    if (far1 && !far2) {
+                        for (int x = last + 1 - CH; x < CH; ++x) b1[at(x)] -= a + CH + x;
+                        if (last < 2 * CH - 1) end1 -= a + 2 * CH - 1;
+                    }
+                    if (fits && !far1) {
+                        for (int x = last + 1; x < CH; ++x) b0[at(x)] -= a + x;
+                        if (last < CH - 1) end0 -= a + CH - 1;
+                    }
                 }
                 const int reach = fits ? last : 0;
                 if (fits) {
@@ -335,13 +359,16 @@ k3_lane_moves(const LaneParams P) {
                 next = fetch(q + 1);
                 // bounds of the far chunks the new windows reach
 #pragma unroll
-                for (int c0 = 0; c0 < NF; c0 += 8) {
+                for (int c0 = 0; c0 < NF; c0 += 4) {
                     if (reach_max < CH * (c0 + 2)) break;
 #pragma unroll
-                    for (int c = c0; c < c0 + 8; ++c)
-                        if (reach >= CH * (c + 2)) { U[c] += a + CH * (c + 3) - 1; Uall = max(Uall, U[c]); }
+                    for (int c = c0; c < c0 + 4; c += 2) {
+                        if (reach >= CH * (c + 2)) U[c] += a + CH * (c + 3) - 1;
+                        if (reach >= CH * (c + 3)) U[c + 1] += a + CH * (c + 4) - 1;
+                        Uall = __vimax3_s32(Uall, U[c], U[c + 1]);
+                    }
                 }
-                if (guard > kv_loop_cap(1 << 28)) { if (lane == 0) atomicExch(P.m.status, KV_DEV_LOOP_CAP); break; }
+                if (guard > most_turns) { if (lane == 0) atomicExch(P.m.status, KV_DEV_LOOP_CAP); break; }
             }
             if (!__any_sync(KV_FULL, q < n)) break;
             if (chunk > kv_loop_cap((i64)(1 << 30))) { if (lane == 0) atomicExch(P.m.status, KV_DEV_LOOP_CAP); break; }
@@ -351,6 +378,7 @@ k3_lane_moves(const LaneParams P) {
             int* const x = b0; b0 = b1; b1 = x;
             dA0 = dA1; dC0 = dC1; dA1 = 0; dC1 = 0;
             W0 = W1 - CH;
+            end0 = end1;
             W1 = build(b1, slot) + CH;
             slot = slot + 1 == NCH ? 0 : slot + 1;
 #pragma unroll
