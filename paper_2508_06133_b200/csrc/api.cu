@@ -40,6 +40,8 @@ const int kDeviceCheckMax = 1 << 20;        // requests whose bits fit a CTA's s
 const i64 kHostCheckMax = 1 << 13;          // ids or starts checked by the host: 8 us, a launch and a read-back 13
 const i64 kAcceptSmall = 16384;              // sweep results that one CTA reduces (4 us against a launch of its own)
 const int kSnapshots = 256;                 // states of the base run kept for the sweeps (chunked simulator)
+const int kLeadingFrom = 2048;              // requests from which the quantile solver's keys are made beforehand: 2 and more per thread
+const size_t kLeadingBytes = 64ull << 20;   // of them, at most
 const int kSnapStrideHyb = 8;               // positions per state (hybrid simulator)
 const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
 
@@ -1225,13 +1227,26 @@ static int phase1_quantile(sched_handle h, u64 seed) {
     KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, 0}, n, 1, h->d_keys_a, h->d_vals_a, h->d_keys_more, h->d_vals_more, by_size));
     KV_TRY(sort_rows(h, K2qSlotKey{h->d_s, h->d_o, list, F}, n, 1, h->d_keys_a, h->d_vals_a, h->d_keys_more, h->d_vals_more, by_ratio));
     const size_t bytes = k2q_bytes<unsigned short>(n), room = (size_t)h->smem_optin - sizeof(K2qShared) - 1024;
+    const unsigned* leading = nullptr;
+    int batches = 0;
+    if (n >= kLeadingFrom) {
+        // as many batches as there may be: the requests' sizes over M, a third of every batch unused
+        const double most = fmin(16.0 + 1.5 * (double)n * (h->mean_s + h->mean_o) / (double)h->M, (double)(kLeadingBytes / ((size_t)n * sizeof(unsigned))));
+        batches = most < n ? (int)most : n;
+        if (batches > 0) {
+            KV_TRY(ensure_stage(h, (size_t)batches * n * sizeof(unsigned)));
+            leading = (const unsigned*)h->d_stage;
+            k2q_leading<<<2 * h->sm_count, 256, 0, st>>>(list, n, batches, seed, (unsigned*)h->d_stage);
+            KV_TRY(check_launch(h));
+        }
+    }
     if (n < 65536 && bytes <= room) {
         KV_CUDA(cudaFuncSetAttribute(k2_quantile<unsigned short>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
-        k2_quantile<unsigned short><<<1, K2Q_THREADS, bytes, st>>>(h->d_s, h->d_o, list, by_size, by_ratio, n, h->M, seed, nullptr,
+        k2_quantile<unsigned short><<<1, K2Q_THREADS, bytes, st>>>(h->d_s, h->d_o, list, by_size, by_ratio, n, h->M, seed, nullptr, leading, batches,
                                                                   h->d_vals_a, h->d_batch_off, h->d_num_batches, h->d_status);
     } else {
         if (!h->d_ls) KV_TRY(dev_alloc(&h->d_ls, 7 * (size_t)n + 32));
-        k2_quantile<int><<<1, K2Q_THREADS, 0, st>>>(h->d_s, h->d_o, list, by_size, by_ratio, n, h->M, seed, h->d_ls,
+        k2_quantile<int><<<1, K2Q_THREADS, 0, st>>>(h->d_s, h->d_o, list, by_size, by_ratio, n, h->M, seed, h->d_ls, leading, batches,
                                                     h->d_vals_a, h->d_batch_off, h->d_num_batches, h->d_status);
     }
     return check_launch(h);

@@ -170,6 +170,21 @@ def test_solvers_beyond_shared_memory():
     assert (order == ref[0]).all() and (offs == ref[1]).all()
 
 
+@pytest.mark.parametrize("n,M,alone", [(2047, 30000, False), (2048, 30000, False), (3000, (1 << 21) - 1, False),
+                                       (3000, 1 << 21, False), (2100, 4000, True)])
+def test_quantile_sizes(n, M, alone):
+    """The first length whose keys are made beforehand and the last that goes without, sums of a tile in 32 and in 64 bits, and
+    a list with more batches (one request each) than keys are made for."""
+    rng = np.random.default_rng(n + M)
+    s = rng.integers(M // 2 + 1, M // 2 + 400, n).astype(np.int32) if alone else rng.integers(1, M // 20, n).astype(np.int32)
+    o = rng.integers(1, 300, n).astype(np.int32)
+    with kv.Scheduler(s, o, M) as h:
+        order, offs, _ = h.sorted_f_quantile(11)
+    ref = orc.sorted_f_quantile(s, o, M, 11)
+    assert (order == ref[0]).all() and (offs == ref[1]).all()
+    assert not alone or len(offs) == n + 1
+
+
 @pytest.mark.parametrize("n,M", [(9, 200), (40, 600), (24, 1100), (24, 1250)])
 def test_dynamic_programme_sizes(n, M):
     """The last tables that fit shared memory and the first that do not."""
