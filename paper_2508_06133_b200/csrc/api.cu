@@ -1233,8 +1233,11 @@ static int phase1_quantile(sched_handle h, u64 seed) {
         // as many batches as there may be: the requests' sizes over M, a third of every batch unused
         const double most = fmin(16.0 + 1.5 * (double)n * (h->mean_s + h->mean_o) / (double)h->M, (double)(kLeadingBytes / ((size_t)n * sizeof(unsigned))));
         batches = most < n ? (int)most : n;
+        if (batches > 0 && ensure_stage(h, (size_t)batches * n * sizeof(unsigned)) != SCHED_OK) {
+            cudaGetLastError();                          // without memory for them the solver makes its keys itself
+            batches = 0;
+        }
         if (batches > 0) {
-            KV_TRY(ensure_stage(h, (size_t)batches * n * sizeof(unsigned)));
             leading = (const unsigned*)h->d_stage;
             k2q_leading<<<2 * h->sm_count, 256, 0, st>>>(list, n, batches, seed, (unsigned*)h->d_stage);
             KV_TRY(check_launch(h));
