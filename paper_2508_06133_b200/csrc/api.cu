@@ -283,14 +283,16 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
     if (M >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
     const i64 total = (i64)B * n;
     KV_TRY(validate_instance(total, s, o, M));
-    int omax = 0, least = INT32_MAX; i64 sum_max = 0; double volume = 0;
+    int omax = 0, omin = INT32_MAX, least = INT32_MAX; i64 sum_max = 0, brief = 0; double volume = 0;
     for (int b = 0; b < B; ++b) {
         i64 sum = 0;
         for (int i = 0; i < n; ++i) {
             const int v = o[(i64)b * n + i], size = s[(i64)b * n + i] + v;
             sum += v;
             volume += (double)v * (size - 0.5 * v);
+            brief += v < 64 ? size - v + 1 : 0;
             omax = v > omax ? v : omax;
+            omin = v < omin ? v : omin;
             least = size < least ? size : least;
         }
         if (sum > sum_max) sum_max = sum;
@@ -313,7 +315,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) {
             rc = kv_cuda_fail(cudaGetLastError(), "cudaDeviceGetAttribute"); break;
         }
-        h->B = B; h->n = n; h->M = M; h->omax = omax; h->least = least; h->volume = volume; h->sum_o_max = sum_max;
+        h->B = B; h->n = n; h->M = M; h->omax = omax; h->omin = omin; h->least = least; h->volume = volume; h->brief_tokens = (double)brief; h->sum_o_max = sum_max;
         h->mean_s = some_s / looked_at; h->mean_o = some_o / looked_at; h->short_share = short_o / looked_at;
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
@@ -559,7 +561,7 @@ bool short_windows(const sched_ctx* h, bool want_starts) { return !want_starts &
 //   longer than a decode: otherwise nearly everything runs side by side.
 // Longer decodes than its ring of events, schedules with more rounds per request than
 // were measured (14.8 for decodes beyond 1,025), and backlogs whose candidate could pass 32 bits of waiting
-// time in its sum of starts keep the warp.
+// time in its sum of starts or of tokens in a chunk (lane_sums_fit) keep the warp.
 constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.55;
 
 // candidates from which on a thread each is the faster one
@@ -586,9 +588,19 @@ double lanes_from(const sched_ctx* h) {
     return need;
 }
 
+// A thread keeps the bound of the chunk that t lies in, and its cells less the ramps that have come in since, in 32 bits.
+// Both take s + 1 and up to a chunk's rounds from every request that starts in the chunk: those that outlast it
+// hold M tokens at most, those that end in it M per round of the chunk.  Beyond 2^30 (budgets from 2^24 on, and then
+// only with decodes of a few rounds) the warp has to do it: its cells are exact.
+bool lane_sums_fit(const sched_ctx* h) {
+    const double rounds = h->nm == 1 ? 32.0 : 64.0, M = (double)h->M;
+    const double ends = fmin(h->brief_tokens, M * rounds / h->omin), starts = fmin((double)h->n, 0.5 * (ends + M));
+    return 2.0 * M + ends + rounds * (starts + 2.0) < 1073741824.0;
+}
+
 bool lanes_fit(const sched_ctx* h, i64 count, bool want_starts) {
     if (want_starts || (h->nm != 1 && h->nm != 2) || count <= ordered_from(h)) return false;
-    return (double)count >= lanes_from(h) && (i64)h->n * (h->omax + 64) <= INT32_MAX;
+    return (double)count >= lanes_from(h) && (i64)h->n * (h->omax + 64) <= INT32_MAX && lane_sums_fit(h);
 }
 
 // The handle's block of rings in device memory, of at least `bytes`; false if there is no memory for it.

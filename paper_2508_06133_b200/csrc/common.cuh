@@ -28,6 +28,8 @@ struct sched_ctx {
     i64 M;
     int omax;                // largest decode length over all instances
     int least;               // smallest s+o over all instances
+    int omin;                // smallest decode length
+    double brief_tokens;     // sum of s + 1 over the decodes of fewer than 64 rounds
     double volume;           // tokens times rounds: sum of s o + o^2 / 2 over all instances
     double mean_s, mean_o;   // of some 4,096 requests spread over all instances
     double short_share;      // mean of min(1, 32 / o) over the same

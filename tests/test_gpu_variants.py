@@ -271,6 +271,29 @@ def test_moves_by_lanes(omax, least):
         assert (tel[0] == np.concatenate(parts)).all()
 
 
+@pytest.mark.parametrize("M,omax,thread", [(1 << 23, 2, True), (1 << 24, 3, True), (1 << 26, 2, False), (1 << 27, 40, False),
+                                           ((1 << 30) - 1, 2, False), ((1 << 30) - 1, 1500, False), (1 << 28, 1500, True)])
+def test_moves_on_the_largest_budgets(M, omax, thread):
+    """Prefills of a third of the budget and less, with decodes of one and more rounds: the tokens of all that starts in the
+    rounds of one chunk pass 32 bits.  Those backlogs keep the warp; the others (the last one has no decode below 700) are
+    counted right by a thread each."""
+    rng = np.random.default_rng(omax)
+    n = 150
+    least, most = (M // 60, M // 40) if omax == 1500 else (M // 5, M // 3)
+    s = rng.integers(least, most, n).astype(np.int32)
+    o = rng.integers(700 if thread and omax == 1500 else 1, omax + 1, n).astype(np.int32)
+    o[::20] = omax
+    base = rng.permutation(n).astype(np.int32)
+    codes = np.arange(3 * n * (n - 1) // 2, dtype=np.int64)
+    with kv.Scheduler(s, o, M) as h:
+        h.set_base_order(base)
+        (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, np.tile(codes, 5)))
+    assert ("k3_lane_moves" in names) == thread, names
+    tel = tel.reshape(5, -1)
+    assert (tel == tel[0]).all()
+    assert (tel[0, ::11] == oracle_moves(s, o, M, base, codes[::11])).all()
+
+
 @pytest.mark.parametrize("omax,median,smax,rounds,count,thread", [
     (1024, 200, 4000, 3.0, 24000, True), (1024, 200, 4000, 3.0, 18000, False),
     (64, 16, 2000, 2.0, 40000, False), (64, 16, 2000, 2.0, 95000, True),      # short decodes
