@@ -262,6 +262,26 @@ int k3_warps(const sched_ctx* h) {
     return w;
 }
 
+// The base run's kernel for a handle (sim_chunk.cuh, run_alone): a form each for backlogs of which more than half decode for up
+// to 64 rounds and more than a quarter for 1,025 and more.
+typedef void (*BaseRunKernel)(BaseRunParams);
+template <int NM>
+BaseRunKernel base_run_form(const sched_ctx* h) {
+    typedef ChunkSim<NM> S;
+    if (h->brief_share > 0.5) return k3_base_run<S, S::kBrief>;
+    if (NM > 1 && h->lengthy_share > 0.25) return k3_base_run<S, (NM > 1 ? S::kLengthy : S::kPlain)>;
+    return k3_base_run<S, S::kPlain>;
+}
+BaseRunKernel base_run_kernel(const sched_ctx* h) {
+    switch (h->nm) {
+        case 1: return base_run_form<1>(h);
+        case 2: return base_run_form<2>(h);
+        case 4: return base_run_form<4>(h);
+        case 8: return base_run_form<8>(h);
+        default: return k3_base_run<HybSim, -1>;
+    }
+}
+
 size_t k3_smem_bytes(const sched_ctx* h) { return (size_t)k3_warps(h) * h->ring_cells * sizeof(int); }
 
 // A sort of rows of n entries merges more than once: it needs a second pair of buffers.
@@ -298,9 +318,10 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         if (sum > sum_max) sum_max = sum;
     }
     // of some 4,096 requests spread over all: enough for a rule, and these sums over all of 1,000,000 are 2 ms
-    double short_o = 0, some_s = 0, some_o = 0, looked_at = 0;
+    double short_o = 0, brief_o = 0, lengthy_o = 0, some_s = 0, some_o = 0, looked_at = 0;
     for (i64 k = 0, step = 1 + total / 4096; k < total; k += step) {
         short_o += o[k] <= 32 ? 1.0 : 32.0 / o[k];
+        brief_o += o[k] <= 64; lengthy_o += o[k] > 1024;
         some_s += s[k]; some_o += o[k]; looked_at += 1.0;
     }
     if (sum_max + omax >= (1ll << 30)) return SCHED_E_UNSUPPORTED;
@@ -317,6 +338,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         }
         h->B = B; h->n = n; h->M = M; h->omax = omax; h->omin = omin; h->least = least; h->volume = volume; h->brief_tokens = (double)brief; h->sum_o_max = sum_max;
         h->mean_s = some_s / looked_at; h->mean_o = some_o / looked_at; h->short_share = short_o / looked_at;
+        h->brief_share = brief_o / looked_at; h->lengthy_share = lengthy_o / looked_at;
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
         h->nm = slots <= 32 ? 1 : slots <= 256 ? slots / 32 : 0;
@@ -406,7 +428,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
             if (e2 == cudaSuccess) e2 = cudaFuncSetAttribute(k3_eval_orders<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn); \
             e3 = cudaFuncSetAttribute(k3_eval_policy<N, int>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn - 2048); \
             if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(k3_eval_policy<N, i64>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn - 2048); \
-            e4 = cudaFuncSetAttribute(k3_base_run<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)
+            e4 = cudaFuncSetAttribute(base_run_kernel(h), cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)
             KV_DISPATCH_SIM(h, SETATTR);
 #undef SETATTR
             if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess) {
@@ -466,9 +488,7 @@ BaseRunParams base_run_params(sched_ctx* h) {
 }
 
 int run_base(sched_ctx* h, const BaseRunParams& p) {
-#define RUN(N) k3_base_run<N><<<1, K3B_THREADS, (size_t)h->ring_cells * sizeof(int), h->stream>>>(p)
-    KV_DISPATCH_SIM(h, RUN);
-#undef RUN
+    base_run_kernel(h)<<<1, K3B_THREADS, (size_t)h->ring_cells * sizeof(int), h->stream>>>(p);
     return check_launch(h);
 }
 

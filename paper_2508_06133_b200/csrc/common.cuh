@@ -33,6 +33,7 @@ struct sched_ctx {
     double volume;           // tokens times rounds: sum of s o + o^2 / 2 over all instances
     double mean_s, mean_o;   // of some 4,096 requests spread over all instances
     double short_share;      // mean of min(1, 32 / o) over the same
+    double brief_share, lengthy_share;   // decodes of up to 64 and of more than 1,024 rounds among the same
     int L;                   // ints per simulator state
     int nm;                  // chunked simulator with this many far registers per lane; 0: hybrid simulator
     int ring_cells;          // shared-memory ints one simulator needs

@@ -123,7 +123,7 @@ __device__ bool k3_accept(const BaseRunParams& p) {
     return true;
 }
 
-template <class SIM>
+template <class SIM, int kForm>
 __global__ void __launch_bounds__(K3B_THREADS)
 k3_base_run(const BaseRunParams p) {
     if (p.accept && !k3_accept(p)) return;
@@ -144,6 +144,8 @@ k3_base_run(const BaseRunParams p) {
     i64 tel = 0;                                         // this lane's share of the completion times so far
     int2 next = lane < n ? tbl_base[lane] : make_int2(1, 1);
     int to_snap = 0, idx = 0;                            // positions until the next snapshot, its number
+    bool calm = true;                                    // nothing has waited, or not since the last snapshot
+    int t_snap = 0;
     for (int q0 = 0; q0 < n;) {
         const int2 so = next;
         // a block ends where a snapshot is due
@@ -154,10 +156,14 @@ k3_base_run(const BaseRunParams p) {
             sim.store(snap_ring + (size_t)i * L, snap_hdr + i, before);
             ++idx;
             to_snap = stride;
+            calm = calm || (sim.start() == t_snap && (idx & 7) == 0);        // a mistake costs a block of four
+            t_snap = sim.start();
         }
         const int cnt = min(min(32, n - q0), to_snap);
         if (q0 + cnt + lane < n) next = tbl_base[q0 + cnt + lane];
-        const int mine = sim.template run<true>(so, cnt, status);
+        int mine;
+        if constexpr (kForm < 0) mine = sim.run(so, cnt, status);
+        else mine = calm ? sim.run_together(so, cnt, calm, status) : sim.template run_alone<kForm>(so, cnt, status);
         if (lane < cnt) base_starts_pos[q0 + lane] = mine;
         if (lane < cnt) tel += (i64)mine + so.y;
         q0 += cnt;
@@ -230,7 +236,7 @@ k3_eval_moves(const MoveEvalParams p) {
         }
         const int cnt = min(32, n - q0);
         if (lane < cnt) sum_o += so.y;
-        const int mine = sim.template run<false>(so, cnt, p.status);
+        const int mine = sim.run(so, cnt, p.status);
         if (kStarts && lane < cnt) starts[KV_IDX(id, n, 405)] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
@@ -308,7 +314,7 @@ k3_eval_orders(const OrderEvalParams p) {
         }
         const int cnt = min(32, n - q0);
         if (lane < cnt) sum_o += so.y;
-        const int mine = sim.template run<false>(so, cnt, p.status);
+        const int mine = sim.run(so, cnt, p.status);
         if (kStarts && lane < cnt) starts[id] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);

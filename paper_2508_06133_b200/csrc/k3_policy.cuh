@@ -213,7 +213,7 @@ k3_eval_policy(const int* __restrict__ s_all, const int* __restrict__ o_all, int
         int2 so = make_int2(1, 1);
         const int cnt = min(32, n - q0);
         if (lane < cnt) { id = (int)KV_IDX(fin[q0 + lane], n, 906); so = make_int2(s[id], o[id]); sum_o += so.y; }
-        const int mine = sim.template run<false>(so, cnt, status);
+        const int mine = sim.run(so, cnt, status);
         if (starts && lane < cnt) starts[id] = mine;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);

@@ -38,11 +38,16 @@
 // 75 to 95 of them; the exact wait, windows of 64 rounds and more without masks, and two turns of the loop in a row leave 60
 // to 80.  Sweeps with a warp each: 16,384 moves of 10,000 requests (decodes to 1,024) 8.71 -> 7.26 ms, 16,000
 // of 1,000 1.23 -> 1.01 ms, 7,000 of 100,000 (decodes to 4,096) 40.5 -> 35.9 ms.  One run
-// that stands alone (run<true>) is bound by the latency of one admission: the part behind the two chunks is put while the
+// that stands alone (run_alone) is bound by the latency of one admission: the part behind the two chunks is put while the
 // next request's reduction is under way, and a branch on fresh data costs 28 cycles, so there is one.  Cycles per
-// admission 367 -> 216 (1,000 requests, 13 rounds per request), 278 -> 150 (10,000, 3 rounds), 269 -> 157 (100,000, 1 round).
-// Tried without gain: two to eight requests in a row without a branch (their conditions cost more: 172 to 257 for
-// the 10,000), t moving over several chunks at once (sweeps 82 -> 85 issue slots per admission).
+// admission 367 -> 216 (1,000 requests, 13 rounds per request), 278 -> 150 (10,000, 3 rounds), 269 -> 155 (100,000, 1 round).
+// Three kinds of backlog leave that loop for nearly every request, at the price of two branches and a second question, so
+// they have loops of their own, which cost the others up to 0.03 (10,000 requests, cycles per admission with the loop
+// for the rest -> theirs): nothing waits (run_together: decodes to 2,048 rounds 236 -> 155, to 1,024 148 -> 116); windows of less
+// than 64 rounds wait inside the chunk (kBrief: up to 20 rounds, one beside the other, 758 -> 300; up to 64, 706 -> 433);
+// windows of 1,025 rounds and more (kLengthy: half of them such, 0.05 / 1 rounds per request, 236 -> 202 / 336 -> 267).
+// Tried without gain: two to eight requests in a row without a branch where some of them wait (their conditions cost more:
+// 172 to 257 for the 10,000), t moving over several chunks at once (sweeps 82 -> 85 issue slots per admission).
 //
 // Sums may wrap; V itself fits 31 bits (the host checks M, sum of o and n), so arithmetic modulo 2^32
 // gives it exactly.
@@ -64,6 +69,7 @@ struct ChunkSim {
     static constexpr int kMeta = 64 + 96 * NM;                      // state ints besides the ring
     __host__ __device__ static constexpr int ring_cells(int L) { return L - kMeta; }   // shared-memory ints per warp
     static constexpr int kAsk = 128;                                // "look closer": above every wait in the two chunks
+    enum { kPlain, kBrief, kLengthy };                              // forms of run_alone, see there
     static constexpr int kLong = 64;                                // om from which every window covers what is left of the two chunks and ends behind them
 
     int lane;
@@ -291,6 +297,19 @@ struct ChunkSim {
         raise(cells_of(last), a + x, last >= 64 && x <= last);
     }
 
+    // Whether requests of `size` tokens in all (s + o each), the longest with om = o - 1, certainly fit at t
+    // one beside the other: none of them uses more than its s + o in any round.
+    __device__ __forceinline__ bool surely(int size, int om) const {
+        const int a0 = size - tau, last = tau + om;
+        bool over = lane >= tau && lane <= last && cur > -a0;
+        over = over || (lane + 32 <= last && nxt > -a0) || (X <= last && a0 > W[0]);
+        if (NM > 1 && om >= 1024) {
+#pragma unroll
+            for (int m = 1; m < NM; ++m) over = over || (X + 1024 * m <= last && a0 > W[m]);
+        }
+        return !__any_sync(KV_FULL, over);
+    }
+
     // Takes back what is left (from t on) of a window whose ramp is a + x in round x, counted from T0, and whose last
     // round is `last`.  The bounds fall by the least the ramp has in a chunk it covers whole.
     __device__ __forceinline__ void remove(int a, int last) {
@@ -319,92 +338,163 @@ struct ChunkSim {
 
     // Up to 32 consecutive requests of a list, each at its earliest start: (s, o) of the k-th in lane k.  Returns
     // the start of the k-th in lane k.
-    template <bool kAlone>
     __device__ __forceinline__ int run(int2 so, int cnt, int* status) {
         const int sp_l = so.x + 1, om_l = so.y - 1, T_first = T0;
         const int cap = kv_loop_cap(32 * mask + 2048);
         int mine = 0, k = 0, turns = 0;
         acc = 0;
-        if constexpr (kAlone) {
-            int sp = __shfl_sync(KV_FULL, sp_l, 0), om = __shfl_sync(KV_FULL, om_l, 0);
-            int pa = 0, plast = -1;                      // the admission whose part behind the two chunks is still to be put
-            auto put_far = [&]() {
-                if (X + 31 < plast) { A[0] += pa; C[0] += 1; }
-                const int x = (plast & ~31) + lane;
-                raise(cells_of(plast), pa + x, plast >= 64 && x <= plast);
-            };
-            for (;;) {
-                int v, sp_next, om_next;
-                for (;;) {
-                    const int a0 = sp - tau, end = tau + om, r = lane + 1 - tau;
-                    v = __viaddmin_s32(cur, a0, lane <= end ? r : 0);
-                    v = max(v, __viaddmin_s32(nxt, a0, lane + 32 <= end ? r + 32 : 0));
-                    if (X - 64 <= om && a0 > W[0]) v = kAsk;
-                    v = kv_warp_max(v);
-                    put_far();
-                    plast = -1;
-                    sp_next = __shfl_sync(KV_FULL, sp_l, (k + 1) & 31); om_next = __shfl_sync(KV_FULL, om_l, (k + 1) & 31);
-                    const int most = NM > 1 && om >= 1024 ? -1 : om >= kLong ? 31 : tau;
-                    const int at = __viaddmax_s32(v, tau, tau);
-                    if (at > most) break;
-                    tau = at;
-                    pa = sp - tau; plast = tau + om;
-                    if (lane >= tau && lane <= plast) cur += pa + lane;
-                    if (lane + 32 <= plast) nxt += pa + (lane + 32);
-                    if (X <= plast) W[0] -= pa + (X + 31);
-                    if (lane == k) mine = T0 + tau;
-                    acc += (unsigned)tau;
-                    turns = 0;
-                    sp = sp_next; om = om_next;
-                    if (++k >= cnt) break;
-                }
-                if (k >= cnt) break;
-                bool in = false;
-                if (NM > 1 && om >= 1024) {
-                    v = ask<true>(sp, om);
-                    in = tau + v <= 31;
-                    if (in) { tau += max(v, 0); put<true>(sp, om); }
-                }
-                if (in || step(sp, om, v, cnt - k)) {
-                    if (lane == k) mine = T0 + tau;
-                    acc += (unsigned)tau;
-                    turns = 0;
-                    sp = sp_next; om = om_next;
-                    if (++k >= cnt) break;
-                } else if (++turns > cap) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
-            }
-            put_far();
-        } else {
-            for (;;) {
-                int sp = 0, om = 0, v = 0;
+        for (;;) {
+            int sp = 0, om = 0, v = 0;
 #pragma unroll 2
-                for (; k < cnt; ++k) {                   // as long as t stays in its chunk and no far bound is in the way
-                    sp = __shfl_sync(KV_FULL, sp_l, k); om = __shfl_sync(KV_FULL, om_l, k);
-                    if (om >= kLong) {
-                        v = ask<true>(sp, om);
-                        const int at = __viaddmax_s32(v, tau, tau);
-                        if (at > 31) break;
-                        tau = at;
-                        put<true>(sp, om);
-                    } else {
-                        for (;;) {                       // a wait inside the chunk: ask again from there
-                            v = ask<false>(sp, om);
-                            if (kGlobal || v <= 0 || tau + v > 31) break;
-                            tau += v;
-                        }
-                        if (v > 0) break;
-                        put<false>(sp, om);
+            for (; k < cnt; ++k) {                   // as long as t stays in its chunk and no far bound is in the way
+                sp = __shfl_sync(KV_FULL, sp_l, k); om = __shfl_sync(KV_FULL, om_l, k);
+                if (om >= kLong) {
+                    v = ask<true>(sp, om);
+                    const int at = __viaddmax_s32(v, tau, tau);
+                    if (at > 31) break;
+                    tau = at;
+                    put<true>(sp, om);
+                } else {
+                    for (;;) {                       // a wait inside the chunk: ask again from there
+                        v = ask<false>(sp, om);
+                        if (kGlobal || v <= 0 || tau + v > 31) break;
+                        tau += v;
                     }
-                    acc += (unsigned)tau;
-                    if (lane == k) mine = T0 + tau;
+                    if (v > 0) break;
+                    put<false>(sp, om);
                 }
-                if (k >= cnt) break;
-                if (step(sp, om, v, cnt - k)) {
-                    acc += (unsigned)tau;
-                    if (lane == k) mine = T0 + tau;
-                    ++k;
-                    turns = 0;
-                } else if (++turns > cap) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
+                acc += (unsigned)tau;
+                if (lane == k) mine = T0 + tau;
+            }
+            if (k >= cnt) break;
+            if (step(sp, om, v, cnt - k)) {
+                acc += (unsigned)tau;
+                if (lane == k) mine = T0 + tau;
+                ++k;
+                turns = 0;
+            } else if (++turns > cap) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
+        }
+        tel += (i64)T_first * cnt + (i64)acc;
+        return mine;
+    }
+
+    // The same for a run that stands alone: one branch for a request that neither waits for another chunk nor meets a far
+    // bound.  What leaves the loop otherwise, and stays in it by kForm: kBrief: a window of less than 64 rounds that
+    // waits inside the chunk; kLengthy: windows of 1,025 rounds and more.
+    template <int kForm>
+    __device__ __forceinline__ int run_alone(int2 so, int cnt, int* status) {
+        constexpr bool kBriefs = kForm == kBrief, kFar = NM > 1 && kForm == kLengthy;
+        const int sp_l = so.x + 1, om_l = so.y - 1, T_first = T0;
+        const int cap = kv_loop_cap(32 * mask + 2048);
+        // far rounds that may matter: a short window ends in round om + 31 at the latest, a long one waits for up to 64.
+        // From the lane that has it: worked out in every turn it lies in front of the reduction.
+        const int far_l = om_l + (om_l >= kLong ? 64 : 31);
+        int mine = 0, k = 0, turns = 0;
+        acc = 0;
+        int sp = __shfl_sync(KV_FULL, sp_l, 0), om = __shfl_sync(KV_FULL, om_l, 0), far_to = kBriefs ? __shfl_sync(KV_FULL, far_l, 0) : 0;
+        int pa = 0, plast = -1;                          // the admission whose part behind the two chunks is still to be put
+        auto put_far = [&]() {
+            if (X + 31 < plast) { A[0] += pa; C[0] += 1; }
+            const int x = (plast & ~31) + lane;
+            raise(cells_of(plast), pa + x, plast >= 64 && x <= plast);
+        };
+        while (kForm == kPlain || k < cnt) {             // of the two ways to write it the faster one for each form, by up to a half
+            int v, sp_next, om_next, far_next = 0;
+            for (;;) {
+                const int a0 = sp - tau, end = tau + om, r = lane + 1 - tau;
+                v = __viaddmin_s32(cur, a0, lane <= end ? r : 0);
+                v = max(v, __viaddmin_s32(nxt, a0, lane + 32 <= end ? r + 32 : 0));
+                if ((kBriefs ? X <= far_to : X - 64 <= om) && a0 > W[0]) v = kAsk;
+                if (kFar && om >= 1024) {
+#pragma unroll
+                    for (int m = 1; m < NM; ++m) if (X + 1024 * m - om <= 64 && a0 > W[m]) v = kAsk;
+                }
+                v = kv_warp_max(v);
+                put_far();
+                plast = -1;
+                sp_next = __shfl_sync(KV_FULL, sp_l, (k + 1) & 31); om_next = __shfl_sync(KV_FULL, om_l, (k + 1) & 31);
+                if (kBriefs) far_next = __shfl_sync(KV_FULL, far_l, (k + 1) & 31);
+                const int most = NM > 1 && !kFar && om >= 1024 ? -1 : om >= kLong ? 31 : tau;
+                const int at = __viaddmax_s32(v, tau, tau);
+                if (at > most) {
+                    if (!kBriefs || om >= kLong || at > 31) break;
+                    tau = at;                            // asked again from there
+                    continue;
+                }
+                tau = at;
+                pa = sp - tau; plast = tau + om;
+                if (lane >= tau && lane <= plast) cur += pa + lane;
+                if (lane + 32 <= plast) nxt += pa + (lane + 32);
+                if (X <= plast) W[0] -= pa + (X + 31);
+                if (kFar && om >= 1024) {
+#pragma unroll
+                    for (int m = 1; m < NM; ++m) {
+                        if (X + 1024 * m <= plast) W[m] -= pa + (X + 1024 * m + 31);
+                        if (X + 1024 * m + 31 < plast) { A[m] += pa; C[m] += 1; }
+                    }
+                }
+                if (lane == k) mine = T0 + tau;
+                acc += (unsigned)tau;
+                turns = 0;
+                sp = sp_next; om = om_next; far_to = far_next;
+                if (++k >= cnt) break;
+            }
+            if (k >= cnt) break;
+            bool in = false;
+            if (NM > 1 && !kFar && om >= 1024) {
+                v = ask<true>(sp, om);
+                in = tau + v <= 31;
+                if (in) { tau += max(v, 0); put<true>(sp, om); }
+            }
+            if (in || step(sp, om, v, cnt - k)) {
+                if (lane == k) mine = T0 + tau;
+                acc += (unsigned)tau;
+                turns = 0;
+                sp = sp_next; om = om_next; far_to = far_next;
+                ++k;
+                if (kForm == kPlain && k >= cnt) break;
+            } else if (++turns > cap) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
+        }
+        put_far();
+        tel += (i64)T_first * cnt + (i64)acc;
+        return mine;
+    }
+
+    // The same where nothing has waited for a while: four at a time are asked for together and put without a question each, as
+    // long as that goes well; calm tells afterwards whether it did.
+    __device__ __forceinline__ int run_together(int2 so, int cnt, bool& calm, int* status) {
+        constexpr int kMost = (1 << 29) - 1;             // four of them fit 31 bits; a group of so much is none
+        const int sp_l = so.x + 1, om_l = so.y - 1, t_first = T0 + tau, T_first = T0;
+        int size = min(so.x + so.y, kMost), longest = om_l;                  // of the aligned four this lane is in
+        size += __shfl_xor_sync(KV_FULL, size, 1); size += __shfl_xor_sync(KV_FULL, size, 2);
+        if (size >= kMost) size = INT_MAX;
+        longest = max(longest, __shfl_xor_sync(KV_FULL, longest, 1));
+        longest = max(longest, __shfl_xor_sync(KV_FULL, longest, 2));
+        int mine = 0, k = 0, turns = 0;
+        acc = 0;
+        for (; calm && k + 4 <= cnt; k += 4) {
+            int s4[4], o4[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { s4[j] = __shfl_sync(KV_FULL, sp_l, k + j); o4[j] = __shfl_sync(KV_FULL, om_l, k + j); }
+            calm = surely(__shfl_sync(KV_FULL, size, k), __shfl_sync(KV_FULL, longest, k));
+            if (!calm) break;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) add(s4[j], o4[j]);
+            acc += 4u * (unsigned)tau;
+        }
+        if (lane < k) mine = t_first;
+        while (k < cnt) {
+            const int sp = __shfl_sync(KV_FULL, sp_l, k & 31), om = __shfl_sync(KV_FULL, om_l, k & 31), v = need(sp, om);
+            if (v <= 0) {
+                add(sp, om);
+                if (lane == k) mine = T0 + tau;
+                acc += (unsigned)tau;
+                ++k;
+                turns = 0;
+            } else {
+                calm = false;
+                advance(v, cnt - k);
+                if (++turns > kv_loop_cap(32 * mask + 2048)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
             }
         }
         tel += (i64)T_first * cnt + (i64)acc;

@@ -134,7 +134,6 @@ struct HybSim {
     static constexpr int kWarps = 24;                 // 33 timeline registers + the ring bookkeeping need more than 64 registers
     static constexpr int kMinCtas = 1;
     static constexpr bool kGlobal = false;
-    static constexpr bool kGroups = false;
     __host__ __device__ static constexpr int ring_cells(int L) { return L - 32 * NREG; }
 
     int R[NREG];
@@ -310,7 +309,6 @@ struct HybSim {
     }
 
     // Up to 32 consecutive requests of a list, (s, o) of the k-th in lane k.  Returns the start of the k-th in lane k.
-    template <bool kAlone>
     __device__ __forceinline__ int run(int2 so, int cnt, int* status) {
         const int sp = so.x + 1, om = so.y - 1;
         int mine = 0;

@@ -85,6 +85,39 @@ def test_waits_in_and_behind_the_near_chunks(omax, beside):
     assert (mtel == oracle_moves(s, o, M, orders[0], codes)).all()
 
 
+@pytest.mark.parametrize("omax,beside", [(1, 1), (20, 1), (20, 3), (64, 2), (64, 400), (300, 1), (1024, 400), (2049, 400), (4097, 60),
+                                         (8193, 400), (8194, 20)])
+def test_runs_that_stand_alone(omax, beside):
+    """The base run where nothing waits (requests go four at a time), where a burst of large requests ends that and small
+    ones begin it again, and where nearly every request waits for a few rounds: TEL, and moves from its snapshots."""
+    rng = np.random.default_rng(omax + beside)
+    n = 397
+    o = rng.integers(1, omax + 1, n).astype(np.int32)
+    s = rng.integers(1, 40, n).astype(np.int32)
+    o[100:110] = o[301] = omax
+    s[100:110] += 20 * omax
+    M = max(int((s + o).max()), int(beside * (s + o).mean()))
+    codes = np.arange(0, 3 * n * (n - 1) // 2, 1999, dtype=np.int64)
+    for base in (np.arange(n, dtype=np.int32), rng.permutation(n).astype(np.int32)):
+        with kv.Scheduler(s, o, M) as h:
+            final, tel, _, _ = h.local_search(kv.NBHD_SWAP, 0, order=base)
+            mtel = h.eval_batch(kv.CAND_MOVE, codes)[0]
+        assert (final == base).all() and tel == orc.list_schedule_rounds(s, o, M, base)[1]
+        assert (mtel == oracle_moves(s, o, M, base, codes)).all()
+
+
+@pytest.mark.parametrize("part", [2, 3, 8])
+def test_runs_that_stand_alone_on_the_largest_budget(part):
+    """Four requests in a row hold more tokens than 31 bits count."""
+    M, n = (1 << 30) - 1, 70
+    rng = np.random.default_rng(part)
+    s = (M // part - rng.integers(20, 60, n)).astype(np.int32)
+    o = rng.integers(1, 20, n).astype(np.int32)
+    base = rng.permutation(n).astype(np.int32)
+    with kv.Scheduler(s, o, M) as h:
+        assert h.local_search(kv.NBHD_SWAP, 0, order=base)[1] == orc.list_schedule_rounds(s, o, M, base)[1]
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 127, 128, 129, 400, 4096])
 def test_amin_running_lists(n):
     """Evictions from lists of running requests at and beside the multiples of what the warps of a CTA look at
