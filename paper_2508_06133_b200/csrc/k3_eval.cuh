@@ -369,8 +369,7 @@ k3_check_starts(const StartsEvalParams p) {
             const int wait = __shfl_sync(KV_FULL, pi, k) - sim.start();
             if (wait < 0) { ok = false; break; }
             if (wait > 0) sim.skip(wait, M);
-            if (sim.need(sp, om) > 0) ok = false;
-            else sim.add(sp, om);
+            ok = sim.put_if_fits(sp, om);
         }
     }
     for (int d = 16; d >= 1; d >>= 1) tel += __shfl_xor_sync(KV_FULL, tel, d);

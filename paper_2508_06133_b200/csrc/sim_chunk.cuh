@@ -297,8 +297,8 @@ struct ChunkSim {
         raise(cells_of(last), a + x, last >= 64 && x <= last);
     }
 
-    // Whether requests of `size` tokens in all (s + o each), the longest with om = o - 1, certainly fit at t
-    // one beside the other: none of them uses more than its s + o in any round.
+    // Whether a request of (size, om) certainly fits at t; or several, `size` the sum of their s + o, the longest with
+    // om = o - 1, one beside the other: none of them uses more than its s + o in any round.
     __device__ __forceinline__ bool surely(int size, int om) const {
         const int a0 = size - tau, last = tau + om;
         bool over = lane >= tau && lane <= last && cur > -a0;
@@ -308,6 +308,23 @@ struct ChunkSim {
             for (int m = 1; m < NM; ++m) over = over || (X + 1024 * m <= last && a0 > W[m]);
         }
         return !__any_sync(KV_FULL, over);
+    }
+
+    // Starts (sp, om) at t if it fits there: a vote, since no wait is asked for, and no second chunk for a window that is put
+    // in the first.  Windows of 64 rounds and more take a path of their own as long as their bounds are one register (with more of
+    // them, on fewer warps, it was no gain).  2,000 schedules of 1,000 requests, decodes to 20 / 256 / 1,024 / 4,096, with the
+    // question that answers a wait -> this: 428 -> 304, 366 -> 311, 367 -> 331, 522 -> 510 us.
+    __device__ __forceinline__ bool put_if_fits(int sp, int om) {
+        const int a0 = sp - tau, last = tau + om;
+        if (NM == 1 && om >= kLong) {
+            const bool over = (lane >= tau && cur > -a0) || nxt > -a0 || (X <= last && a0 > W[0]);
+            if (__any_sync(KV_FULL, over) && test(sp, om) > 0) return false;
+            put<true>(sp, om);
+            return true;
+        }
+        if (!surely(sp, om) && test(sp, om) > 0) return false;
+        if (NM == 1) put<false>(sp, om); else add(sp, om);
+        return true;
     }
 
     // Takes back what is left (from t on) of a window whose ramp is a + x in round x, counted from T0, and whose last
