@@ -296,6 +296,13 @@ size_t result_bytes(int n) { return offsets_at(n) + ((size_t)n + 1) * sizeof(int
 // copied from and to the caller's memory (pinning 128 MB for 10,000,000 requests takes sched_init 100 ms).
 bool reads_through_pinned(int n) { return 256 + result_bytes(n) <= ((size_t)32 << 20); }
 
+// The chunked simulator's bounds are a round (below 2^30, as are M and the sum of all decodes) plus tokens in use (M) plus
+// at most 31 for every request that is resident at the same time (two tokens each): V fits 31 bits, and its bound has to.
+bool chunk_sums_fit(i64 n, i64 M) {
+    const i64 beside = n < M / 2 ? n : M / 2;
+    return M + 32 * n + 32768 < (1ll << 31) && (1ll << 30) + 31 * beside + 65536 < (1ll << 31);
+}
+
 int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t* o, i64 M) {
     if (!out) return SCHED_E_INVAL;
     *out = nullptr;
@@ -342,8 +349,7 @@ int create_common(sched_ctx** out, int B, int n, const int32_t* s, const int32_t
         h->g_num = 0; h->g_den = 1;
         const int slots = sim_pick_slots(omax);
         h->nm = slots <= 32 ? 1 : slots <= 256 ? slots / 32 : 0;
-        // the chunked simulator's bounds (M, rounds ahead, at most 31 more per admission) have to fit 31 bits
-        if (M + 32ll * n + 32768 >= (1ll << 31)) h->nm = 0;
+        if (!chunk_sums_fit(n, M)) h->nm = 0;
         if (const char* kind = getenv("KVSCHED_SIM"))               // testing knob: force the hybrid simulator
             if (strcmp(kind, "hybrid") == 0) h->nm = 0;
         // ints per simulator state, and the part of it that lives in shared memory

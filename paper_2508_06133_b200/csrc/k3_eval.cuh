@@ -301,7 +301,7 @@ k3_eval_orders(const OrderEvalParams p) {
     const int* ord = p.orders + (size_t)c * n;
     int* starts = kStarts ? p.starts_out + (size_t)c * n : nullptr;
     sim.reset(M);
-    int bad = 0;
+    int bad = 0, base = 0;                                // rounds are counted from `base` on (0 in permutations)
     i64 sum_o = 0;
     for (int q0 = 0; q0 < n; q0 += 32) {
         const int qq = q0 + lane;
@@ -313,9 +313,10 @@ k3_eval_orders(const OrderEvalParams p) {
             return;
         }
         const int cnt = min(32, n - q0);
-        if (lane < cnt) sum_o += so.y;
+        base += sim.rebase();
+        if (lane < cnt) sum_o += (i64)so.y + (unsigned)base;
         const int mine = sim.run(so, cnt, p.status);
-        if (kStarts && lane < cnt) starts[id] = mine;
+        if (kStarts && lane < cnt) starts[id] = mine + base;
     }
     for (int d = 16; d >= 1; d >>= 1) sum_o += __shfl_xor_sync(KV_FULL, sum_o, d);
     if (lane == 0) p.tel_out[c] = sim.total(sum_o);
@@ -356,6 +357,7 @@ k3_check_starts(const StartsEvalParams p) {
     sim.reset(M);
     i64 tel = 0;
     bool ok = true;
+    int base = 0;                                                              // rounds are counted from here on
     int id_next = lane < n ? ids[lane] : 0;
     for (int q0 = 0; q0 < n; q0 += 32) {
         const int cnt = min(32, n - q0), id = id_next;
@@ -364,11 +366,13 @@ k3_check_starts(const StartsEvalParams p) {
         int pi = 0;
         if (lane < cnt) { so = p.tbl_id[KV_IDX(id, n, 407)]; pi = st_c[id]; tel += (i64)pi + so.y; }
         if (__any_sync(KV_FULL, pi < 0)) ok = false;                           // the simulator cannot go back
+        base += sim.rebase();
         for (int k = 0; k < cnt && ok; ++k) {
             const int sp = __shfl_sync(KV_FULL, so.x, k) + 1, om = __shfl_sync(KV_FULL, so.y, k) - 1;
-            const int wait = __shfl_sync(KV_FULL, pi, k) - sim.start();
+            const int wait = __shfl_sync(KV_FULL, pi, k) - base - sim.start();
             if (wait < 0) { ok = false; break; }
-            if (wait > 0) sim.skip(wait, M);
+            if (wait > sim.mask + 128) { base += sim.start() + wait; sim.reset(M); }          // nothing is resident any more
+            else if (wait > 0) sim.advance(wait);
             ok = sim.put_if_fits(sp, om);
         }
     }

@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
         // decision (or ends the run).
         const int head_s = head < n ? ps[head] : 0;
         for (;;) {
-            const bool live = lane >= sim.tau;
-            const int round = sim.T0 + lane, k = round & mask;
+            const bool live = sim.x0 >= sim.t;
+            const int round = sim.x0, k = round & mask;
             int es = live ? ev[k] : 0;
             unsigned as = live ? dA[k] : 0u;
             if (__any_sync(KV_FULL, es != 0 || as != 0u)) {
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             }
             const unsigned cnt_l = cnt + (unsigned)(es >> 16), A_l = A + as;
             const int rem_l = remaining - (es & 0xffff);
-            const int u = sim.cur + M - lane + (int)(A_l + cnt_l * (unsigned)round);
+            const int u = sim.cur + M - round + (int)(A_l + cnt_l * (unsigned)round);
             const bool end = live && rem_l == 0;
             // the head's first round is the current one: if it does not fit there, the window test cannot
             // succeed in this iteration
@@ -193,16 +193,16 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             A = __shfl_sync(KV_FULL, A_l, src);
             remaining = __shfl_sync(KV_FULL, rem_l, src);
             if (first < 32) {
-                if (lane == first) sim.cur = u + lane - M;                              // step 1 of the round that is decided
-                sim.advance(first - sim.tau, 0);
+                if (lane == first) sim.cur = u + round - M;                             // step 1 of the round that is decided
+                sim.advance(sim.tn - 32 + first - sim.t);
                 if ((ends >> first) & 1u) done = true;
                 else if (!((works >> first) & 1u)) failed = true;
                 break;
             }
-            sim.advance(32 - sim.tau, 0);
+            sim.advance(sim.tn - sim.t);
         }
         if (done || failed) break;
-        const int t = sim.T0 + sim.tau;
+        const int t = sim.t;
 
         // ---- step 2: admissions of iteration t
         if (head < n && t >= t_ok) {
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
 
         // ---- step 3: ordered eviction while round t is over budget
         for (;;) {
-            const int used = __shfl_sync(KV_FULL, sim.cur + M - lane, sim.tau);
+            const int used = __shfl_sync(KV_FULL, sim.cur + M - sim.x0, sim.t & 31);
             if (used <= M) { peak = max(peak, used); break; }
             // smallest (estimate, request id) among the running
             if (lane == 0) { scan.t = t; scan.nrun = nrun; }
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             const int at = scan.at[__ffs(__ballot_sync(KV_FULL, key == least)) - 1];
             const int q = run[KV_IDX(at, nm, 1103)];
             const int p = pp[q], s = ps[q], o = po[q], e0 = pe[q];
-            sim.remove(s - (p - sim.T0), p + est - sim.T0);        // what is left of its projection
+            sim.remove(s - p, p + est);        // what is left of its projection
             const unsigned v = (unsigned)(s - p);
             const bool overdue = e0 < o && t >= p + e0 + 1;
             if (overdue) { cnt -= 1u; A -= v; }
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
         }
         if (failed) break;
         // ---- step 4: the round runs
-        sim.advance(1, 0);
+        sim.advance(1);
     }
     if (lane == 0) scan.nrun = -1;
     __syncthreads();

@@ -30,9 +30,9 @@
 // answers "when", not only "whether" (see ask).  A request that waits for longer than the two chunks
 // takes its bound from A + C x of the far ones: a few steps, however long it waits.
 //
-// Rounds and starts (and with them V, A and W) are counted from T0 = t rounded down to a multiple of 32, so that
-// an admission is a handful of three-input additions of per-lane constants; entering the next chunk takes 32
-// off every V and puts 32 (C - 1) on A.  A request is passed as sp = s + 1 and om = o - 1.
+// Rounds are counted from 0 throughout, so nothing that a lane keeps changes when t moves on (counted from the beginning of
+// t's chunk, entering the next one had to correct A, W, X and both chunks: 26 instead of 19 instructions, 1.6 times per
+// admission where memory is short).  A request is passed as sp = s + 1 and om = o - 1.
 //
 // What bounds it: instructions.  With one near chunk, tested again after every wait, an admission of k3_eval_moves took
 // 75 to 95 of them; the exact wait, windows of 64 rounds and more without masks, and two turns of the loop in a row leave 60
@@ -50,7 +50,7 @@
 // 172 to 257 for the 10,000), t moving over several chunks at once (sweeps 82 -> 85 issue slots per admission).
 //
 // Sums may wrap; V itself fits 31 bits (the host checks M, sum of o and n), so arithmetic modulo 2^32
-// gives it exactly.
+// gives it exactly.  U may exceed it by 31 for every request that is resident in a chunk's first round (chunk_sums_fit, api.cu).
 #pragma once
 
 #include "common.cuh"
@@ -73,12 +73,14 @@ struct ChunkSim {
     static constexpr int kLong = 64;                                // om from which every window covers what is left of the two chunks and ends behind them
 
     int lane;
-    int T0, tau;             // t = T0 + tau, 0 <= tau < 32
+    int t;                   // the round the next request may start at
+    int tn;                  // first round of the chunk behind the one t lies in
     int M;
+    int x0;                  // this lane's round of the chunk t lies in
     int cur, nxt;            // V - M of this lane's round of the two chunks
     int X;                   // first round of this lane's far chunk; register m: the chunk 1024 m rounds behind it
     int A[NM], C[NM], W[NM]; // W = M - U
-    unsigned acc;            // of a block of up to 32 admissions: sum of their starts, less the T0 it began with
+    unsigned acc;            // of a block of up to 32 admissions: sum of their starts
     i64 tel;                 // sum of starts in front of the block
     int* ring;               // this lane's column
     int mask;                // ring ints - 1, without the lane bits
@@ -88,23 +90,24 @@ struct ChunkSim {
         ring = ring_ + lane;
         mask = (ring_cells(L) - 1) & ~31;
     }
-    __device__ __forceinline__ int* cells_of(int x) const { return ring + KV_IDX((T0 + x) & mask, mask + 32, 151); }
+    __device__ __forceinline__ int* cells_of(int x) const { return ring + KV_IDX(x & mask, mask + 32, 151); }
     __device__ __forceinline__ static int cell(const int* p) { return kGlobal ? __ldcg(p) : *p; }
     // *p += v where `on`: an atomic without a result, so nothing waits for the old value, and without a branch
     __device__ __forceinline__ static void raise(int* p, int v, bool on) {
         if (kGlobal) asm volatile("{ .reg .pred q; setp.ne.s32 q, %2, 0; @q red.global.add.s32 [%0], %1; }" :: "l"(p), "r"(v), "r"((int)on) : "memory");
         else atomicAdd(p, on ? v : 0);
     }
-    __device__ __forceinline__ void set_time(int t, int M_) {
-        T0 = t & ~31; tau = t & 31; M = M_;
-        X = 64 + 32 * ((lane - (T0 >> 5) - 2) & 31);
+    __device__ __forceinline__ void set_time(int t_, int M_) {
+        t = t_; M = M_;
+        x0 = (t & ~31) + lane; tn = (t & ~31) + 32;
+        X = tn + 32 + 32 * ((lane - (tn >> 5) - 1) & 31);
     }
-    __device__ __forceinline__ int start() const { return T0 + tau; }      // of the request admitted last
+    __device__ __forceinline__ int start() const { return t; }             // of the request admitted last
 
     // nothing is resident at t or later
-    __device__ __forceinline__ void reset(int M_, int t = 0) {
-        set_time(t, M_);
-        cur = lane - M; nxt = cur + 32; tel = 0;
+    __device__ __forceinline__ void reset(int M_, int t_ = 0) {
+        set_time(t_, M_);
+        cur = x0 - M; nxt = cur + 32; tel = 0;
 #pragma unroll
         for (int m = 0; m < NM; ++m) { A[m] = -M; C[m] = 1; W[m] = M - (X + 1024 * m + 31); }
         for (int k = 0; k <= mask; k += 32) ring[KV_IDX(k, mask + 32, 152)] = 0;
@@ -140,7 +143,7 @@ struct ChunkSim {
             snap[64 + 96 * m + lane] = A[m]; snap[96 + 96 * m + lane] = C[m]; snap[128 + 96 * m + lane] = W[m];
         }
         if (lane == 0) {
-            SnapHeader h; h.t = T0 + tau;
+            SnapHeader h; h.t = t;
             h.tel_lo = (int)(tel_before & 0xffffffffll); h.tel_hi = (int)(tel_before >> 32);
             *hdr = h;
         }
@@ -148,41 +151,58 @@ struct ChunkSim {
     // sum of the completion times of all requests; sum_o: decode lengths of those admitted here
     __device__ __forceinline__ i64 total(i64 sum_o) const { return tel + sum_o; }
 
-    // this lane's first far chunk is none any more
-    __device__ __forceinline__ void next_chunk() {
-        X += 1024;
+    __device__ __forceinline__ static int pick(int on, int a, int b) {     // a select that stays one
+        int r;
+        asm("{ .reg .pred q; setp.ne.s32 q, %1, 0; selp.s32 %0, %2, %3, q; }" : "=r"(r) : "r"(on), "r"(a), "r"(b));
+        return r;
+    }
+    // on: this lane's first far chunk is none any more.  With several registers as selects by all lanes: as a branch that one lane
+    // takes alone it held up the other 31 (10,000 requests on short prefills, 20 rounds per request, 6,000 moves, decodes to
+    // 2,048 / 4,096 / 8,192: 6.55 -> 6.26, 9.57 -> 7.29, 22.0 -> 14.6 ms).
+    __device__ __forceinline__ void next_chunk(int on) {
+        if (NM == 1) {
+            if (on) { X += 1024; A[0] = -M; C[0] = 1; W[0] = M - (X + 31); }
+            return;
+        }
+        X += on << 10;
 #pragma unroll
-        for (int m = 0; m + 1 < NM; ++m) { A[m] = A[m + 1]; C[m] = C[m + 1]; W[m] = W[m + 1]; }
-        A[NM - 1] = -M; C[NM - 1] = 1; W[NM - 1] = M - (X + (1024 * (NM - 1) + 31));
+        for (int m = 0; m + 1 < NM; ++m) { A[m] = pick(on, A[m + 1], A[m]); C[m] = pick(on, C[m + 1], C[m]); W[m] = pick(on, W[m + 1], W[m]); }
+        A[NM - 1] = pick(on, -M, A[NM - 1]); C[NM - 1] = pick(on, 1, C[NM - 1]);
+        W[NM - 1] = pick(on, M - (X + (1024 * (NM - 1) + 31)), W[NM - 1]);
     }
     // t has left its chunk: the next one takes its place, the first far chunk that one's, and the lane that held it
-    // gets the chunk 1024 NM rounds further on.  left: requests of the block still to be admitted
-    __device__ __forceinline__ void rotate(int left) {
-        T0 += 32; tau -= 32;
-        acc += 32u * (unsigned)left;
-        const int j = ((T0 >> 5) + 1) & 31;
-        int* const p = cells_of(32);
+    // gets the chunk 1024 NM rounds further on
+    __device__ __forceinline__ void rotate() {
+        tn += 32; x0 += 32;
+        const int j = (tn >> 5) & 31;
+        int* const p = cells_of(tn);
         const int own = cell(p);
         *p = 0;
-        X -= 32;
-#pragma unroll
-        for (int m = 0; m < NM; ++m) { A[m] += 32 * C[m] - 32; W[m] += 32; }
         const int a = __shfl_sync(KV_FULL, A[0], j), c = __shfl_sync(KV_FULL, C[0], j);
-        cur = nxt - 32;
-        nxt = own + a + c * (32 + lane);
-        if (lane == j) next_chunk();
+        cur = nxt;
+        nxt = own + a + c * (x0 + 32);
+        next_chunk(lane == j);
     }
     // t moves on by d rounds
-    __device__ __forceinline__ void advance(int d, int left) {
-        tau += d;
-        while (tau >= 32) rotate(left);
+    __device__ __forceinline__ void advance(int d) {
+        t += d;
+        while (t >= tn) rotate();
     }
     // the same for any d: a gap longer than every window leaves nothing resident
     __device__ __forceinline__ void skip(int d, int M) {
-        if (d > mask + 128) reset(M, T0 + tau + d);
-        else advance(d, 0);
+        if (d > mask + 128) reset(M, t + d);
+        else advance(d);
     }
-
+    // Lists whose schedules may go on for 2^30 rounds and more (orders with an id many times over, any start times) count
+    // their rounds from a later one now and then: taken off t, a multiple of every ring's length and of the 32 lanes' chunks.
+    __device__ __forceinline__ int rebase() {
+        if (t < (1 << 29)) return 0;
+        const int d = t & ~8191;
+        t -= d; tn -= d; x0 -= d; X -= d; cur -= d; nxt -= d;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) { A[m] += (C[m] - 1) * d; W[m] += d; }
+        return d;
+    }
     // far chunks of the window whose bound does not clear it: exact maximum into W, wait bound of their cells
     __device__ __forceinline__ int far_need(int a0, int last) {
         int d = 0;
@@ -197,7 +217,7 @@ struct ChunkSim {
                 const int v = cell(cells_of(x)) + a + c * x;
                 const int vmax = kv_warp_max(v);
                 if (lane == j) W[m] = -vmax;
-                if (x <= last) d = max(d, __viaddmin_s32(v, a0, x - tau + 1));
+                if (x <= last) d = max(d, __viaddmin_s32(v, a0, x - t + 1));
             }
         }
         return kv_warp_max(d);
@@ -205,17 +225,17 @@ struct ChunkSim {
     // 0: (sp, om) fits at t; otherwise a lower bound of the rounds it has to wait.  A far chunk that may be over says
     // what the windows that cover it whole use in its last round of the window: a long wait is a few steps.
     __device__ __forceinline__ int test(int sp, int om) {
-        const int a0 = sp - tau, last = tau + om;        // it fits  <=>  V[x] - M + a0 <= 0 in every round of the window
-        const int r = lane + 1 - tau;
-        int v = lane <= last ? __viaddmin_s32(cur, a0, r) : 0;
-        if (lane + 32 <= last) v = max(v, __viaddmin_s32(nxt, a0, r + 32));
+        const int a0 = sp - t, last = t + om;            // it fits  <=>  V[x] - M + a0 <= 0 in every round of the window
+        const int r = x0 + 1 - t;
+        int v = x0 <= last ? __viaddmin_s32(cur, a0, r) : 0;
+        if (x0 + 32 <= last) v = max(v, __viaddmin_s32(nxt, a0, r + 32));
         bool far = false;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
             const int x = X + 1024 * m;
             if (x <= last && a0 > W[m]) {
                 const int e = min(x + 31, last);
-                v = max(v, __viaddmin_s32(A[m] + C[m] * e, a0, e - tau + 1));
+                v = max(v, __viaddmin_s32(A[m] + C[m] * e, a0, e - t + 1));
                 far = true;
             }
         }
@@ -230,26 +250,26 @@ struct ChunkSim {
     // asked here, at the limit of t, which only rises.
     template <bool kWhole>
     __device__ __forceinline__ int ask(int sp, int om) const {
-        const int a0 = sp - tau, last = tau + om, r = lane + 1 - tau;
-        int v = __viaddmin_s32(cur, a0, kWhole || lane <= last ? r : 0);           // rounds before t: 0 or less
-        if (kShort && !kWhole && last < 32) return kv_warp_max(v);
-        v = max(v, __viaddmin_s32(nxt, a0, kWhole || lane + 32 <= last ? r + 32 : 0));
-        if (X <= (kWhole ? om + 64 : last) && a0 > W[0]) v = kAsk;
+        const int a0 = sp - t, last = t + om, r = x0 + 1 - t;
+        int v = __viaddmin_s32(cur, a0, kWhole || x0 <= last ? r : 0);             // rounds before t: 0 or less
+        if (kShort && !kWhole && last < tn) return kv_warp_max(v);
+        v = max(v, __viaddmin_s32(nxt, a0, kWhole || x0 + 32 <= last ? r + 32 : 0));
+        if (X <= (kWhole ? tn + 32 + om : last) && a0 > W[0]) v = kAsk;
         if (kWhole && NM > 1 && om >= 1024) {
 #pragma unroll
-            for (int m = 1; m < NM; ++m) if (X + 1024 * m <= om + 64 && a0 > W[m]) v = kAsk;
+            for (int m = 1; m < NM; ++m) if (X + 1024 * m <= tn + 32 + om && a0 > W[m]) v = kAsk;
         }
         return kv_warp_max(v);
     }
     // the same for any window without a branch but for long ones: where one run stands alone a branch takes longer
     __device__ __forceinline__ int ask(int sp, int om) const {
-        const int a0 = sp - tau, last = tau + om, r = lane + 1 - tau;
-        int v = __viaddmin_s32(cur, a0, lane <= last ? r : 0);
-        v = max(v, __viaddmin_s32(nxt, a0, lane + 32 <= last ? r + 32 : 0));
-        if (X - 64 <= om && a0 > W[0]) v = kAsk;
+        const int a0 = sp - t, last = t + om, r = x0 + 1 - t;
+        int v = __viaddmin_s32(cur, a0, x0 <= last ? r : 0);
+        v = max(v, __viaddmin_s32(nxt, a0, x0 + 32 <= last ? r + 32 : 0));
+        if (X <= tn + 32 + om && a0 > W[0]) v = kAsk;
         if (NM > 1 && om >= 1024) {
 #pragma unroll
-            for (int m = 1; m < NM; ++m) if (X + 1024 * m <= om + 64 && a0 > W[m]) v = kAsk;
+            for (int m = 1; m < NM; ++m) if (X + 1024 * m <= tn + 32 + om && a0 > W[m]) v = kAsk;
         }
         return kv_warp_max(v);
     }
@@ -261,11 +281,11 @@ struct ChunkSim {
     // (sp, om) starts at t
     template <bool kWhole>
     __device__ __forceinline__ void put(int sp, int om) {
-        const int a = sp - tau, last = tau + om;
-        if (kWhole ? lane >= tau : (unsigned)(lane - tau) <= (unsigned)om) cur += a + lane;
-        if (kShort && !kWhole && last < 32) return;
-        if (kWhole || lane + 32 <= last) nxt += a + lane + 32;
-        if (!kWhole && last < 64) return;
+        const int a = sp - t, last = t + om;
+        if (kWhole ? x0 >= t : (unsigned)(x0 - t) <= (unsigned)om) cur += a + x0;
+        if (kShort && !kWhole && last < tn) return;
+        if (kWhole || x0 + 32 <= last) nxt += a + x0 + 32;
+        if (!kWhole && last < tn + 32) return;
         if (X <= last) W[0] -= a + X + 31;
         if (kWhole) {                                                   // a short one covers no far chunk whole
             if (X + 31 < last) { A[0] += a; C[0] += 1; }
@@ -281,9 +301,9 @@ struct ChunkSim {
         raise(cells_of(last), a + x, x <= last);
     }
     __device__ __forceinline__ void add(int sp, int om) {                // the same for any window
-        const int a = sp - tau, last = tau + om;
-        if (lane >= tau && lane <= last) cur += a + lane;
-        if (lane + 32 <= last) nxt += a + lane + 32;
+        const int a = sp - t, last = t + om;
+        if (x0 >= t && x0 <= last) cur += a + x0;
+        if (x0 + 32 <= last) nxt += a + x0 + 32;
         if (X <= last) W[0] -= a + X + 31;
         if (X + 31 < last) { A[0] += a; C[0] += 1; }
         if (NM > 1 && om >= 1024) {
@@ -294,15 +314,15 @@ struct ChunkSim {
             }
         }
         const int x = (last & ~31) + lane;
-        raise(cells_of(last), a + x, last >= 64 && x <= last);
+        raise(cells_of(last), a + x, last >= tn + 32 && x <= last);
     }
 
     // Whether a request of (size, om) certainly fits at t; or several, `size` the sum of their s + o, the longest with
     // om = o - 1, one beside the other: none of them uses more than its s + o in any round.
     __device__ __forceinline__ bool surely(int size, int om) const {
-        const int a0 = size - tau, last = tau + om;
-        bool over = lane >= tau && lane <= last && cur > -a0;
-        over = over || (lane + 32 <= last && nxt > -a0) || (X <= last && a0 > W[0]);
+        const int a0 = size - t, last = t + om;
+        bool over = x0 >= t && x0 <= last && cur > -a0;
+        over = over || (x0 + 32 <= last && nxt > -a0) || (X <= last && a0 > W[0]);
         if (NM > 1 && om >= 1024) {
 #pragma unroll
             for (int m = 1; m < NM; ++m) over = over || (X + 1024 * m <= last && a0 > W[m]);
@@ -315,9 +335,9 @@ struct ChunkSim {
     // them, on fewer warps, it was no gain).  2,000 schedules of 1,000 requests, decodes to 20 / 256 / 1,024 / 4,096, with the
     // question that answers a wait -> this: 428 -> 304, 366 -> 311, 367 -> 331, 522 -> 510 us.
     __device__ __forceinline__ bool put_if_fits(int sp, int om) {
-        const int a0 = sp - tau, last = tau + om;
+        const int a0 = sp - t, last = t + om;
         if (NM == 1 && om >= kLong) {
-            const bool over = (lane >= tau && cur > -a0) || nxt > -a0 || (X <= last && a0 > W[0]);
+            const bool over = (x0 >= t && cur > -a0) || nxt > -a0 || (X <= last && a0 > W[0]);
             if (__any_sync(KV_FULL, over) && test(sp, om) > 0) return false;
             put<true>(sp, om);
             return true;
@@ -327,11 +347,11 @@ struct ChunkSim {
         return true;
     }
 
-    // Takes back what is left (from t on) of a window whose ramp is a + x in round x, counted from T0, and whose last
-    // round is `last`.  The bounds fall by the least the ramp has in a chunk it covers whole.
+    // Takes back what is left (from t on) of a window whose ramp is a + x in round x and whose last round is `last`.  The
+    // bounds fall by the least the ramp has in a chunk it covers whole.
     __device__ __forceinline__ void remove(int a, int last) {
-        if (lane >= tau && lane <= last) cur -= a + lane;
-        if (lane + 32 <= last) nxt -= a + lane + 32;
+        if (x0 >= t && x0 <= last) cur -= a + x0;
+        if (x0 + 32 <= last) nxt -= a + x0 + 32;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
             const int x = X + 1024 * m;
@@ -339,24 +359,30 @@ struct ChunkSim {
             if (x + 31 < last) { A[m] -= a; C[m] -= 1; }
         }
         const int x = (last & ~31) + lane;                          // the chunk the window ends in
-        raise(cells_of(last), -(a + x), last >= 64 && x <= last);
+        raise(cells_of(last), -(a + x), last >= tn + 32 && x <= last);
     }
 
     // The request at hand stays where `run` has left it: t moves on to the next round that is worth a question (false), or it
     // fits although a far bound does not clear it and has been admitted (true).  v: the answer that was neither
     // "fits" nor a wait that ends in t's chunk.
-    __device__ __forceinline__ bool step(int sp, int om, int v, int left) {
+    __device__ __forceinline__ bool step(int sp, int om, int v) {
         if (v >= kAsk) v = test(sp, om);
-        else if (om >= kLong) { advance(v, left); put<true>(sp, om); return true; }
+        else if (om >= kLong) { advance(v); put<true>(sp, om); return true; }
         if (v <= 0) { add(sp, om); return true; }
-        advance(v, left);
+        advance(v);
         return false;
+    }
+
+    // acc counts modulo 2^32; the starts of a block lie less than 2^27 rounds apart
+    __device__ __forceinline__ void add_block(int t_first, int cnt) {
+        const unsigned base = (unsigned)t_first * (unsigned)cnt;
+        tel += (i64)t_first * cnt + (i64)(acc - base);
     }
 
     // Up to 32 consecutive requests of a list, each at its earliest start: (s, o) of the k-th in lane k.  Returns
     // the start of the k-th in lane k.
     __device__ __forceinline__ int run(int2 so, int cnt, int* status) {
-        const int sp_l = so.x + 1, om_l = so.y - 1, T_first = T0;
+        const int sp_l = so.x + 1, om_l = so.y - 1, t_first = t;
         const int cap = kv_loop_cap(32 * mask + 2048);
         int mine = 0, k = 0, turns = 0;
         acc = 0;
@@ -367,31 +393,31 @@ struct ChunkSim {
                 sp = __shfl_sync(KV_FULL, sp_l, k); om = __shfl_sync(KV_FULL, om_l, k);
                 if (om >= kLong) {
                     v = ask<true>(sp, om);
-                    const int at = __viaddmax_s32(v, tau, tau);
-                    if (at > 31) break;
-                    tau = at;
+                    const int at = __viaddmax_s32(v, t, t);
+                    if (at >= tn) break;
+                    t = at;
                     put<true>(sp, om);
                 } else {
                     for (;;) {                       // a wait inside the chunk: ask again from there
                         v = ask<false>(sp, om);
-                        if (kGlobal || v <= 0 || tau + v > 31) break;
-                        tau += v;
+                        if (kGlobal || v <= 0 || t + v >= tn) break;
+                        t += v;
                     }
                     if (v > 0) break;
                     put<false>(sp, om);
                 }
-                acc += (unsigned)tau;
-                if (lane == k) mine = T0 + tau;
+                acc += (unsigned)t;
+                if (lane == k) mine = t;
             }
             if (k >= cnt) break;
-            if (step(sp, om, v, cnt - k)) {
-                acc += (unsigned)tau;
-                if (lane == k) mine = T0 + tau;
+            if (step(sp, om, v)) {
+                acc += (unsigned)t;
+                if (lane == k) mine = t;
                 ++k;
                 turns = 0;
             } else if (++turns > cap) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
         }
-        tel += (i64)T_first * cnt + (i64)acc;
+        add_block(t_first, cnt);
         return mine;
     }
 
@@ -401,11 +427,12 @@ struct ChunkSim {
     template <int kForm>
     __device__ __forceinline__ int run_alone(int2 so, int cnt, int* status) {
         constexpr bool kBriefs = kForm == kBrief, kFar = NM > 1 && kForm == kLengthy;
-        const int sp_l = so.x + 1, om_l = so.y - 1, T_first = T0;
+        const int sp_l = so.x + 1, om_l = so.y - 1, t_first = t;
         const int cap = kv_loop_cap(32 * mask + 2048);
-        // far rounds that may matter: a short window ends in round om + 31 at the latest, a long one waits for up to 64.
+        // far rounds that may matter, from tn on: a short window ends om + 31 rounds behind the chunk's beginning at the
+        // latest, a long one waits for up to 64.
         // From the lane that has it: worked out in every turn it lies in front of the reduction.
-        const int far_l = om_l + (om_l >= kLong ? 64 : 31);
+        const int far_l = om_l + (om_l >= kLong ? 32 : -1);
         int mine = 0, k = 0, turns = 0;
         acc = 0;
         int sp = __shfl_sync(KV_FULL, sp_l, 0), om = __shfl_sync(KV_FULL, om_l, 0), far_to = kBriefs ? __shfl_sync(KV_FULL, far_l, 0) : 0;
@@ -413,35 +440,35 @@ struct ChunkSim {
         auto put_far = [&]() {
             if (X + 31 < plast) { A[0] += pa; C[0] += 1; }
             const int x = (plast & ~31) + lane;
-            raise(cells_of(plast), pa + x, plast >= 64 && x <= plast);
+            raise(cells_of(plast), pa + x, plast >= tn + 32 && x <= plast);
         };
         while (kForm == kPlain || k < cnt) {             // of the two ways to write it the faster one for each form, by up to a half
             int v, sp_next, om_next, far_next = 0;
             for (;;) {
-                const int a0 = sp - tau, end = tau + om, r = lane + 1 - tau;
-                v = __viaddmin_s32(cur, a0, lane <= end ? r : 0);
-                v = max(v, __viaddmin_s32(nxt, a0, lane + 32 <= end ? r + 32 : 0));
-                if ((kBriefs ? X <= far_to : X - 64 <= om) && a0 > W[0]) v = kAsk;
+                const int a0 = sp - t, end = t + om, r = x0 + 1 - t;
+                v = __viaddmin_s32(cur, a0, x0 <= end ? r : 0);
+                v = max(v, __viaddmin_s32(nxt, a0, x0 + 32 <= end ? r + 32 : 0));
+                if (X - tn <= (kBriefs ? far_to : om + 32) && a0 > W[0]) v = kAsk;
                 if (kFar && om >= 1024) {
 #pragma unroll
-                    for (int m = 1; m < NM; ++m) if (X + 1024 * m - om <= 64 && a0 > W[m]) v = kAsk;
+                    for (int m = 1; m < NM; ++m) if (X + 1024 * m - tn <= om + 32 && a0 > W[m]) v = kAsk;
                 }
                 v = kv_warp_max(v);
                 put_far();
                 plast = -1;
                 sp_next = __shfl_sync(KV_FULL, sp_l, (k + 1) & 31); om_next = __shfl_sync(KV_FULL, om_l, (k + 1) & 31);
                 if (kBriefs) far_next = __shfl_sync(KV_FULL, far_l, (k + 1) & 31);
-                const int most = NM > 1 && !kFar && om >= 1024 ? -1 : om >= kLong ? 31 : tau;
-                const int at = __viaddmax_s32(v, tau, tau);
+                const int most = NM > 1 && !kFar && om >= 1024 ? t - 1 : om >= kLong ? tn - 1 : t;
+                const int at = __viaddmax_s32(v, t, t);
                 if (at > most) {
-                    if (!kBriefs || om >= kLong || at > 31) break;
-                    tau = at;                            // asked again from there
+                    if (!kBriefs || om >= kLong || at >= tn) break;
+                    t = at;                            // asked again from there
                     continue;
                 }
-                tau = at;
-                pa = sp - tau; plast = tau + om;
-                if (lane >= tau && lane <= plast) cur += pa + lane;
-                if (lane + 32 <= plast) nxt += pa + (lane + 32);
+                t = at;
+                pa = sp - t; plast = t + om;
+                if (x0 >= t && x0 <= plast) cur += pa + x0;
+                if (x0 + 32 <= plast) nxt += pa + (x0 + 32);
                 if (X <= plast) W[0] -= pa + (X + 31);
                 if (kFar && om >= 1024) {
 #pragma unroll
@@ -450,8 +477,8 @@ struct ChunkSim {
                         if (X + 1024 * m + 31 < plast) { A[m] += pa; C[m] += 1; }
                     }
                 }
-                if (lane == k) mine = T0 + tau;
-                acc += (unsigned)tau;
+                if (lane == k) mine = t;
+                acc += (unsigned)t;
                 turns = 0;
                 sp = sp_next; om = om_next; far_to = far_next;
                 if (++k >= cnt) break;
@@ -460,12 +487,12 @@ struct ChunkSim {
             bool in = false;
             if (NM > 1 && !kFar && om >= 1024) {
                 v = ask<true>(sp, om);
-                in = tau + v <= 31;
-                if (in) { tau += max(v, 0); put<true>(sp, om); }
+                in = t + v < tn;
+                if (in) { t += max(v, 0); put<true>(sp, om); }
             }
-            if (in || step(sp, om, v, cnt - k)) {
-                if (lane == k) mine = T0 + tau;
-                acc += (unsigned)tau;
+            if (in || step(sp, om, v)) {
+                if (lane == k) mine = t;
+                acc += (unsigned)t;
                 turns = 0;
                 sp = sp_next; om = om_next; far_to = far_next;
                 ++k;
@@ -473,7 +500,7 @@ struct ChunkSim {
             } else if (++turns > cap) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
         }
         put_far();
-        tel += (i64)T_first * cnt + (i64)acc;
+        add_block(t_first, cnt);
         return mine;
     }
 
@@ -481,7 +508,7 @@ struct ChunkSim {
     // long as that goes well; calm tells afterwards whether it did.
     __device__ __forceinline__ int run_together(int2 so, int cnt, bool& calm, int* status) {
         constexpr int kMost = (1 << 29) - 1;             // four of them fit 31 bits; a group of so much is none
-        const int sp_l = so.x + 1, om_l = so.y - 1, t_first = T0 + tau, T_first = T0;
+        const int sp_l = so.x + 1, om_l = so.y - 1, t_first = t;
         int size = min(so.x + so.y, kMost), longest = om_l;                  // of the aligned four this lane is in
         size += __shfl_xor_sync(KV_FULL, size, 1); size += __shfl_xor_sync(KV_FULL, size, 2);
         if (size >= kMost) size = INT_MAX;
@@ -497,24 +524,24 @@ struct ChunkSim {
             if (!calm) break;
 #pragma unroll
             for (int j = 0; j < 4; ++j) add(s4[j], o4[j]);
-            acc += 4u * (unsigned)tau;
+            acc += 4u * (unsigned)t;
         }
         if (lane < k) mine = t_first;
         while (k < cnt) {
             const int sp = __shfl_sync(KV_FULL, sp_l, k & 31), om = __shfl_sync(KV_FULL, om_l, k & 31), v = need(sp, om);
             if (v <= 0) {
                 add(sp, om);
-                if (lane == k) mine = T0 + tau;
-                acc += (unsigned)tau;
+                if (lane == k) mine = t;
+                acc += (unsigned)t;
                 ++k;
                 turns = 0;
             } else {
                 calm = false;
-                advance(v, cnt - k);
+                advance(v);
                 if (++turns > kv_loop_cap(32 * mask + 2048)) { if (lane == 0) atomicExch(status, KV_DEV_LOOP_CAP); break; }
             }
         }
-        tel += (i64)T_first * cnt + (i64)acc;
+        add_block(t_first, cnt);
         return mine;
     }
 };

@@ -308,6 +308,8 @@ struct HybSim {
         }
     }
 
+    __device__ __forceinline__ int rebase() { return 0; }
+
     // Up to 32 consecutive requests of a list, (s, o) of the k-th in lane k.  Returns the start of the k-th in lane k.
     __device__ __forceinline__ int run(int2 so, int cnt, int* status) {
         const int sp = so.x + 1, om = so.y - 1;

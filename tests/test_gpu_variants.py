@@ -496,3 +496,46 @@ def test_orders_that_do_not_pass_through_pinned_memory():
         with pytest.raises(kv.SchedError) as e:
             h.local_search(kv.NBHD_SAMPLED, 1, order=np.zeros(n, dtype=np.int32), seed=1, samples_per_iter=64)
         assert e.value.code == kv.E_NOT_PERMUTATION
+
+
+@pytest.mark.parametrize("omax", [1, 300, 1500, 5000])
+def test_schedules_of_more_rounds_than_a_permutation_has(omax):
+    """Device form: orders that repeat one long request (they are not detected) and start times up to 2^31, sparse and one behind the
+    other, in rounds that the permutations of the list never reach."""
+    n, M, far = 700, 40000, (1 << 31) - 1 - omax
+    s = np.full(n, M // 3, np.int32)
+    o = np.full(n, omax, np.int32)
+    rng = np.random.default_rng(omax)
+    gap = omax if omax > 1 else 2
+    rows = np.stack([np.sort(rng.integers(0, far, n)), far - gap * np.arange(n - 1, -1, -1), far - (gap - 1) * np.arange(n - 1, -1, -1),
+                     (1 << 29) - 350 * gap + gap * np.arange(n), np.full(n, far)]).astype(np.int32)
+    starts = torch.from_numpy(rows).cuda()
+    tel = torch.zeros(len(rows), dtype=torch.int64, device="cuda")
+    ok = torch.zeros(len(rows), dtype=torch.uint8, device="cuda")
+    with kv.Scheduler(s, o, M) as h:
+        h.eval_batch_dev(kv.CAND_START_TIMES, len(rows), starts, tel, ok, None)
+        h.sync()
+    for r, good, total in zip(rows.astype(np.int64), ok.tolist(), tel.tolist()):
+        ends = r + omax                                       # memory is fullest in somebody's last round
+        beside = (r[None] < ends[:, None]) & (ends[:, None] <= ends[None])
+        most = np.where(beside, s[0] + ends[:, None] - r[None], 0).sum(1).max()
+        assert bool(good) == (most <= M) and total == int((r + omax).sum())
+
+
+def test_orders_that_go_on_for_two_to_the_thirty_rounds():
+    """Device form: one request of 8,000 rounds 150,000 times over, each alone in the memory, between others that run once."""
+    n, M = 150000, 16000
+    s, o = np.full(n, 10, np.int32), np.full(n, 7, np.int32)
+    s[0], o[0] = 8000, 8000
+    order = np.zeros(n, np.int32)
+    order[-40:] = np.arange(1, 41)
+    with kv.Scheduler(s, o, M) as h:
+        tel = torch.zeros(1, dtype=torch.int64, device="cuda")
+        starts = torch.zeros((1, n), dtype=torch.int32, device="cuda")
+        h.eval_batch_dev(kv.CAND_ORDER, 1, torch.from_numpy(order[None]).cuda(), tel, None, starts)
+        h.sync()
+    p = 8000 * np.arange(n, dtype=np.int64)
+    p[-40:] = p[-41]                                          # 40 requests of 17 tokens fit beside the last long one at once
+    assert p[-1] > 1 << 30
+    assert (starts.cpu().numpy()[0, 1:41] == p[-1]).all()
+    assert tel.item() == int(p.sum()) + 8000 * (n - 40) + 7 * 40
