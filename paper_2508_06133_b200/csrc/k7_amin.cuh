@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
         // decision (or ends the run).
         const int head_s = head < n ? ps[head] : 0;
         for (;;) {
-            const bool live = sim.x0 >= sim.t;
+            const int tau = sim.t & 31;
+            const bool live = lane >= tau;
             const int round = sim.x0, k = round & mask;
             int es = live ? ev[k] : 0;
             unsigned as = live ? dA[k] : 0u;
@@ -194,12 +195,12 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
             remaining = __shfl_sync(KV_FULL, rem_l, src);
             if (first < 32) {
                 if (lane == first) sim.cur = u + round - M;                             // step 1 of the round that is decided
-                sim.advance(sim.tn - 32 + first - sim.t);
+                sim.t += first - tau;
                 if ((ends >> first) & 1u) done = true;
                 else if (!((works >> first) & 1u)) failed = true;
                 break;
             }
-            sim.advance(sim.tn - sim.t);
+            sim.t = sim.tn; sim.rotate();
         }
         if (done || failed) break;
         const int t = sim.t;
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(32 * K7_WARPS) k7_amin(const AminParams P) {
         }
         if (failed) break;
         // ---- step 4: the round runs
-        sim.advance(1);
+        if (++sim.t == sim.tn) sim.rotate();
     }
     if (lane == 0) scan.nrun = -1;
     __syncthreads();

@@ -266,10 +266,10 @@ struct ChunkSim {
         const int a0 = sp - t, last = t + om, r = x0 + 1 - t;
         int v = __viaddmin_s32(cur, a0, x0 <= last ? r : 0);
         v = max(v, __viaddmin_s32(nxt, a0, x0 + 32 <= last ? r + 32 : 0));
-        if (X <= tn + 32 + om && a0 > W[0]) v = kAsk;
+        if (X - tn <= om + 32 && a0 > W[0]) v = kAsk;
         if (NM > 1 && om >= 1024) {
 #pragma unroll
-            for (int m = 1; m < NM; ++m) if (X + 1024 * m <= tn + 32 + om && a0 > W[m]) v = kAsk;
+            for (int m = 1; m < NM; ++m) if (X + 1024 * m - tn <= om + 32 && a0 > W[m]) v = kAsk;
         }
         return kv_warp_max(v);
     }
