@@ -31,6 +31,10 @@
  *     that where M * M over the smallest s+o passes some 2^31), 16 KB beyond; 412, 495 (824, 989) and 512 MB
  *     at most.  It is allocated by the first such sweep of a handle and kept until sched_destroy(); where
  *     there is no memory for it the sweep runs without.
+ *   - sched_sorted_f_quantile() on 2,048 requests and more keeps the leading halves of its random keys in the
+ *     handle's staging block: 4 n bytes for each of some 16 + 1.5 n mean(s+o) / M batches, at most 64 MiB; it goes
+ *     without where the batches to be expected need more, or where there is no memory for them.  The staging block (the
+ *     largest that any call has needed) stays with the handle until sched_destroy().
  *   - A handle is tied to the CUDA device that was current in sched_init(); calls on one handle
  *     must not overlap in time.
  *   - Arrays are dense, row-major, int32 unless stated; TELs are int64.
@@ -317,7 +321,7 @@ int sched_online_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const
  * All pointers are host memory; the call allocates and frees its own device buffers and synchronises
  * the device.  SCHED_E_INVAL: bad sizes, s < 1, lower < 1, lower > o, s + o > M;
  * SCHED_E_NOT_PERMUTATION: a row of order is not a permutation; SCHED_E_UNSUPPORTED: n_max > 4096,
- * o > 8192, M >= 2^30, or rows too large for the shared memory of one CTA (20 n_max + 12 L + 128 R bytes,
+ * o > 8192, M >= 2^30, or rows too large for the shared memory of one CTA (20 n_max + 8 L + 128 R bytes,
  * L = the power of two >= max o + 2, R = the one >= (max o + 30) / 32); SCHED_E_INTERNAL: a scenario did not finish within
  * 16 + (n+1) sum(o) rounds (capped at 2^30). */
 int sched_amin_simulate(int32_t B, int32_t n_max, const int32_t* n_each, const int32_t* s, const int32_t* lower,

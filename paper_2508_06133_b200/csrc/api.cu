@@ -41,7 +41,7 @@ const i64 kHostCheckMax = 1 << 13;          // ids or starts checked by the host
 const i64 kAcceptSmall = 16384;              // sweep results that one CTA reduces (4 us against a launch of its own)
 const int kSnapshots = 256;                 // states of the base run kept for the sweeps (chunked simulator)
 const int kLeadingFrom = 2048;              // requests from which the quantile solver's keys are made beforehand: 2 and more per thread
-const size_t kLeadingBytes = 64ull << 20;   // of them, at most
+const size_t kLeadingBytes = 64ull << 20;   // of them, at most; without them where that is not all batches there may well be
 const int kSnapStrideHyb = 8;               // positions per state (hybrid simulator)
 const size_t kSnapBudget = 512ull << 20;    // bytes of snapshot memory
 
@@ -99,6 +99,8 @@ void pool_trim_locked(int device) {             // device < 0: every device
 
 cudaError_t kv_malloc(void** out, size_t bytes) {
     *out = nullptr;
+    if (const char* least = getenv("KVSCHED_REFUSE_MB"))        // testing knob: there is no memory for blocks of this size and more
+        if (bytes >= (size_t)atoll(least) << 20) return cudaErrorMemoryAllocation;
     if (bytes < kPoolMinBlock || pool_cap_bytes() == 0) return cudaMalloc(out, bytes);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1268,9 +1270,10 @@ static int phase1_quantile(sched_handle h, u64 seed) {
     const unsigned* leading = nullptr;
     int batches = 0;
     if (n >= kLeadingFrom) {
-        // as many batches as there may be: the requests' sizes over M, a third of every batch unused
-        const double most = fmin(16.0 + 1.5 * (double)n * (h->mean_s + h->mean_o) / (double)h->M, (double)(kLeadingBytes / ((size_t)n * sizeof(unsigned))));
-        batches = most < n ? (int)most : n;
+        // as many batches as there may be: the requests' sizes over M, and half as many again for what batches leave unused
+        const double expected = (double)n * (h->mean_s + h->mean_o) / (double)h->M, room_for = (double)(kLeadingBytes / ((size_t)n * sizeof(unsigned)));
+        const double most = fmin(16.0 + 1.5 * expected, fmin(room_for, (double)n));
+        batches = room_for >= expected ? (int)most : 0;
         if (batches > 0 && ensure_stage(h, (size_t)batches * n * sizeof(unsigned)) != SCHED_OK) {
             cudaGetLastError();                          // without memory for them the solver makes its keys itself
             batches = 0;

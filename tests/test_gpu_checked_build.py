@@ -23,7 +23,7 @@ SMALL_CASES = ("small_random or paper_example or long_waits or every_simulator_s
 # the kernels that only larger calls take, and the edges of what each variant covers
 VARIANT_CASES = ("moves_by_lanes or largest_budgets or device_rings or short_windows or beyond_the_registers or timeline_sizes or sorting or "
                  "several_merges or longest_lists or candidates_are_checked or dynamic_programme or online_windows or "
-                 "local_swap_sizes or beyond_shared_memory or near_chunks or stand_alone or schedules_of_more or amin_running")
+                 "local_swap_sizes or beyond_shared_memory or near_chunks or stand_alone or schedules_of_more or amin_running or quantile_sizes")
 
 _PROBE = r"""
 import sys

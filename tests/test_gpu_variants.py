@@ -218,6 +218,45 @@ def test_quantile_sizes(n, M, alone):
     assert not alone or len(offs) == n + 1
 
 
+@pytest.mark.parametrize("n,M,beforehand", [(2048, 20000, True), (20000, 60000, False), (16000, 400000, True)])
+def test_quantile_keys_where_they_cover_the_batches(monkeypatch, n, M, beforehand):
+    """Keys are made beforehand where 64 MiB hold those of all batches there may well be (20,000 requests at a budget of 60,000:
+    some 900 batches of 80 KB), and the same batches come without memory for them."""
+    inst = W.mixed_backlog(n, 3, M)
+    with kv.Scheduler(inst.s, inst.o, M) as h:
+        (order, offs, tel), names = kernels_of(lambda: h.sorted_f_quantile(5))
+    assert ("k2q_leading" in names) == beforehand, names
+    with kv.Scheduler(inst.s, inst.o, M) as h:
+        monkeypatch.setenv("KVSCHED_REFUSE_MB", "1")
+        (order2, offs2, tel2), names = kernels_of(lambda: h.sorted_f_quantile(5))
+    assert "k2q_leading" not in names, names
+    assert (order == order2).all() and (offs == offs2).all() and tel == tel2
+    if n <= 16000:
+        ref = orc.sorted_f_quantile(inst.s, inst.o, M, 5)
+        assert (order == ref[0]).all() and (offs == ref[1]).all()
+
+
+def test_sweeps_without_memory_for_rings(monkeypatch):
+    """The forms that keep state in device memory, with memory and without: the same TELs from a warp per candidate."""
+    for inst, count, kernel in ((W.mixed_backlog(1000, 4, 65536), 60000, "k3_lane_moves"),
+                                (W.mixed_backlog(3000, 4, 4194304, **dict(chat_o=(5.5, 1.0, 8, 4096))), 6000, "ChunkSim<4, true")):
+        best = torch.zeros(2, dtype=torch.int64, device="cuda")
+        tels = []
+        for refuse in (False, True):
+            tel = torch.empty(count, dtype=torch.int64, device="cuda")
+            with kv.Scheduler(inst.s, inst.o, inst.M) as h:
+                h.sorted_f()
+                h.sweep_dev(64, best, sampled=True, seed=3, iteration=1)
+                h.sync()
+                if refuse:
+                    monkeypatch.setenv("KVSCHED_REFUSE_MB", "4")
+                _, names = kernels_of(lambda: (h.sweep_dev(count, best, sampled=True, seed=3, iteration=1, tel_out=tel), h.sync()))
+            monkeypatch.delenv("KVSCHED_REFUSE_MB", raising=False)
+            assert (kernel in names) != refuse, names
+            tels.append(tel)
+        assert torch.equal(*tels)
+
+
 @pytest.mark.parametrize("n,M", [(9, 200), (40, 600), (24, 1100), (24, 1250)])
 def test_dynamic_programme_sizes(n, M):
     """The last tables that fit shared memory and the first that do not."""
