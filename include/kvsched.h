@@ -25,7 +25,7 @@
  *     scratch, outgrown staging buffers) are kept in a process-wide per-device cache -- at most
  *     KVSCHED_POOL_MB MiB in total (environment variable, default 1024, 0 disables the cache) -- and
  *     reused by later calls; sched_release_cached_memory() returns them to the driver.
- *   - A large sweep (sched_sweep_dev, sched_local_search, MOVE candidates; more than some 18,000 moves on
+ *   - A large sweep (sched_sweep_dev, sched_local_search, MOVE candidates; more than some 15,000 moves on
  *     decodes up to 2,049 rounds, more than some 4,000 on decodes up to 4,097) keeps simulator state in
  *     device memory: 4.3 KB per move side by side for decodes up to 1,025 rounds, 8.5 KB up to 2,049 (twice
  *     that where M * M over the smallest s+o passes some 2^31), 16 KB beyond; 412, 495 (824, 989) and 512 MB

@@ -555,10 +555,10 @@ int order_candidates(sched_ctx* h, const MoveSource& src, i64 count) {
     return SCHED_OK;
 }
 
-// Moves with a warp each on the simulator for short windows (sim_chunk.cuh)?  Measured over 225 sweeps of random
-// backlogs, the share of short decodes (mean of min(1, 32 / o)) against the time with it over that without: 0.995 and
-// more 0.87 (0.75 to 0.99), 0.96 to 0.995 0.98 (0.84 to 1.05), below 1.02 to 1.08.
-bool short_windows(const sched_ctx* h, bool want_starts) { return !want_starts && h->nm == 1 && h->short_share >= 0.985; }
+// Moves with a warp each on the simulator for short windows (sim_chunk.cuh)?  Measured over 216 sweeps of 16,000 moves, the
+// share of short decodes (mean of min(1, 32 / o)) against the time with it over that without: 0.985 and more 0.79 to 0.92,
+// 0.95 to 0.985 0.94 (0.92 to 0.98), 0.94 0.98 (0.95 to 1.01), 0.90 1.00 (0.98 to 1.03), below 1.03 (1.01 to 1.05).
+bool short_windows(const sched_ctx* h, bool want_starts) { return !want_starts && h->nm == 1 && h->short_share >= 0.93; }
 
 // One thread per candidate instead of one warp (k3_lanes.cuh)?  Its work goes with the rounds that pass, the
 // other kernel's with the admissions: rounds per request is the backlog's volume (sum of s o + o^2 / 2) over
@@ -577,42 +577,40 @@ bool short_windows(const sched_ctx* h, bool want_starts) { return !want_starts &
 //   96,000               11.4 /  5.7       15.1 / 12.2    17.4 / 16.4
 // Two kinds of backlog cost a thread more per admission (log-normal decodes, prefills uniform up to 2,000):
 //   short decodes: a window that ends in one of the two chunks kept as cells takes its share back from them one by one,
-//   which the share of decodes up to a chunk (each counted as 32 / o beyond) tells.  Mean 21 (share 0.94): 40,000 moves of
-//   10,000, 0.5 / 2 / 6 rounds per request 16.5 / 19.6, 20.3 / 31.0, 27.8 / 50.0; mean 87 (0.56): 16.4 / 10.1, 18.5 / 15.1,
-//   21.3 / 24.1;
+//   which the share of decodes up to a chunk (each counted as 32 / o beyond) tells.  Mean 20 (share 0.94): 40,000 moves of
+//   10,000, 0.5 / 2 / 6 rounds per request 16.3 / 20.0, 19.8 / 30.7, 27.6 / 49.7; mean 82 (0.56): 16.4 / 9.3, 18.4 / 14.7,
+//   21.2 / 24.2;
 //   long decodes on short prefills: memory is used by tokens still to come, what a request waits for lies chunks
-//   ahead, and every wait walks the events up to there.  Prefills up to 20, decodes of mean 335, 10,000 requests, 40,000
-//   moves, 0.5 / 1 / 2 / 6 rounds per request 16.0 / 10.5, 16.4 / 14.7, 17.4 / 36, 21.2 / 146; prefills up to 2,000: 15.8 / 6.7,
-//   16.2 / 8.5, 16.8 / 10.8, 19.2 / 24.0; decodes of mean 668 (to 2,048), prefills up to 20: 20.7 / 7.9, 21.3 / 14.7, 22.3 / 17.2,
-//   26.9 / 56.  Use of memory falls by s / rounds per round and varies by (s + o) sqrt(rounds ahead / rounds), hence
+//   ahead, and every wait walks the events up to there.  Prefills up to 20, decodes of mean 344, 10,000 requests, 40,000
+//   moves, 0.5 / 1 / 2 / 6 rounds per request 16.0 / 9.4, 16.4 / 17.8, 17.3 / 43.5, 20.8 / 179; prefills up to 2,000: 16.0 / 6.9,
+//   16.4 / 8.6, 17.0 / 11.6, 19.5 / 28.2; decodes of mean 692 (to 2,048), prefills up to 20: 20.8 / 8.7, 21.2 / 14.7, 22.2 / 19.0,
+//   26.2 / 57.5.  Use of memory falls by s / rounds per round and varies by (s + o) sqrt(rounds ahead / rounds), hence
 //   the form in (1 + o / s) sqrt(rounds); its square and the caps are fitted.  Only where time goes on for
 //   longer than a decode: otherwise nearly everything runs side by side.
-// Longer decodes than its ring of events, schedules with more rounds per request than
-// were measured (14.8 for decodes beyond 1,025), and backlogs whose candidate could pass 32 bits of waiting
-// time in its sum of starts or of tokens in a chunk (lane_sums_fit) keep the warp.
-constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.55;
+// The constants are fitted to 1,164 sweeps of 20,000 to 112,000 moves measured in both forms (mixed backlogs of 3 to 25 rounds
+// per request; decodes of median 8 to 400 on prefills to 20, 200 and 2,000; 60 backlogs drawn at random; in Sorted-F and random
+// order).  10 of them take a thread where a warp is faster by more than a tenth, 22 the other way round; 8 lose more than
+// 0.3, the worst 0.45.  Longer decodes than its ring of events, schedules with more rounds per request than were
+// measured, and backlogs whose candidate could pass 32 bits of waiting time in its sum of starts or of tokens in a chunk
+// (lane_sums_fit) keep the warp.
+constexpr double LANE_ROUNDS = 25.5;
 
 // candidates from which on a thread each is the faster one
 double lanes_from(const sched_ctx* h) {
-    const double rounds = h->volume / ((double)h->n * (double)h->M), n = (double)h->n;
-    double need = LANE_MIN + LANE_MIN_PER_ROUND * rounds, ahead = (1.0 + h->mean_o / h->mean_s) * (1.0 + h->mean_o / h->mean_s);
+    const double rounds = h->volume / ((double)h->n * (double)h->M), n = (double)h->n, share = h->short_share;
+    const double size = 1.0 + h->mean_o / h->mean_s, grow = size * size;
+    double need, ahead;
     if (rounds > LANE_ROUNDS) return INFINITY;
     if (h->nm == 1) {
-        if (h->short_share > 0.3) need += 11000.0 * rounds * (h->short_share - 0.3);
-        if (ahead > 1.3) need += 8700.0 * rounds * (fmin(ahead, 3.0) - 1.3);
-        if (h->short_share > 0.75) need += 150000.0 * (h->short_share - 0.75);
+        need = 15000.0 + 1600.0 * rounds + fmax(share - 0.3, 0.0) * (65000.0 + 9000.0 * rounds) + 4800.0 * rounds * fmax(fmin(grow, 3.0) - 1.3, 0.0);
         if (short_windows(h, false)) need *= 1.3;              // against the warp's simulator for those
-        ahead = fmin(ahead, 8.0);
+        ahead = fmin(grow - 1.0, 8.7);
     } else {
-        need *= LANE_LONG;
-        if (h->short_share > 0.4) need *= 1.0 + (h->short_share - 0.4) * rounds / 3.0;
-        // candidates further apart in a long list also leave one another's rounds: 40,000 moves of 10,000 and of 2,000
-        // requests with a share of 0.72, 6 rounds per request: 28.1 / 60 and 5.6 / 11.4
-        if (h->short_share > 0.4 && n > 2000.0) need *= 1.0 + (n - 2000.0) * rounds / 48000.0;
-        ahead = fmin(0.6 * ahead, 3.6);
+        need = (17000.0 + 2500.0 * rounds) * (1.0 + fmax(share - 0.4, 0.0) * (3.0 + 39.0 * rounds));
+        ahead = fmin(1.65 * (grow - 1.0), 6.1);
     }
     const double far = ahead * sqrt(rounds);
-    if (n * rounds >= (double)h->omax && far > 5.0) need = far > 8.0 ? INFINITY : need * (1.0 + 0.55 * (far - 5.0));
+    if (n * rounds >= (double)h->omax && far > 4.5) need = far > 10.0 ? INFINITY : need * (1.0 + 0.2 * (far - 4.5));
     return need;
 }
 

@@ -370,7 +370,9 @@ def test_moves_on_the_largest_budgets(M, omax, thread):
     (1024, 200, 4000, 3.0, 24000, True), (1024, 200, 4000, 3.0, 18000, False),
     (64, 16, 2000, 2.0, 40000, False), (64, 16, 2000, 2.0, 95000, True),      # short decodes
     (1024, 256, 20, 6.0, 95000, False), (1024, 256, 20, 0.5, 40000, True),    # short prefills: memory grows
-    (2048, 512, 20, 6.0, 95000, False), (2048, 512, 2000, 3.0, 40000, True)])
+    (2048, 512, 20, 6.0, 95000, False), (2048, 512, 2000, 3.0, 40000, True),
+    (1024, 200, 4000, 24.0, 62000, True), (1024, 200, 20, 1.0, 60000, True), (2048, 512, 2000, 0.5, 20000, True),
+    (256, 20, 2000, 0.5, 28000, False)])
 def test_which_form_a_sweep_takes(omax, median, smax, rounds, count, thread):
     """Backlogs on which a thread per candidate is slower than a warp (by up to ten times) keep the warp."""
     rng = np.random.default_rng(omax + median + smax)
@@ -474,6 +476,22 @@ def test_moves_of_short_windows(omax):
     with kv.Scheduler(s, 40 * o, M) as h:
         _, names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, codes))
     assert ("ChunkSim<1, false, false>" if 40 * omax <= 1025 else "ChunkSim<2, false, false>") in names, names
+
+
+@pytest.mark.parametrize("median,short", [(12, True), (16, True), (32, False)])
+def test_backlogs_that_take_the_simulator_of_short_windows(median, short):
+    """Log-normal decodes: shares of short ones of 0.98, 0.96 and 0.84."""
+    rng = np.random.default_rng(median)
+    n = 3000
+    s = rng.integers(1, 500, n).astype(np.int32)
+    o = np.clip(np.round(rng.lognormal(np.log(median), 0.8, n)), 1, 512).astype(np.int32)
+    codes = rng.integers(0, 3 * n * (n - 1) // 2, 3000).astype(np.int64)
+    base = rng.permutation(n).astype(np.int32)
+    with kv.Scheduler(s, o, 30000) as h:
+        h.set_base_order(base)
+        (tel, _, _), names = kernels_of(lambda: h.eval_batch(kv.CAND_MOVE, codes))
+    assert ("ChunkSim<1, false, true>" in names) == short, names
+    assert (tel[::300] == oracle_moves(s, o, 30000, base, codes[::300])).all()
 
 
 @pytest.mark.parametrize("count", [5000, 32768, 32769, 80000])
