@@ -671,9 +671,14 @@ int launch_lanes(sched_ctx* h, const MoveEvalParams& p, bool* done) {
 }
 
 // Moves with a warp each whose rings are in device memory (sim_chunk.cuh)?  32 instead of 13 warps per SM
-// against a wait for memory per 32 rounds.  Measured, shared against device memory, decodes to 4,096: 100,000
-// requests, 7,000 moves, 1.0 rounds per request 53.4 / 45.0 ms; 20,000 requests, 4.2 rounds: 35,000 moves 59.4 /
-// 61.2, 2,400 moves (16 warps per SM) 5.1 / 6.5; 2,000 requests, 16 rounds, 200,000 moves 50.7 / 89.5.
+// against a wait for memory per 32 rounds.  Measured, shared against device memory, decodes to 4,096, ms:
+//   rounds per request             1               2               3               4.2             16
+//   100,000 requests, 7,000 moves  42.7 / 38.5     44.9 / 49.1
+//   20,000, 35,000                 40.0 / 34.9     42.1 / 39.9     44.2 / 49.4     46.7 / 63.4
+//   20,000, 4,000                  4.79 / 4.80     5.03 / 5.58                     5.67 / 8.11
+//   20,000, 2,400                  3.20 / 4.17                                     3.86 / 5.95
+//   2,000, 100,000                 11.4 / 10.1     12.0 / 11.6                     13.4 / 19.0     20.1 / 49.6
+// The two cross near 2 rounds per request and at 27 warps per SM, and differ by a tenth there.
 bool device_rings_fit(const sched_ctx* h, i64 count, bool want_starts) {
     return !want_starts && h->nm == 4 && count >= 27ll * h->sm_count && h->volume <= 2.0 * (double)h->n * (double)h->M;
 }

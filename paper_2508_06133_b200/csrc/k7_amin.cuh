@@ -38,7 +38,8 @@
 // evictions among 620 running, 1,450 walks), so the latency of each of these: about 350 cycles an admission, 750 a walk of up
 // to 32 rounds, and an eviction 4,050 with one warp looking through the list, 1,100 with four.  The events of a round's
 // admissions are put together, a lane each (they were 300 of 890 cycles per admission).  Kernel with 1 / 64 / 592
-// scenarios 2.38 / 2.45 / 4.83 -> 1.61 / 1.65 / 3.31 ms, the call around it 2.51 / 2.97 / 9.03 -> 1.74 / 2.14 / 6.50.
+// scenarios (l uniform in [o / 2, o]) 2.71 / 2.80 / 5.37 -> 1.99 / 2.05 / 3.97 ms, the call around it 2.83 / 3.30 / 9.72 -> 2.12 /
+// 2.57 / 8.2.
 #pragma once
 
 #include "common.cuh"
