@@ -123,7 +123,7 @@ __device__ bool k3_accept(const BaseRunParams& p) {
     return true;
 }
 
-template <class SIM, int kForm>
+template <class SIM, int kForm, bool kTogether>
 __global__ void __launch_bounds__(K3B_THREADS)
 k3_base_run(const BaseRunParams p) {
     if (p.accept && !k3_accept(p)) return;
@@ -144,7 +144,7 @@ k3_base_run(const BaseRunParams p) {
     i64 tel = 0;                                         // this lane's share of the completion times so far
     int2 next = lane < n ? tbl_base[lane] : make_int2(1, 1);
     int to_snap = 0, idx = 0;                            // positions until the next snapshot, its number
-    bool calm = true;                                    // nothing has waited, or not since the last snapshot
+    bool calm = kTogether;                                    // nothing has waited, or not since the last snapshot
     int t_snap = 0;
     for (int q0 = 0; q0 < n;) {
         const int2 so = next;
@@ -156,13 +156,14 @@ k3_base_run(const BaseRunParams p) {
             sim.store(snap_ring + (size_t)i * L, snap_hdr + i, before);
             ++idx;
             to_snap = stride;
-            calm = calm || (sim.start() == t_snap && (idx & 7) == 0);        // a mistake costs a block of four
+            calm = kTogether && (calm || (sim.start() == t_snap && (idx & 7) == 0));       // a mistake costs a block of four
             t_snap = sim.start();
         }
         const int cnt = min(min(32, n - q0), to_snap);
         if (q0 + cnt + lane < n) next = tbl_base[q0 + cnt + lane];
         int mine;
         if constexpr (kForm < 0) mine = sim.run(so, cnt, status);
+        else if constexpr (!kTogether) mine = sim.template run_alone<kForm>(so, cnt, status);
         else mine = calm ? sim.run_together(so, cnt, calm, status) : sim.template run_alone<kForm>(so, cnt, status);
         if (lane < cnt) base_starts_pos[q0 + lane] = mine;
         if (lane < cnt) tel += (i64)mine + so.y;

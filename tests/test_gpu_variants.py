@@ -106,6 +106,25 @@ def test_runs_that_stand_alone(omax, beside):
         assert (mtel == oracle_moves(s, o, M, base, codes)).all()
 
 
+@pytest.mark.parametrize("share", [0.05, 0.099, 0.101])
+@pytest.mark.parametrize("omax,median", [(64, 20), (1025, 200), (2049, 200), (2049, 1500), (4097, 20), (4097, 400), (8193, 4000)])
+def test_runs_that_stand_alone_by_share_of_the_budget(omax, median, share):
+    """Every form of the base run on both sides of the budget from which requests are asked for four at a time."""
+    rng = np.random.default_rng(omax + median)
+    n = 333
+    o = np.clip(rng.lognormal(np.log(median), 1.0, n), 1, omax).astype(np.int32)
+    o[50] = omax
+    s = rng.integers(1, 200, n).astype(np.int32)
+    M = max(int((s + o).max()), int(share * float((s + o).sum())))
+    base = rng.permutation(n).astype(np.int32)
+    codes = np.arange(0, 3 * n * (n - 1) // 2, 4999, dtype=np.int64)
+    with kv.Scheduler(s, o, M) as h:
+        final, tel, _, _ = h.local_search(kv.NBHD_SWAP, 0, order=base)
+        mtel = h.eval_batch(kv.CAND_MOVE, codes)[0]
+    assert (final == base).all() and tel == orc.list_schedule_rounds(s, o, M, base)[1]
+    assert (mtel == oracle_moves(s, o, M, base, codes)).all()
+
+
 @pytest.mark.parametrize("part", [2, 3, 8])
 def test_runs_that_stand_alone_on_the_largest_budget(part):
     """Four requests in a row hold more tokens than 31 bits count."""
