@@ -48,7 +48,7 @@ OPS_PER_CELL = 4.0                       # integer operations of a plain timelin
 # dram__bytes_read.sum + dram__bytes_write.sum of one simulator launch, from a one-pass ncu capture of
 # this very launch (summary under profiles/); keyed by (workload, moves per launch) with a digest of
 # the code lines of the simulator's source files, so that it turns into null when the kernel changes
-K3_TRAFFIC = {("mixed_n10000", 1 << 22): (658.64e9 + 476.68e9, "8fee4ffce4e01b81")}
+K3_TRAFFIC = {("mixed_n10000", 1 << 22): (658.38e9 + 476.35e9, "212cd70ecff1f22c")}
 OPS_PER_ADMISSION = 10.0                 # request read and mapped, one compare per bound, two sums and one cell updated
 DEFAULT_MOVES = {"mixed_10k": 1 << 22, "mixed_1k": 499500, "paper_scale": 1 << 21, "heavy_100k": 1 << 18}
 
