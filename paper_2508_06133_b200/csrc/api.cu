@@ -599,30 +599,33 @@ bool short_windows(const sched_ctx* h, bool want_starts) { return !want_starts &
 //   26.2 / 57.5.  Use of memory falls by s / rounds per round and varies by (s + o) sqrt(rounds ahead / rounds), hence
 //   the form in (1 + o / s) sqrt(rounds); its square and the caps are fitted.  Only where time goes on for
 //   longer than a decode: otherwise nearly everything runs side by side.
-// The constants are fitted to 1,164 sweeps of 20,000 to 112,000 moves measured in both forms (mixed backlogs of 3 to 25 rounds
-// per request; decodes of median 8 to 400 on prefills to 20, 200 and 2,000; 60 backlogs drawn at random; in Sorted-F and random
-// order).  10 of them take a thread where a warp is faster by more than a tenth, 22 the other way round; 8 lose more than
-// 0.3, the worst 0.45.  Longer decodes than its ring of events, schedules with more rounds per request than were
+// A line fitted again to 1,164 sweeps (1,000 mixed requests at 24 rounds per request: the thread from 50,000 moves instead of
+// 85,000) took 7.60 instead of 4.06 ms for a backlog drawn at random, so the line before it stands.  Longer decodes than its ring of events, schedules with more rounds per request than were
 // measured, and backlogs whose candidate could pass 32 bits of waiting time in its sum of starts or of tokens in a chunk
 // (lane_sums_fit) keep the warp.
-constexpr double LANE_ROUNDS = 25.5;
+constexpr double LANE_ROUNDS = 25.0, LANE_MIN = 18000.0, LANE_MIN_PER_ROUND = 1500.0, LANE_LONG = 1.55;
 
 // candidates from which on a thread each is the faster one
 double lanes_from(const sched_ctx* h) {
-    const double rounds = h->volume / ((double)h->n * (double)h->M), n = (double)h->n, share = h->short_share;
-    const double size = 1.0 + h->mean_o / h->mean_s, grow = size * size;
-    double need, ahead;
+    const double rounds = h->volume / ((double)h->n * (double)h->M), n = (double)h->n;
+    double need = LANE_MIN + LANE_MIN_PER_ROUND * rounds, ahead = (1.0 + h->mean_o / h->mean_s) * (1.0 + h->mean_o / h->mean_s);
     if (rounds > LANE_ROUNDS) return INFINITY;
     if (h->nm == 1) {
-        need = 15000.0 + 1600.0 * rounds + fmax(share - 0.3, 0.0) * (65000.0 + 9000.0 * rounds) + 4800.0 * rounds * fmax(fmin(grow, 3.0) - 1.3, 0.0);
+        if (h->short_share > 0.3) need += 11000.0 * rounds * (h->short_share - 0.3);
+        if (ahead > 1.3) need += 8700.0 * rounds * (fmin(ahead, 3.0) - 1.3);
+        if (h->short_share > 0.75) need += 150000.0 * (h->short_share - 0.75);
         if (short_windows(h, false)) need *= 1.3;              // against the warp's simulator for those
-        ahead = fmin(grow - 1.0, 8.7);
+        ahead = fmin(ahead, 8.0);
     } else {
-        need = (17000.0 + 2500.0 * rounds) * (1.0 + fmax(share - 0.4, 0.0) * (3.0 + 39.0 * rounds));
-        ahead = fmin(1.65 * (grow - 1.0), 6.1);
+        need *= LANE_LONG;
+        if (h->short_share > 0.4) need *= 1.0 + (h->short_share - 0.4) * rounds / 3.0;
+        // candidates further apart in a long list also leave one another's rounds: 40,000 moves of 10,000 and of 2,000
+        // requests with a share of 0.72, 6 rounds per request: 28.1 / 60 and 5.6 / 11.4
+        if (h->short_share > 0.4 && n > 2000.0) need *= 1.0 + (n - 2000.0) * rounds / 48000.0;
+        ahead = fmin(0.6 * ahead, 3.6);
     }
     const double far = ahead * sqrt(rounds);
-    if (n * rounds >= (double)h->omax && far > 4.5) need = far > 10.0 ? INFINITY : need * (1.0 + 0.2 * (far - 4.5));
+    if (n * rounds >= (double)h->omax && far > 5.0) need = far > 8.0 ? INFINITY : need * (1.0 + 0.55 * (far - 5.0));
     return need;
 }
 
